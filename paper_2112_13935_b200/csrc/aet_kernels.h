@@ -51,6 +51,8 @@ cudaError_t launch_wait_probe(uint32_t* status, uint32_t max_polls, cudaStream_t
 // how many round-tasks the launch holds.  Asynchronous on s; may start under the tail of the previous kernel in s
 // (programmatic stream serialisation) and waits on the device before reading that kernel's output.
 cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s);
+// at most one round-task per SM: a cluster of up to four CTAs per round-task (see lr_chain_kernel.cu)
+cudaError_t launch_lr_chain_rounds(const RoundLaunch& p, uint32_t sms, cudaStream_t s);
 // lambda = 0, more round-tasks than SMs: update sum in tensor memory, accumulated by tcgen05.mma (tf32 x 3)
 bool lr_tc_eligible(const RoundLaunch& p);
 cudaError_t launch_lr_tc_rounds(const RoundLaunch& p, cudaStream_t s);

@@ -743,44 +743,20 @@ cudaError_t launch_wait_probe(uint32_t* status, uint32_t max_polls, cudaStream_t
 
 cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s) {
   if (p.n_tasks == 0) return cudaSuccess;
-  if (p.l2 == 0.f) {
-    // more than 48 KB of shared memory has to be asked for once per device
-    static bool opted_in[64] = {};
-    static int sm_count[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+  static int sm_count[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const bool known = dev >= 0 && dev < 64;
+  int sms = known ? sm_count[dev] : 0;
+  if (!sms) {
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const bool known = dev >= 0 && dev < 64;
-    int sms = known ? sm_count[dev] : 0;
-    if (!known || !opted_in[dev]) {
-      e = cudaFuncSetAttribute(lr_block_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlkSmem));
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lr_block_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlkSmem));
-      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      if (e != cudaSuccess) return e;
-      if (known) { opted_in[dev] = true; sm_count[dev] = sms; }
-    }
-    // More round-tasks than SMs: the kernel that keeps the update sum in tensor memory.
-    if ((p.n_tasks > (uint32_t)sms || p.crowded_hint) && lr_tc_eligible(p)) return launch_lr_tc_rounds(p, s);
-    // At most one round-task per SM: the variant with a warp of its own for the softmax recurrence.
-    const bool dedicated = p.n_tasks <= (uint32_t)sms;
-    // Programmatic stream serialisation: the grid may start while the kernel before it in the
-    // stream (the aggregation of the previous wave) is still running; lr_block_kernel waits
-    // (griddepcontrol.wait) before it reads anything that kernel writes.
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(p.n_tasks, 1, 1);
-    cfg.blockDim = dim3(dedicated ? 2 * kThreads : kThreads, 1, 1);
-    cfg.dynamicSmemBytes = sizeof(BlkSmem);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return dedicated ? cudaLaunchKernelEx(&cfg, lr_block_kernel<true>, p) : cudaLaunchKernelEx(&cfg, lr_block_kernel<false>, p);
+    if (known) sm_count[dev] = sms;
   }
-  // lambda != 0 couples the steps of a block through the decay of W: step by step.
-  // Enough round-tasks to put two CTAs on every SM: trade latency for instruction count.
+  const bool crowded = p.n_tasks > (uint32_t)sms || p.crowded_hint;
+  if (!crowded) return launch_lr_chain_rounds(p, (uint32_t)sms, s);
+  if (lr_tc_eligible(p)) return launch_lr_tc_rounds(p, s);
   const bool shared = p.n_tasks >= 2 * 148;
   if (shared) lr_round_kernel<true, true><<<p.n_tasks, kThreads, 0, s>>>(p);
   else lr_round_kernel<true, false><<<p.n_tasks, kThreads, 0, s>>>(p);

@@ -1,0 +1,63 @@
+// Warp-level tensor-core products of fp32 operands for the round kernels: m16n8k8 tf32 instructions on split
+// operands, and the cluster-scope barrier wrappers the kernels that split one round-task over CTAs use.
+//
+// Why mma.sync here and not tcgen05: the contractions of a batch-1 regression block are 16 samples x 10 classes
+// (and 16 x 16 Gram matrices).  tcgen05 needs M >= 64, its operands in shared memory in both orientations and its
+// results fetched back from tensor memory; here the update sum's accumulator fragment IS the operand fragment of
+// the next logits product (see frag order below), so nothing moves between the two products of a block.
+// Measured on this part: m16n8k8 tf32 issues every 8 cycles per scheduler (512 multiply-adds per clock and SM),
+// 21 cycles latency.
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace aet {
+namespace mma {
+
+// Nearest tf32 of a finite fp32 (as fp32 bits) and the remainder: v = hi + lo exactly; the tensor cores read the
+// top 19 bits of lo.  hi.hi + hi.lo + lo.hi keeps every product to about 2^-22 of its size.
+struct Split { uint32_t hi, lo; };
+__device__ __forceinline__ Split split(float v) {
+  Split s;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(s.hi) : "f"(v));
+  s.lo = __float_as_uint(v - __uint_as_float(s.hi));
+  return s;
+}
+// d[16 x 8] += a[16 x 8] b[8 x 8]; lane = 4 g + t.  a0 (row g, k t), a1 (g + 8, t), a2 (g, t + 4), a3 (g + 8, t + 4);
+// b0 (k t, col g), b1 (t + 4, g); d0 (row g, col 2t), d1 (g, 2t + 1), d2 (g + 8, 2t), d3 (g + 8, 2t + 1).
+__device__ __forceinline__ void tf32(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// ---- cluster helpers -----------------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t peer_addr(uint32_t saddr, uint32_t rank) {   // shared::cluster address of a peer's copy
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+// 16 bytes into a peer's shared memory; they count towards the transaction bytes of a barrier there (no fence needed)
+__device__ __forceinline__ void send_peer(uint32_t addr, float4 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
+}
+__device__ __forceinline__ bool try_wait_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\t"
+               "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+               "selp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+}  // namespace mma
+}  // namespace aet
