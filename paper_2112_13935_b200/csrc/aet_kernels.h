@@ -53,6 +53,8 @@ cudaError_t launch_wait_probe(uint32_t* status, uint32_t max_polls, cudaStream_t
 cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s);
 // at most one round-task per SM: a cluster of up to four CTAs per round-task (see lr_chain_kernel.cu)
 cudaError_t launch_lr_chain_rounds(const RoundLaunch& p, uint32_t sms, cudaStream_t s);
+// one CTA per round-task; crowded: two CTAs per SM (see lr_block_kernel.cu)
+cudaError_t launch_lr_block_rounds(const RoundLaunch& p, bool crowded, cudaStream_t s);
 // lambda = 0, more round-tasks than SMs: update sum in tensor memory, accumulated by tcgen05.mma (tf32 x 3)
 bool lr_tc_eligible(const RoundLaunch& p);
 cudaError_t launch_lr_tc_rounds(const RoundLaunch& p, cudaStream_t s);

@@ -463,19 +463,27 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
 
     // block kb's logits follow the update by block kb - 2: everything R needs is one block ahead of it
     for (uint32_t kb = 0; kb < nblk + 2; ++kb) {
-      if (kb >= 2) {
-        // ---- U^T = q^nv U^T + sum_s q^(nv-1-s) delta_s x_s ----
-        const uint32_t k = kb - 2, nv = min((uint32_t)kB, n - k * kB);
-        // the block's inputs as the second operand: [sample][pixel], pixel g of the warp's k-steps
-        const float* xb = &sm.rows[k % NS][tt][8 * warp + g];
-        constexpr bool kEarly = KM <= 4;   // room to split the inputs ahead of the wait
-        Split x[kEarly ? KM : 1][4];
-        if (kEarly) {
+      const bool update = kb >= 2, look = kb < nblk;
+      const uint32_t k = update ? kb - 2 : 0, nv = min((uint32_t)kB, n - k * kB);
+      // What does not depend on the deltas comes before the wait for them: the rows of block k as the update's second
+      // operand ([sample][pixel], pixel g of the warp's k-steps), split, and those of block kb.
+      const float* xb = &sm.rows[k % NS][tt][8 * warp + g];
+      const float* xr = &sm.rows[kb % NS][g][8 * warp + 2 * tt];
+      constexpr bool kEarly = KM <= 4;   // room for them in registers
+      Split x[kEarly ? KM : 1][4];
+      float2 r0[kEarly ? KM : 1], r1[kEarly ? KM : 1];
+      if (look) wait(&sm.full[kb % NS], (kb / NS) & 1);
+      if (kEarly) {
 #pragma unroll
-          for (int j = 0; j < (kEarly ? KM : 1); ++j)
+        for (int j = 0; j < (kEarly ? KM : 1); ++j) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) x[j][i] = split(xb[4 * i * S::kPitch + 8 * NM * j]);
+          for (int i = 0; i < 4; ++i) x[j][i] = split(xb[4 * i * S::kPitch + 8 * NM * j]);
+          r0[j] = *reinterpret_cast<const float2*>(xr + 8 * NM * j);
+          r1[j] = *reinterpret_cast<const float2*>(xr + 8 * S::kPitch + 8 * NM * j);
         }
+      }
+      if (update) {
+        // ---- U^T = q^nv U^T + sum_s q^(nv-1-s) delta_s x_s ----
         wait(&sm.delta[k & 1], (k >> 1) & 1);
         Split a[2][4];
         {
@@ -487,7 +495,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
             for (int i = 0; i < 2; ++i) {
               const int s = 8 * m + tt + 4 * i;
               float v0 = sm.dbuf[k & 1][s][col], v1 = two ? sm.dbuf[k & 1][s][g + 11] : 0.f;
-              s0 += v0; s1 += v1;
+              if (biases) { s0 += v0; s1 += v1; }
               if (decay) {
                 const float f = (uint32_t)s < nv ? sm.qp[nv - 1 - s] : 0.f;
                 v0 *= f; v1 *= f;
@@ -500,9 +508,12 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
             ub0 += s0 + shx(s0, 2); ub1 += s1 + shx(s1, 2);
           }
         }
-        float qn = 1.f;
-        if (decay) {
-          qn = sm.qp[nv];
+        if (decay) {   // U decays with the block, and with it the share of the start model
+          const float qn = sm.qp[nv];
+#pragma unroll
+          for (int j = 0; j < KM; ++j)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) U[j][c] *= qn;
           const double qd = 1.0 - (double)eta * (double)p.l2;
 #pragma unroll 1
           for (uint32_t i = 0; i < nv; ++i) qwd *= qd;
@@ -523,22 +534,21 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
           mma::tf32(d[j], a[0][0].hi, a[0][1].hi, a[0][2].hi, a[0][3].hi, v[0].hi, v[1].hi);
           mma::tf32(d[j], a[1][0].hi, a[1][1].hi, a[1][2].hi, a[1][3].hi, v[2].hi, v[3].hi);
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.freed[k % NS]);
 #pragma unroll
         for (int j = 0; j < KM; ++j)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) U[j][c] = fmaf(U[j][c], qn, d[j][c]);
+          for (int c = 0; c < 4; ++c) U[j][c] += d[j][c];
       }
-      if (kb < nblk) {
+      if (look) {
         // ---- logits of block kb with the model W = qw W_start - eta U ----
-        wait(&sm.full[kb % NS], (kb / NS) & 1);
-        const float* xr = &sm.rows[kb % NS][g][8 * warp + 2 * tt];
         float zm[2][4] = {}, zx[2][4] = {};
 #pragma unroll
         for (int j = 0; j < KM; ++j) {
-          const float2 x0 = *reinterpret_cast<const float2*>(xr + 8 * NM * j);
-          const float2 x1 = *reinterpret_cast<const float2*>(xr + 8 * S::kPitch + 8 * NM * j);
+          if (!kEarly) {
+            r0[0] = *reinterpret_cast<const float2*>(xr + 8 * NM * j);
+            r1[0] = *reinterpret_cast<const float2*>(xr + 8 * S::kPitch + 8 * NM * j);
+          }
+          const float2 x0 = r0[kEarly ? j : 0], x1 = r1[kEarly ? j : 0];
           const Split a = split(x0.x), b = split(x0.y), c = split(x1.x), d = split(x1.y);
           const Split w0 = split(fmaf(neta, U[j][0], qw * ws[j][0])), w2 = split(fmaf(neta, U[j][1], qw * ws[j][1]));
           const Split w1 = split(fmaf(neta, U[j][2], qw * ws[j][2])), w3 = split(fmaf(neta, U[j][3], qw * ws[j][3]));
@@ -584,6 +594,10 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
             if (lane == 0) mbar_arrive(&sm.bz[iz]);
           }
         }
+      }
+      if (update) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.freed[k % NS]);
       }
     }
 

@@ -755,12 +755,9 @@ cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s) {
     if (known) sm_count[dev] = sms;
   }
   const bool crowded = p.n_tasks > (uint32_t)sms || p.crowded_hint;
-  if (!crowded) return launch_lr_chain_rounds(p, (uint32_t)sms, s);
-  if (lr_tc_eligible(p)) return launch_lr_tc_rounds(p, s);
-  const bool shared = p.n_tasks >= 2 * 148;
-  if (shared) lr_round_kernel<true, true><<<p.n_tasks, kThreads, 0, s>>>(p);
-  else lr_round_kernel<true, false><<<p.n_tasks, kThreads, 0, s>>>(p);
-  return cudaGetLastError();
+  if (crowded) return launch_lr_block_rounds(p, true, s);
+  if (p.n_tasks * 2 > (uint32_t)(sms - sms / 16)) return launch_lr_block_rounds(p, false, s);
+  return launch_lr_chain_rounds(p, (uint32_t)sms, s);
 }
 
 }  // namespace aet
