@@ -275,16 +275,17 @@ const char* aet_last_error(const aet_handle* h);
  * `client` (Algorithm 3, MainComputeNode) from the model w_in, writing the update
  * sum U_out and the end-of-round model w_out.  x [n, dims[0]] fp32, y [n] int32,
  * w_in, U_out, w_out (n_params floats each) are DEVICE pointers owned by the
- * caller.  The entry point always runs the library's generic fp32 round kernel
- * (any layer widths; not the shape-specialised kernels a handle may pick), so
- * its results agree with aet_debug_run_client_round within fp32 rounding order,
- * not bit for bit.  The kernel's scratch (descriptors, the working model, activations)
+ * caller.  Softmax regression 784 -> 10 with batch 1 and 16-byte aligned x, U_out
+ * and w_out runs the kernel a handle with few clients runs; everything else the
+ * library's generic fp32 round kernel (any layer widths; not the shape-specialised
+ * kernels a handle may pick), so results agree with aet_debug_run_client_round
+ * within fp32 rounding order, not bit for bit.  The kernel's scratch (descriptors, the working model, activations)
  * is a fixed array inside the library image: every GPU that loads the library
  * holds about 1 MB for it until the process exits.  Limits: precision 0, at most
  * 131,072 parameters and 131,072 floats of activation scratch (about
  * 10 x batch x sum of layer widths); larger requests return AET_ERR_CONFIG
  * with the sizes in aet_last_error(NULL).  The call is asynchronous on
- * `cuda_stream`, launches two kernels and calls neither cudaMalloc nor
+ * `cuda_stream`, launches at most two kernels and calls neither cudaMalloc nor
  * cudaFree.  Its first call on a device looks the array's device address up
  * (cudaGetSymbolAddress); make that first call outside any stream capture.
  * All calls share the one array and what the last call left in it (the entry

@@ -5,9 +5,11 @@
 #include <string.h>
 
 #include <chrono>
+#include <mutex>
 #include <new>
 #include <string>
 #include <thread>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/aet.h"
@@ -21,19 +23,83 @@ namespace {
 
 thread_local std::string g_create_error;
 
+// Device memory of destroyed handles, kept for the next one: cudaMalloc and cudaFree of a handle's dozen arrays cost a
+// short job (create, load, run, destroy) more than its run - milliseconds, at times tens of them.  Bounded per process,
+// given back to the driver whenever an allocation fails or the bound is reached; blocks come back only after the device
+// has been synchronised, so any stream may use them next.
+class DevicePool {
+ public:
+  void* get(size_t bytes) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    bytes = (bytes + 511) & ~(size_t)511;
+    std::lock_guard<std::mutex> lock(mu_);
+    size_t best = free_.size();
+    for (size_t i = 0; i < free_.size(); ++i)   // smallest block that fits without wasting more than itself
+      if (free_[i].dev == dev && free_[i].bytes >= bytes && free_[i].bytes <= 2 * bytes + 65536 &&
+          (best == free_.size() || free_[i].bytes < free_[best].bytes)) best = i;
+    if (best < free_.size()) {
+      const Block b = free_[best];
+      free_[best] = free_.back();
+      free_.pop_back();
+      held_ -= b.bytes;
+      live_[b.p] = b;
+      return b.p;
+    }
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      flush();
+      if (cudaMalloc(&p, bytes) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    }
+    live_[p] = Block{p, bytes, dev};
+    return p;
+  }
+  // The caller has synchronised the device since the block's last use.
+  void put(void* p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> lock(mu_);
+    auto it = live_.find(p);
+    if (it == live_.end()) return;
+    const Block b = it->second;
+    live_.erase(it);
+    if (held_ + b.bytes > kMost || free_.size() >= kMostBlocks) { cudaFree(p); return; }
+    held_ += b.bytes;
+    free_.push_back(b);
+  }
+
+ private:
+  struct Block { void* p; size_t bytes; int dev; };
+  static constexpr size_t kMost = 512ull << 20, kMostBlocks = 128;
+  void flush() {
+    for (const Block& b : free_) cudaFree(b.p);
+    free_.clear();
+    held_ = 0;
+  }
+  std::mutex mu_;
+  std::vector<Block> free_;
+  std::unordered_map<void*, Block> live_;
+  size_t held_ = 0;
+};
+DevicePool& pool() {
+  static DevicePool* p = new DevicePool;   // outlives every handle; the driver takes its blocks back with the process
+  return *p;
+}
+
 // Bump allocator over a few large device chunks: client data sets are many
 // small allocations of unknown count, and cudaMalloc per client is slow.
 struct Arena {
   std::vector<void*> chunks;
   char* cur = nullptr;
   size_t left = 0;
-  static constexpr size_t kChunk = 256ull << 20;
+  size_t next = 8ull << 20;   // chunks double from 8 MB to 256 MB: a small job takes a small one
   void* alloc(size_t bytes) {
     bytes = (bytes + 255) & ~(size_t)255;
     if (bytes > left) {
-      size_t want = bytes > kChunk ? bytes : kChunk;
-      void* p = nullptr;
-      if (cudaMalloc(&p, want) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+      size_t want = bytes > next ? bytes : next;
+      if (next < (256ull << 20)) next *= 2;
+      void* p = pool().get(want);
+      if (!p) return nullptr;
       chunks.push_back(p);
       cur = (char*)p;
       left = want;
@@ -44,7 +110,7 @@ struct Arena {
     return r;
   }
   void release() {
-    for (void* p : chunks) cudaFree(p);
+    for (void* p : chunks) pool().put(p);
     chunks.clear();
     cur = nullptr;
     left = 0;
@@ -57,14 +123,13 @@ struct DevBuf {  // grow-only device array
   size_t cap = 0;
   bool reserve(size_t n) {
     if (n <= cap) return true;
-    if (p) cudaFree(p);
-    p = nullptr;
-    cap = 0;
-    if (cudaMalloc((void**)&p, n * sizeof(T)) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (p) { cudaDeviceSynchronize(); release(); }   // an earlier launch may still use the old array
+    p = static_cast<T*>(pool().get(n * sizeof(T)));
+    if (!p) return false;
     cap = n;
     return true;
   }
-  void release() { if (p) cudaFree(p); p = nullptr; cap = 0; }
+  void release() { pool().put(p); p = nullptr; cap = 0; }
 };
 
 struct CachedRingPlan {
@@ -92,6 +157,7 @@ void set_thread_error(const std::string& msg) { g_create_error = msg; }
 
 struct aet_handle {
   aet_config cfg{};
+  int device = 0;
   std::vector<uint32_t> shares;   // copy of cfg.client_shares (cfg.client_shares points here)
   uint32_t P = 0;
   size_t stride = 0;
@@ -131,8 +197,8 @@ struct aet_handle {
   float* w_cur() { return w_buf[w_sel].p; }
   DevBuf<uint32_t> d_status;
   DevBuf<TaskDesc> d_tasks;
-  DevBuf<InflightRef> d_inflight;
-  DevBuf<ApplyDesc> d_applies;
+  DevBuf<char> d_plan;            // topology 0: the plan's tasks, sums in flight and updates
+  std::vector<char> pack;         // the same on the host, for the copy
   DevBuf<TriggerRec> d_trig;
   DevBuf<ApplyRec> d_alog;
   bool clients_dirty = true, have_w0 = false;
@@ -290,13 +356,12 @@ aet_status run_ring_rounds(aet_handle* h, uint32_t n_rounds, cudaStream_t s) {
             h->d_ring_applies.reserve(plan.applies.size() + 1) && h->d_ring_ops.reserve(plan.ops.size() + 1);
   if (ok && !h->lr_fast) ok = h->act.reserve((size_t)plan.max_wave_tasks * h->act_floats());
   if (!ok) return fail(h, AET_ERR_NOMEM, "device allocation failed");
-  if (!cp.uploaded) {
+  if (!cp.uploaded) {   // (a copy from pageable memory has read its source when it returns: no need to wait)
     AET_CUDA(h, cudaMemcpyAsync(h->d_tasks.p, plan.tasks.data(), T * sizeof(TaskDesc), cudaMemcpyHostToDevice, s));
     if (!plan.applies.empty())
       AET_CUDA(h, cudaMemcpyAsync(h->d_ring_applies.p, plan.applies.data(), plan.applies.size() * sizeof(RingApplyDesc), cudaMemcpyHostToDevice, s));
     if (!plan.ops.empty())
       AET_CUDA(h, cudaMemcpyAsync(h->d_ring_ops.p, plan.ops.data(), plan.ops.size() * sizeof(RingOp), cudaMemcpyHostToDevice, s));
-    AET_CUDA(h, cudaStreamSynchronize(s));
     cp.uploaded = true;
   }
   AET_CUDA(h, cudaMemsetAsync(h->d_trig.p, 0, T * sizeof(TriggerRec), s));
@@ -367,6 +432,7 @@ aet_status aet_create(const aet_config* cfg, aet_handle** out) {
   aet_handle* h = new (std::nothrow) aet_handle();
   if (!h) return fail(nullptr, AET_ERR_NOMEM, "out of host memory");
   h->cfg = *cfg;
+  h->device = dev;
   if (cfg->client_shares) {
     h->shares.assign(cfg->client_shares, cfg->client_shares + cfg->n_clients);
     h->cfg.client_shares = h->shares.data();
@@ -412,7 +478,10 @@ aet_status aet_create(const aet_config* cfg, aet_handle** out) {
 aet_status aet_destroy(aet_handle* h) {
   if (!h) return AET_ERR_ARG;
   join_prepare(h);
-  cudaDeviceSynchronize();
+  int before = h->device;
+  cudaGetDevice(&before);
+  if (before != h->device) cudaSetDevice(h->device);
+  cudaDeviceSynchronize();   // nothing uses the handle's memory any more when it goes back to the pool
   collect_timings(h);
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
   h->arena.release();
@@ -420,9 +489,10 @@ aet_status aet_destroy(aet_handle* h) {
   h->w_buf[0].release(); h->w_buf[1].release(); h->totals.release(); h->d_status.release(); h->w0.release(); h->snaps.release(); h->U.release();
   h->work.release(); h->act.release(); h->dbg.release();
   h->node_w.release(); h->d_ring_applies.release(); h->d_ring_ops.release();
-  h->d_tasks.release(); h->d_inflight.release(); h->d_applies.release();
+  h->d_tasks.release(); h->d_plan.release();
   h->d_trig.release(); h->d_alog.release();
   cudaGetLastError();
+  if (before != h->device) cudaSetDevice(before);
   delete h;
   return AET_OK;
 }
@@ -566,17 +636,22 @@ aet_status aet_run_rounds(aet_handle* h, uint32_t n_rounds, void* cuda_stream) {
   // ---- device buffers ----
   aet_status st_up = upload_clients(h, s);
   if (st_up != AET_OK) return st_up;
+  // tasks, sums in flight and updates side by side: one copy
+  const size_t off_in = E * sizeof(TaskDesc), off_ap = off_in + plan.inflight.size() * sizeof(InflightRef);
+  const size_t plan_bytes = off_ap + E * sizeof(ApplyDesc);
   bool ok = h->snaps.reserve((size_t)plan.n_snap * h->stride) && h->U.reserve((size_t)plan.n_u_rows * h->stride) &&
-            h->d_tasks.reserve(E) && h->d_inflight.reserve(plan.inflight.size() + 1) &&
-            h->d_applies.reserve(E) && h->d_trig.reserve(E) && h->d_alog.reserve(E);
+            h->d_plan.reserve(plan_bytes) &&
+            h->d_trig.reserve(E) && h->d_alog.reserve(E);
   if (ok && !h->lr_fast) ok = h->act.reserve((size_t)plan.max_wave_tasks * h->act_floats());
   if (!ok) return fail(h, AET_ERR_NOMEM, "device allocation failed");
   if (!cp.uploaded) {
-    AET_CUDA(h, cudaMemcpyAsync(h->d_tasks.p, plan.tasks.data(), E * sizeof(TaskDesc), cudaMemcpyHostToDevice, s));
-    if (!plan.inflight.empty())
-      AET_CUDA(h, cudaMemcpyAsync(h->d_inflight.p, plan.inflight.data(), plan.inflight.size() * sizeof(InflightRef), cudaMemcpyHostToDevice, s));
-    AET_CUDA(h, cudaMemcpyAsync(h->d_applies.p, plan.applies.data(), E * sizeof(ApplyDesc), cudaMemcpyHostToDevice, s));
-    AET_CUDA(h, cudaStreamSynchronize(s));
+    std::vector<char>& pack = h->pack;
+    pack.resize(plan_bytes);
+    memcpy(pack.data(), plan.tasks.data(), off_in);
+    if (off_ap > off_in) memcpy(pack.data() + off_in, plan.inflight.data(), off_ap - off_in);
+    memcpy(pack.data() + off_ap, plan.applies.data(), plan_bytes - off_ap);
+    // (a copy from pageable memory has read its source when it returns: no need to wait)
+    AET_CUDA(h, cudaMemcpyAsync(h->d_plan.p, pack.data(), plan_bytes, cudaMemcpyHostToDevice, s));
     cp.uploaded = true;
   }
   AET_CUDA(h, cudaMemsetAsync(h->d_trig.p, 0, E * sizeof(TriggerRec), s));
@@ -584,14 +659,15 @@ aet_status aet_run_rounds(aet_handle* h, uint32_t n_rounds, void* cuda_stream) {
   AET_CUDA(h, cudaMemcpyAsync(h->snaps.p, h->w_cur(), h->stride * sizeof(float), cudaMemcpyDeviceToDevice, s));
 
   RoundLaunch r{};
-  r.tasks = h->d_tasks.p; r.inflight = h->d_inflight.p; r.clients = h->d_clients.p;
+  r.tasks = reinterpret_cast<const TaskDesc*>(h->d_plan.p);
+  r.inflight = reinterpret_cast<const InflightRef*>(h->d_plan.p + off_in); r.clients = h->d_clients.p;
   r.sample_keys = h->d_keys.p; r.snaps = h->snaps.p; r.U = h->U.p; r.w_end = nullptr;
   r.trig = h->d_trig.p; r.status = h->d_status.p; r.stride = h->stride; r.l2 = h->cfg.l2;
   r.debug_checks = (h->cfg.flags & AET_FLAG_DEBUG_CHECKS) ? 1u : 0u;
   r.step_by_step = (h->cfg.flags & AET_FLAG_STEPWISE_RECURRENCE) ? 1u : 0u;
   r.n_u_rows = plan.n_u_rows; r.n_snap = plan.n_snap;
   ApplyLaunch a{};
-  a.applies = h->d_applies.p; a.U = h->U.p; a.snaps = h->snaps.p; a.totals = h->totals.p;
+  a.applies = reinterpret_cast<const ApplyDesc*>(h->d_plan.p + off_ap); a.U = h->U.p; a.snaps = h->snaps.p; a.totals = h->totals.p;
   a.H = h->d_H.p; a.log = h->d_alog.p; a.status = h->d_status.p; a.stride = h->stride; a.n_params = h->P;
 
   // ---- waves: a3/a4 local SGD of independent round-tasks, then a6 aggregation ----

@@ -40,6 +40,12 @@ struct RoundLaunch {
   uint32_t n_u_rows, n_snap;     // extents of U and snaps (for the debug checks)
   uint32_t crowded_hint;         // non-zero: pick the kernel a full wave of this run's clients would get,
                                  // however few tasks this launch holds (single-task parity runs)
+  // One round-task with its descriptors in the launch itself (n_tasks 1, no sums in flight; lr_chain_kernel only):
+  // nothing has to be in device memory beforehand.
+  uint32_t by_value;
+  TaskDesc one_task;
+  ClientData one_client;
+  uint64_t one_key;
   uint32_t step_by_step;         // non-zero: the recurrence of a block is always walked step by step
   float l2;
 };

@@ -7,6 +7,7 @@
 // golden-ratio-spaced inputs.  Delays are integer ticks computed without
 // floating point, so the event order is identical on every machine.
 #pragma once
+#include <math.h>
 #include <stdint.h>
 
 #if defined(__CUDACC__)
@@ -45,10 +46,18 @@ AET_HD uint32_t sample_index(uint64_t r, uint32_t n) {
 // Host only (the delay model is part of the host scheduler).
 // -log2(x / 2^64) in Q32, x = r (1 when r == 0): integer part from the leading
 // bit, 32 fraction bits by squaring the Q1.63 mantissa and watching for >= 2.
+//
+// The squaring truncates, so its 32 bits are floor(2^32 (log2 m - d)) with 0 <= d < 2^-61.  A double-precision log2 is
+// within 2^-50 of log2 m, so the same bits follow from it unless 2^32 log2 m lies within 2^-17 of an integer (one draw
+// in 2^16), where the squaring decides.  (About 10 ns instead of 60 ns; the delay draws were most of a first run.)
 inline uint64_t neg_log2_q32(uint64_t r) {
   uint64_t x = r ? r : 1;
   int e = 63 - __builtin_clzll(x);
   uint64_t m = x << (63 - e);
+  {
+    const double y = log2((double)m * 0x1p-63) * 0x1p32, whole = floor(y), part = y - whole;
+    if (part > 0x1p-17 && part < 1.0 - 0x1p-17) return ((uint64_t)(64 - e) << 32) - (uint64_t)whole;
+  }
   uint64_t f = 0;
   for (int it = 0; it < 32; ++it) {
     unsigned __int128 p = (unsigned __int128)m * m;

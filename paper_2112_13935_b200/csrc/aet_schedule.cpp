@@ -157,8 +157,12 @@ void fill_delays(const aet_config& c, uint32_t first, uint32_t last, DelayCache&
       net.push_back(dm.network(draw(kn, round)));
     }
   };
-  unsigned hw = std::thread::hardware_concurrency();
-  unsigned nt = std::max(1u, std::min({hw ? hw : 1u, n, 32u}));
+  // A draw takes some 15 ns and a thread some 20 us to start: threads only for long fills.
+  uint64_t draws = 0;
+  for (uint32_t rel = cache.busy[0].size(); rel < need; ++rel) draws += sample_size(c, c.round_base + rel) / c.batch;
+  if (!c.split_mode) draws *= n;
+  const unsigned hw = std::thread::hardware_concurrency();
+  const unsigned nt = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>({hw ? hw : 1u, n, 32u, draws / 8192}));
   if (nt == 1) { for (uint32_t cl = 0; cl < n; ++cl) work(cl); return; }
   std::vector<std::thread> pool;
   for (unsigned t = 0; t < nt; ++t)
@@ -200,31 +204,50 @@ bool simulate(const aet_config& c, uint32_t n_rounds, SchedState& st, DelayCache
   const bool never_wait = c.max_lag_d == AET_NEVER_WAIT;
   uint32_t seq = 0, n_blocked = 0;
 
+  // How many clients stand at each history count, the smallest count and how many stand there: the minimum over the
+  // others in constant time per event (a scan over the clients per event was most of the schedule of 1,024 clients).
+  std::vector<uint32_t> standing;
+  uint32_t m1 = *std::min_element(H.begin(), H.end()), m2 = 0;
+  const uint32_t h0 = m1;
+  auto stand = [&](uint32_t h) -> uint32_t& {
+    if (h - h0 >= standing.size()) standing.resize(h - h0 + 1, 0);
+    return standing[h - h0];
+  };
+  for (uint32_t e = 0; e < n; ++e) stand(H[e]) += 1;
+  // min over e != cl of H_e: m1 unless cl alone stands there, then the next occupied count (UINT32_MAX: nobody else)
+  auto second = [&]() -> uint32_t {
+    for (size_t h = m1 - h0 + 1; h < standing.size(); ++h) if (standing[h]) return h0 + (uint32_t)h;
+    return UINT32_MAX;
+  };
   auto lag_of = [&](uint32_t cl, uint32_t round) -> uint32_t {
     if (n == 1) return 0;
-    uint32_t m = UINT32_MAX;
-    for (uint32_t e = 0; e < n; ++e) if (e != cl && H[e] < m) m = H[e];
-    uint32_t rel = round - c.round_base;
+    const uint32_t m = H[cl] == m1 && standing[m1 - h0] == 1 ? second() : m1;
+    const uint32_t rel = round - c.round_base;
     return rel > m ? rel - m : 0;
   };
+  bool alone = standing[0] == 1;
+  m2 = alone ? second() : 0;
 
   while (!q.empty()) {
     QItem it = q.top();
     q.pop();
     if (it.kind == kApply) {
+      stand(H[it.client]) -= 1;
       H[it.client] += 1;
+      stand(H[it.client]) += 1;
+      bool moved = false;   // can a blocked client's lag have changed?
+      while (!standing[m1 - h0]) { ++m1; moved = true; }
+      {
+        const bool a = standing[m1 - h0] == 1;
+        const uint32_t s = a ? second() : 0;
+        moved |= a != alone || s != m2;
+        alone = a; m2 = s;
+      }
       out.events[ev_of[(size_t)it.client * n_rounds + (it.round - first)]].seq = seq++;
-      if (n_blocked) {
-        // min and second min of H once, then an O(1) test per blocked client
-        uint32_t m1 = UINT32_MAX, m2 = UINT32_MAX, c1 = 0;
-        for (uint32_t e = 0; e < n; ++e) {
-          if (H[e] < m1) { m2 = m1; m1 = H[e]; c1 = 1; }
-          else if (H[e] == m1) { ++c1; }
-          else if (H[e] < m2) { m2 = H[e]; }
-        }
+      if (n_blocked && moved) {
         for (uint32_t b = 0; b < n; ++b) {
           if (blocked[b] < 0) continue;
-          uint32_t mo = (H[b] == m1 && c1 == 1) ? m2 : m1;
+          uint32_t mo = H[b] == m1 && alone ? m2 : m1;
           uint32_t rel = (uint32_t)blocked[b] - c.round_base;
           uint32_t lag = rel > mo ? rel - mo : 0;
           if (never_wait || lag <= c.max_lag_d) {

@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   typename S::Smem& sm = *reinterpret_cast<typename S::Smem*>(smem_raw);
 
-  const TaskDesc t = p.tasks[p.task_begin + blockIdx.x / CL];
+  const TaskDesc t = p.by_value ? p.one_task : p.tasks[p.task_begin + blockIdx.x / CL];
   if (!debug_task_ok(p, t)) return;
   const uint32_t rank = CL > 1 ? mma::cluster_rank() : 0;
   if (t.n_samples == 0) {
@@ -268,8 +268,8 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
     }
   } else if (role == kProd) {
     // ================= producer: rows and labels =================
-    const ClientData cd = p.clients[t.client];
-    const uint64_t key = p.sample_keys[t.client];
+    const ClientData cd = p.by_value ? p.one_client : p.clients[t.client];
+    const uint64_t key = p.by_value ? p.one_key : p.sample_keys[t.client];
     const float* xrows = reinterpret_cast<const float*>(cd.x) + 8 * ks0;
     const uint32_t bytes = 32u * cnt;
     for (uint32_t kb = 0; kb < nblk; ++kb) {
@@ -603,8 +603,11 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
 
     // ---- event trigger: h reached s_{i,c}; publish U_i (and the end model) ----
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (ok) {
-      const float c1 = decay ? (float)((1.0 - qwd) / (double)eta) : 0.f;
+    {
+      // a round whose copies never came leaves NaN behind, for callers that have no status word to look at
+      const float bad = ok ? 0.f : __int_as_float(0x7FFFFFFF);
+      const float c1 = (decay ? (float)((1.0 - qwd) / (double)eta) : 0.f) + bad;
+      qw += bad;
 #pragma unroll 1
       for (int pass = 0; pass < (p.w_end ? 2 : 1); ++pass) {
         float* row = (pass == 0 ? p.U : p.w_end) + (size_t)t.u_row * p.stride;
@@ -626,7 +629,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
         if (biases) {
           if (tt == 0) row[kD * kC + g] = fmaf(fu, ub0, pass == 0 ? 0.f : b0);
           if (tt == 0 && two) row[kD * kC + 8 + g] = fmaf(fu, ub1, pass == 0 ? 0.f : b1);
-          if (lane < kStageFloats - kParams) row[kParams + lane] = 0.f;   // the row's padding
+          if (p.stride && lane < kStageFloats - kParams) row[kParams + lane] = 0.f;   // the row's padding
         }
       }
     }
