@@ -92,12 +92,12 @@ struct Arena {
   std::vector<void*> chunks;
   char* cur = nullptr;
   size_t left = 0;
-  size_t next = 8ull << 20;   // chunks double from 8 MB to 256 MB: a small job takes a small one
+  size_t next = 8ull << 20;   // chunks grow from 8 MB to 256 MB: a small job takes a small one
   void* alloc(size_t bytes) {
     bytes = (bytes + 255) & ~(size_t)255;
     if (bytes > left) {
       size_t want = bytes > next ? bytes : next;
-      if (next < (256ull << 20)) next *= 2;
+      if (next < (256ull << 20)) next = next * 4 < (256ull << 20) ? next * 4 : 256ull << 20;
       void* p = pool().get(want);
       if (!p) return nullptr;
       chunks.push_back(p);
@@ -186,6 +186,7 @@ struct aet_handle {
 
   Arena arena;
   std::vector<ClientData> h_clients;
+  std::vector<uint64_t> keys;
   DevBuf<ClientData> d_clients;
   DevBuf<uint64_t> d_keys;
   DevBuf<uint32_t> d_H;
@@ -271,11 +272,11 @@ aet_status upload_clients(aet_handle* h, cudaStream_t s) {
   if (!h->clients_dirty) return AET_OK;
   const uint32_t n = h->cfg.n_clients;
   if (!h->d_clients.reserve(n) || !h->d_keys.reserve(n)) return fail(h, AET_ERR_NOMEM, "device allocation failed");
-  std::vector<uint64_t> keys(n);
+  std::vector<uint64_t>& keys = h->keys;
+  keys.resize(n);
   for (uint32_t c = 0; c < n; ++c) keys[c] = stream_key(h->cfg.seed, kStreamSample, c);
   AET_CUDA(h, cudaMemcpyAsync(h->d_clients.p, h->h_clients.data(), n * sizeof(ClientData), cudaMemcpyHostToDevice, s));
   AET_CUDA(h, cudaMemcpyAsync(h->d_keys.p, keys.data(), n * sizeof(uint64_t), cudaMemcpyHostToDevice, s));
-  AET_CUDA(h, cudaStreamSynchronize(s));  // the host vectors above go out of scope
   h->clients_dirty = false;
   return AET_OK;
 }

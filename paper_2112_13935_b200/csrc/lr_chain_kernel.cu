@@ -48,6 +48,7 @@ namespace {
 using namespace lr;
 using mma::Split;
 using mma::split;
+using mma::split_t;
 
 constexpr int kB = 16;                       // samples per block
 constexpr int kSteps8 = kD / 8;              // 98 k-steps of 8 inputs
@@ -58,6 +59,7 @@ constexpr int kOffC = kB * kGp;
 constexpr int kQuadZ = kZ / 4;               // the logits as 16-byte pieces; a matrix has 64
 // bytes a CTA sends about a block: the own couplings' pieces that reach below the diagonal, and the others'
 constexpr uint32_t kSendG0 = 16 * 36, kSendG = kSendG0 + 16 * 64;
+constexpr int kDbuf = 2 * kB * kCh;
 constexpr float kTol = 2e-7f * kLog2e;       // logits are kept in units of log2
 
 // CL CTAs per round-task; per CTA NM model warps with KM k-steps each, NG Gram warps with KG each, NS blocks of rows.
@@ -73,10 +75,10 @@ struct Shape {
   // Rings of what CTAs send one another.  A CTA that has the deltas of block k knows that its peers have taken what
   // belongs to block k - 2; it may itself be sending logits of block k + 2 and couplings of block k + NS.
   static constexpr int kInZ = CL > 1 ? 4 : 2, kInG = CL > 1 ? NS + 2 : NS;
-  static constexpr int kWarps = QUIET ? 16 : NM + NG + (CL > 1 ? 3 : 2);
+  static constexpr int kWarps = QUIET ? (NM + NG + 2) / 3 * 4 : NM + NG + (CL > 1 ? 3 : 2);
   static constexpr int kThreads = kWarps * 32;
   static constexpr bool kCarry = KG <= 7;   // Gram warps keep the split rows of the block before in registers
-  static_assert(!QUIET || NM + NG == 12, "three schedulers for the products");
+  static_assert(!QUIET || (NM + NG > 6 && NM + NG <= 12), "three schedulers for the products, the fourth for the rest");
   static_assert(NM >= 2 && NG >= 4, "one 16-byte piece per thread");
   static_assert(NM * KM >= kMost && NG * KG >= kMost, "every k-step has a warp");
   struct __align__(128) Smem {
@@ -86,7 +88,8 @@ struct Shape {
     float zin[kInZ][CL][kZ];        // per CTA of the cluster
     float gin[kInG][CL][kCoup];
     float coup[CL > 1 ? 2 : 1][CL > 1 ? kCoup : 4];   // summed over the cluster
-    float dbuf[2][kB][16];          // delta[s][class]: class c at c (c < 5) or c + 3
+    float zsum[CL > 1 ? 2 : 1][CL > 1 ? kZ : 4];
+    float dbuf[2][2][kB * kCh];     // deltas by parity of the block and class half: [sample][five classes]
     uint32_t amax[kInG][16];        // largest coupling, as bits: per Gram warp (one CTA), or [0] (cluster)
     float qp[32];                   // powers of q
     int ys[8][kB];
@@ -117,12 +120,12 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
   {
     const int w = threadIdx.x >> 5;
     int id;         // products first, then the others
-    if (S::kQuiet) id = (w & 3) == 3 ? NM + NG + (w >> 2) : (w >> 2) * 3 + (w & 3);
+    if (S::kQuiet) id = (w & 3) == 3 ? NM + NG + (w >> 2) : (w >> 2) * 3 + (w & 3) < NM + NG ? (w >> 2) * 3 + (w & 3) : NM + NG + 3;
     else id = w;
     if (id < NM) { role = kModel; warp = id; }
     else if (id < NM + NG) { role = kGram; warp = id - NM; }
-    else { role = kRec + (id - NM - NG); warp = 0; }
-    if (CL == 1 && role >= kSum) role = kIdle;
+    else { role = min(kRec + (id - NM - NG), (int)kIdle); warp = 0; }
+    if (CL == 1 && role == kSum) role = kIdle;
   }
   const uint32_t n = t.n_samples, nblk = (n + kB - 1) / kB;
   const float eta = t.eta, neta = -t.eta;
@@ -140,7 +143,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
     double q = 1.0 - (double)eta * (double)p.l2, v = 1.0;
     for (int i = 0; i < 32; ++i) { sm.qp[i] = (float)v; v *= q; }
   }
-  for (int i = threadIdx.x; i < 2 * kB * 16; i += S::kThreads) (&sm.dbuf[0][0][0])[i] = 0.f;
+  for (int i = threadIdx.x; i < 2 * kDbuf; i += S::kThreads) (&sm.dbuf[0][0][0])[i] = 0.f;
   for (int i = threadIdx.x; i < NS * kB; i += S::kThreads)   // columns no copy writes: inputs that add nothing
     for (int c = 8 * cnt; c < S::kCols; ++c) sm.rows[i / kB][i % kB][c] = 0.f;
   if (CL > 1) mma::cluster_sync(); else __syncthreads();   // a peer's barriers exist before anything is sent to it
@@ -161,38 +164,51 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
   if (role == kRec) {
     // ================= R: the recurrence; lane = (sample, class half) =================
     const int s_mine = lane & 15, h = lane >> 4;
+    const float* dall0 = &sm.dbuf[0][h][0];
     for (uint32_t k = 0; k < nblk; ++k) {
       const int b = k & 1, ig = k % S::kInG, iz = k % S::kInZ;
       const uint32_t nv = min((uint32_t)kB, n - k * kB);
+      if (CL > 1) {
+        wait(&sm.ready[b], (k >> 1) & 1);
+      } else {
+        wait(&sm.bg[ig], (k / S::kInG) & 1);
+        wait(&sm.bz[iz], (k / S::kInZ) & 1);
+      }
       const float* in = CL > 1 ? sm.coup[b] : sm.gin[ig][0];
-      if (CL > 1) wait(&sm.ready[b], (k >> 1) & 1); else wait(&sm.bg[ig], (k / S::kInG) & 1);
+      const float* zi = CL > 1 ? sm.zsum[b] : sm.zin[iz][0];
+      float z0[kCh], L[kB];
+#pragma unroll
+      for (int c = 0; c < kCh; ++c) z0[c] = zi[(h * kCh + c) * kB + s_mine];
+      const float4* lr4 = reinterpret_cast<const float4*>(in + s_mine * kGp);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 v = lr4[i];
+        L[4 * i] = v.x; L[4 * i + 1] = v.y; L[4 * i + 2] = v.z; L[4 * i + 3] = v.w;
+      }
       const float amax = __uint_as_float(CL > 1 ? sm.amax[b][0] : warp_max(lane < NG ? sm.amax[ig][lane] : 0u));
       const int y = sm.ys[k & 7][s_mine];
-      float L[kB];
-      {
-        const float4* lr4 = reinterpret_cast<const float4*>(in + s_mine * kGp);
+      // acc[c] += sum over s < cnt of f[s] delta[s][c]; deltas lie [sample][class] in a class half, five apart
+      auto add_deltas = [&](const float* d, const float (&f)[kB], float (&acc)[kCh]) {
+        float v[4 * ((kB * kCh + 3) / 4)];
+#pragma unroll
+        for (int i = 0; i < kB * kCh / 4; ++i) {
+          const float4 x = reinterpret_cast<const float4*>(d)[i];
+          v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
+        }
+#pragma unroll
+        for (int s = 0; s < kB; ++s)
+#pragma unroll
+          for (int c = 0; c < kCh; ++c) acc[c] = fmaf(f[s], v[s * kCh + c], acc[c]);
+      };
+      if (k) {   // what the deltas of the block before add
+        float cf[kB];
+        const float4* cr = reinterpret_cast<const float4*>(in + kOffC + s_mine * kGp);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const float4 v = lr4[i];
-          L[4 * i] = v.x; L[4 * i + 1] = v.y; L[4 * i + 2] = v.z; L[4 * i + 3] = v.w;
+          const float4 v = cr[i];
+          cf[4 * i] = v.x; cf[4 * i + 1] = v.y; cf[4 * i + 2] = v.z; cf[4 * i + 3] = v.w;
         }
-      }
-      float z0[kCh] = {};
-      if (k) {   // what the deltas of the block before add
-        const float4* cr = reinterpret_cast<const float4*>(in + kOffC + s_mine * kGp);
-        const float* dp = &sm.dbuf[b ^ 1][0][h * 8];
-#pragma unroll
-        for (int s4 = 0; s4 < 4; ++s4) {
-          const float4 cv = cr[s4];
-          const float cf[4] = {cv.x, cv.y, cv.z, cv.w};
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float4 d = *reinterpret_cast<const float4*>(dp + (4 * s4 + i) * 16);
-            const float d4 = dp[(4 * s4 + i) * 16 + 4];
-            z0[0] = fmaf(cf[i], d.x, z0[0]); z0[1] = fmaf(cf[i], d.y, z0[1]); z0[2] = fmaf(cf[i], d.z, z0[2]);
-            z0[3] = fmaf(cf[i], d.w, z0[3]); z0[4] = fmaf(cf[i], d4, z0[4]);
-          }
-        }
+        add_deltas(dall0 + (b ^ 1) * kDbuf, cf, z0);
       }
       // amax is in units of log2 as the logits are; (1 + a)^15 <= exp(15 a)
       const float gain = 7.5f / kLog2e * amax * ex2(fminf(7.5f * amax, 60.f));
@@ -204,19 +220,6 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
         float m = fmaxf(fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3])), z[4]);
         return fmaxf(m, shx(m, 16));
       };
-      if (CL > 1) {
-        if (lane == 0) mbar_expect_tx(&sm.bz[iz], CL * kZ * 4);
-        wait_cluster(&sm.bz[iz], (k / S::kInZ) & 1);
-      } else {
-        wait(&sm.bz[iz], (k / S::kInZ) & 1);
-      }
-#pragma unroll
-      for (int c = 0; c < kCh; ++c) {
-        float v = sm.zin[iz][0][(h * kCh + c) * kB + s_mine];
-#pragma unroll
-        for (int r = 1; r < CL; ++r) v += sm.zin[iz][r][(h * kCh + c) * kB + s_mine];
-        z0[c] += v;
-      }
       {
         const float m = top(z0);
 #pragma unroll
@@ -225,16 +228,21 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
       float z[kCh], d[kCh];
 #pragma unroll
       for (int c = 0; c < kCh; ++c) z[c] = z0[c];
-      float* dmine = &sm.dbuf[b][s_mine][h * 8];
-      const float* dall = &sm.dbuf[b][0][h * 8];
+      const float* dall = dall0 + b * kDbuf;
+      float* dmine = const_cast<float*>(dall) + s_mine * kCh;
       const bool live = (uint32_t)s_mine < nv;
+      const float need = live ? kTol : 3e38f;
       uint32_t left = nv - 1;   // sweeps that can still be needed
       while (true) {
-        float m = 0.f;
-        if (wild) m = top(z);
         float e[kCh];
+        if (wild) {
+          const float m = top(z);
 #pragma unroll
-        for (int c = 0; c < kCh; ++c) e[c] = ex2(z[c] - m);
+          for (int c = 0; c < kCh; ++c) e[c] = ex2(z[c] - m);
+        } else {
+#pragma unroll
+          for (int c = 0; c < kCh; ++c) e[c] = ex2(z[c]);
+        }
         float sum = ((e[0] + e[1]) + (e[2] + e[3])) + e[4];
         sum += shx(sum, 16);
         const float inv = rcp(sum);
@@ -242,27 +250,22 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
         for (int c = 0; c < kCh; ++c) d[c] = fmaf(e[c], inv, oh[c]);
         if (!left) break;
         --left;
-        *reinterpret_cast<float4*>(dmine) = make_float4(d[0], d[1], d[2], d[3]);
-        dmine[4] = d[4];
+#pragma unroll
+        for (int c = 0; c < kCh; ++c) dmine[c] = d[c];
         __syncwarp();
         float zn[kCh];
 #pragma unroll
         for (int c = 0; c < kCh; ++c) zn[c] = z0[c];
+        add_deltas(dall, L, zn);   // (L is zero from the diagonal on)
+        const float change = fmaxf(fmaxf(fmaxf(fabsf(zn[0] - z[0]), fabsf(zn[1] - z[1])), fmaxf(fabsf(zn[2] - z[2]), fabsf(zn[3] - z[3]))),
+                                   fabsf(zn[4] - z[4]));
 #pragma unroll
-        for (int s = 0; s < kB - 1; ++s) {
-          const float4 dv = *reinterpret_cast<const float4*>(dall + s * 16);
-          const float d4 = dall[s * 16 + 4];
-          zn[0] = fmaf(L[s], dv.x, zn[0]); zn[1] = fmaf(L[s], dv.y, zn[1]); zn[2] = fmaf(L[s], dv.z, zn[2]);
-          zn[3] = fmaf(L[s], dv.w, zn[3]); zn[4] = fmaf(L[s], d4, zn[4]);
-        }
-        float change = 0.f;
-#pragma unroll
-        for (int c = 0; c < kCh; ++c) { change = fmaxf(change, fabsf(zn[c] - z[c])); z[c] = zn[c]; }
-        if (!__any_sync(0xffffffffu, live && !(change * gain <= kTol)) && !p.step_by_step) left = 0;
+        for (int c = 0; c < kCh; ++c) z[c] = zn[c];
+        if (!__any_sync(0xffffffffu, !(change * gain <= need)) && !p.step_by_step) left = 0;
         __syncwarp();
       }
-      *reinterpret_cast<float4*>(dmine) = live ? make_float4(d[0], d[1], d[2], d[3]) : make_float4(0.f, 0.f, 0.f, 0.f);
-      dmine[4] = live ? d[4] : 0.f;
+#pragma unroll
+      for (int c = 0; c < kCh; ++c) dmine[c] = live ? d[c] : 0.f;
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.delta[b]);
     }
@@ -290,10 +293,14 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
       if (lane == 0) mbar_arrive(&sm.full[sb]);
     }
   } else if (CL > 1 && role == kSum) {
-    // ================= the CTAs' parts of the couplings, summed in rank order =================
+    // ================= the CTAs' parts, summed in rank order =================
+    if (lane == 0) {
+      mbar_expect_tx(&sm.bg[0], CL * kSendG0);
+      mbar_expect_tx(&sm.bz[0], CL * kZ * 4);
+    }
     for (uint32_t k = 0; k < nblk; ++k) {
       const int ig = k % S::kInG, b = k & 1;
-      if (lane == 0) mbar_expect_tx(&sm.bg[ig], CL * (k ? kSendG : kSendG0));
+      const int iz = k % S::kInZ;
       wait_cluster(&sm.bg[ig], (k / S::kInG) & 1);
       if (k >= 2) wait(&sm.delta[b], ((k >> 1) - 1) & 1);   // R has taken block k - 2
       float* out = sm.coup[b];
@@ -312,6 +319,18 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
       }
       const uint32_t m = warp_max(__float_as_uint(big));
       if (lane == 0) sm.amax[b][0] = m;
+      wait_cluster(&sm.bz[iz], (k / S::kInZ) & 1);
+#pragma unroll
+      for (int i = 0; i < kZ / 32; ++i) {
+        float v = sm.zin[iz][0][lane + 32 * i];
+#pragma unroll
+        for (int r = 1; r < CL; ++r) v += sm.zin[iz][r][lane + 32 * i];
+        sm.zsum[b][lane + 32 * i] = v;
+      }
+      if (lane == 0 && k + 1 < nblk) {
+        mbar_expect_tx(&sm.bg[(k + 1) % S::kInG], CL * kSendG);
+        mbar_expect_tx(&sm.bz[(k + 1) % S::kInZ], CL * kZ * 4);
+      }
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.ready[b]);
     }
@@ -328,7 +347,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
       for (int j = 0; j < KG; ++j) {
         const float2 x0 = *reinterpret_cast<const float2*>(xr + 8 * NG * j);
         const float2 x1 = *reinterpret_cast<const float2*>(xr + 8 * S::kPitch + 8 * NG * j);
-        const Split a = split(x0.x), b = split(x0.y), c = split(x1.x), d = split(x1.y);
+        const Split a = split_t(x0.x), b = split_t(x0.y), c = split_t(x1.x), d = split_t(x1.y);
         mma::tf32(gh[0], a.hi, c.hi, b.hi, d.hi, a.hi, b.hi);
         mma::tf32(gh[1], a.hi, c.hi, b.hi, d.hi, c.hi, d.hi);
         mma::tf32(gs[0], a.hi, c.hi, b.hi, d.hi, a.lo, b.lo);
@@ -340,7 +359,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
           } else {
             const float2 y0 = *reinterpret_cast<const float2*>(pr + 8 * NG * j);
             const float2 y1 = *reinterpret_cast<const float2*>(pr + 8 * S::kPitch + 8 * NG * j);
-            e = split(y0.x); f = split(y0.y); u = split(y1.x); v = split(y1.y);
+            e = split_t(y0.x); f = split_t(y0.y); u = split_t(y1.x); v = split_t(y1.y);
           }
           mma::tf32(hh[0], a.hi, c.hi, b.hi, d.hi, e.hi, f.hi);
           mma::tf32(hh[1], a.hi, c.hi, b.hi, d.hi, u.hi, v.hi);
@@ -470,14 +489,14 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
       const float* xb = &sm.rows[k % NS][tt][8 * warp + g];
       const float* xr = &sm.rows[kb % NS][g][8 * warp + 2 * tt];
       constexpr bool kEarly = KM <= 4;   // room for them in registers
-      Split x[kEarly ? KM : 1][4];
+      Split x[kEarly ? KM : 2][4];
       float2 r0[kEarly ? KM : 1], r1[kEarly ? KM : 1];
       if (look) wait(&sm.full[kb % NS], (kb / NS) & 1);
       if (kEarly) {
 #pragma unroll
         for (int j = 0; j < (kEarly ? KM : 1); ++j) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) x[j][i] = split(xb[4 * i * S::kPitch + 8 * NM * j]);
+          for (int i = 0; i < 4; ++i) x[j][i] = split_t(xb[4 * i * S::kPitch + 8 * NM * j]);
           r0[j] = *reinterpret_cast<const float2*>(xr + 8 * NM * j);
           r1[j] = *reinterpret_cast<const float2*>(xr + 8 * S::kPitch + 8 * NM * j);
         }
@@ -487,14 +506,15 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
         wait(&sm.delta[k & 1], (k >> 1) & 1);
         Split a[2][4];
         {
-          const int col = g < kCh ? g : g + 3;
+          const float* d0 = &sm.dbuf[k & 1][g / kCh][g % kCh];
+          const float* d1 = &sm.dbuf[k & 1][1][two ? g + 3 : 0];   // classes 8, 9
           float s0 = 0.f, s1 = 0.f;
 #pragma unroll
           for (int m = 0; m < 2; ++m)
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
               const int s = 8 * m + tt + 4 * i;
-              float v0 = sm.dbuf[k & 1][s][col], v1 = two ? sm.dbuf[k & 1][s][g + 11] : 0.f;
+              float v0 = d0[s * kCh], v1 = two ? d1[s * kCh] : 0.f;
               if (biases) { s0 += v0; s1 += v1; }
               if (decay) {
                 const float f = (uint32_t)s < nv ? sm.qp[nv - 1 - s] : 0.f;
@@ -519,25 +539,34 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
           for (uint32_t i = 0; i < nv; ++i) qwd *= qd;
           qw = (float)qwd;
         }
-        float d[KM][4] = {};
+        // the six products of a k-step depend on one another: several k-steps side by side
+        constexpr int kSide = kEarly ? KM : 2;
 #pragma unroll
-        for (int j = 0; j < KM; ++j) {
+        for (int j0 = 0; j0 < KM; j0 += kSide) {
+          float d[kSide][4] = {};
           if (!kEarly) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) x[0][i] = split(xb[4 * i * S::kPitch + 8 * NM * j]);
+            for (int jj = 0; jj < kSide; ++jj)
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                if (j0 + jj < KM) x[jj][i] = split_t(xb[4 * i * S::kPitch + 8 * NM * (j0 + jj)]);
           }
-          const Split (&v)[4] = x[kEarly ? j : 0];
-          mma::tf32(d[j], a[0][0].lo, a[0][1].lo, a[0][2].lo, a[0][3].lo, v[0].hi, v[1].hi);
-          mma::tf32(d[j], a[0][0].hi, a[0][1].hi, a[0][2].hi, a[0][3].hi, v[0].lo, v[1].lo);
-          mma::tf32(d[j], a[1][0].lo, a[1][1].lo, a[1][2].lo, a[1][3].lo, v[2].hi, v[3].hi);
-          mma::tf32(d[j], a[1][0].hi, a[1][1].hi, a[1][2].hi, a[1][3].hi, v[2].lo, v[3].lo);
-          mma::tf32(d[j], a[0][0].hi, a[0][1].hi, a[0][2].hi, a[0][3].hi, v[0].hi, v[1].hi);
-          mma::tf32(d[j], a[1][0].hi, a[1][1].hi, a[1][2].hi, a[1][3].hi, v[2].hi, v[3].hi);
+#pragma unroll
+          for (int term = 0; term < 6; ++term)
+#pragma unroll
+            for (int jj = 0; jj < kSide; ++jj) {
+              if (j0 + jj >= KM) continue;
+              const int m = term & 1, i = 2 * m;   // which eight samples
+              if (term < 2) mma::tf32(d[jj], a[m][0].lo, a[m][1].lo, a[m][2].lo, a[m][3].lo, x[jj][i].hi, x[jj][i + 1].hi);
+              else if (term < 4) mma::tf32(d[jj], a[m][0].hi, a[m][1].hi, a[m][2].hi, a[m][3].hi, x[jj][i].lo, x[jj][i + 1].lo);
+              else mma::tf32(d[jj], a[m][0].hi, a[m][1].hi, a[m][2].hi, a[m][3].hi, x[jj][i].hi, x[jj][i + 1].hi);
+            }
+#pragma unroll
+          for (int jj = 0; jj < kSide; ++jj)
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              if (j0 + jj < KM) U[j0 + jj][c] += d[jj][c];
         }
-#pragma unroll
-        for (int j = 0; j < KM; ++j)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) U[j][c] += d[j][c];
       }
       if (look) {
         // ---- logits of block kb with the model W = qw W_start - eta U ----
@@ -549,9 +578,9 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
             r1[0] = *reinterpret_cast<const float2*>(xr + 8 * S::kPitch + 8 * NM * j);
           }
           const float2 x0 = r0[kEarly ? j : 0], x1 = r1[kEarly ? j : 0];
-          const Split a = split(x0.x), b = split(x0.y), c = split(x1.x), d = split(x1.y);
-          const Split w0 = split(fmaf(neta, U[j][0], qw * ws[j][0])), w2 = split(fmaf(neta, U[j][1], qw * ws[j][1]));
-          const Split w1 = split(fmaf(neta, U[j][2], qw * ws[j][2])), w3 = split(fmaf(neta, U[j][3], qw * ws[j][3]));
+          const Split a = split_t(x0.x), b = split_t(x0.y), c = split_t(x1.x), d = split_t(x1.y);
+          const Split w0 = split_t(fmaf(neta, U[j][0], qw * ws[j][0])), w2 = split_t(fmaf(neta, U[j][1], qw * ws[j][1]));
+          const Split w1 = split_t(fmaf(neta, U[j][2], qw * ws[j][2])), w3 = split_t(fmaf(neta, U[j][3], qw * ws[j][3]));
           mma::tf32(zm[0], w0.hi, w1.hi, w2.hi, w3.hi, a.hi, b.hi);
           mma::tf32(zm[1], w0.hi, w1.hi, w2.hi, w3.hi, c.hi, d.hi);
           mma::tf32(zx[0], w0.lo, w1.lo, w2.lo, w3.lo, a.hi, b.hi);
@@ -650,7 +679,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
 
 typedef Shape<1, 10, 10, 4, 25, 3, false> One;
 typedef Shape<2, 7, 7, 6, 9, 4, false> Two;
-typedef Shape<4, 7, 4, 5, 5, 4, true> Four;
+typedef Shape<4, 5, 5, 4, 7, 4, true> Four;
 
 template <class S>
 cudaError_t launch(const RoundLaunch& p, cudaStream_t s) {
