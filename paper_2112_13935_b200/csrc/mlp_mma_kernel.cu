@@ -1,0 +1,846 @@
+// Local-SGD round of one client for ReLU MLPs on minibatches of up to 64 samples (fp32, or bf16 operands with fp32
+// masters): the first layer stays on the chip for the whole round, spread over a cluster.
+//
+// Algorithm 3, MainComputeNode, inner loop with xi a minibatch: g = mean gradient (+ lambda W), w_c -= eta_i g,
+// U_i += g, repeated s_{i,c} / B times; then (c, U_i, i) is sent.
+//
+// A cluster of CL CTAs of 16 warps per round-task.  CTA r owns a range of the inputs (whole units of 16); it copies only
+// these columns of the minibatch rows (one iteration ahead) and holds the rows of W_0 they meet - in transposed fragments,
+// each thread its own entries, in TENSOR MEMORY used as a register file of 128 words per thread (tcgen05.ld / st; what
+// does not fit goes on in shared memory): nothing of W_0 moves between start and trigger.  Per iteration:
+//   1  Z_0^T += W_0^T X^T over the CTA's inputs (warp = hidden tile x input part), summed over the parts in shared
+//      memory, each CTA's share sent to the CTA that owns the hidden row (st.async, counted by an mbarrier there);
+//   2  the owner adds the CTAs' parts in rank order, bias, ReLU, and sends its rows of A_0 to every CTA;
+//   3  every CTA runs the narrow layers, the softmax and the backward pass down to dZ_0 redundantly (same inputs, same
+//      order: the same bits in every CTA);
+//   4  dW_0^T = dZ_0^T X over the CTA's inputs: the accumulator fragment is the thread's own piece of W_0^T - update in place.
+// The hand-overs need no cluster barrier: a CTA sends its part of Z_0 for the next iteration only after it has all of A_0
+// of this one, which the owners sent after taking everybody's part.
+//
+// Products are m16n8k16 bf16, or m16n8k8 tf32 on split fp32 operands (mma_common.cuh).  The transposed orientation puts
+// hidden units on M, samples (forward) or inputs (gradient) on N: the fragment of a thread is the same in both products.
+// tcgen05 would need W_0 as an operand in shared memory (bf16 image or hi/lo pair) rewritten every iteration and 64-row
+// tiles; at 16-64 samples per iteration the warp-level instructions' rate (1,024 bf16 / 512 tf32 multiply-adds per clock
+// and SM) is not what limits a round: hand-overs, updates and the narrow layers are.
+//
+// precision 1: the update sum of W_0 is (W_start - W_end) / eta; everything else accumulates U.
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include "aet_kernels.h"
+#include "aet_rng.h"
+#include "lr_common.cuh"
+#include "mma_common.cuh"
+
+namespace aet {
+namespace {
+
+using lr::kWaitLimit;
+using lr::mbar_expect_tx;
+using lr::mbar_init;
+using lr::smem_addr;
+using mma::Split;
+using mma::split;
+using mma::split_t;
+
+constexpr int kWarps = 16, kThreads = kWarps * 32;
+constexpr int kTmemWords = 128;     // per thread: 512 columns over the four warps that share 32 lanes
+constexpr int kMaxL = AET_MAX_LAYERS;
+
+struct MmaPlan {
+  int nl, d[8], B, Bp, bt;
+  int CL, units, upc, upw;          // 16-input units: all, per CTA, per warp
+  int MT, WM, WK;                   // hidden tiles of 16; warps over tiles, over input parts
+  int rgs;                          // hidden rows owned per CTA, in groups of 8
+  int xpitch, xbufs;                // minibatch columns: elements per row, buffers
+  int ap[kMaxL], zp[kMaxL], wp[kMaxL], np[kMaxL];   // pitches of A_l, dZ_l, W_l (l >= 1), padded rows of W_l
+  int ext;                          // words per thread beyond tensor memory
+  // offsets in floats
+  int o_x, o_in, o_part, o_a[kMaxL], o_z[kMaxL], o_w[kMaxL], o_u[kMaxL], o_b, o_ub, o_gb, o_logit, o_ext, o_idx, o_bar, total;
+  int boff[kMaxL];                  // of layer l's biases in the bias arrays
+};
+
+__host__ __device__ inline int up(int v, int m) { return (v + m - 1) / m * m; }
+
+// Whether and how a shape runs on clusters of cl CTAs; total == 0: it does not.
+MmaPlan make_plan(const MlpShape& s, int cl) {
+  MmaPlan p{};
+  const bool bf = s.precision == 1;
+  p.nl = (int)s.n_layers;
+  for (int i = 0; i <= p.nl; ++i) p.d[i] = (int)s.dims[i];
+  p.B = (int)s.batch;
+  p.Bp = up(p.B, bf ? 16 : 8);
+  p.bt = p.Bp / 8;
+  p.CL = cl;
+  p.MT = (p.d[1] + 15) / 16;
+  const int mpw = (p.MT + 7) / 8;
+  if (p.B > 64 || p.MT > 16 || (!bf && (p.MT > 8)) || p.d[p.nl] > 32 || (bf && p.d[0] % 8)) return p;
+  p.WM = (p.MT + mpw - 1) / mpw;
+  p.WK = kWarps / p.WM;
+  p.units = (p.d[0] + 15) / 16;
+  p.upc = (p.units + cl - 1) / cl;
+  p.upw = (p.upc + p.WK - 1) / p.WK;
+  if (cl > 1 && p.upc * (cl - 1) >= p.units) return p;   // the last CTA would have nothing
+  const int words = p.upw * mpw * 8 * (bf ? 1 : 2);
+  p.ext = words > kTmemWords ? words - kTmemWords : 0;
+  p.rgs = (2 * p.MT + cl - 1) / cl;
+  int o = 0;
+  auto take = [&](int floats) { const int at = o; o += up(floats, 4); return at; };
+  const int elems = bf ? 2 : 1;      // elements per float
+  p.xpitch = 16 * p.upc + 8;         // 8 mod 16 elements: fragment loads hit different banks
+  p.xbufs = 2;
+  p.o_bar = take(16);
+  p.o_idx = take(4 * 64);
+  p.o_x = take(p.xbufs * p.Bp * p.xpitch / elems);
+  p.o_in = take(cl * p.rgs * 8 * p.Bp);
+  int part = (p.WK - 1) * p.WM * mpw * p.bt * 128;
+  for (int l = 0; l < p.nl; ++l) {
+    const int n = up(p.d[l + 1], 16);
+    p.ap[l] = p.zp[l] = n + 8;
+    if (l + 1 < p.nl) p.o_a[l] = take(p.Bp * p.ap[l] / elems);
+    else if (l == 0) p.o_a[0] = take(p.Bp * p.ap[0]);   // no hidden layer: the logits, fp32
+    if (l > 0) {
+      p.o_z[l] = take(p.Bp * p.zp[l] / elems);
+      p.wp[l] = up(p.d[l], 16) + 8;
+      p.np[l] = n;
+      p.o_w[l] = take(n * p.wp[l]);
+      p.o_u[l] = take(n * p.wp[l]);
+    }
+  }
+  // dZ_0 and the partial products of the input parts are never needed at the same time
+  const int z0 = p.Bp * p.zp[0] / elems;
+  p.o_part = p.o_z[0] = take(part > z0 ? part : z0);
+  int nb = 0;
+  for (int l = 0; l < p.nl; ++l) { p.boff[l] = nb; nb += up(p.d[l + 1], 16); }
+  p.o_b = take(nb); p.o_ub = take(nb); p.o_gb = take(nb);
+  p.o_logit = take(p.Bp * 33);
+  p.o_ext = take(p.ext * kThreads);
+  p.total = o;
+  if ((size_t)o * 4 > 227 * 1024) p.total = 0;
+  return p;
+}
+
+// ---- fragments -----------------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldmatrix4t(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldmatrix2t(uint32_t (&r)[2], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr) : "memory");
+}
+
+// One operand fragment set of a k-step (fp32: 8 wide, head and remainder; bf16: 16 wide).
+template <bool BF> struct FragA;
+template <> struct FragA<false> { Split v[4]; };
+template <> struct FragA<true> { uint32_t v[4]; };
+template <bool BF> struct FragB;
+template <> struct FragB<false> { Split v[2]; };
+template <> struct FragB<true> { uint32_t v[2]; };
+
+// d += a b; fp32: the two cross terms into x (which may be d itself)
+__device__ __forceinline__ void product(float (&d)[4], float (&x)[4], const FragA<false>& a, const FragB<false>& b) {
+  mma::tf32(x, a.v[0].lo, a.v[1].lo, a.v[2].lo, a.v[3].lo, b.v[0].hi, b.v[1].hi);
+  mma::tf32(x, a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].lo, b.v[1].lo);
+  mma::tf32(d, a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].hi, b.v[1].hi);
+}
+__device__ __forceinline__ void product(float (&d)[4], float (&)[4], const FragA<true>& a, const FragB<true>& b) {
+  mma_bf16(d, a.v, b.v[0], b.v[1]);
+}
+
+template <bool BF> struct Elem { typedef float T; static constexpr int kStep = 8; };
+template <> struct Elem<true> { typedef __nv_bfloat16 T; static constexpr int kStep = 16; };
+
+// First operand from an fp32 weight array [row][k] (rows g, g + 8; the k index of a step is read as pairs 2t | 2t + 1)
+__device__ __forceinline__ void load_w(FragA<false>& f, const float* w, int pitch, int g, int tt) {
+  const float2 a = *reinterpret_cast<const float2*>(w + g * pitch + 2 * tt), b = *reinterpret_cast<const float2*>(w + (g + 8) * pitch + 2 * tt);
+  f.v[0] = split(a.x); f.v[1] = split(b.x); f.v[2] = split(a.y); f.v[3] = split(b.y);
+}
+__device__ __forceinline__ void load_w(FragA<true>& f, const float* w, int pitch, int g, int tt) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const float2 a = *reinterpret_cast<const float2*>(w + g * pitch + 8 * h + 2 * tt), b = *reinterpret_cast<const float2*>(w + (g + 8) * pitch + 8 * h + 2 * tt);
+    f.v[2 * h] = pack_bf16(a.x, a.y); f.v[2 * h + 1] = pack_bf16(b.x, b.y);
+  }
+}
+// First operand W^T: rows are the k index of an fp32 array [n][row], k = n in pairs
+__device__ __forceinline__ void load_wt(FragA<false>& f, const float* w, int pitch, int g, int tt) {
+  const float* p = w + 2 * tt * pitch + g;
+  f.v[0] = split(p[0]); f.v[1] = split(p[8]); f.v[2] = split(p[pitch]); f.v[3] = split(p[pitch + 8]);
+}
+__device__ __forceinline__ void load_wt(FragA<true>& f, const float* w, int pitch, int g, int tt) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const float* p = w + (8 * h + 2 * tt) * pitch + g;
+    f.v[2 * h] = pack_bf16(p[0], p[pitch]); f.v[2 * h + 1] = pack_bf16(p[8], p[pitch + 8]);
+  }
+}
+// Second operand from samples [sample][k], column = sample g
+__device__ __forceinline__ void load_s(FragB<false>& f, const float* x, int pitch, int g, int tt) {
+  const float2 a = *reinterpret_cast<const float2*>(x + g * pitch + 2 * tt);
+  f.v[0] = split_t(a.x); f.v[1] = split_t(a.y);
+}
+__device__ __forceinline__ void load_s(FragB<true>& f, const __nv_bfloat16* x, int pitch, int g, int tt) {
+  f.v[0] = *reinterpret_cast<const uint32_t*>(x + g * pitch + 2 * tt);
+  f.v[1] = *reinterpret_cast<const uint32_t*>(x + g * pitch + 8 + 2 * tt);
+}
+// First operand dZ^T: rows are columns of an array [sample][n], k = sample
+__device__ __forceinline__ void load_zt(FragA<false>& f, const float* z, int pitch, int lane) {
+  const float* p = z + (lane & 3) * pitch + (lane >> 2);
+  f.v[0] = split(p[0]); f.v[1] = split(p[8]); f.v[2] = split(p[4 * pitch]); f.v[3] = split(p[4 * pitch + 8]);
+}
+__device__ __forceinline__ void load_zt(FragA<true>& f, const __nv_bfloat16* z, int pitch, int lane) {
+  const int i = lane >> 3, r = lane & 7;
+  ldmatrix4t(f.v, smem_addr(z + ((i >> 1) * 8 + r) * pitch + (i & 1) * 8));
+}
+// Second operand from an array [sample][n], k = sample, column = n
+__device__ __forceinline__ void load_st(FragB<false>& f, const float* x, int pitch, int lane) {
+  const float* p = x + (lane & 3) * pitch + (lane >> 2);
+  f.v[0] = split_t(p[0]); f.v[1] = split_t(p[4 * pitch]);
+}
+__device__ __forceinline__ void load_st(FragB<true>& f, const __nv_bfloat16* x, int pitch, int lane) {
+  const int r = lane & 15;
+  ldmatrix2t(f.v, smem_addr(x + r * pitch));
+}
+__device__ __forceinline__ void put(float* p, float v) { *p = v; }
+__device__ __forceinline__ void put(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ float get(const float* p) { return *p; }
+__device__ __forceinline__ float get(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+
+// ---- a thread's own words: tensor memory, then shared memory ----------------------------------------------------------
+struct Own {
+  uint32_t tmem;     // this thread's lane and first column
+  float* ext;        // word i at ext[i * kThreads]
+  __device__ __forceinline__ void load_issue(int group, float (&v)[8]) const {
+    if (group < kTmemWords / 8) {
+      uint32_t r[8];
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\ttcgen05.wait::ld.sync.aligned;"
+                   : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                   : "r"(tmem + 8u * group) : "memory");
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = ext[(8 * group - kTmemWords + i) * kThreads];
+    }
+  }
+  __device__ __forceinline__ void store(int group, const float (&v)[8]) const {
+    if (group < kTmemWords / 8) {
+      asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                   ::"r"(tmem + 8u * group), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
+                     "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])) : "memory");
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) ext[(8 * group - kTmemWords + i) * kThreads] = v[i];
+    }
+  }
+  __device__ __forceinline__ void store_wait() const { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+};
+
+__device__ __forceinline__ void send2(uint32_t addr, uint32_t a, uint32_t b, uint32_t bar) {   // 8 bytes to a peer
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+               ::"r"(addr), "r"(a), "r"(b), "r"(bar) : "memory");
+}
+
+struct MmaLaunch {
+  RoundLaunch r;
+  MmaPlan m;
+};
+
+template <bool BF, int MPW, int BT>
+__global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_constant__ MmaLaunch p) {
+  typedef typename Elem<BF>::T T;
+  constexpr int kStep = Elem<BF>::kStep;
+  extern __shared__ __align__(128) float smem[];
+  const MmaPlan& m = p.m;
+  const int CL = m.CL, B = m.B, Bp = m.Bp, bt = m.bt, nl = m.nl, N1 = m.d[1], D0 = m.d[0];
+
+  const TaskDesc t = p.r.tasks[p.r.task_begin + blockIdx.x / CL];
+  if (!debug_task_ok(p.r, t)) return;   // the whole cluster alike
+  const uint32_t rank = CL > 1 ? mma::cluster_rank() : 0;
+  if (t.steps == 0) {
+    int P = 0;
+    for (int l = 0; l < nl; ++l) P += m.d[l] * m.d[l + 1] + m.d[l + 1];
+    if (rank == 0) publish_empty_round(p.r, t, (uint32_t)P);
+    return;
+  }
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tt = lane & 3;
+  const float eta = t.eta, lambda = p.r.l2;
+
+  T* const xb0 = reinterpret_cast<T*>(smem + m.o_x);
+  float* const inbox = smem + m.o_in;
+  float* const part = smem + m.o_part;
+  float* const bias = smem + m.o_b;
+  float* const ubias = smem + m.o_ub;
+  float* const gbias = smem + m.o_gb;
+  float* const logit = smem + m.o_logit;
+  int* const idx = reinterpret_cast<int*>(smem + m.o_idx);        // [2][64] row numbers, then [2][64] labels
+  uint64_t* const bars = reinterpret_cast<uint64_t*>(smem + m.o_bar);   // [0] parts of Z_0, [1] A_0
+  uint32_t* const tmem_at = reinterpret_cast<uint32_t*>(bars + 2);
+  auto A = [&](int l) { return reinterpret_cast<T*>(smem + m.o_a[l]); };
+  auto Z = [&](int l) { return reinterpret_cast<T*>(smem + m.o_z[l]); };
+
+  const int u0 = min(m.units, (int)rank * m.upc), nu = min(m.units, u0 + m.upc) - u0;   // this CTA's input units
+  const int x0 = 16 * u0, nx = min(D0, x0 + 16 * nu) - x0;                              // ... and columns
+  const int wm = warp % m.WM, wk = warp / m.WM;
+  const bool mine = wk < m.WK;                                                          // (some warps hold no tile)
+  const int w0 = mine ? min(nu, wk * m.upw) : nu, wn = min(nu, w0 + m.upw) - w0;        // this warp's units
+  const int rg0 = min(2 * m.MT, (int)rank * m.rgs), nrg = min(2 * m.MT, rg0 + m.rgs) - rg0;   // owned groups of 8 hidden rows
+
+  for (int i = tid; i < m.total; i += kThreads) smem[i] = 0.f;
+  __syncthreads();
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_addr(tmem_at)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 0) {
+    mbar_init(&bars[0], 1);
+    mbar_init(&bars[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (CL > 1) mma::cluster_sync(); else __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t in_bytes = (uint32_t)(CL * nrg * 8 * Bp * 4), a_bytes = (uint32_t)(16 * m.MT * Bp * (nl > 1 ? sizeof(T) : sizeof(float)));
+  if (tid == 0) {
+    if (nrg > 0) mbar_expect_tx(&bars[0], in_bytes);
+    mbar_expect_tx(&bars[1], a_bytes);
+  }
+
+  Own own;
+  own.tmem = *tmem_at + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * kTmemWords;
+  own.ext = smem + m.o_ext + tid;
+  const int ug = m.upw * MPW;   // first group of the update sum (fp32)
+
+  bool ok = true;
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    const uint32_t at = smem_addr(bar);
+    for (uint32_t i = 0; ok; ++i) {
+      if (mma::try_wait_cluster(at, parity)) break;
+      if (i >= kWaitLimit) ok = false;
+    }
+  };
+
+  const ClientData cd = p.r.clients[t.client];
+  const uint64_t key = p.r.sample_keys[t.client];
+  // Row numbers and labels of iteration it, then this CTA's columns of its rows into a buffer (asynchronous copies).
+  auto draw_rows = [&](uint32_t it) {
+    if (tid < B) {
+      const uint32_t id = sample_index(draw(key, t.sample_ctr0 + (uint64_t)it * B + tid), cd.n);
+      idx[(it & 1) * 64 + tid] = (int)id;
+      idx[128 + (it & 1) * 64 + tid] = __ldg(cd.y + id);
+    }
+  };
+  constexpr int kChunk = 16 / (int)sizeof(T);
+  const bool whole = (D0 * sizeof(T)) % 16 == 0;
+  auto copy_rows = [&](uint32_t it) {
+    T* x = xb0 + (it % m.xbufs) * Bp * m.xpitch;
+    const T* src = reinterpret_cast<const T*>(cd.x) + x0;
+    for (int r = warp; r < B; r += kWarps) {
+      const T* row = src + (size_t)idx[(it & 1) * 64 + r] * D0;
+      if (whole) {
+        for (int c = lane * kChunk; c < nx; c += 32 * kChunk)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(x + r * m.xpitch + c)), "l"(row + c) : "memory");
+      } else {
+        for (int c = lane; c < nx; c += 32) x[r * m.xpitch + c] = row[c];
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+  // ---- start model: snapshot minus own update sums still in flight ----
+  const float* snap = p.r.snaps + (size_t)t.snap_slot * p.r.stride;
+  auto start_value = [&](size_t at) {
+    float v = snap[at];
+    for (uint32_t f = 0; f < t.inflight_cnt; ++f) {
+      const InflightRef ref = p.r.inflight[t.inflight_off + f];
+      v = fmaf(-ref.eta, p.r.U[(size_t)ref.row * p.r.stride + at], v);
+    }
+    return v;
+  };
+  // Parameter of W_0 behind word i of group (unit u, tile j): hidden unit n, input x; false if there is none
+  auto place = [&](int u, int j, int i, size_t& at) {
+    const int n = 16 * (wm * MPW + j) + g + ((i & 2) ? 8 : 0), x = 16 * (u0 + w0 + u) + 2 * tt + (i & 1) + ((i & 4) ? 8 : 0);
+    at = (size_t)x * N1 + n;
+    return n < N1 && x < D0;
+  };
+  // W_start of `n` groups from `first` on: all loads of a chunk on their way before the first is used
+  constexpr int kChunkG = 4;
+  auto start_groups = [&](int first, int n, float (&v)[kChunkG][8]) {
+#pragma unroll
+    for (int q = 0; q < kChunkG; ++q)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        size_t at;
+        v[q][i] = q < n && place((first + q) / MPW, (first + q) % MPW, i, at) ? snap[at] : 0.f;
+      }
+    for (uint32_t f = 0; f < t.inflight_cnt; ++f) {
+      const InflightRef ref = p.r.inflight[t.inflight_off + f];
+      const float* us = p.r.U + (size_t)ref.row * p.r.stride;
+      float x[kChunkG][8];
+#pragma unroll
+      for (int q = 0; q < kChunkG; ++q)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          size_t at;
+          x[q][i] = q < n && place((first + q) / MPW, (first + q) % MPW, i, at) ? us[at] : 0.f;
+        }
+#pragma unroll
+      for (int q = 0; q < kChunkG; ++q)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[q][i] = fmaf(-ref.eta, x[q][i], v[q][i]);
+    }
+  };
+  draw_rows(0);
+  for (int g0 = 0; g0 < wn * MPW; g0 += kChunkG) {
+    const int n = min(kChunkG, wn * MPW - g0);
+    float v[kChunkG][8], zero[8] = {};
+    start_groups(g0, n, v);
+#pragma unroll
+    for (int q = 0; q < kChunkG; ++q)
+      if (q < n) {
+        own.store(g0 + q, v[q]);
+        if (!BF) own.store(ug + g0 + q, zero);
+      }
+  }
+  own.store_wait();
+  {
+    size_t o = (size_t)D0 * N1;
+    for (int l = 0; l < nl; ++l) {
+      const int K = m.d[l], N = m.d[l + 1];
+      if (l > 0) {
+        for (int e0 = tid; e0 < K * N; e0 += 8 * kThreads) {
+          float v[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) v[q] = e0 + q * kThreads < K * N ? start_value(o + e0 + q * kThreads) : 0.f;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const int e = e0 + q * kThreads;
+            if (e < K * N) smem[m.o_w[l] + (e % N) * m.wp[l] + e / N] = v[q];
+          }
+        }
+        o += (size_t)K * N;
+      }
+      for (int e = tid; e < N; e += kThreads) bias[m.boff[l] + e] = start_value(o + e);
+      o += N;
+    }
+  }
+  __syncthreads();
+  copy_rows(0);
+
+  for (uint32_t it = 0; it < t.steps; ++it) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (it + 1 < t.steps) draw_rows(it + 1);
+    __syncthreads();   // this iteration's rows are in, the next one's numbers too; everybody is done with the last one
+    const T* X = xb0 + (it % m.xbufs) * Bp * m.xpitch;
+    if (it + 1 < t.steps) copy_rows(it + 1);
+
+    // ================= 1: this CTA's part of Z_0^T =================
+    {
+      float acc[MPW][BT][4], crs[BF ? 1 : MPW][BF ? 1 : BT][4];
+#pragma unroll
+      for (int j = 0; j < MPW; ++j)
+#pragma unroll
+        for (int b = 0; b < BT; ++b)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) { acc[j][b][c] = 0.f; if (!BF) crs[BF ? 0 : j][BF ? 0 : b][c] = 0.f; }
+      for (int u = 0; u < wn; ++u) {
+        const T* xu = X + 16 * (w0 + u);
+        FragA<BF> a[MPW][16 / kStep];
+#pragma unroll
+        for (int j = 0; j < MPW; ++j) {
+          float w[8];
+          own.load_issue(u * MPW + j, w);
+          if constexpr (BF) {
+            a[j][0].v[0] = pack_bf16(w[0], w[1]); a[j][0].v[1] = pack_bf16(w[2], w[3]);
+            a[j][0].v[2] = pack_bf16(w[4], w[5]); a[j][0].v[3] = pack_bf16(w[6], w[7]);
+          } else {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              a[j][h].v[0] = split(w[4 * h]); a[j][h].v[1] = split(w[4 * h + 2]);
+              a[j][h].v[2] = split(w[4 * h + 1]); a[j][h].v[3] = split(w[4 * h + 3]);
+            }
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 16 / kStep; ++h)
+#pragma unroll
+          for (int b = 0; b < BT; ++b)
+            if (b < bt) {
+              FragB<BF> f;
+              load_s(f, xu + 8 * b * m.xpitch + 8 * h, m.xpitch, g, tt);
+#pragma unroll
+              for (int j = 0; j < MPW; ++j) product(acc[j][b], crs[BF ? 0 : j][BF ? 0 : b], a[j][h], f);
+            }
+      }
+      if (!BF) {
+#pragma unroll
+        for (int j = 0; j < MPW; ++j)
+#pragma unroll
+          for (int b = 0; b < BT; ++b)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[j][b][c] += crs[BF ? 0 : j][BF ? 0 : b][c];
+      }
+      float* pp = part + ((wk - 1) * m.WM + wm) * MPW * bt * 128 + lane;
+      if (mine && wk > 0) {
+#pragma unroll
+        for (int j = 0; j < MPW; ++j)
+#pragma unroll
+          for (int b = 0; b < BT; ++b)
+            if (b < bt)
+#pragma unroll
+              for (int c = 0; c < 4; ++c) pp[((j * bt + b) * 4 + c) * 32] = acc[j][b][c];
+      }
+      __syncthreads();
+      if (wk == 0) {
+        for (int k = 1; k < m.WK; ++k) {
+          const float* q = part + ((k - 1) * m.WM + wm) * MPW * bt * 128 + lane;
+#pragma unroll
+          for (int j = 0; j < MPW; ++j)
+#pragma unroll
+            for (int b = 0; b < BT; ++b)
+              if (b < bt)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[j][b][c] += q[((j * bt + b) * 4 + c) * 32];
+        }
+        // rows g and g + 8 of the tile to the owners of their groups of eight
+#pragma unroll
+        for (int j = 0; j < MPW; ++j)
+#pragma unroll
+          for (int r2 = 0; r2 < 2; ++r2) {
+            const int rg = 2 * (wm * MPW + j) + r2;
+            if (rg >= 2 * m.MT) continue;
+            const uint32_t to = (uint32_t)(rg / m.rgs);
+            float* dst = inbox + ((int)rank * m.rgs * 8 + (rg % m.rgs) * 8 + g) * Bp + 2 * tt;
+            const uint32_t da = mma::peer_addr(smem_addr(dst), to), db = mma::peer_addr(smem_addr(&bars[0]), to);
+#pragma unroll
+            for (int b = 0; b < BT; ++b)
+              if (b < bt) send2(da + 32u * b, __float_as_uint(acc[j][b][2 * r2]), __float_as_uint(acc[j][b][2 * r2 + 1]), db);
+          }
+      }
+    }
+
+    // ================= 2: owned rows: sum over the CTAs, bias, ReLU; A_0 (or the logits) to every CTA =================
+    if (nrg > 0) {
+      wait(&bars[0], it & 1);
+      if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[0], in_bytes);
+      const int quads = nrg * 2;      // four rows each
+      for (int e = tid; e < quads * Bp; e += kThreads) {
+        const int q = e / Bp, b = e - q * Bp, n = 8 * rg0 + 4 * q;
+        float v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = bias[n + i];
+        for (int r = 0; r < CL; ++r)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) v[i] += inbox[(r * m.rgs * 8 + 4 * q + i) * Bp + b];
+        if (nl > 1) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) v[i] = fmaxf(v[i], 0.f);
+        }
+        // (without hidden layers these are the logits: fp32 whatever the operands)
+        if (BF && nl > 1) {
+          const uint32_t at = smem_addr(reinterpret_cast<__nv_bfloat16*>(A(0)) + b * m.ap[0] + n), lo = pack_bf16(v[0], v[1]), hi = pack_bf16(v[2], v[3]);
+          for (int r = 0; r < CL; ++r) send2(mma::peer_addr(at, r), lo, hi, mma::peer_addr(smem_addr(&bars[1]), r));
+        } else {
+          const uint32_t at = smem_addr(smem + m.o_a[0] + b * m.ap[0] + n);
+          for (int r = 0; r < CL; ++r)
+            mma::send_peer(mma::peer_addr(at, r), make_float4(v[0], v[1], v[2], v[3]), mma::peer_addr(smem_addr(&bars[1]), r));
+        }
+      }
+    }
+    wait(&bars[1], it & 1);
+    if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[1], a_bytes);
+
+    // ================= 3: narrow layers, redundantly in every CTA =================
+    for (int l = 1; l < nl; ++l) {
+      const int mt = m.np[l] / 16, K = up(m.d[l], kStep);
+      const bool last = l + 1 == nl;
+      for (int e = warp; e < mt * bt; e += kWarps) {
+        const int i = e % mt, b = e / mt;
+        float acc[4] = {}, crs[4] = {};
+        const float* w = smem + m.o_w[l] + 16 * i * m.wp[l];
+        const T* a = A(l - 1) + 8 * b * m.ap[l - 1];
+#pragma unroll 2
+        for (int k = 0; k < K; k += kStep) {
+          FragA<BF> fa;
+          FragB<BF> fb;
+          load_w(fa, w + k, m.wp[l], g, tt);
+          load_s(fb, a + k, m.ap[l - 1], g, tt);
+          product(acc, crs, fa, fb);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
+          float v = acc[c] + (BF ? 0.f : crs[c]) + bias[m.boff[l] + n];
+          if (!last) put(A(l) + s * m.ap[l] + n, fmaxf(v, 0.f));
+          else if (n < m.d[nl]) logit[s * 33 + n] = v;
+        }
+      }
+      __syncthreads();
+    }
+    {   // softmax cross-entropy: dZ = (p - onehot) / B; four lanes per sample
+      const int C = m.d[nl], s = tid >> 2, q = tid & 3;
+      const float* z = nl > 1 ? logit + s * 33 : smem + m.o_a[0] + s * m.ap[0];
+      T* dz = Z(nl - 1) + s * m.zp[nl - 1];
+      if (s < Bp) {
+        float mx = -3e38f, sum = 0.f;
+        for (int c = q; c < C; c += 4) mx = fmaxf(mx, z[c]);
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        for (int c = q; c < C; c += 4) sum += __expf(z[c] - mx);
+        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+        const float inv = 1.f / sum, fb = s < B ? 1.f / (float)B : 0.f;
+        const int y = idx[128 + (it & 1) * 64 + s];
+        for (int c = q; c < up(C, 16); c += 4) {
+          const float d = c < C ? (__expf(z[c] - mx) * inv - (c == y ? 1.f : 0.f)) * fb : 0.f;
+          put(dz + c, d);
+          if (c < C) logit[s * 33 + c] = d;   // unrounded, for the bias gradient (z of this sample has been read by its four lanes)
+        }
+      }
+    }
+    __syncthreads();
+    for (int c = warp; c < m.d[nl]; c += kWarps) {   // bias gradient of the last layer
+      float v = 0.f;
+      for (int s = lane; s < B; s += 32) v += logit[s * 33 + c];
+#pragma unroll
+      for (int k = 16; k; k >>= 1) v += __shfl_xor_sync(0xffffffffu, v, k);
+      if (lane == 0) gbias[m.boff[nl - 1] + c] = v;
+    }
+    for (int l = nl - 1; l >= 1; --l) {
+      // dZ_{l-1}^T = [A_{l-1} > 0] W_l dZ_l^T: a warp takes 16 inputs and all samples, and so has their bias gradients
+      const int mi = up(m.d[l], 16) / 16, K = up(m.d[l + 1], kStep);
+      for (int i = warp; i < mi; i += kWarps) {
+        float s0 = 0.f, s1 = 0.f;
+        for (int b = 0; b < bt; ++b) {
+          float acc[4] = {}, crs[4] = {};
+#pragma unroll 2
+          for (int k = 0; k < K; k += kStep) {
+            FragA<BF> fa;
+            FragB<BF> fb;
+            load_wt(fa, smem + m.o_w[l] + k * m.wp[l] + 16 * i, m.wp[l], g, tt);
+            load_s(fb, Z(l) + 8 * b * m.zp[l] + k, m.zp[l], g, tt);
+            product(acc, crs, fa, fb);
+          }
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
+            const float v = get(A(l - 1) + s * m.ap[l - 1] + n) > 0.f ? acc[c] + (BF ? 0.f : crs[c]) : 0.f;
+            put(Z(l - 1) + s * m.zp[l - 1] + n, v);
+            if (c & 2) s1 += v; else s0 += v;
+          }
+        }
+        s0 += __shfl_xor_sync(0xffffffffu, s0, 1); s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
+        s0 += __shfl_xor_sync(0xffffffffu, s0, 2); s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
+        if (tt == 0) { gbias[m.boff[l - 1] + 16 * i + g] = s0; gbias[m.boff[l - 1] + 16 * i + g + 8] = s1; }
+      }
+      __syncthreads();
+      // dW_l^T = dZ_l^T A_{l-1}, update
+      const int mt = m.np[l] / 16, ni = up(m.d[l], 16) / 8;
+      for (int e = warp; e < mt * ni; e += kWarps) {
+        const int i = e % mt, j = e / mt;
+        float acc[4] = {}, crs[4] = {};
+#pragma unroll 2
+        for (int k = 0; k < Bp; k += kStep) {
+          FragA<BF> fa;
+          FragB<BF> fb;
+          load_zt(fa, Z(l) + k * m.zp[l] + 16 * i, m.zp[l], lane);
+          load_st(fb, A(l - 1) + k * m.ap[l - 1] + 8 * j, m.ap[l - 1], lane);
+          product(acc, crs, fa, fb);
+        }
+#pragma unroll
+        for (int r2 = 0; r2 < 2; ++r2) {
+          const int at = (16 * i + g + 8 * r2) * m.wp[l] + 8 * j + 2 * tt;
+          float2* w = reinterpret_cast<float2*>(smem + m.o_w[l] + at);
+          float2* u = reinterpret_cast<float2*>(smem + m.o_u[l] + at);
+          float2 wv = *w, uv = *u;
+          const float g0 = fmaf(lambda, wv.x, acc[2 * r2] + (BF ? 0.f : crs[2 * r2])), g1 = fmaf(lambda, wv.y, acc[2 * r2 + 1] + (BF ? 0.f : crs[2 * r2 + 1]));
+          wv.x = fmaf(-eta, g0, wv.x); wv.y = fmaf(-eta, g1, wv.y);
+          uv.x += g0; uv.y += g1;
+          *w = wv; *u = uv;
+        }
+      }
+    }
+    // biases: every layer's gradient is in (the barriers above lie between)
+    if (nl == 1) __syncthreads();
+    for (int l = 0; l < nl; ++l)
+      for (int e = tid; e < m.d[l + 1]; e += kThreads) {
+        const float gb = gbias[m.boff[l] + e];
+        bias[m.boff[l] + e] = fmaf(-eta, gb, bias[m.boff[l] + e]);
+        ubias[m.boff[l] + e] += gb;
+      }
+
+    // ================= 4: dW_0^T over this CTA's inputs, update in place =================
+    if (wn > 0) {
+      constexpr int kBk = 8 * BT / kStep;   // k-steps over the samples at most
+      FragA<BF> a[MPW][BF ? kBk : 1];
+      if (BF) {
+#pragma unroll
+        for (int j = 0; j < MPW; ++j)
+#pragma unroll
+          for (int k = 0; k < kBk; ++k)
+            if (k * kStep < Bp) load_zt(a[j][BF ? k : 0], Z(0) + k * kStep * m.zp[0] + 16 * (wm * MPW + j), m.zp[0], lane);
+      }
+      for (int u = 0; u < wn; ++u) {
+        const T* xu = X + 16 * (w0 + u);
+        float acc[MPW][2][4] = {}, crs[MPW][2][4] = {};
+#pragma unroll
+        for (int k = 0; k < kBk; ++k)
+          if (k * kStep < Bp) {
+            if (!BF) {
+#pragma unroll
+              for (int j = 0; j < MPW; ++j) load_zt(a[j][0], Z(0) + k * kStep * m.zp[0] + 16 * (wm * MPW + j), m.zp[0], lane);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              FragB<BF> f;
+              load_st(f, xu + k * kStep * m.xpitch + 8 * h, m.xpitch, lane);
+#pragma unroll
+              for (int j = 0; j < MPW; ++j) product(acc[j][h], crs[j][h], a[j][BF ? k : 0], f);
+            }
+          }
+#pragma unroll
+        for (int j = 0; j < MPW; ++j) {
+          float w[8], us[8];
+          own.load_issue(u * MPW + j, w);
+          if (!BF) own.load_issue(ug + u * MPW + j, us);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float gr = fmaf(lambda, w[i], acc[j][i >> 2][i & 3] + (BF ? 0.f : crs[j][i >> 2][i & 3]));
+            w[i] = fmaf(-eta, gr, w[i]);
+            if (!BF) us[i] += gr;
+          }
+          own.store(u * MPW + j, w);
+          if (!BF) own.store(ug + u * MPW + j, us);
+        }
+      }
+      own.store_wait();
+    }
+  }
+
+  // ---- event trigger: h reached s_{i,c}; publish U_i (and the end model) ----
+  __syncthreads();
+  {
+    // a round whose hand-overs gave up leaves NaN behind as well as the status bit
+    const float bad = ok ? 0.f : __int_as_float(0x7FFFFFFF);
+    float* Urow = p.r.U + (size_t)t.u_row * p.r.stride;
+    float* wrow = p.r.w_end ? p.r.w_end + (size_t)t.u_row * p.r.stride : nullptr;
+    const float inv_eta = 1.f / eta;
+    for (int g0 = 0; g0 < wn * MPW; g0 += kChunkG) {
+      const int n = min(kChunkG, wn * MPW - g0);
+      float us[kChunkG][8];
+      if (BF) start_groups(g0, n, us);
+#pragma unroll
+      for (int q = 0; q < kChunkG; ++q)
+        if (q < n) {
+          float w[8];
+          own.load_issue(g0 + q, w);
+          if (!BF) own.load_issue(ug + g0 + q, us[q]);
+          else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) us[q][i] = (us[q][i] - w[i]) * inv_eta;
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            size_t at;
+            if (!place((g0 + q) / MPW, (g0 + q) % MPW, i, at)) continue;
+            Urow[at] = us[q][i] + bad;
+            if (wrow) wrow[at] = w[i] + bad;
+          }
+        }
+    }
+    if (rank == 0) {
+      size_t o = (size_t)D0 * N1;
+      for (int l = 0; l < nl; ++l) {
+        const int K = m.d[l], N = m.d[l + 1];
+        if (l > 0) {
+          for (int e = tid; e < K * N; e += kThreads) {
+            const int at = (e % N) * m.wp[l] + e / N;
+            Urow[o + e] = smem[m.o_u[l] + at] + bad;
+            if (wrow) wrow[o + e] = smem[m.o_w[l] + at] + bad;
+          }
+          o += (size_t)K * N;
+        }
+        for (int e = tid; e < N; e += kThreads) {
+          Urow[o + e] = ubias[m.boff[l] + e] + bad;
+          if (wrow) wrow[o + e] = bias[m.boff[l] + e] + bad;
+        }
+        o += N;
+      }
+    }
+  }
+  if (!ok && p.r.status && lane == 0) atomicOr(p.r.status, 1u);
+  if (tid == 0 && rank == 0) {
+    TriggerRec rec;
+    rec.client = t.client; rec.round = t.round; rec.samples_done = t.steps * (uint32_t)B; rec.flags = 1;
+    p.r.trig[t.seq] = rec;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if (CL > 1) mma::cluster_sync(); else __syncthreads();   // no CTA leaves while a peer may still send to it
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(*tmem_at) : "memory");
+}
+
+template <bool BF, int MPW, int BT>
+cudaError_t launch(const MmaLaunch& p, cudaStream_t s) {
+  const size_t smem = (size_t)p.m.total * sizeof(float);
+  cudaError_t e = cudaFuncSetAttribute(mlp_mma_kernel<BF, MPW, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(p.r.n_tasks * p.m.CL, 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = p.m.CL;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = p.m.CL > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, mlp_mma_kernel<BF, MPW, BT>, p);
+}
+
+// The widest cluster that leaves every round-task of the launch its own SMs; where none does, the smallest that holds
+// the first layer.
+MmaPlan pick_plan(const MlpShape& s, uint32_t n_tasks, uint32_t sms) {
+  MmaPlan last{};
+  for (int cl = 8; cl >= 1; cl >>= 1) {
+    const MmaPlan p = make_plan(s, cl);
+    if (!p.total) continue;
+    last = p;
+    if (n_tasks * cl <= sms) return p;
+  }
+  return last;
+}
+
+}  // namespace
+
+bool mlp_mma_eligible(const MlpShape& shape) {
+  for (int cl = 8; cl >= 1; cl >>= 1)
+    if (make_plan(shape, cl).total) return true;
+  return false;
+}
+
+cudaError_t launch_mlp_mma_rounds(const MlpLaunch& p, cudaStream_t s) {
+  int sms = 0, dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  MmaLaunch q;
+  q.r = p.r;
+  q.m = pick_plan(p.shape, p.r.n_tasks, (uint32_t)sms);
+  if (!q.m.total) return cudaErrorInvalidConfiguration;
+  const bool small = q.m.bt <= 4;
+  if (p.shape.precision == 0) return small ? launch<false, 1, 4>(q, s) : launch<false, 1, 8>(q, s);
+  if (q.m.MT <= 8) return small ? launch<true, 1, 4>(q, s) : launch<true, 1, 8>(q, s);
+  return small ? launch<true, 2, 4>(q, s) : launch<true, 2, 8>(q, s);
+}
+
+}  // namespace aet
