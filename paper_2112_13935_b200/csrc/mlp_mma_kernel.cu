@@ -23,7 +23,7 @@
 // tiles; at 16-64 samples per iteration the warp-level instructions' rate (1,024 bf16 / 512 tf32 multiply-adds per clock
 // and SM) is not what limits a round: hand-overs, updates and the narrow layers are.
 //
-// precision 1: the update sum of W_0 is (W_start - W_end) / eta; everything else accumulates U.
+// precision 1: the update sums of the weights are (W_start - W_end) / eta; everything else accumulates U.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -56,7 +56,7 @@ struct MmaPlan {
   int ap[kMaxL], zp[kMaxL], wp[kMaxL], np[kMaxL];   // pitches of A_l, dZ_l, W_l (l >= 1), padded rows of W_l
   int ext;                          // words per thread beyond tensor memory
   // offsets in floats
-  int o_x, o_in, o_part, o_a[kMaxL], o_z[kMaxL], o_w[kMaxL], o_u[kMaxL], o_b, o_ub, o_gb, o_logit, o_ext, o_idx, o_bar, total;
+  int o_x, o_in, o_part, o_a[kMaxL], o_z[kMaxL], o_w[kMaxL], o_u[kMaxL], o_b, o_ub, o_gb, o_gb2, nb, o_logit, o_ext, o_idx, o_bar, total;
   int boff[kMaxL];                  // of layer l's biases in the bias arrays
 };
 
@@ -73,15 +73,14 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
   p.bt = p.Bp / 8;
   p.CL = cl;
   p.MT = (p.d[1] + 15) / 16;
-  const int mpw = (p.MT + 7) / 8;
   if (p.B > 64 || p.MT > 16 || (!bf && (p.MT > 8)) || p.d[p.nl] > 32 || (bf && p.d[0] % 8)) return p;
-  p.WM = (p.MT + mpw - 1) / mpw;
+  p.WM = p.MT;
   p.WK = kWarps / p.WM;
   p.units = (p.d[0] + 15) / 16;
   p.upc = (p.units + cl - 1) / cl;
   p.upw = (p.upc + p.WK - 1) / p.WK;
   if (cl > 1 && p.upc * (cl - 1) >= p.units) return p;   // the last CTA would have nothing
-  const int words = p.upw * mpw * 8 * (bf ? 1 : 2);
+  const int words = p.upw * 8 * (bf ? 1 : 2);
   p.ext = words > kTmemWords ? words - kTmemWords : 0;
   p.rgs = (2 * p.MT + cl - 1) / cl;
   int o = 0;
@@ -93,7 +92,7 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
   p.o_idx = take(4 * 64);
   p.o_x = take(p.xbufs * p.Bp * p.xpitch / elems);
   p.o_in = take(cl * p.rgs * 8 * p.Bp);
-  int part = (p.WK - 1) * p.WM * mpw * p.bt * 128;
+  const int part = (p.WK - 1) * p.WM * p.bt * 128;
   for (int l = 0; l < p.nl; ++l) {
     const int n = up(p.d[l + 1], 16);
     p.ap[l] = p.zp[l] = n + 8;
@@ -104,15 +103,16 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
       p.wp[l] = up(p.d[l], 16) + 8;
       p.np[l] = n;
       p.o_w[l] = take(n * p.wp[l]);
-      p.o_u[l] = take(n * p.wp[l]);
+      if (!bf) p.o_u[l] = take(n * p.wp[l]);
     }
   }
   // dZ_0 and the partial products of the input parts are never needed at the same time
-  const int z0 = p.Bp * p.zp[0] / elems;
-  p.o_part = p.o_z[0] = take(part > z0 ? part : z0);
+  const int z0 = up(p.Bp * p.zp[0], elems) / elems, least = kWarps * 128;
+  p.o_part = p.o_z[0] = take(part > z0 ? (part > least ? part : least) : (z0 > least ? z0 : least));
   int nb = 0;
   for (int l = 0; l < p.nl; ++l) { p.boff[l] = nb; nb += up(p.d[l + 1], 16); }
-  p.o_b = take(nb); p.o_ub = take(nb); p.o_gb = take(nb);
+  p.nb = nb;
+  p.o_b = take(nb); p.o_ub = take(nb); p.o_gb = take(nb); p.o_gb2 = take(nb);
   p.o_logit = take(p.Bp * 33);
   p.o_ext = take(p.ext * kThreads);
   p.total = o;
@@ -146,15 +146,24 @@ template <bool BF> struct FragB;
 template <> struct FragB<false> { Split v[2]; };
 template <> struct FragB<true> { uint32_t v[2]; };
 
-// d += a b; fp32: the two cross terms into x (which may be d itself)
-__device__ __forceinline__ void product(float (&d)[4], float (&x)[4], const FragA<false>& a, const FragB<false>& b) {
-  mma::tf32(x, a.v[0].lo, a.v[1].lo, a.v[2].lo, a.v[3].lo, b.v[0].hi, b.v[1].hi);
-  mma::tf32(x, a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].lo, b.v[1].lo);
-  mma::tf32(d, a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].hi, b.v[1].hi);
+// d[i] += a b[i] for N column tiles; fp32: the two cross terms into x1 and x2.  Term by term, so that no
+// instruction waits for the one before it.
+template <int N>
+__device__ __forceinline__ void products(float (&d)[N][4], float (&x1)[N][4], float (&x2)[N][4], const FragA<false>& a, const FragB<false> (&b)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma::tf32(d[i], a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b[i].v[0].hi, b[i].v[1].hi);
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma::tf32(x1[i], a.v[0].lo, a.v[1].lo, a.v[2].lo, a.v[3].lo, b[i].v[0].hi, b[i].v[1].hi);
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma::tf32(x2[i], a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b[i].v[0].lo, b[i].v[1].lo);
 }
-__device__ __forceinline__ void product(float (&d)[4], float (&)[4], const FragA<true>& a, const FragB<true>& b) {
-  mma_bf16(d, a.v, b.v[0], b.v[1]);
+template <int N>
+__device__ __forceinline__ void products(float (&d)[N][4], float (&)[N][4], float (&)[N][4], const FragA<true>& a, const FragB<true> (&b)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma_bf16(d[i], a.v, b[i].v[0], b[i].v[1]);
 }
+// the sum over the terms of one entry
+template <bool BF> __device__ __forceinline__ float term(float d, float x1, float x2) { return BF ? d : d + (x1 + x2); }
 
 template <bool BF> struct Elem { typedef float T; static constexpr int kStep = 8; };
 template <> struct Elem<true> { typedef __nv_bfloat16 T; static constexpr int kStep = 16; };
@@ -210,6 +219,16 @@ __device__ __forceinline__ void load_st(FragB<true>& f, const __nv_bfloat16* x, 
   const int r = lane & 15;
   ldmatrix2t(f.v, smem_addr(x + r * pitch));
 }
+// ... two column tiles side by side
+__device__ __forceinline__ void load_st2(FragB<false> (&f)[2], const float* x, int pitch, int lane) {
+  load_st(f[0], x, pitch, lane);
+  load_st(f[1], x + 8, pitch, lane);
+}
+__device__ __forceinline__ void load_st2(FragB<true> (&f)[2], const __nv_bfloat16* x, int pitch, int lane) {
+  uint32_t r[4];
+  ldmatrix4t(r, smem_addr(x + (lane & 15) * pitch + (lane >> 4) * 8));
+  f[0].v[0] = r[0]; f[0].v[1] = r[1]; f[1].v[0] = r[2]; f[1].v[1] = r[3];
+}
 __device__ __forceinline__ void put(float* p, float v) { *p = v; }
 __device__ __forceinline__ void put(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
 __device__ __forceinline__ float get(const float* p) { return *p; }
@@ -219,18 +238,22 @@ __device__ __forceinline__ float get(const __nv_bfloat16* p) { return __bfloat16
 struct Own {
   uint32_t tmem;     // this thread's lane and first column
   float* ext;        // word i at ext[i * kThreads]
-  __device__ __forceinline__ void load_issue(int group, float (&v)[8]) const {
+  // the words of a group; they may be used after wait() (other work goes between the two)
+  __device__ __forceinline__ void issue(int group, uint32_t (&r)[8]) const {
     if (group < kTmemWords / 8) {
-      uint32_t r[8];
-      asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\ttcgen05.wait::ld.sync.aligned;"
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                    : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                    : "r"(tmem + 8u * group) : "memory");
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
     } else {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = ext[(8 * group - kTmemWords + i) * kThreads];
+      for (int i = 0; i < 8; ++i) r[i] = __float_as_uint(ext[(8 * group - kTmemWords + i) * kThreads]);
     }
+  }
+  __device__ __forceinline__ void wait(uint32_t (&r)[8], float (&v)[8]) const {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]) : : "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
   }
   __device__ __forceinline__ void store(int group, const float (&v)[8]) const {
     if (group < kTmemWords / 8) {
@@ -255,13 +278,16 @@ struct MmaLaunch {
   MmaPlan m;
 };
 
-template <bool BF, int MPW, int BT>
+template <bool BF, int BT>
 __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_constant__ MmaLaunch p) {
   typedef typename Elem<BF>::T T;
   constexpr int kStep = Elem<BF>::kStep;
   extern __shared__ __align__(128) float smem[];
   const MmaPlan& m = p.m;
-  const int CL = m.CL, B = m.B, Bp = m.Bp, bt = m.bt, nl = m.nl, N1 = m.d[1], D0 = m.d[0];
+  // the number of sample tiles is a constant: run-time guards around single instructions cut the code into blocks of
+  // one instruction each (three times slower)
+  constexpr int bt = BT, Bp = 8 * BT;
+  const int CL = m.CL, B = m.B, nl = m.nl, N1 = m.d[1], D0 = m.d[0];
 
   const TaskDesc t = p.r.tasks[p.r.task_begin + blockIdx.x / CL];
   if (!debug_task_ok(p.r, t)) return;   // the whole cluster alike
@@ -318,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   Own own;
   own.tmem = *tmem_at + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * kTmemWords;
   own.ext = smem + m.o_ext + tid;
-  const int ug = m.upw * MPW;   // first group of the update sum (fp32)
+  const int ug = m.upw;   // first group of the update sum (fp32)
 
   bool ok = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) {
@@ -336,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     if (tid < B) {
       const uint32_t id = sample_index(draw(key, t.sample_ctr0 + (uint64_t)it * B + tid), cd.n);
       idx[(it & 1) * 64 + tid] = (int)id;
-      idx[128 + (it & 1) * 64 + tid] = __ldg(cd.y + id);
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(idx + 128 + (it & 1) * 64 + tid)), "l"(cd.y + id) : "memory");
     }
   };
   constexpr int kChunk = 16 / (int)sizeof(T);
@@ -366,9 +392,9 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     }
     return v;
   };
-  // Parameter of W_0 behind word i of group (unit u, tile j): hidden unit n, input x; false if there is none
-  auto place = [&](int u, int j, int i, size_t& at) {
-    const int n = 16 * (wm * MPW + j) + g + ((i & 2) ? 8 : 0), x = 16 * (u0 + w0 + u) + 2 * tt + (i & 1) + ((i & 4) ? 8 : 0);
+  // Parameter of W_0 behind word i of group (unit) u: hidden unit n, input x; false if there is none
+  auto place = [&](int u, int i, size_t& at) {
+    const int n = 16 * wm + g + ((i & 2) ? 8 : 0), x = 16 * (u0 + w0 + u) + 2 * tt + (i & 1) + ((i & 4) ? 8 : 0);
     at = (size_t)x * N1 + n;
     return n < N1 && x < D0;
   };
@@ -380,7 +406,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         size_t at;
-        v[q][i] = q < n && place((first + q) / MPW, (first + q) % MPW, i, at) ? snap[at] : 0.f;
+        v[q][i] = q < n && place(first + q, i, at) ? snap[at] : 0.f;
       }
     for (uint32_t f = 0; f < t.inflight_cnt; ++f) {
       const InflightRef ref = p.r.inflight[t.inflight_off + f];
@@ -391,7 +417,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           size_t at;
-          x[q][i] = q < n && place((first + q) / MPW, (first + q) % MPW, i, at) ? us[at] : 0.f;
+          x[q][i] = q < n && place(first + q, i, at) ? us[at] : 0.f;
         }
 #pragma unroll
       for (int q = 0; q < kChunkG; ++q)
@@ -400,8 +426,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     }
   };
   draw_rows(0);
-  for (int g0 = 0; g0 < wn * MPW; g0 += kChunkG) {
-    const int n = min(kChunkG, wn * MPW - g0);
+  for (int g0 = 0; g0 < wn; g0 += kChunkG) {
+    const int n = min(kChunkG, wn - g0);
     float v[kChunkG][8], zero[8] = {};
     start_groups(g0, n, v);
 #pragma unroll
@@ -436,6 +462,17 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   __syncthreads();
   copy_rows(0);
 
+  // Where this warp's rows g and g + 8 of Z_0 go: their owners' inboxes and barriers (warps of the first input part).
+  uint32_t row_at[2], row_bar[2];
+#pragma unroll
+  for (int r2 = 0; r2 < 2; ++r2) {
+    const int rg = min(2 * wm + r2, 2 * m.MT - 1);
+    const uint32_t to = (uint32_t)(rg / m.rgs);
+    row_at[r2] = mma::peer_addr(smem_addr(inbox + ((int)rank * m.rgs * 8 + (rg % m.rgs) * 8 + g) * Bp + 2 * tt), to);
+    row_bar[r2] = mma::peer_addr(smem_addr(&bars[0]), to);
+  }
+  const int own_q = tid / Bp, own_b = tid - own_q * Bp;   // this thread's four owned rows and sample in step 2
+
   for (uint32_t it = 0; it < t.steps; ++it) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (it + 1 < t.steps) draw_rows(it + 1);
@@ -445,86 +482,68 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
 
     // ================= 1: this CTA's part of Z_0^T =================
     {
-      float acc[MPW][BT][4], crs[BF ? 1 : MPW][BF ? 1 : BT][4];
+      float acc[BT][4], crs[BT][4];
 #pragma unroll
-      for (int j = 0; j < MPW; ++j)
+      for (int b = 0; b < BT; ++b)
 #pragma unroll
-        for (int b = 0; b < BT; ++b)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) { acc[j][b][c] = 0.f; if (!BF) crs[BF ? 0 : j][BF ? 0 : b][c] = 0.f; }
+        for (int c = 0; c < 4; ++c) { acc[b][c] = 0.f; crs[b][c] = 0.f; }
       for (int u = 0; u < wn; ++u) {
         const T* xu = X + 16 * (w0 + u);
-        FragA<BF> a[MPW][16 / kStep];
+        uint32_t r[8];
+        float w[8];
+        own.issue(u, r);
+        FragB<BF> f[BT];
 #pragma unroll
-        for (int j = 0; j < MPW; ++j) {
-          float w[8];
-          own.load_issue(u * MPW + j, w);
+        for (int b = 0; b < BT; ++b)
+          load_s(f[b], xu + 8 * b * m.xpitch, m.xpitch, g, tt);
+        own.wait(r, w);
+#pragma unroll
+        for (int h = 0; h < 16 / kStep; ++h) {
+          FragA<BF> a;
           if constexpr (BF) {
-            a[j][0].v[0] = pack_bf16(w[0], w[1]); a[j][0].v[1] = pack_bf16(w[2], w[3]);
-            a[j][0].v[2] = pack_bf16(w[4], w[5]); a[j][0].v[3] = pack_bf16(w[6], w[7]);
+            a.v[0] = pack_bf16(w[0], w[1]); a.v[1] = pack_bf16(w[2], w[3]);
+            a.v[2] = pack_bf16(w[4], w[5]); a.v[3] = pack_bf16(w[6], w[7]);
           } else {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              a[j][h].v[0] = split(w[4 * h]); a[j][h].v[1] = split(w[4 * h + 2]);
-              a[j][h].v[2] = split(w[4 * h + 1]); a[j][h].v[3] = split(w[4 * h + 3]);
-            }
+            a.v[0] = split(w[4 * h]); a.v[1] = split(w[4 * h + 2]);
+            a.v[2] = split(w[4 * h + 1]); a.v[3] = split(w[4 * h + 3]);
           }
+          if (h) {
+#pragma unroll
+            for (int b = 0; b < BT; ++b)
+              load_s(f[b], xu + 8 * b * m.xpitch + 8 * h, m.xpitch, g, tt);
+          }
+          products(acc, crs, crs, a, f);
         }
-#pragma unroll
-        for (int h = 0; h < 16 / kStep; ++h)
-#pragma unroll
-          for (int b = 0; b < BT; ++b)
-            if (b < bt) {
-              FragB<BF> f;
-              load_s(f, xu + 8 * b * m.xpitch + 8 * h, m.xpitch, g, tt);
-#pragma unroll
-              for (int j = 0; j < MPW; ++j) product(acc[j][b], crs[BF ? 0 : j][BF ? 0 : b], a[j][h], f);
-            }
       }
       if (!BF) {
 #pragma unroll
-        for (int j = 0; j < MPW; ++j)
+        for (int b = 0; b < BT; ++b)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[b][c] += crs[b][c];
+      }
+      if (m.WK > 1) {
+        if (mine && wk > 0) {
+          float* pp = part + ((wk - 1) * m.WM + wm) * bt * 128 + lane;
 #pragma unroll
           for (int b = 0; b < BT; ++b)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[j][b][c] += crs[BF ? 0 : j][BF ? 0 : b][c];
+              for (int c = 0; c < 4; ++c) pp[(b * 4 + c) * 32] = acc[b][c];
+        }
+        __syncthreads();
       }
-      float* pp = part + ((wk - 1) * m.WM + wm) * MPW * bt * 128 + lane;
-      if (mine && wk > 0) {
-#pragma unroll
-        for (int j = 0; j < MPW; ++j)
-#pragma unroll
-          for (int b = 0; b < BT; ++b)
-            if (b < bt)
-#pragma unroll
-              for (int c = 0; c < 4; ++c) pp[((j * bt + b) * 4 + c) * 32] = acc[j][b][c];
-      }
-      __syncthreads();
       if (wk == 0) {
         for (int k = 1; k < m.WK; ++k) {
-          const float* q = part + ((k - 1) * m.WM + wm) * MPW * bt * 128 + lane;
+          const float* q = part + ((k - 1) * m.WM + wm) * bt * 128 + lane;
 #pragma unroll
-          for (int j = 0; j < MPW; ++j)
+          for (int b = 0; b < BT; ++b)
 #pragma unroll
-            for (int b = 0; b < BT; ++b)
-              if (b < bt)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) acc[j][b][c] += q[((j * bt + b) * 4 + c) * 32];
+              for (int c = 0; c < 4; ++c) acc[b][c] += q[(b * 4 + c) * 32];
         }
-        // rows g and g + 8 of the tile to the owners of their groups of eight
 #pragma unroll
-        for (int j = 0; j < MPW; ++j)
+        for (int r2 = 0; r2 < 2; ++r2)
 #pragma unroll
-          for (int r2 = 0; r2 < 2; ++r2) {
-            const int rg = 2 * (wm * MPW + j) + r2;
-            if (rg >= 2 * m.MT) continue;
-            const uint32_t to = (uint32_t)(rg / m.rgs);
-            float* dst = inbox + ((int)rank * m.rgs * 8 + (rg % m.rgs) * 8 + g) * Bp + 2 * tt;
-            const uint32_t da = mma::peer_addr(smem_addr(dst), to), db = mma::peer_addr(smem_addr(&bars[0]), to);
-#pragma unroll
-            for (int b = 0; b < BT; ++b)
-              if (b < bt) send2(da + 32u * b, __float_as_uint(acc[j][b][2 * r2]), __float_as_uint(acc[j][b][2 * r2 + 1]), db);
-          }
+          for (int b = 0; b < BT; ++b)
+            send2(row_at[r2] + 32u * b, __float_as_uint(acc[b][2 * r2]), __float_as_uint(acc[b][2 * r2 + 1]), row_bar[r2]);
       }
     }
 
@@ -532,27 +551,29 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     if (nrg > 0) {
       wait(&bars[0], it & 1);
       if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[0], in_bytes);
-      const int quads = nrg * 2;      // four rows each
-      for (int e = tid; e < quads * Bp; e += kThreads) {
-        const int q = e / Bp, b = e - q * Bp, n = 8 * rg0 + 4 * q;
-        float v[4];
+      int q = own_q, b = own_b;
+      for (int e = tid; e < nrg * 2 * Bp; e += kThreads) {
+        if (e >= kThreads) { q = e / Bp; b = e - q * Bp; }
+        const int n = 8 * rg0 + 4 * q;
+        const float4 b4 = *reinterpret_cast<const float4*>(bias + n);
+        float v[4] = {b4.x, b4.y, b4.z, b4.w};
+        const float* in = inbox + 4 * q * Bp + b;
+#pragma unroll 4
+        for (int r = 0; r < CL; ++r, in += m.rgs * 8 * Bp)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = bias[n + i];
-        for (int r = 0; r < CL; ++r)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) v[i] += inbox[(r * m.rgs * 8 + 4 * q + i) * Bp + b];
+          for (int i = 0; i < 4; ++i) v[i] += in[i * Bp];
         if (nl > 1) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) v[i] = fmaxf(v[i], 0.f);
         }
         // (without hidden layers these are the logits: fp32 whatever the operands)
+        const uint32_t bar = smem_addr(&bars[1]);
         if (BF && nl > 1) {
           const uint32_t at = smem_addr(reinterpret_cast<__nv_bfloat16*>(A(0)) + b * m.ap[0] + n), lo = pack_bf16(v[0], v[1]), hi = pack_bf16(v[2], v[3]);
-          for (int r = 0; r < CL; ++r) send2(mma::peer_addr(at, r), lo, hi, mma::peer_addr(smem_addr(&bars[1]), r));
+          for (int r = 0; r < CL; ++r) send2(mma::peer_addr(at, r), lo, hi, mma::peer_addr(bar, r));
         } else {
           const uint32_t at = smem_addr(smem + m.o_a[0] + b * m.ap[0] + n);
-          for (int r = 0; r < CL; ++r)
-            mma::send_peer(mma::peer_addr(at, r), make_float4(v[0], v[1], v[2], v[3]), mma::peer_addr(smem_addr(&bars[1]), r));
+          for (int r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(at, r), make_float4(v[0], v[1], v[2], v[3]), mma::peer_addr(bar, r));
         }
       }
     }
@@ -561,54 +582,83 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
 
     // ================= 3: narrow layers, redundantly in every CTA =================
     for (int l = 1; l < nl; ++l) {
-      const int mt = m.np[l] / 16, K = up(m.d[l], kStep);
+      const int mt = m.np[l] / 16, ks = up(m.d[l], kStep) / kStep, items = mt * bt;
       const bool last = l + 1 == nl;
-      for (int e = warp; e < mt * bt; e += kWarps) {
-        const int i = e % mt, b = e / mt;
-        float acc[4] = {}, crs[4] = {};
+      // few output tiles: several warps share one, each with its part of the inputs.  (The area of the partial Z_0 is
+      // free: A_0 is complete, so every part has been sent.)
+      const int kp = items >= kWarps ? 1 : min(kWarps / items, ks);
+      for (int e = warp; e < items * kp; e += kWarps) {
+        const int part_k = e / items, i = (e % items) % mt, b = (e % items) / mt;
+        float acc[1][4] = {}, x1[1][4] = {}, x2[1][4] = {};
         const float* w = smem + m.o_w[l] + 16 * i * m.wp[l];
         const T* a = A(l - 1) + 8 * b * m.ap[l - 1];
-#pragma unroll 2
-        for (int k = 0; k < K; k += kStep) {
+        const int k1 = ks * (part_k + 1) / kp;
+#pragma unroll 4
+        for (int k = ks * part_k / kp; k < k1; ++k) {
           FragA<BF> fa;
-          FragB<BF> fb;
-          load_w(fa, w + k, m.wp[l], g, tt);
-          load_s(fb, a + k, m.ap[l - 1], g, tt);
-          product(acc, crs, fa, fb);
+          FragB<BF> fb[1];
+          load_w(fa, w + k * kStep, m.wp[l], g, tt);
+          load_s(fb[0], a + k * kStep, m.ap[l - 1], g, tt);
+          products(acc, x1, x2, fa, fb);
+        }
+        if (kp > 1) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) part[e * 128 + c * 32 + lane] = term<BF>(acc[0][c], x1[0][c], x2[0][c]);
+          continue;
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
-          float v = acc[c] + (BF ? 0.f : crs[c]) + bias[m.boff[l] + n];
+          const float v = term<BF>(acc[0][c], x1[0][c], x2[0][c]) + bias[m.boff[l] + n];
           if (!last) put(A(l) + s * m.ap[l] + n, fmaxf(v, 0.f));
           else if (n < m.d[nl]) logit[s * 33 + n] = v;
         }
       }
       __syncthreads();
+      if (kp > 1) {
+        for (int e = tid; e < items * 128; e += kThreads) {
+          const int item = e >> 7, c = (e >> 5) & 3, i = item % mt, b = item / mt;
+          const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
+          float v = bias[m.boff[l] + n];
+          for (int k = 0; k < kp; ++k) v += part[k * items * 128 + e];
+          if (!last) put(A(l) + s * m.ap[l] + n, fmaxf(v, 0.f));
+          else if (n < m.d[nl]) logit[s * 33 + n] = v;
+        }
+        __syncthreads();
+      }
     }
     {   // softmax cross-entropy: dZ = (p - onehot) / B; four lanes per sample
       const int C = m.d[nl], s = tid >> 2, q = tid & 3;
-      const float* z = nl > 1 ? logit + s * 33 : smem + m.o_a[0] + s * m.ap[0];
-      T* dz = Z(nl - 1) + s * m.zp[nl - 1];
       if (s < Bp) {
-        float mx = -3e38f, sum = 0.f;
-        for (int c = q; c < C; c += 4) mx = fmaxf(mx, z[c]);
+        const float* z = nl > 1 ? logit + s * 33 : smem + m.o_a[0] + s * m.ap[0];
+        T* dz = Z(nl - 1) + s * m.zp[nl - 1];
+        float v[8], mx = -3e38f, sum = 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          v[i] = q + 4 * i < C ? z[q + 4 * i] : -3e38f;
+          mx = fmaxf(mx, v[i]);
+        }
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        for (int c = q; c < C; c += 4) sum += __expf(z[c] - mx);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (4 * i < C) { v[i] = lr::ex2((v[i] - mx) * lr::kLog2e); sum += v[i]; }
         sum += __shfl_xor_sync(0xffffffffu, sum, 1);
         sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-        const float inv = 1.f / sum, fb = s < B ? 1.f / (float)B : 0.f;
+        const float fb = s < B ? 1.f / (float)B : 0.f, inv = lr::rcp(sum);
         const int y = idx[128 + (it & 1) * 64 + s];
-        for (int c = q; c < up(C, 16); c += 4) {
-          const float d = c < C ? (__expf(z[c] - mx) * inv - (c == y ? 1.f : 0.f)) * fb : 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int c = q + 4 * i;
+          if (4 * i >= up(C, 16)) continue;
+          const float d = c < C ? (v[i] * inv - (c == y ? 1.f : 0.f)) * fb : 0.f;
           put(dz + c, d);
-          if (c < C) logit[s * 33 + c] = d;   // unrounded, for the bias gradient (z of this sample has been read by its four lanes)
+          if (c < C) logit[s * 33 + c] = d;   // unrounded, for the bias gradient (the four lanes have read the sample's logits)
         }
       }
     }
     __syncthreads();
-    for (int c = warp; c < m.d[nl]; c += kWarps) {   // bias gradient of the last layer
+    for (int c = kWarps - 1 - warp; c < m.d[nl]; c += kWarps) {   // bias gradient of the last layer
       float v = 0.f;
       for (int s = lane; s < B; s += 32) v += logit[s * 33 + c];
 #pragma unroll
@@ -616,110 +666,116 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       if (lane == 0) gbias[m.boff[nl - 1] + c] = v;
     }
     for (int l = nl - 1; l >= 1; --l) {
-      // dZ_{l-1}^T = [A_{l-1} > 0] W_l dZ_l^T: a warp takes 16 inputs and all samples, and so has their bias gradients
+      // dZ_{l-1}^T = [A_{l-1} > 0] W_l dZ_l^T: a warp takes 16 inputs and all samples, or half of them, and so has its
+      // share of their bias gradients
       const int mi = up(m.d[l], 16) / 16, K = up(m.d[l + 1], kStep);
-      for (int i = warp; i < mi; i += kWarps) {
+      constexpr int kHalf = BT % 2 == 0 ? BT / 2 : BT;
+      const int halves = BT / kHalf;
+      for (int e = warp; e < mi * halves; e += kWarps) {
+        const int i = e % mi, half = e / mi, b0 = half * kHalf;
         float s0 = 0.f, s1 = 0.f;
-        for (int b = 0; b < bt; ++b) {
-          float acc[4] = {}, crs[4] = {};
-#pragma unroll 2
-          for (int k = 0; k < K; k += kStep) {
-            FragA<BF> fa;
-            FragB<BF> fb;
-            load_wt(fa, smem + m.o_w[l] + k * m.wp[l] + 16 * i, m.wp[l], g, tt);
-            load_s(fb, Z(l) + 8 * b * m.zp[l] + k, m.zp[l], g, tt);
-            product(acc, crs, fa, fb);
-          }
+        float acc[kHalf][4] = {}, crs[kHalf][4] = {};
+        for (int k = 0; k < K; k += kStep) {
+          FragA<BF> fa;
+          FragB<BF> fb[kHalf];
+          load_wt(fa, smem + m.o_w[l] + k * m.wp[l] + 16 * i, m.wp[l], g, tt);
+#pragma unroll
+          for (int b = 0; b < kHalf; ++b) load_s(fb[b], Z(l) + 8 * (b0 + b) * m.zp[l] + k, m.zp[l], g, tt);
+          products(acc, crs, crs, fa, fb);
+        }
+#pragma unroll
+        for (int b = 0; b < kHalf; ++b)
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
-            const float v = get(A(l - 1) + s * m.ap[l - 1] + n) > 0.f ? acc[c] + (BF ? 0.f : crs[c]) : 0.f;
+            const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * (b0 + b) + 2 * tt + (c & 1);
+            const float v = get(A(l - 1) + s * m.ap[l - 1] + n) > 0.f ? acc[b][c] + (BF ? 0.f : crs[b][c]) : 0.f;
             put(Z(l - 1) + s * m.zp[l - 1] + n, v);
             if (c & 2) s1 += v; else s0 += v;
           }
-        }
         s0 += __shfl_xor_sync(0xffffffffu, s0, 1); s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
         s0 += __shfl_xor_sync(0xffffffffu, s0, 2); s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
-        if (tt == 0) { gbias[m.boff[l - 1] + 16 * i + g] = s0; gbias[m.boff[l - 1] + 16 * i + g + 8] = s1; }
+        if (tt == 0) {
+          float* gb = smem + (half ? m.o_gb2 : m.o_gb) + m.boff[l - 1] + 16 * i + g;
+          gb[0] = s0; gb[8] = s1;
+        }
       }
       __syncthreads();
       // dW_l^T = dZ_l^T A_{l-1}, update
       const int mt = m.np[l] / 16, ni = up(m.d[l], 16) / 8;
       for (int e = warp; e < mt * ni; e += kWarps) {
         const int i = e % mt, j = e / mt;
-        float acc[4] = {}, crs[4] = {};
+        float acc[1][4] = {}, x1[1][4] = {}, x2[1][4] = {};
 #pragma unroll 2
         for (int k = 0; k < Bp; k += kStep) {
           FragA<BF> fa;
-          FragB<BF> fb;
+          FragB<BF> fb[1];
           load_zt(fa, Z(l) + k * m.zp[l] + 16 * i, m.zp[l], lane);
-          load_st(fb, A(l - 1) + k * m.ap[l - 1] + 8 * j, m.ap[l - 1], lane);
-          product(acc, crs, fa, fb);
+          load_st(fb[0], A(l - 1) + k * m.ap[l - 1] + 8 * j, m.ap[l - 1], lane);
+          products(acc, x1, x2, fa, fb);
         }
 #pragma unroll
         for (int r2 = 0; r2 < 2; ++r2) {
-          const int at = (16 * i + g + 8 * r2) * m.wp[l] + 8 * j + 2 * tt;
+          const int at = (16 * i + g + 8 * r2) * m.wp[l] + 8 * j + 2 * tt, c = 2 * r2;
           float2* w = reinterpret_cast<float2*>(smem + m.o_w[l] + at);
-          float2* u = reinterpret_cast<float2*>(smem + m.o_u[l] + at);
-          float2 wv = *w, uv = *u;
-          const float g0 = fmaf(lambda, wv.x, acc[2 * r2] + (BF ? 0.f : crs[2 * r2])), g1 = fmaf(lambda, wv.y, acc[2 * r2 + 1] + (BF ? 0.f : crs[2 * r2 + 1]));
+          float2 wv = *w;
+          const float g0 = fmaf(lambda, wv.x, term<BF>(acc[0][c], x1[0][c], x2[0][c]));
+          const float g1 = fmaf(lambda, wv.y, term<BF>(acc[0][c + 1], x1[0][c + 1], x2[0][c + 1]));
           wv.x = fmaf(-eta, g0, wv.x); wv.y = fmaf(-eta, g1, wv.y);
-          uv.x += g0; uv.y += g1;
-          *w = wv; *u = uv;
+          *w = wv;
+          if (!BF) {
+            float2* u = reinterpret_cast<float2*>(smem + m.o_u[l] + at);
+            float2 uv = *u;
+            uv.x += g0; uv.y += g1;
+            *u = uv;
+          }
         }
       }
     }
     // biases: every layer's gradient is in (the barriers above lie between)
     if (nl == 1) __syncthreads();
-    for (int l = 0; l < nl; ++l)
-      for (int e = tid; e < m.d[l + 1]; e += kThreads) {
-        const float gb = gbias[m.boff[l] + e];
-        bias[m.boff[l] + e] = fmaf(-eta, gb, bias[m.boff[l] + e]);
-        ubias[m.boff[l] + e] += gb;
-      }
+    for (int e = tid; e < m.nb; e += kThreads) {
+      const float gb = gbias[e] + smem[m.o_gb2 + e];
+      bias[e] = fmaf(-eta, gb, bias[e]);
+      ubias[e] += gb;
+    }
 
     // ================= 4: dW_0^T over this CTA's inputs, update in place =================
     if (wn > 0) {
       constexpr int kBk = 8 * BT / kStep;   // k-steps over the samples at most
-      FragA<BF> a[MPW][BF ? kBk : 1];
-      if (BF) {
+      constexpr bool kHold = BF || BT <= 4;   // room for all of dZ_0's fragments
+      FragA<BF> a[kHold ? kBk : 1];
+      if (kHold) {
 #pragma unroll
-        for (int j = 0; j < MPW; ++j)
-#pragma unroll
-          for (int k = 0; k < kBk; ++k)
-            if (k * kStep < Bp) load_zt(a[j][BF ? k : 0], Z(0) + k * kStep * m.zp[0] + 16 * (wm * MPW + j), m.zp[0], lane);
+        for (int k = 0; k < kBk; ++k)
+          load_zt(a[kHold ? k : 0], Z(0) + k * kStep * m.zp[0] + 16 * wm, m.zp[0], lane);
       }
       for (int u = 0; u < wn; ++u) {
         const T* xu = X + 16 * (w0 + u);
-        float acc[MPW][2][4] = {}, crs[MPW][2][4] = {};
+        uint32_t r[8];
+        own.issue(u, r);
+        float acc[2][4] = {}, x1[2][4] = {}, x2[2][4] = {};
 #pragma unroll
-        for (int k = 0; k < kBk; ++k)
-          if (k * kStep < Bp) {
-            if (!BF) {
-#pragma unroll
-              for (int j = 0; j < MPW; ++j) load_zt(a[j][0], Z(0) + k * kStep * m.zp[0] + 16 * (wm * MPW + j), m.zp[0], lane);
-            }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              FragB<BF> f;
-              load_st(f, xu + k * kStep * m.xpitch + 8 * h, m.xpitch, lane);
-#pragma unroll
-              for (int j = 0; j < MPW; ++j) product(acc[j][h], crs[j][h], a[j][BF ? k : 0], f);
-            }
+        for (int k = 0; k < kBk; ++k) {
+            if (!kHold) load_zt(a[0], Z(0) + k * kStep * m.zp[0] + 16 * wm, m.zp[0], lane);
+            FragB<BF> f[2];
+            load_st2(f, xu + k * kStep * m.xpitch, m.xpitch, lane);
+            products(acc, x1, x2, a[kHold ? k : 0], f);
           }
+        float w[8], us[8];
+        own.wait(r, w);
+        if (!BF) own.issue(ug + u, r);
 #pragma unroll
-        for (int j = 0; j < MPW; ++j) {
-          float w[8], us[8];
-          own.load_issue(u * MPW + j, w);
-          if (!BF) own.load_issue(ug + u * MPW + j, us);
+        for (int i = 0; i < 8; ++i) {
+          us[i] = fmaf(lambda, w[i], term<BF>(acc[i >> 2][i & 3], x1[i >> 2][i & 3], x2[i >> 2][i & 3]));   // the gradient
+          w[i] = fmaf(-eta, us[i], w[i]);
+        }
+        own.store(u, w);
+        if (!BF) {
+          float v[8];
+          own.wait(r, v);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float gr = fmaf(lambda, w[i], acc[j][i >> 2][i & 3] + (BF ? 0.f : crs[j][i >> 2][i & 3]));
-            w[i] = fmaf(-eta, gr, w[i]);
-            if (!BF) us[i] += gr;
-          }
-          own.store(u * MPW + j, w);
-          if (!BF) own.store(ug + u * MPW + j, us);
+          for (int i = 0; i < 8; ++i) us[i] += v[i];
+          own.store(ug + u, us);
         }
       }
       own.store_wait();
@@ -734,24 +790,28 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     float* Urow = p.r.U + (size_t)t.u_row * p.r.stride;
     float* wrow = p.r.w_end ? p.r.w_end + (size_t)t.u_row * p.r.stride : nullptr;
     const float inv_eta = 1.f / eta;
-    for (int g0 = 0; g0 < wn * MPW; g0 += kChunkG) {
-      const int n = min(kChunkG, wn * MPW - g0);
+    for (int g0 = 0; g0 < wn; g0 += kChunkG) {
+      const int n = min(kChunkG, wn - g0);
       float us[kChunkG][8];
       if (BF) start_groups(g0, n, us);
 #pragma unroll
       for (int q = 0; q < kChunkG; ++q)
         if (q < n) {
           float w[8];
-          own.load_issue(g0 + q, w);
-          if (!BF) own.load_issue(ug + g0 + q, us[q]);
-          else {
+          uint32_t r[8];
+          own.issue(g0 + q, r);
+          own.wait(r, w);
+          if (!BF) {
+            own.issue(ug + g0 + q, r);
+            own.wait(r, us[q]);
+          } else {
 #pragma unroll
             for (int i = 0; i < 8; ++i) us[q][i] = (us[q][i] - w[i]) * inv_eta;
           }
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             size_t at;
-            if (!place((g0 + q) / MPW, (g0 + q) % MPW, i, at)) continue;
+            if (!place(g0 + q, i, at)) continue;
             Urow[at] = us[q][i] + bad;
             if (wrow) wrow[at] = w[i] + bad;
           }
@@ -764,7 +824,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         if (l > 0) {
           for (int e = tid; e < K * N; e += kThreads) {
             const int at = (e % N) * m.wp[l] + e / N;
-            Urow[o + e] = smem[m.o_u[l] + at] + bad;
+            Urow[o + e] = (BF ? (start_value(o + e) - smem[m.o_w[l] + at]) * inv_eta : smem[m.o_u[l] + at]) + bad;
             if (wrow) wrow[o + e] = smem[m.o_w[l] + at] + bad;
           }
           o += (size_t)K * N;
@@ -788,10 +848,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(*tmem_at) : "memory");
 }
 
-template <bool BF, int MPW, int BT>
+template <bool BF, int BT>
 cudaError_t launch(const MmaLaunch& p, cudaStream_t s) {
   const size_t smem = (size_t)p.m.total * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(mlp_mma_kernel<BF, MPW, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(mlp_mma_kernel<BF, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(p.r.n_tasks * p.m.CL, 1, 1);
@@ -804,7 +864,7 @@ cudaError_t launch(const MmaLaunch& p, cudaStream_t s) {
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = p.m.CL > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, mlp_mma_kernel<BF, MPW, BT>, p);
+  return cudaLaunchKernelEx(&cfg, mlp_mma_kernel<BF, BT>, p);
 }
 
 // The widest cluster that leaves every round-task of the launch its own SMs; where none does, the smallest that holds
@@ -837,10 +897,24 @@ cudaError_t launch_mlp_mma_rounds(const MlpLaunch& p, cudaStream_t s) {
   q.r = p.r;
   q.m = pick_plan(p.shape, p.r.n_tasks, (uint32_t)sms);
   if (!q.m.total) return cudaErrorInvalidConfiguration;
-  const bool small = q.m.bt <= 4;
-  if (p.shape.precision == 0) return small ? launch<false, 1, 4>(q, s) : launch<false, 1, 8>(q, s);
-  if (q.m.MT <= 8) return small ? launch<true, 1, 4>(q, s) : launch<true, 1, 8>(q, s);
-  return small ? launch<true, 2, 4>(q, s) : launch<true, 2, 8>(q, s);
+  if (p.shape.precision == 0) {
+    switch (q.m.bt) {
+      case 1: return launch<false, 1>(q, s);
+      case 2: return launch<false, 2>(q, s);
+      case 3: return launch<false, 3>(q, s);
+      case 4: return launch<false, 4>(q, s);
+      case 5: return launch<false, 5>(q, s);
+      case 6: return launch<false, 6>(q, s);
+      case 7: return launch<false, 7>(q, s);
+      default: return launch<false, 8>(q, s);
+    }
+  }
+  switch (q.m.bt) {
+    case 2: return launch<true, 2>(q, s);
+    case 4: return launch<true, 4>(q, s);
+    case 6: return launch<true, 6>(q, s);
+    default: return launch<true, 8>(q, s);
+  }
 }
 
 }  // namespace aet
