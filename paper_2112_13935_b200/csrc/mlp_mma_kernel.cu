@@ -57,6 +57,7 @@ struct MmaPlan {
   int ext;                          // words per thread beyond tensor memory
   // offsets in floats
   int o_x, o_in, o_part, o_a[kMaxL], o_z[kMaxL], o_w[kMaxL], o_u[kMaxL], o_b, o_ub, o_gb, o_gb2, nb, o_logit, o_ext, o_idx, o_bar, total;
+  int imt[kMaxL], iitems[kMaxL], kp[kMaxL];   // ceil(2^20 / tiles of outputs | items); parts of the inputs
   int boff[kMaxL];                  // of layer l's biases in the bias arrays
 };
 
@@ -109,6 +110,12 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
   // dZ_0 and the partial products of the input parts are never needed at the same time
   const int z0 = up(p.Bp * p.zp[0], elems) / elems, least = kWarps * 128;
   p.o_part = p.o_z[0] = take(part > z0 ? (part > least ? part : least) : (z0 > least ? z0 : least));
+  for (int l = 1; l < p.nl; ++l) {
+    auto inv = [](int d) { return ((1 << 20) + d - 1) / d; };
+    const int mt = p.np[l] / 16, items = mt * p.bt, ks = up(p.d[l], bf ? 16 : 8) / (bf ? 16 : 8);
+    p.imt[l] = inv(mt); p.iitems[l] = inv(items);
+    p.kp[l] = items >= kWarps ? 1 : (kWarps / items < ks ? kWarps / items : ks);
+  }
   int nb = 0;
   for (int l = 0; l < p.nl; ++l) { p.boff[l] = nb; nb += up(p.d[l + 1], 16); }
   p.nb = nb;
@@ -272,6 +279,10 @@ __device__ __forceinline__ void send2(uint32_t addr, uint32_t a, uint32_t b, uin
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
                ::"r"(addr), "r"(a), "r"(b), "r"(bar) : "memory");
 }
+
+// n / d for 0 <= n < 2^13 by a multiplication with ceil(2^20 / d) (d <= 128: exact); a hardware division of integers is
+// some twenty dependent instructions, and every phase of the narrow layers needs a few
+__device__ __forceinline__ int div20(int n, int inv) { return (int)(((uint32_t)n * (uint32_t)inv) >> 20); }
 
 struct MmaLaunch {
   RoundLaunch r;
@@ -462,14 +473,13 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   __syncthreads();
   copy_rows(0);
 
-  // Where this warp's rows g and g + 8 of Z_0 go: their owners' inboxes and barriers (warps of the first input part).
-  uint32_t row_at[2], row_bar[2];
-#pragma unroll
-  for (int r2 = 0; r2 < 2; ++r2) {
-    const int rg = min(2 * wm + r2, 2 * m.MT - 1);
+  // Where this lane's row of Z_0 (g, or g + 8 for odd lanes) goes: its owner's inbox and barrier (warps of the first part).
+  uint32_t row_at, row_bar;
+  {
+    const int rg = min(2 * wm + (tt & 1), 2 * m.MT - 1);
     const uint32_t to = (uint32_t)(rg / m.rgs);
-    row_at[r2] = mma::peer_addr(smem_addr(inbox + ((int)rank * m.rgs * 8 + (rg % m.rgs) * 8 + g) * Bp + 2 * tt), to);
-    row_bar[r2] = mma::peer_addr(smem_addr(&bars[0]), to);
+    row_at = mma::peer_addr(smem_addr(inbox + ((int)rank * m.rgs * 8 + (rg % m.rgs) * 8 + g) * Bp + 4 * (tt >> 1)), to);
+    row_bar = mma::peer_addr(smem_addr(&bars[0]), to);
   }
   const int own_q = tid / Bp, own_b = tid - own_q * Bp;   // this thread's four owned rows and sample in step 2
 
@@ -540,10 +550,12 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
               for (int c = 0; c < 4; ++c) acc[b][c] += q[(b * 4 + c) * 32];
         }
 #pragma unroll
-        for (int r2 = 0; r2 < 2; ++r2)
-#pragma unroll
-          for (int b = 0; b < BT; ++b)
-            send2(row_at[r2] + 32u * b, __float_as_uint(acc[b][2 * r2]), __float_as_uint(acc[b][2 * r2 + 1]), row_bar[r2]);
+        for (int b = 0; b < BT; ++b) {
+          // neighbouring lanes trade pairs: the even one then has four samples of row g, the odd one of row g + 8
+          const bool odd = tt & 1;
+          const float r0 = __shfl_xor_sync(0xffffffffu, odd ? acc[b][0] : acc[b][2], 1), r1 = __shfl_xor_sync(0xffffffffu, odd ? acc[b][1] : acc[b][3], 1);
+          mma::send_peer(row_at + 32u * b, odd ? make_float4(r0, r1, acc[b][2], acc[b][3]) : make_float4(acc[b][0], acc[b][1], r0, r1), row_bar);
+        }
       }
     }
 
@@ -586,15 +598,15 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       const bool last = l + 1 == nl;
       // few output tiles: several warps share one, each with its part of the inputs.  (The area of the partial Z_0 is
       // free: A_0 is complete, so every part has been sent.)
-      const int kp = items >= kWarps ? 1 : min(kWarps / items, ks);
+      const int kp = m.kp[l];
       for (int e = warp; e < items * kp; e += kWarps) {
-        const int part_k = e / items, i = (e % items) % mt, b = (e % items) / mt;
+        const int part_k = kp > 1 ? div20(e, m.iitems[l]) : 0, item = e - part_k * items, b = div20(item, m.imt[l]), i = item - b * mt;
         float acc[1][4] = {}, x1[1][4] = {}, x2[1][4] = {};
         const float* w = smem + m.o_w[l] + 16 * i * m.wp[l];
         const T* a = A(l - 1) + 8 * b * m.ap[l - 1];
-        const int k1 = ks * (part_k + 1) / kp;
+        const int per = (ks + kp - 1) / kp, k1 = min(ks, per * (part_k + 1));
 #pragma unroll 4
-        for (int k = ks * part_k / kp; k < k1; ++k) {
+        for (int k = per * part_k; k < k1; ++k) {
           FragA<BF> fa;
           FragB<BF> fb[1];
           load_w(fa, w + k * kStep, m.wp[l], g, tt);
@@ -617,7 +629,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       __syncthreads();
       if (kp > 1) {
         for (int e = tid; e < items * 128; e += kThreads) {
-          const int item = e >> 7, c = (e >> 5) & 3, i = item % mt, b = item / mt;
+          const int item = e >> 7, c = (e >> 5) & 3, b = div20(item, m.imt[l]), i = item - b * mt;
           const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
           float v = bias[m.boff[l] + n];
           for (int k = 0; k < kp; ++k) v += part[k * items * 128 + e];
@@ -672,7 +684,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       constexpr int kHalf = BT % 2 == 0 ? BT / 2 : BT;
       const int halves = BT / kHalf;
       for (int e = warp; e < mi * halves; e += kWarps) {
-        const int i = e % mi, half = e / mi, b0 = half * kHalf;
+        const int half = halves > 1 && e >= mi ? 1 : 0, i = e - half * mi, b0 = half * kHalf;
         float s0 = 0.f, s1 = 0.f;
         float acc[kHalf][4] = {}, crs[kHalf][4] = {};
         for (int k = 0; k < K; k += kStep) {
@@ -703,7 +715,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       // dW_l^T = dZ_l^T A_{l-1}, update
       const int mt = m.np[l] / 16, ni = up(m.d[l], 16) / 8;
       for (int e = warp; e < mt * ni; e += kWarps) {
-        const int i = e % mt, j = e / mt;
+        const int j = div20(e, m.imt[l]), i = e - j * mt;
         float acc[1][4] = {}, x1[1][4] = {}, x2[1][4] = {};
 #pragma unroll 2
         for (int k = 0; k < Bp; k += kStep) {
@@ -751,8 +763,9 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       }
       for (int u = 0; u < wn; ++u) {
         const T* xu = X + 16 * (w0 + u);
-        uint32_t r[8];
+        uint32_t r[8], rs[8];
         own.issue(u, r);
+        if (!BF) own.issue(ug + u, rs);
         float acc[2][4] = {}, x1[2][4] = {}, x2[2][4] = {};
 #pragma unroll
         for (int k = 0; k < kBk; ++k) {
@@ -763,7 +776,6 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           }
         float w[8], us[8];
         own.wait(r, w);
-        if (!BF) own.issue(ug + u, r);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           us[i] = fmaf(lambda, w[i], term<BF>(acc[i >> 2][i & 3], x1[i >> 2][i & 3], x2[i >> 2][i & 3]));   // the gradient
@@ -772,7 +784,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         own.store(u, w);
         if (!BF) {
           float v[8];
-          own.wait(r, v);
+          own.wait(rs, v);
 #pragma unroll
           for (int i = 0; i < 8; ++i) us[i] += v[i];
           own.store(ug + u, us);
