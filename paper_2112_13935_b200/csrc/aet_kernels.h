@@ -110,6 +110,9 @@ uint32_t cnn_n_params(const CnnShape& s);
 size_t cnn_act_floats(const CnnShape& s);
 const char* cnn_check_shape(const CnnShape& s);   // null if the kernel can run it
 cudaError_t launch_cnn_rounds(const CnnLaunch& p, cudaStream_t s);
+// The LeNet shape, minibatches of up to 24 samples, on clusters of 8 or 4 CTAs (see cnn_mma_kernel.cu); 0: not eligible
+uint32_t cnn_mma_cluster(const CnnShape& s, uint32_t n_tasks, uint32_t sms);
+cudaError_t launch_cnn_mma_rounds(const CnnLaunch& p, uint32_t cluster, cudaStream_t s);
 
 // Ordered aggregation: for seq in [lo, hi): w -= eta_seq * U[seq]; keep a copy
 // where a later round starts from it; bump H and log the apply.

@@ -559,6 +559,7 @@ cudaError_t launch_cnn_rounds(const CnnLaunch& p0, cudaStream_t s) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
   }
+  if (const uint32_t c = cnn_mma_cluster(p0.shape, p0.r.n_tasks, (uint32_t)sms)) return launch_cnn_mma_rounds(p0, c, s);
   // CTAs per round-task: as many as the minibatch has samples and the launch leaves SMs for
   uint32_t cl = kMaxCl;
   while (cl > 1 && (cl > p0.shape.batch || p0.r.n_tasks * cl > (uint32_t)sms)) cl >>= 1;
