@@ -41,7 +41,7 @@ using mma::split_t;
 constexpr int kWarps = 16, kThreads = kWarps * 32;
 constexpr int kS = 28, kC1 = 6, kP1 = 12, kC2 = 16, kFlat = 256, kF1 = 120, kF2 = 84, kN = 10;
 constexpr int kX = kS * kS, kQ1 = kC1 * kP1 * kP1;      // values of a row, of the first pooled maps
-constexpr int kPw2 = 152, kW2c = kC2 * kPw2, kW1c = 256;   // conv 2: [plane][tap, bias, 0]; conv 1: [tap, bias][4 (c / 3) + c % 3]
+constexpr int kPw2 = 152, kW2c = kC2 * kPw2, kW1c = 256;   // conv 2: [plane][tap, bias, 0]; conv 1: [tap, bias][8 planes, 6 used]
 constexpr int kQuads = (kW2c + kW1c) / 4;               // the convolutions' parameters as 16-byte pieces
 constexpr int kPq2 = 264, kPh1 = 120, kPh2 = 88, kPdz = 72, kPcol = 72;   // row pitches: fragment loads hit different banks
 constexpr int kMaxPer = 4;                              // samples per CTA
@@ -78,6 +78,11 @@ __device__ __forceinline__ void mul(float (&d)[4], float (&x)[4], const FA& a, c
   mma::tf32(x, a.v[0].lo, a.v[1].lo, a.v[2].lo, a.v[3].lo, b.v[0].hi, b.v[1].hi);
   mma::tf32(x, a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].lo, b.v[1].lo);
 }
+__device__ __forceinline__ void mul3(float (&d)[3][4], const FA& a, const FB& b) {   // a term an accumulator: three short chains
+  mma::tf32(d[0], a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].hi, b.v[1].hi);
+  mma::tf32(d[1], a.v[0].lo, a.v[1].lo, a.v[2].lo, a.v[3].lo, b.v[0].hi, b.v[1].hi);
+  mma::tf32(d[2], a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].lo, b.v[1].lo);
+}
 __device__ __forceinline__ void send1(uint32_t addr, float v, uint32_t bar) {   // 4 bytes to a peer
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(__float_as_uint(v)), "r"(bar) : "memory");
 }
@@ -89,7 +94,7 @@ struct Lay {   // shared memory, in floats
   static constexpr int kPd1 = 16 * MT1 + 8;
   static constexpr int wc = 0, w1 = wc + kW2c + kW1c, w2 = w1 + 16 * MT1 * kPq2, w3 = w2 + 88 * kPh1, b1 = w3 + kF2 * kN,
                        b2 = b1 + 16 * MT1, b3 = b2 + 96, x = b3 + 16, q1 = x + kPer * kX, m1 = q1 + kPer * kQ1,
-                       m2 = m1 + kPer * kQ1 / 4, dz2 = m2 + kPer * kFlat / 4, dq1 = dz2 + kC2 * kPdz, dense = dq1 + kQ1;
+                       m2 = m1 + kPer * kQ1 / 4, dz2 = m2 + kPer * kFlat / 4, dq1 = dz2 + kC2 * kPdz, dense = dq1 + (kPer > 1 ? 2 : 1) * kQ1;
   // q2, h1, h2, dh2 of all samples; once the dense layers are done the convolutions' gradient parts lie there
   static constexpr int q2 = dense, h1 = q2 + Bp * kPq2, h2 = h1 + Bp * kPh1, dh2 = h2 + Bp * kPh2, dense_end0 = dh2 + Bp * kPh2 + 8;
   static constexpr int g2 = dense, g1 = g2 + 2 * kW2c, dense_end1 = g1 + kWarps * kW1c;
@@ -125,22 +130,27 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
   uint8_t* const m1 = reinterpret_cast<uint8_t*>(sm + M::m1);         // signs of the four outputs behind a pooled one
   uint8_t* const m2 = reinterpret_cast<uint8_t*>(sm + M::m2);
 
+#pragma unroll 1
   for (int i = tid; i < M::total; i += kThreads) sm[i] = 0.f;
   __syncthreads();
+#pragma unroll 1
   for (int k = tid; k < kPw2; k += kThreads) off[k] = k < 150 ? (uint16_t)((k / 25) * 144 + ((k % 25) / 5) * 12 + k % 5) : 0;
   if (tid == 0) {
+#pragma unroll 1
     for (int i = 0; i < 5; ++i) mbar_init(&bars[i], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   mma::cluster_sync();
   const uint32_t bytes[5] = {(uint32_t)(B * kFlat * 4), (uint32_t)(kF1 * Bp * 4), (uint32_t)(CL * nb * kFlat * 4), (uint32_t)(CL * kOwn * 16), (uint32_t)(kQuads * 16)};
   if (tid == 0) {
+#pragma unroll 1
     for (int i = 0; i < 5; ++i)
       if (bytes[i]) mbar_expect_tx(&bars[i], bytes[i]);
   }
   bool ok = true;
   auto wait = [&](int i, uint32_t parity) {
     const uint32_t at = smem_addr(&bars[i]);
+#pragma unroll 1
     for (uint32_t k = 0; ok; ++k) {
       if (mma::try_wait_cluster(at, parity)) break;
       if (k >= kWaitLimit) ok = false;
@@ -151,6 +161,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
   const float* snap = p.r.snaps + (size_t)t.snap_slot * p.r.stride;
   auto start_value = [&](int at) {
     float v = snap[at];
+#pragma unroll 1
     for (uint32_t f = 0; f < t.inflight_cnt; ++f) {
       const InflightRef ref = p.r.inflight[t.inflight_off + f];
       v = fmaf(-ref.eta, p.r.U[(size_t)ref.row * p.r.stride + at], v);
@@ -163,12 +174,13 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
       const int c = e / kPw2, k = e - c * kPw2;
       return k < 150 ? kOW2 + c * 150 + k : (k == 150 ? kOb2 + c : -1);
     }
-    const int q = e - kW2c, tap = q >> 3, cc = q & 7, c = (cc >> 2) * 3 + (cc & 3);
-    return (cc & 3) == 3 || tap > 25 ? -1 : (tap < 25 ? kOW1 + c * 25 + tap : kOb1 + c);
+    const int q = e - kW2c, tap = q >> 3, c = q & 7;
+    return c >= kC1 || tap > 25 ? -1 : (tap < 25 ? kOW1 + c * 25 + tap : kOb1 + c);
   };
   {
     constexpr int kTrip = 4;
     auto fill = [&](int count, auto place, auto dest) {   // kTrip loads on their way before the first store
+#pragma unroll 1
       for (int e0 = tid; e0 < count; e0 += kTrip * kThreads) {
         float v[kTrip];
 #pragma unroll
@@ -200,6 +212,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     }
   };
   auto copy_rows = [&](uint32_t it) {
+#pragma unroll 1
     for (int e = tid; e < nb * (kX / 4); e += kThreads) {
       const int b = e / (kX / 4), c = e - b * (kX / 4);
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(sm + M::x + 4 * e)), "l"(xrows + (size_t)idx[(it & 1) * 64 + b] * kX + 4 * c) : "memory");
@@ -222,6 +235,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     }
   }
 
+#pragma unroll 1
   for (uint32_t it = 0; it < t.steps; ++it) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (it) {
@@ -231,12 +245,13 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     if (it + 1 < t.steps) draw_rows(it + 1);
     __syncthreads();
 
-    // ================= conv 1, ReLU, pooling: three planes of a pooled output per thread =================
-    for (int e = tid; e < nb * 288; e += kThreads) {
-      const int b = e / 288, r = e - b * 288, grp = r >= 144 ? 1 : 0, pos = r - grp * 144, py = pos / kP1, px = pos - py * kP1;
+    // ================= conv 1, ReLU, pooling: two planes of a pooled output per thread =================
+#pragma unroll 1
+    for (int e = tid; e < nb * 432; e += kThreads) {
+      const int b = e / 432, r = e - b * 432, grp = r / 144, pos = r - grp * 144, py = pos / kP1, px = pos - py * kP1;
       const float* xp = sm + M::x + b * kX + 2 * py * kS + 2 * px;
-      const float* w = sm + M::wc + kW2c + 4 * grp;
-      float patch[6][6], z[3][4];
+      const float* w = sm + M::wc + kW2c + 2 * grp;
+      float patch[6][6], z[2][4];
 #pragma unroll
       for (int i = 0; i < 6; ++i)
 #pragma unroll
@@ -245,30 +260,30 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
           patch[i][2 * j] = v.x; patch[i][2 * j + 1] = v.y;
         }
       {
-        const float4 bias = *reinterpret_cast<const float4*>(w + 25 * 8);
+        const float2 bias = *reinterpret_cast<const float2*>(w + 25 * 8);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) { z[0][q] = bias.x; z[1][q] = bias.y; z[2][q] = bias.z; }
+        for (int q = 0; q < 4; ++q) { z[0][q] = bias.x; z[1][q] = bias.y; }
       }
 #pragma unroll
       for (int dy = 0; dy < 5; ++dy)
 #pragma unroll
         for (int dx = 0; dx < 5; ++dx) {
-          const float4 wv = *reinterpret_cast<const float4*>(w + (dy * 5 + dx) * 8);
+          const float2 wv = *reinterpret_cast<const float2*>(w + (dy * 5 + dx) * 8);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const float v = patch[dy + (q >> 1)][dx + (q & 1)];
-            z[0][q] = fmaf(wv.x, v, z[0][q]); z[1][q] = fmaf(wv.y, v, z[1][q]); z[2][q] = fmaf(wv.z, v, z[2][q]);
+            z[0][q] = fmaf(wv.x, v, z[0][q]); z[1][q] = fmaf(wv.y, v, z[1][q]);
           }
         }
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
+      for (int c = 0; c < 2; ++c) {
         uint32_t bits = 0;
         float sum = 0.f;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           if (z[c][q] > 0.f) { bits |= 1u << q; sum += z[c][q]; }
         }
-        const int at = b * kQ1 + (3 * grp + c) * 144 + pos;
+        const int at = b * kQ1 + (2 * grp + c) * 144 + pos;
         sm[M::q1 + at] = 0.25f * sum;
         m1[at] = (uint8_t)bits;
       }
@@ -276,12 +291,14 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     __syncthreads();
 
     // ================= conv 2, ReLU, pooling: a warp takes two rows of a sample's 8 x 8 outputs, all planes =================
-    for (int e = warp; e < 4 * nb; e += kWarps) {
-      const int b = e >> 2, yp = e & 3;
+    // (with at most two samples two warps share an item, each with half of the taps)
+    constexpr bool kShare = kPer <= 2;
+    float acc2[2][4] = {}, crs2[2][4] = {};
+    const int e_half = kShare ? warp >> 3 : 0;
+    auto conv2 = [&](int b, int yp, int s0, int s1, float (&acc)[2][4], float (&crs)[2][4]) {
       const float* q = sm + M::q1 + b * kQ1 + 2 * yp * kP1 + g;
-      float acc[2][4] = {}, crs[2][4] = {};
-#pragma unroll 3
-      for (int s = 0; s < kPw2 / 8; ++s) {
+#pragma unroll 5
+      for (int s = s0; s < s1; ++s) {
         const FA a = a_rows(sm + M::wc + 8 * s, kPw2, g, tt);
         const uint32_t o2 = *reinterpret_cast<const uint32_t*>(off + 8 * s + 2 * tt);
         const float* i0 = q + (o2 & 0xFFFF);
@@ -292,6 +309,31 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
           const FB f = {split_t(last ? 1.f : i0[kP1 * r]), split_t(last ? 0.f : i1[kP1 * r])};
           mul(acc[r], crs[r], a, f);
         }
+      }
+    };
+    if (kShare) {
+      const int e = warp & 7;
+      if (e < 4 * nb) {
+        if (e_half == 0) conv2(e >> 2, e & 3, 0, 9, acc2, crs2);
+        else conv2(e >> 2, e & 3, 9, kPw2 / 8, acc2, crs2);
+        if (e_half) {
+          float* d = sm + M::col + kWarps * 64 + e * 256 + lane;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) d[32 * i] = acc2[i >> 2][i & 3] + crs2[i >> 2][i & 3];
+        }
+      }
+      __syncthreads();
+    }
+#pragma unroll 1
+    for (int e = warp; e < 4 * nb; e += kWarps) {
+      const int b = e >> 2, yp = e & 3;
+      float acc[2][4] = {}, crs[2][4] = {};
+      if (kShare) {
+        const float* d = sm + M::col + kWarps * 64 + e * 256 + lane;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { acc[i >> 2][i & 3] = acc2[i >> 2][i & 3] + crs2[i >> 2][i & 3]; crs[i >> 2][i & 3] = d[32 * i]; }
+      } else {
+        conv2(b, yp, 0, kPw2 / 8, acc, crs);
       }
       float* st = sm + M::col + warp * 64;
 #pragma unroll
@@ -344,6 +386,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
                 make_float2(acc[i][b][2 * r] + crs[i][b][2 * r], acc[i][b][2 * r + 1] + crs[i][b][2 * r + 1]);
     }
     __syncthreads();
+#pragma unroll 1
     for (int e = tid; e < N1 * Bp; e += kThreads) {
       const int n = e / Bp, b = e % Bp;
       float v = sm[M::b1 + n];
@@ -358,19 +401,21 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[1], bytes[1]);
 
     // ================= dense 2, dense 3, softmax, in every CTA =================
+#pragma unroll 1
     for (int e = warp; e < 6 * BT; e += kWarps) {
       const int i = e % 6, b = e / 6;
-      float acc[4] = {}, crs[4] = {};
-#pragma unroll 5
+      float acc[3][4] = {};
+#pragma unroll
       for (int s = 0; s < kF1 / 8; ++s)
-        mul(acc, crs, a_rows(sm + M::w2 + 16 * i * kPh1 + 8 * s, kPh1, g, tt), b_rows(sm + M::h1 + 8 * b * kPh1 + 8 * s, kPh1, g, tt));
+        mul3(acc, a_rows(sm + M::w2 + 16 * i * kPh1 + 8 * s, kPh1, g, tt), b_rows(sm + M::h1 + 8 * b * kPh1 + 8 * s, kPh1, g, tt));
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
-        if (n < kPh2) sm[M::h2 + s * kPh2 + n] = n < kF2 ? fmaxf(acc[c] + crs[c] + sm[M::b2 + n], 0.f) : 0.f;
+        if (n < kPh2) sm[M::h2 + s * kPh2 + n] = n < kF2 ? fmaxf(acc[0][c] + (acc[1][c] + acc[2][c]) + sm[M::b2 + n], 0.f) : 0.f;
       }
     }
     __syncthreads();
+#pragma unroll 1
     for (int e = tid; e < Bp * kN * 2; e += kThreads) {   // two lanes per logit (whole warps: Bp is a multiple of 8, 160 | Bp * 20)
       const int o = e >> 1, b = o / kN, c = o % kN, i0 = (e & 1) * (kF2 / 2);
       const float* h = sm + M::h2 + b * kPh2 + i0;
@@ -407,6 +452,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     __syncthreads();
 
     // ================= backward through the dense layers =================
+#pragma unroll 1
     for (int e = tid; e < Bp * kPh2; e += kThreads) {   // dh2
       const int b = e / kPh2, i = e % kPh2;
       float v = 0.f;
@@ -420,16 +466,17 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     }
     __syncthreads();
     if (warp < 4) {   // dh1 of the own outputs
+#pragma unroll 1
       for (int e = warp; e < MT1 * BT; e += 4) {
         const int i = e / BT, b = e % BT;
-        float acc[4] = {}, crs[4] = {};
+        float acc[3][4] = {};
 #pragma unroll
         for (int s = 0; s < kPh2 / 8; ++s)
-          mul(acc, crs, a_cols(sm + M::w2 + 8 * s * kPh1 + rank * N1 + 16 * i, kPh1, g, tt), b_rows(sm + M::dh2 + 8 * b * kPh2 + 8 * s, kPh2, g, tt));
+          mul3(acc, a_cols(sm + M::w2 + 8 * s * kPh1 + rank * N1 + 16 * i, kPh1, g, tt), b_rows(sm + M::dh2 + 8 * b * kPh2 + 8 * s, kPh2, g, tt));
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
-          sm[M::dh1 + s * kPd1 + n] = n < N1 && sm[M::h1 + s * kPh1 + rank * N1 + n] > 0.f ? acc[c] + crs[c] : 0.f;
+          sm[M::dh1 + s * kPd1 + n] = n < N1 && sm[M::h1 + s * kPh1 + rank * N1 + n] > 0.f ? acc[0][c] + (acc[1][c] + acc[2][c]) : 0.f;
         }
       }
     } else {          // dense 3 and the biases of layers 2 and 3
@@ -502,22 +549,25 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
           u1[i][h][2 * r] += g0; u1[i][h][2 * r + 1] += g1;
         }
     }
+    {   // dense 2: 6 x 15 tiles, all of a warp's products before its first update (stores would hold the loads back)
+      float acc[6][4] = {};
 #pragma unroll
-    for (int r = 0; r < 6; ++r) {   // dense 2: 6 x 15 tiles
-      const int e = warp + kWarps * r;
-      if (e < 90) {
-        const int j = e / 6, i = e - 6 * j;
-        float acc[4] = {}, crs[4] = {};
+      for (int r = 0; r < 6; ++r) {
+        const int e = min(warp + kWarps * r, 89), j = e / 6, i = e - 6 * j;
 #pragma unroll
         for (int s = 0; s < BT; ++s)
-          mul(acc, crs, a_cols_k(sm + M::dh2 + 8 * s * kPh2 + 16 * i, kPh2, g, tt), b_cols_k(sm + M::h1 + 8 * s * kPh1 + 8 * j, kPh1, g, tt));
+          mul(acc[r], acc[r], a_cols_k(sm + M::dh2 + 8 * s * kPh2 + 16 * i, kPh2, g, tt), b_cols_k(sm + M::h1 + 8 * s * kPh1 + 8 * j, kPh1, g, tt));
+      }
+#pragma unroll
+      for (int r = 0; r < 6; ++r) {
+        const int e = warp + kWarps * r, j = e / 6, i = e - 6 * j;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const int n = 16 * i + g + 8 * q;
-          if (n < kF2) {
+          if (e < 90 && n < kF2) {
             float2* w = reinterpret_cast<float2*>(sm + M::w2 + n * kPh1 + 8 * j + 2 * tt);
             float2 v = *w;
-            const float g0 = fmaf(lambda, v.x, acc[2 * q] + crs[2 * q]), g1 = fmaf(lambda, v.y, acc[2 * q + 1] + crs[2 * q + 1]);
+            const float g0 = fmaf(lambda, v.x, acc[r][2 * q]), g1 = fmaf(lambda, v.y, acc[r][2 * q + 1]);
             v.x = fmaf(-eta, g0, v.x); v.y = fmaf(-eta, g1, v.y);
             *w = v;
             if (r % CL == rank) { u2[r / CL][2 * q] += g0; u2[r / CL][2 * q + 1] += g1; }
@@ -554,47 +604,53 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     int o2[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) o2[i] = off[min(8 * ((warp + kWarps * i) >> 1) + g, kPw2 - 1)];
-    for (int b = 0; b <= nb; ++b) {
-      if (b < nb) {   // dz2 = [z2 > 0] dq2 / 4
+    auto put_dz2 = [&](int b) {   // dz2 = [z2 > 0] dq2 / 4
 #pragma unroll
-        for (int r = 0; r < kMaxPer / 2; ++r) {
-          const int e = tid + kThreads * r;
-          if ((e >> 8) == b) {
-            const int k = e & 255, c = k >> 4, py = (k >> 2) & 3, px = k & 3;
-            const uint32_t bits = m2[e];
-            float2* d = reinterpret_cast<float2*>(sm + M::dz2 + c * kPdz + 16 * py + 2 * px);
-            d[0] = make_float2(bits & 1 ? vq[r] : 0.f, bits & 2 ? vq[r] : 0.f);
-            d[4] = make_float2(bits & 4 ? vq[r] : 0.f, bits & 8 ? vq[r] : 0.f);
-          }
+      for (int r = 0; r < kMaxPer / 2; ++r) {
+        const int e = tid + kThreads * r;
+        if ((e >> 8) == b) {
+          const int k = e & 255, c = k >> 4, py = (k >> 2) & 3, px = k & 3;
+          const uint32_t bits = m2[e];
+          float2* d = reinterpret_cast<float2*>(sm + M::dz2 + c * kPdz + 16 * py + 2 * px);
+          d[0] = make_float2(bits & 1 ? vq[r] : 0.f, bits & 2 ? vq[r] : 0.f);
+          d[4] = make_float2(bits & 4 ? vq[r] : 0.f, bits & 8 ? vq[r] : 0.f);
         }
       }
-      if (b > 0) {    // conv 1's gradient of the sample before: dW1^T[tap x plane] += im2col(x)^T dz1, eight outputs of a row a step
-        const float* xp = sm + M::x + (b - 1) * kX;
-        const int c = (g >> 2) * 3 + (g & 3);
-        const bool plane = (g & 3) < 3;
-        const int tap1 = g + 8;
-        const int oa = (g / 5) * kS + g % 5, ob = (tap1 / 5) * kS + tap1 % 5, oc = ((g + 16) / 5) * kS + (g + 16) % 5, od = 4 * kS + 4;
-        for (int u = warp; u < 36; u += kWarps) {
-          const int py = u / 3, s3 = u - 3 * py, px = 4 * s3 + tt;
-          const float v = plane ? 0.25f * sm[M::dq1 + c * 144 + py * kP1 + px] : 0.f;
-          const uint32_t bits = plane ? m1[(b - 1) * kQ1 + c * 144 + py * kP1 + px] : 0;
+    };
+    // Conv 1's gradient of the samples from s0 (an even one) to s1 (at most two): dW1^T[tap x plane] += im2col(x)^T dz1,
+    // eight outputs of a row a step; dz1 from dq1 and the sign bits.
+    auto conv1_grad = [&](int s0, int s1) {
+      const bool plane = g < kC1;
+      const int tap1 = g + 8, tap2 = g + 16;
+      const int oa = (g / 5) * kS + g % 5, ob = (tap1 / 5) * kS + tap1 % 5, oc = (tap2 / 5) * kS + tap2 % 5, od = 4 * kS + 4;
+#pragma unroll 2
+      for (int u = warp; u < 36 * (s1 - s0); u += kWarps) {
+        const int hi = u >= 36 ? 1 : 0, v36 = u - 36 * hi, py = v36 / 3, px = 4 * (v36 - 3 * py) + tt;
+        const float* xp = sm + M::x + (s0 + hi) * kX + 2 * px;
+        const int at = (plane ? g : 0) * 144 + py * kP1 + px;
+        const float v = plane ? 0.25f * sm[M::dq1 + hi * kQ1 + at] : 0.f;
+        const uint32_t bits = m1[(s0 + hi) * kQ1 + at];
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const FB f = {split_t(bits & (1u << (2 * h)) ? v : 0.f), split_t(bits & (2u << (2 * h)) ? v : 0.f)};
-            const float* xi = xp + (2 * py + h) * kS + 2 * px;
-            mul(a1[0], x1[0], {split(xi[oa]), split(xi[ob]), split(xi[oa + 1]), split(xi[ob + 1])}, f);
-            // taps 16 .. 23, then 24, the bias (an input of 1) and none
-            const float t0 = g == 0 ? xi[od] : (g == 1 ? 1.f : 0.f), t1 = g == 0 ? xi[od + 1] : (g == 1 ? 1.f : 0.f);
-            mul(a1[1], x1[1], {split(xi[oc]), split(t0), split(xi[oc + 1]), split(t1)}, f);
-          }
+        for (int h = 0; h < 2; ++h) {
+          const FB f = {split(bits & (1u << (2 * h)) ? v : 0.f), split(bits & (2u << (2 * h)) ? v : 0.f)};
+          const float* xi = xp + (2 * py + h) * kS;
+          mul(a1[0], x1[0], {split_t(xi[oa]), split_t(xi[ob]), split_t(xi[oa + 1]), split_t(xi[ob + 1])}, f);
+          // taps 16 .. 23, then 24, the bias (an input of 1) and none
+          const float t0 = g == 0 ? xi[od] : (g == 1 ? 1.f : 0.f), t1 = g == 0 ? xi[od + 1] : (g == 1 ? 1.f : 0.f);
+          mul(a1[1], x1[1], {split_t(xi[oc]), split_t(t0), split_t(xi[oc + 1]), split_t(t1)}, f);
         }
       }
-      __syncthreads();
-      if (b == nb) break;
+    };
+    __syncthreads();   // dq2's parts have been read: col may take their place
+    if (nb > 0) put_dz2(0);
+    __syncthreads();
+#pragma unroll 1
+    for (int b = 0; b < nb; ++b) {
       const float* q1 = sm + M::q1 + b * kQ1;
       // col[tap x output] = W2^T dz2: items of 16 taps x 16 outputs; the warps with fewer gradient tiles take more
       {
         const int first = warp < 6 ? 2 * warp : 12 + 3 * (warp - 6), n = min(40, first + (warp < 6 ? 2 : 3));
+#pragma unroll 1
         for (int e = first; e < n; ++e) {
           const int i = e >> 2, y = 2 * (e & 3);
           const FA f0 = a_cols_k(sm + M::wc + 16 * i, kPw2, g, tt), f1 = a_cols_k(sm + M::wc + 8 * kPw2 + 16 * i, kPw2, g, tt);
@@ -610,15 +666,16 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
         }
       }
       // dW2[plane x tap] += dz2 im2col(q1)^T over four rows of outputs
+      const int y0 = 4 * (warp & 1);   // (the same half for all of a warp's tiles)
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const int q = warp + kWarps * i;
-        if (q < 38) {
-          const int n = 8 * (q >> 1) + g, y0 = 4 * (q & 1);
-          const float* in = q1 + o2[i] + 2 * tt;
+      for (int y = 0; y < 4; ++y) {
+        const FA f = a_rows(sm + M::dz2 + 8 * (y0 + y), kPdz, g, tt);
 #pragma unroll
-          for (int y = 0; y < 4; ++y) {
-            const FA f = a_rows(sm + M::dz2 + 8 * (y0 + y), kPdz, g, tt);
+        for (int i = 0; i < 3; ++i) {
+          const int q = warp + kWarps * i;
+          if (q < 38) {
+            const int n = 8 * (q >> 1) + g;
+            const float* in = q1 + o2[i] + 2 * tt;
             float v0 = in[(y0 + y) * kP1], v1 = in[(y0 + y) * kP1 + 1];
             if (n >= 150) v0 = v1 = n == 150 ? 1.f : 0.f;   // the bias
             mul(a2[i], x2[i], f, {split_t(v0), split_t(v1)});
@@ -626,6 +683,8 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
         }
       }
       __syncthreads();
+      if (b + 1 < nb) put_dz2(b + 1);
+#pragma unroll 1
       for (int e = tid; e < kQ1; e += kThreads) {   // dq1: every input of conv 2 adds up the entries of col it is part of
         const int c = e / 144, r = e - 144 * c, y = r / kP1, x = r - kP1 * y;
         const float* cp = sm + M::col + c * 25 * kPcol + y * 8 + x;
@@ -640,11 +699,13 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
               if (dx & 1) w += q; else v += q;
             }
         }
-        sm[M::dq1 + e] = v + w;
+        sm[M::dq1 + (b & 1) * kQ1 + e] = v + w;
       }
       __syncthreads();
+      if ((b & 1) || b + 1 == nb) conv1_grad(b & ~1, b + 1);   // (the barriers of the next sample lie before dq1 is written again)
     }
-    if (it + 1 < t.steps) copy_rows(it + 1);   // the rows have served: the next iteration's
+    __syncthreads();   // the rows have been read
+    if (it + 1 < t.steps) copy_rows(it + 1);
 
     // ================= the convolutions' gradients to their owners, the new weights back =================
     // (the dense layers' activations are dead: every CTA has sent its part of dq2 and used its own)
@@ -664,6 +725,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
       *reinterpret_cast<float2*>(d + 64) = make_float2(a1[i][2] + x1[i][2], a1[i][3] + x1[i][3]);
     }
     __syncthreads();
+#pragma unroll 1
     for (int e = tid; e < kQuads; e += kThreads) {
       float4 v;
       if (e < kW2c / 4) {
@@ -797,6 +859,7 @@ constexpr bool kFits[2][3] = {{Lay<8, 1>::fits, Lay<8, 2>::fits, Lay<8, 3>::fits
 // GPCs: with eight CTAs a few SMs stay unused, so a launch that needs nearly all of them takes four.
 uint32_t cnn_mma_cluster(const CnnShape& s, uint32_t n_tasks, uint32_t sms) {
   constexpr uint32_t lenet[7] = {kS, 1, kC1, kC2, kF1, kF2, kN};
+#pragma unroll 1
   for (int i = 0; i < 7; ++i)
     if (s.dims[i] != lenet[i]) return 0;
   const uint32_t bt = (s.batch + 7) / 8;

@@ -305,6 +305,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   const uint32_t rank = CL > 1 ? mma::cluster_rank() : 0;
   if (t.steps == 0) {
     int P = 0;
+#pragma unroll 1
     for (int l = 0; l < nl; ++l) P += m.d[l] * m.d[l + 1] + m.d[l + 1];
     if (rank == 0) publish_empty_round(p.r, t, (uint32_t)P);
     return;
@@ -332,6 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   const int w0 = mine ? min(nu, wk * m.upw) : nu, wn = min(nu, w0 + m.upw) - w0;        // this warp's units
   const int rg0 = min(2 * m.MT, (int)rank * m.rgs), nrg = min(2 * m.MT, rg0 + m.rgs) - rg0;   // owned groups of 8 hidden rows
 
+#pragma unroll 1
   for (int i = tid; i < m.total; i += kThreads) smem[i] = 0.f;
   __syncthreads();
   if (warp == 0) {
@@ -360,6 +362,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   bool ok = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) {
     const uint32_t at = smem_addr(bar);
+#pragma unroll 1
     for (uint32_t i = 0; ok; ++i) {
       if (mma::try_wait_cluster(at, parity)) break;
       if (i >= kWaitLimit) ok = false;
@@ -381,12 +384,15 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   auto copy_rows = [&](uint32_t it) {
     T* x = xb0 + (it % m.xbufs) * Bp * m.xpitch;
     const T* src = reinterpret_cast<const T*>(cd.x) + x0;
+#pragma unroll 1
     for (int r = warp; r < B; r += kWarps) {
       const T* row = src + (size_t)idx[(it & 1) * 64 + r] * D0;
       if (whole) {
+#pragma unroll 1
         for (int c = lane * kChunk; c < nx; c += 32 * kChunk)
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(x + r * m.xpitch + c)), "l"(row + c) : "memory");
       } else {
+#pragma unroll 1
         for (int c = lane; c < nx; c += 32) x[r * m.xpitch + c] = row[c];
       }
     }
@@ -397,6 +403,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   const float* snap = p.r.snaps + (size_t)t.snap_slot * p.r.stride;
   auto start_value = [&](size_t at) {
     float v = snap[at];
+#pragma unroll 1
     for (uint32_t f = 0; f < t.inflight_cnt; ++f) {
       const InflightRef ref = p.r.inflight[t.inflight_off + f];
       v = fmaf(-ref.eta, p.r.U[(size_t)ref.row * p.r.stride + at], v);
@@ -419,6 +426,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         size_t at;
         v[q][i] = q < n && place(first + q, i, at) ? snap[at] : 0.f;
       }
+#pragma unroll 1
     for (uint32_t f = 0; f < t.inflight_cnt; ++f) {
       const InflightRef ref = p.r.inflight[t.inflight_off + f];
       const float* us = p.r.U + (size_t)ref.row * p.r.stride;
@@ -437,6 +445,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     }
   };
   draw_rows(0);
+#pragma unroll 1
   for (int g0 = 0; g0 < wn; g0 += kChunkG) {
     const int n = min(kChunkG, wn - g0);
     float v[kChunkG][8], zero[8] = {};
@@ -451,9 +460,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   own.store_wait();
   {
     size_t o = (size_t)D0 * N1;
+#pragma unroll 1
     for (int l = 0; l < nl; ++l) {
       const int K = m.d[l], N = m.d[l + 1];
       if (l > 0) {
+#pragma unroll 1
         for (int e0 = tid; e0 < K * N; e0 += 8 * kThreads) {
           float v[8];
 #pragma unroll
@@ -466,6 +477,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         }
         o += (size_t)K * N;
       }
+#pragma unroll 1
       for (int e = tid; e < N; e += kThreads) bias[m.boff[l] + e] = start_value(o + e);
       o += N;
     }
@@ -483,6 +495,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   }
   const int own_q = tid / Bp, own_b = tid - own_q * Bp;   // this thread's four owned rows and sample in step 2
 
+#pragma unroll 1
   for (uint32_t it = 0; it < t.steps; ++it) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (it + 1 < t.steps) draw_rows(it + 1);
@@ -497,6 +510,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       for (int b = 0; b < BT; ++b)
 #pragma unroll
         for (int c = 0; c < 4; ++c) { acc[b][c] = 0.f; crs[b][c] = 0.f; }
+#pragma unroll 1
       for (int u = 0; u < wn; ++u) {
         const T* xu = X + 16 * (w0 + u);
         uint32_t r[8];
@@ -542,6 +556,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         __syncthreads();
       }
       if (wk == 0) {
+#pragma unroll 1
         for (int k = 1; k < m.WK; ++k) {
           const float* q = part + ((k - 1) * m.WM + wm) * bt * 128 + lane;
 #pragma unroll
@@ -564,6 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       wait(&bars[0], it & 1);
       if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[0], in_bytes);
       int q = own_q, b = own_b;
+#pragma unroll 1
       for (int e = tid; e < nrg * 2 * Bp; e += kThreads) {
         if (e >= kThreads) { q = e / Bp; b = e - q * Bp; }
         const int n = 8 * rg0 + 4 * q;
@@ -582,9 +598,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         const uint32_t bar = smem_addr(&bars[1]);
         if (BF && nl > 1) {
           const uint32_t at = smem_addr(reinterpret_cast<__nv_bfloat16*>(A(0)) + b * m.ap[0] + n), lo = pack_bf16(v[0], v[1]), hi = pack_bf16(v[2], v[3]);
+#pragma unroll 1
           for (int r = 0; r < CL; ++r) send2(mma::peer_addr(at, r), lo, hi, mma::peer_addr(bar, r));
         } else {
           const uint32_t at = smem_addr(smem + m.o_a[0] + b * m.ap[0] + n);
+#pragma unroll 1
           for (int r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(at, r), make_float4(v[0], v[1], v[2], v[3]), mma::peer_addr(bar, r));
         }
       }
@@ -593,12 +611,14 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[1], a_bytes);
 
     // ================= 3: narrow layers, redundantly in every CTA =================
+#pragma unroll 1
     for (int l = 1; l < nl; ++l) {
       const int mt = m.np[l] / 16, ks = up(m.d[l], kStep) / kStep, items = mt * bt;
       const bool last = l + 1 == nl;
       // few output tiles: several warps share one, each with its part of the inputs.  (The area of the partial Z_0 is
       // free: A_0 is complete, so every part has been sent.)
       const int kp = m.kp[l];
+#pragma unroll 1
       for (int e = warp; e < items * kp; e += kWarps) {
         const int part_k = kp > 1 ? div20(e, m.iitems[l]) : 0, item = e - part_k * items, b = div20(item, m.imt[l]), i = item - b * mt;
         float acc[1][4] = {}, x1[1][4] = {}, x2[1][4] = {};
@@ -628,10 +648,12 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       }
       __syncthreads();
       if (kp > 1) {
+#pragma unroll 1
         for (int e = tid; e < items * 128; e += kThreads) {
           const int item = e >> 7, c = (e >> 5) & 3, b = div20(item, m.imt[l]), i = item - b * mt;
           const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
           float v = bias[m.boff[l] + n];
+#pragma unroll 1
           for (int k = 0; k < kp; ++k) v += part[k * items * 128 + e];
           if (!last) put(A(l) + s * m.ap[l] + n, fmaxf(v, 0.f));
           else if (n < m.d[nl]) logit[s * 33 + n] = v;
@@ -670,23 +692,28 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       }
     }
     __syncthreads();
+#pragma unroll 1
     for (int c = kWarps - 1 - warp; c < m.d[nl]; c += kWarps) {   // bias gradient of the last layer
       float v = 0.f;
+#pragma unroll 1
       for (int s = lane; s < B; s += 32) v += logit[s * 33 + c];
 #pragma unroll
       for (int k = 16; k; k >>= 1) v += __shfl_xor_sync(0xffffffffu, v, k);
       if (lane == 0) gbias[m.boff[nl - 1] + c] = v;
     }
+#pragma unroll 1
     for (int l = nl - 1; l >= 1; --l) {
       // dZ_{l-1}^T = [A_{l-1} > 0] W_l dZ_l^T: a warp takes 16 inputs and all samples, or half of them, and so has its
       // share of their bias gradients
       const int mi = up(m.d[l], 16) / 16, K = up(m.d[l + 1], kStep);
       constexpr int kHalf = BT % 2 == 0 ? BT / 2 : BT;
       const int halves = BT / kHalf;
+#pragma unroll 1
       for (int e = warp; e < mi * halves; e += kWarps) {
         const int half = halves > 1 && e >= mi ? 1 : 0, i = e - half * mi, b0 = half * kHalf;
         float s0 = 0.f, s1 = 0.f;
         float acc[kHalf][4] = {}, crs[kHalf][4] = {};
+#pragma unroll 1
         for (int k = 0; k < K; k += kStep) {
           FragA<BF> fa;
           FragB<BF> fb[kHalf];
@@ -714,6 +741,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       __syncthreads();
       // dW_l^T = dZ_l^T A_{l-1}, update
       const int mt = m.np[l] / 16, ni = up(m.d[l], 16) / 8;
+#pragma unroll 1
       for (int e = warp; e < mt * ni; e += kWarps) {
         const int j = div20(e, m.imt[l]), i = e - j * mt;
         float acc[1][4] = {}, x1[1][4] = {}, x2[1][4] = {};
@@ -745,6 +773,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     }
     // biases: every layer's gradient is in (the barriers above lie between)
     if (nl == 1) __syncthreads();
+#pragma unroll 1
     for (int e = tid; e < m.nb; e += kThreads) {
       const float gb = gbias[e] + smem[m.o_gb2 + e];
       bias[e] = fmaf(-eta, gb, bias[e]);
@@ -761,6 +790,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         for (int k = 0; k < kBk; ++k)
           load_zt(a[kHold ? k : 0], Z(0) + k * kStep * m.zp[0] + 16 * wm, m.zp[0], lane);
       }
+#pragma unroll 1
       for (int u = 0; u < wn; ++u) {
         const T* xu = X + 16 * (w0 + u);
         uint32_t r[8], rs[8];
@@ -802,6 +832,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     float* Urow = p.r.U + (size_t)t.u_row * p.r.stride;
     float* wrow = p.r.w_end ? p.r.w_end + (size_t)t.u_row * p.r.stride : nullptr;
     const float inv_eta = 1.f / eta;
+#pragma unroll 1
     for (int g0 = 0; g0 < wn; g0 += kChunkG) {
       const int n = min(kChunkG, wn - g0);
       float us[kChunkG][8];
@@ -831,9 +862,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     }
     if (rank == 0) {
       size_t o = (size_t)D0 * N1;
+#pragma unroll 1
       for (int l = 0; l < nl; ++l) {
         const int K = m.d[l], N = m.d[l + 1];
         if (l > 0) {
+#pragma unroll 1
           for (int e = tid; e < K * N; e += kThreads) {
             const int at = (e % N) * m.wp[l] + e / N;
             Urow[o + e] = (BF ? (start_value(o + e) - smem[m.o_w[l] + at]) * inv_eta : smem[m.o_u[l] + at]) + bad;
@@ -841,6 +874,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           }
           o += (size_t)K * N;
         }
+#pragma unroll 1
         for (int e = tid; e < N; e += kThreads) {
           Urow[o + e] = ubias[m.boff[l] + e] + bad;
           if (wrow) wrow[o + e] = bias[m.boff[l] + e] + bad;
@@ -883,6 +917,7 @@ cudaError_t launch(const MmaLaunch& p, cudaStream_t s) {
 // the first layer.
 MmaPlan pick_plan(const MlpShape& s, uint32_t n_tasks, uint32_t sms) {
   MmaPlan last{};
+#pragma unroll 1
   for (int cl = 8; cl >= 1; cl >>= 1) {
     const MmaPlan p = make_plan(s, cl);
     if (!p.total) continue;
@@ -895,6 +930,7 @@ MmaPlan pick_plan(const MlpShape& s, uint32_t n_tasks, uint32_t sms) {
 }  // namespace
 
 bool mlp_mma_eligible(const MlpShape& shape) {
+#pragma unroll 1
   for (int cl = 8; cl >= 1; cl >>= 1)
     if (make_plan(shape, cl).total) return true;
   return false;
