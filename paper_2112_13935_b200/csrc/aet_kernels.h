@@ -80,6 +80,9 @@ cudaError_t launch_mlp_rounds(const MlpLaunch& p, cudaStream_t s);
 size_t mlp_act_floats(const MlpShape& shape);
 uint32_t mlp_pick_cluster(const MlpShape& shape, uint32_t n_clients);
 const char* mlp_check_shape(const MlpShape& shape);  // null if the kernel can run it
+// bf16 D0-256-(128-)C models, batch 32 or 64: the first layer streams through a cluster (see mlp_wide_kernel.cu)
+bool mlp_wide_eligible(const MlpShape& shape);
+cudaError_t launch_mlp_wide_rounds(const MlpLaunch& p, cudaStream_t s);
 // minibatches of up to 64 samples, first hidden layer of at most 128 units (bf16: 256): the first layer stays on the chip,
 // spread over a cluster (see mlp_mma_kernel.cu)
 bool mlp_mma_eligible(const MlpShape& shape);
