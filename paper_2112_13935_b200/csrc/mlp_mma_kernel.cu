@@ -23,7 +23,8 @@
 // tiles; at 16-64 samples per iteration the warp-level instructions' rate (1,024 bf16 / 512 tf32 multiply-adds per clock
 // and SM) is not what limits a round: hand-overs, updates and the narrow layers are.
 //
-// precision 1: the update sums of the weights are (W_start - W_end) / eta; everything else accumulates U.
+// precision 1: the update sum of W_0 is (W_start - W_end) / eta; everything else accumulates U (the narrow layers' sums
+// beside W_0 in tensor memory).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -60,6 +61,7 @@ struct MmaPlan {
   int ext;                          // words per thread beyond tensor memory
   // offsets in floats
   int o_x, o_in, o_part, o_a[kMaxL], o_z[kMaxL], o_w[kMaxL], o_u[kMaxL], o_b, o_ub, o_gb, o_gb2, nb, o_logit, o_ext, o_idx, o_bar, total;
+  int useg, us[kMaxL];              // bf16: first 4-word piece of the narrow layers' update sums, of layer l's
   int imt[kMaxL], iitems[kMaxL], kp[kMaxL];   // ceil(2^20 / tiles of outputs | items); parts of the inputs
   int boff[kMaxL];                  // of layer l's biases in the bias arrays
 };
@@ -85,6 +87,7 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
   p.upw = (p.upc + p.WK - 1) / p.WK;
   if (cl > 1 && p.upc * (cl - 1) >= p.units) return p;   // the last CTA would have nothing
   const int words = p.upw * 8 * (bf ? 1 : 2);
+  p.useg = words / 4;
   p.ext = words > kTmemWords ? words - kTmemWords : 0;
   p.rgs = (2 * p.MT + cl - 1) / cl;
   int o = 0;
@@ -118,6 +121,15 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
     const int mt = p.np[l] / 16, items = mt * p.bt, ks = up(p.d[l], bf ? 16 : 8) / (bf ? 16 : 8);
     p.imt[l] = inv(mt); p.iitems[l] = inv(items);
     p.kp[l] = items >= kWarps ? 1 : (kWarps / items < ks ? kWarps / items : ks);
+  }
+  if (bf) {   // the narrow layers' update sums beside W_0 in tensor memory, a piece per tile of 16 x 8
+    int at = p.useg;
+    for (int l = 1; l < p.nl; ++l) {
+      p.us[l] = at;
+      at += (p.np[l] / 16 * (up(p.d[l], 16) / 8) + kWarps - 1) / kWarps;
+    }
+    p.us[0] = at;   // (the end)
+    if (p.ext || 4 * at > kTmemWords) return p;
   }
   int nb = 0;
   for (int l = 0; l < p.nl; ++l) { p.boff[l] = nb; nb += up(p.d[l + 1], 16); }
@@ -261,6 +273,17 @@ struct Own {
 #pragma unroll
       for (int i = 0; i < 8; ++i) ext[(8 * group - kTmemWords + i) * kThreads] = v[i];
     }
+  }
+  __device__ __forceinline__ void load4(int piece, float (&v)[4]) const {
+    uint32_t r[4];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n\ttcgen05.wait::ld.sync.aligned;"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tmem + 4u * piece) : "memory");
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+  }
+  __device__ __forceinline__ void store4(int piece, const float (&v)[4]) const {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};\n\ttcgen05.wait::st.sync.aligned;"
+                 ::"r"(tmem + 4u * piece), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])) : "memory");
   }
   __device__ __forceinline__ void store_wait() const { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 };
@@ -446,6 +469,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         own.store(g0 + q, v[q]);
         if (!BF) own.store(ug + g0 + q, zero);
       }
+  }
+  if (BF) {
+    const float zero[4] = {};
+#pragma unroll 1
+    for (int q = m.useg; q < m.us[0]; ++q) own.store4(q, zero);
   }
   own.store_wait();
   {
@@ -743,6 +771,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           load_st(fb[0], A(l - 1) + k * m.ap[l - 1] + 8 * j, m.ap[l - 1], lane);
           products(acc, x1, x2, fa, fb);
         }
+        float uq[4];
+        if (BF) own.load4(m.us[l] + (e >> 4), uq);
 #pragma unroll
         for (int r2 = 0; r2 < 2; ++r2) {
           const int at = (16 * i + g + 8 * r2) * m.wp[l] + 8 * j + 2 * tt, c = 2 * r2;
@@ -752,13 +782,16 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           const float g1 = fmaf(lambda, wv.y, term<BF>(acc[0][c + 1], x1[0][c + 1], x2[0][c + 1]));
           wv.x = fmaf(-eta, g0, wv.x); wv.y = fmaf(-eta, g1, wv.y);
           *w = wv;
-          if (!BF) {
+          if (BF) {
+            uq[c] += g0; uq[c + 1] += g1;
+          } else {
             float2* u = reinterpret_cast<float2*>(smem + m.o_u[l] + at);
             float2 uv = *u;
             uv.x += g0; uv.y += g1;
             *u = uv;
           }
         }
+        if (BF) own.store4(m.us[l] + (e >> 4), uq);
       }
     }
     // biases: every layer's gradient is in (the barriers above lie between)
@@ -859,8 +892,22 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
 #pragma unroll 1
           for (int e = tid; e < K * N; e += kThreads) {
             const int at = (e % N) * m.wp[l] + e / N;
-            Urow[o + e] = (BF ? (start_value(o + e) - smem[m.o_w[l] + at]) * inv_eta : smem[m.o_u[l] + at]) + bad;
+            if (!BF) Urow[o + e] = smem[m.o_u[l] + at] + bad;
             if (wrow) wrow[o + e] = smem[m.o_w[l] + at] + bad;
+          }
+          if (BF) {
+            const int mt = m.np[l] / 16, tiles = mt * (up(K, 16) / 8);
+#pragma unroll 1
+            for (int e = warp; e < tiles; e += kWarps) {
+              const int j = div20(e, m.imt[l]), i = e - j * mt;
+              float uq[4];
+              own.load4(m.us[l] + (e >> 4), uq);
+#pragma unroll
+              for (int c = 0; c < 4; ++c) {
+                const int n = 16 * i + g + ((c & 2) ? 8 : 0), k = 8 * j + 2 * tt + (c & 1);
+                if (n < N && k < K) Urow[o + (size_t)k * N + n] = uq[c] + bad;
+              }
+            }
           }
           o += (size_t)K * N;
         }

@@ -19,8 +19,8 @@
 // same order: the same bits).  Memory is reused without cluster barriers: parts are sent only after every peer's warps have
 // said that they are done with what lies there.
 //
-// The update sums of the weights are (W_start - W_end) / eta (w -= eta g and U += g in the same step); the biases'
-// are accumulated.
+// The update sums of the two wide layers are (W_start - W_end) / eta (w -= eta g and U += g in the same step); the class
+// layer's and the biases' are accumulated.
 //
 // What bounds it: HBM - W_0 is read and written once per iteration, 6.3 MB per client at D0 = 3072 - as long as the launch has
 // enough clients; with few, the warp-level tensor rate (16 instructions of 8 cycles per 16 x 16 entries and scheduler).
@@ -86,7 +86,7 @@ struct Lay {   // shared memory, in bytes
   static constexpr int bias = z2 + Bp * kPz * 2, ub = bias + kNb * 4, gb = ub + kNb * 4, gb2 = gb + kNb * 4;
   static constexpr int kStage = 2 * Bp * kPx * 2;
   static constexpr int ring = (gb2 + kNb * 4 + 15) / 16 * 16, idx = ring + kRing * kStage, bars = idx + 4 * 64 * 4, total = bars + 128;
-  static constexpr int kRes = MID ? 8 : 16;    // units of W_0 in tensor memory (a group each), beside W_1's 8 groups
+  static constexpr int kRes = MID ? 6 : 14;    // units of W_0 in tensor memory (a group each); then W_1's 8 groups, W_2's update sum
   static_assert(z0 % 16 == 0 && z1 % 16 == 0 && a1 % 16 == 0 && w2 % 16 == 0 && logit % 16 == 0 && z2 % 16 == 0 && bias % 16 == 0 && idx % 16 == 0 && bars % 8 == 0, "alignment");
   static_assert(total <= 227 * 1024, "fits an SM");
 };
@@ -100,7 +100,7 @@ struct WideLaunch {
 template <int BT, bool MID>
 __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_constant__ WideLaunch p) {
   typedef Lay<BT, MID> M;
-  constexpr int Bp = M::Bp, K2 = M::K2, kPw2 = M::kPw2, KS = BT / 2, kRes = M::kRes;
+  constexpr int Bp = M::Bp, K2 = M::K2, kPw2 = M::kPw2, KS = BT / 2, kRes = M::kRes, kU2 = kRes + (MID ? 8 : 0);
   extern __shared__ __align__(128) unsigned char smem[];
   const int CL = p.CL, C = p.C, D0 = p.D0;
   const TaskDesc t = p.r.tasks[p.r.task_begin + blockIdx.x / CL];
@@ -237,6 +237,11 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
     *reinterpret_cast<uint32_t*>(d + 8) = pack_bf16(w[4], w[5]);
     *reinterpret_cast<uint32_t*>(d + 8 * kP0 + 8) = pack_bf16(w[6], w[7]);
   };
+  {
+    const float zero[8] = {};
+    own.store(kU2, zero);
+    own.store_wait();
+  }
   draw_rows(0);
   if (MID) {
 #pragma unroll 1
@@ -547,16 +552,22 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
         mma_bf16(acc[0], f, x[0], x[1]);
         mma_bf16(acc[1], f, x[2], x[3]);
       }
+      float us[8];
+      own.load(kU2, us);
 #pragma unroll
       for (int h = 0; h < 2; ++h)
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           float2* w = reinterpret_cast<float2*>(W2 + (g + 8 * q) * kPw2 + 16 * warp + 8 * h + 2 * tt);
           float2 v = *w;
-          v.x = fmaf(-eta, fmaf(lambda, v.x, acc[h][2 * q]), v.x);
-          v.y = fmaf(-eta, fmaf(lambda, v.y, acc[h][2 * q + 1]), v.y);
+          const float g0 = fmaf(lambda, v.x, acc[h][2 * q]), g1 = fmaf(lambda, v.y, acc[h][2 * q + 1]);
+          v.x = fmaf(-eta, g0, v.x);
+          v.y = fmaf(-eta, g1, v.y);
           *w = v;
+          us[4 * h + 2 * q] += g0; us[4 * h + 2 * q + 1] += g1;
         }
+      own.store(kU2, us);
+      own.store_wait();
     }
     if (MID) {
       {   // dZ_0 = relu' (W_1 dZ_1): a warp has 16 hidden units of layer 0, all samples
@@ -634,11 +645,17 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
   }
   if (rank == 0) {
     const float bad = ok ? 0.f : __int_as_float(0x7FFFFFFF);
-#pragma unroll 1
-    for (int e = tid; e < K2 * C; e += kThreads) {
-      const float w = W2[(e % C) * kPw2 + e / C];
-      Urow[oW2 + e] = (start_value(oW2 + e) - w) * inv_eta + bad;
-      if (wrow) wrow[oW2 + e] = w + bad;
+    if (warp < K2 / 16) {
+      float us[8];
+      own.load(kU2, us);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int k = 16 * warp + 2 * tt + (i & 1) + ((i & 4) ? 8 : 0), c = g + ((i & 2) ? 8 : 0);
+        if (c < C) {
+          Urow[oW2 + (size_t)k * C + c] = us[i] + bad;
+          if (wrow) wrow[oW2 + (size_t)k * C + c] = W2[c * kPw2 + k] + bad;
+        }
+      }
     }
     if (tid < kNb && (MID || tid < kB1 || tid >= kB2) && tid < kB2 + C) {
       const size_t at = tid < kB1 ? ob0 + tid : (tid < kB2 ? ob1 + tid - kB1 : ob2 + tid - kB2);
