@@ -81,6 +81,7 @@ struct Lay {   // shared memory, in bytes
   // dZ_0, dZ_1, A_1: dead during a pass, whose parts of Z_0 come in there: up to 7 / 8 of 16 tiles of 16 x Bp
   static constexpr int z0 = a0 + Bp * kP0 * 2, z1 = z0 + Bp * kP0 * 2, a1 = z1 + (MID ? Bp * kP1 * 2 : 0), dead_end = a1 + (MID ? Bp * kP1 * 2 : 0);
   static constexpr int in_end = z0 + 14 * BT * 512;
+  static_assert(!MID || BT != 8 || dead_end - z1 >= kWarps * 2048, "two units per warp");
   static constexpr int part = MID ? z1 : z0;   // the class layer's partial sums: before dZ of the layer below is written
   static constexpr int w2 = dead_end > in_end ? dead_end : in_end, logit = w2 + 16 * kPw2 * 4, z2 = logit + Bp * 17 * 4;
   static constexpr int bias = z2 + Bp * kPz * 2, ub = bias + kNb * 4, gb = ub + kNb * 4, gb2 = gb + kNb * 4;
@@ -278,6 +279,9 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
     }
   };
 
+  // With at most two CTAs the parts of Z_0 leave dZ_1's and A_1's place free during a pass: 2 KB per warp
+  const bool deep = MID && BT == 8 && CL <= 2;
+  float* const deep_at = reinterpret_cast<float*>(smem + M::z1) + warp * 512 + lane * 4;
   // One pass over the CTA's inputs.  GRAD: the gradient of iteration itc and the update (otherwise the start model comes
   // in); LOOK: the forward product of iteration itc + 1 and its hand-over (otherwise the update sums go out).
   auto pass = [&](auto grad_, auto look_, int itc) {
@@ -293,16 +297,31 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
       __syncwarp();
       if (lane < CL && lane != rank) mma::arrive_peer(mma::peer_addr(smem_addr(b_free), lane));
     }
-    float4 wb[2][2];   // the master two units ahead
+    // The master two units ahead in registers; with `deep` the two units behind those are on their way into shared memory
+    // (each lane copies and reads its own 32 bytes of a unit).  A group of copies per unit.
+    float4 wb[2][2];
     auto fetch = [&](int u, float4 (&d)[2]) {
       const float4* s = reinterpret_cast<const float4*>(master + (size_t)u * (kWarps * 256));
       d[0] = __ldcg(s);
       d[1] = __ldcg(s + 32);
     };
+    auto stage = [&](int u) {
+      const float* s = master + (size_t)u * (kWarps * 256);
+      const uint32_t d = smem_addr(deep_at + (u & 1) * 256);
+      if (u < nu) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(s) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 512), "l"(s + 128) : "memory");
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     if (GRAD) {
 #pragma unroll
       for (int j = 0; j < 2; ++j)
         if (kRes + j < nu) fetch(kRes + j, wb[j]);
+      if (deep) {
+        stage(kRes + 2);
+        stage(kRes + 3);
+      }
     }
 #pragma unroll 1
     for (int c = 0; c < nch; ++c) {
@@ -311,7 +330,6 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
 #pragma unroll
         for (int j = 0; j < 2; ++j) start_words(nat + (size_t)(2 * c + j) * (16 * kH0), kH0, sv[GRAD && LOOK ? 0 : j]);
       }
-      if (c + 2 < nch) issue(c + 2, itc, GRAD, LOOK);
       wait(&full[qc % kRing], (qc / kRing) & 1);
       const bf16* xc = ring + (qc % kRing) * 2 * Bp * kPx;
       const bf16* xn = xc + Bp * kPx;
@@ -327,7 +345,15 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
         } else {
           w[0] = wb[j][0].x; w[1] = wb[j][0].y; w[2] = wb[j][0].z; w[3] = wb[j][0].w;
           w[4] = wb[j][1].x; w[5] = wb[j][1].y; w[6] = wb[j][1].z; w[7] = wb[j][1].w;
-          if (u + 2 < nu) fetch(u + 2, wb[j]);
+          if (deep) {
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            const float4* s = reinterpret_cast<const float4*>(deep_at + (u & 1) * 256);
+            wb[j][0] = s[0];
+            wb[j][1] = s[32];
+            stage(u + 4);
+          } else if (u + 2 < nu) {
+            fetch(u + 2, wb[j]);
+          }
         }
         if (GRAD) {
           float gr[2][4] = {};
@@ -364,6 +390,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
       ++qc;
       __syncwarp();
       if (lane == 0) mbar_arrive(&freed[(qc - 1) % kRing]);
+      // at the end of a chunk the slot of the one before is free without a wait: every warp is about as far
+      if (c + 2 < nch) issue(c + 2, itc, GRAD, LOOK);
     }
     if (!LOOK) return;
     own.store_wait();
@@ -628,6 +656,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
       bias[tid] = fmaf(-eta, gr, bias[tid]);
       ubias[tid] += gr;
     }
+    if (MID) __syncthreads();   // dZ_1 and A_1 have been read
     if (more) pass(Yes(), Yes(), (int)it);
     else pass(Yes(), No(), (int)it);
   }
