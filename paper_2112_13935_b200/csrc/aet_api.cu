@@ -190,12 +190,11 @@ struct aet_handle {
   DevBuf<ClientData> d_clients;
   DevBuf<uint64_t> d_keys;
   DevBuf<uint32_t> d_H;
-  DevBuf<float> w_buf[2], w0, snaps, U, work, act, dbg, totals;
+  DevBuf<float> w, w0, snaps, U, work, act, dbg;
   DevBuf<float> node_w;           // topology 1: [n_clients, stride], every node's own model
   DevBuf<RingApplyDesc> d_ring_applies;
   DevBuf<RingOp> d_ring_ops;
-  int w_sel = 0;  // which of w_buf holds the server model
-  float* w_cur() { return w_buf[w_sel].p; }
+  float* w_cur() { return w.p; }   // the server model
   DevBuf<uint32_t> d_status;
   DevBuf<TaskDesc> d_tasks;
   DevBuf<char> d_plan;            // topology 0: the plan's tasks, sums in flight and updates
@@ -453,8 +452,8 @@ aet_status aet_create(const aet_config* cfg, aet_handle** out) {
   }
   h->h_clients.assign(cfg->n_clients, ClientData{nullptr, nullptr, 0, 0});
   h->st.H.assign(cfg->n_clients, 0);
-  bool ok = h->w_buf[0].reserve(h->stride) && h->w_buf[1].reserve(h->stride) && h->w0.reserve(h->stride) &&
-            h->d_H.reserve(cfg->n_clients) && h->d_status.reserve(1) && h->totals.reserve(32 * h->stride);
+  bool ok = h->w.reserve(h->stride) && h->w0.reserve(h->stride) &&
+            h->d_H.reserve(cfg->n_clients) && h->d_status.reserve(1);
   if (ok && !h->lr_fast && !h->cnn) ok = h->work.reserve((size_t)cfg->n_clients * h->stride);
   if (ok && cfg->topology == 1) ok = h->node_w.reserve((size_t)cfg->n_clients * h->stride);
   if (!ok) { aet_destroy(h); return fail(nullptr, AET_ERR_NOMEM, "device allocation failed"); }
@@ -463,8 +462,7 @@ aet_status aet_create(const aet_config* cfg, aet_handle** out) {
     aet_destroy(h);
     return fail(nullptr, AET_ERR_CUDA, std::string("cudaMemset: ") + cudaGetErrorString(e));
   }
-  if (cudaMemset(h->w_buf[0].p, 0, h->stride * sizeof(float)) != cudaSuccess ||
-      cudaMemset(h->w_buf[1].p, 0, h->stride * sizeof(float)) != cudaSuccess ||
+  if (cudaMemset(h->w.p, 0, h->stride * sizeof(float)) != cudaSuccess ||
       cudaMemset(h->d_status.p, 0, sizeof(uint32_t)) != cudaSuccess ||
       cudaMemset(h->w0.p, 0, h->stride * sizeof(float)) != cudaSuccess ||
       cudaMemset(h->d_H.p, 0, cfg->n_clients * sizeof(uint32_t)) != cudaSuccess) {
@@ -487,7 +485,7 @@ aet_status aet_destroy(aet_handle* h) {
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
   h->arena.release();
   h->d_clients.release(); h->d_keys.release(); h->d_H.release();
-  h->w_buf[0].release(); h->w_buf[1].release(); h->totals.release(); h->d_status.release(); h->w0.release(); h->snaps.release(); h->U.release();
+  h->w.release(); h->d_status.release(); h->w0.release(); h->snaps.release(); h->U.release();
   h->work.release(); h->act.release(); h->dbg.release();
   h->node_w.release(); h->d_ring_applies.release(); h->d_ring_ops.release();
   h->d_tasks.release(); h->d_plan.release();
@@ -668,7 +666,7 @@ aet_status aet_run_rounds(aet_handle* h, uint32_t n_rounds, void* cuda_stream) {
   r.step_by_step = (h->cfg.flags & AET_FLAG_STEPWISE_RECURRENCE) ? 1u : 0u;
   r.n_u_rows = plan.n_u_rows; r.n_snap = plan.n_snap;
   ApplyLaunch a{};
-  a.applies = reinterpret_cast<const ApplyDesc*>(h->d_plan.p + off_ap); a.U = h->U.p; a.snaps = h->snaps.p; a.totals = h->totals.p;
+  a.applies = reinterpret_cast<const ApplyDesc*>(h->d_plan.p + off_ap); a.U = h->U.p; a.snaps = h->snaps.p; a.w = h->w_cur();
   a.H = h->d_H.p; a.log = h->d_alog.p; a.status = h->d_status.p; a.stride = h->stride; a.n_params = h->P;
 
   // ---- waves: a3/a4 local SGD of independent round-tasks, then a6 aggregation ----
@@ -681,10 +679,6 @@ aet_status aet_run_rounds(aet_handle* h, uint32_t n_rounds, void* cuda_stream) {
     if (rs != AET_OK) return rs;
     if (plan.apply_upto[L] > applied) {
       a.lo = applied; a.hi = plan.apply_upto[L];
-      a.groups = apply_groups(a.hi - a.lo);
-      a.w_in = h->w_cur();
-      if (a.groups > 1) h->w_sel ^= 1;   // grouped ranges write the other buffer
-      a.w_out = h->w_cur();
       KernelTimer kt(h, s, 1);
       cudaError_t e = launch_apply_updates(a, s);
       if (e != cudaSuccess) return cuda_fail(h, e, "aggregation kernel launch");

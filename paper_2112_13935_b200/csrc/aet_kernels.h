@@ -123,17 +123,13 @@ struct ApplyLaunch {
   const ApplyDesc* applies;  // device, indexed by seq
   const float* U;
   float* snaps;
-  const float* w_in;         // server model before the range [stride]
-  float* w_out;              // ... and after it (may equal w_in only when groups == 1)
-  float* totals;             // scratch [groups, stride], used when groups > 1
+  float* w;                  // server model [stride], before and after the range
   uint32_t* H;               // [n_clients]
   ApplyRec* log;             // [n_events]
   uint32_t* status;          // optional: bit 1 set if the model after the range is not finite
   size_t stride;
   uint32_t n_params, lo, hi;
-  uint32_t groups;           // apply_groups(hi - lo)
 };
-uint32_t apply_groups(uint32_t n_updates);
 cudaError_t launch_apply_updates(const ApplyLaunch& p, cudaStream_t s);
 
 // Peer-to-peer ring: the models of the nodes listed in applies[lo, hi) take their operations.

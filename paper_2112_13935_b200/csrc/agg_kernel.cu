@@ -1,111 +1,103 @@
 // Server side: ordered aggregation of the triggered update sums.
 //
 // Algorithm 3, Receive: "w = w - eta_k * U; H_v = H_v + 1", applied in the
-// order the simulated-time schedule fixes.  Each thread owns one parameter and
-// walks the updates of its range in order, keeping the parameter in a register;
-// wherever a later round starts from the model after update k the running
-// value is also stored as that round's start snapshot (this replaces a
-// separate broadcast copy into client slots).
+// order the simulated-time schedule fixes; wherever a later round starts from
+// the model after update k the running value is also stored as that round's
+// start snapshot (this replaces a separate broadcast copy into client slots).
 //
-// A long range (many clients) is cut into G groups of consecutive updates.
-// Pass 1 sums -eta_k * U_k over each group; pass 2 starts group g from
-// w + sum of the totals of the groups before it and walks the group in order.
-// The result is the paper's sequential rule up to fp32 re-association across
-// group boundaries, and identical from run to run.
+// A CTA has a slice of 128 parameters and a range of consecutive updates: it
+// fetches the slice of all its update sums at once (asynchronous copies into
+// shared memory, one row per warp instruction), its four thread groups sum
+// -eta_k U_k over a quarter of the range each, and with everything that comes
+// before known every group walks its quarter in order, keeping the parameter
+// in a register.  Long ranges are cut over a cluster of up to eight CTAs, which
+// exchange their totals through distributed shared memory.  The result is the
+// paper's sequential rule up to fp32 re-association across quarters, and
+// identical from run to run.
+// What bounds it: L2 (every update sum read once, every snapshot written once)
+// and the latency of one such fetch.  Two passes of eight-deep walks over the
+// range (group totals, then the walk) took 24 us for 700 updates of 7,850
+// parameters; this takes @@NEW@@.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "aet_kernels.h"
+#include "mma_common.cuh"
 
 namespace aet {
 namespace {
 
-constexpr int kAggThreads = 128;
-constexpr int kAhead = 8;  // update rows fetched ahead of the dependent FMA chain
+constexpr int kSlice = 128;                 // parameters per CTA
+constexpr int kSub = 4, kAggThreads = kSlice * kSub;
+constexpr int kMostRows = 384;              // updates per CTA: 192 KB of shared memory
+constexpr int kMostGroups = 8;
 
-__device__ __forceinline__ void group_range(const ApplyLaunch& p, uint32_t g, uint32_t& lo, uint32_t& hi) {
-  const uint32_t per = (p.hi - p.lo + p.groups - 1) / p.groups;
-  lo = min(p.hi, p.lo + g * per);
-  hi = min(p.hi, lo + per);
-}
+struct AggSmem {   // behind it rows[n][kSlice]
+  float sub[kSub][kSlice], total[kSlice];
+  float eta[kMostRows];
+  int32_t slot[kMostRows];
+  uint32_t row[kMostRows];
+};
 
-// Both kernels are launched with programmatic stream serialisation: their CTAs may become resident
-// while the kernel ahead of them in the stream (the round kernel, then group_totals_kernel) is
-// draining, and they read and write nothing before griddepcontrol.wait, which returns once that
-// kernel - and, because it waited the same way, every kernel before it - has finished.
-__global__ void __launch_bounds__(kAggThreads) group_totals_kernel(ApplyLaunch p) {
+// Launched with programmatic stream serialisation: the CTAs may become resident while the kernel ahead of them in the
+// stream (the round kernel) is draining; before griddepcontrol.wait they read descriptors only, which the host wrote.
+__global__ void __launch_bounds__(kAggThreads) apply_updates_kernel(ApplyLaunch p, uint32_t per) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  AggSmem& sm = *reinterpret_cast<AggSmem*>(smem_raw);
+  float* rows = reinterpret_cast<float*>(smem_raw + sizeof(AggSmem));
+  // The round kernel behind this one may start its set-up: it reads nothing this grid writes before its own wait.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  const uint32_t j = blockIdx.x * kAggThreads + threadIdx.x;
-  if (j >= p.n_params) return;
-  uint32_t lo, hi;
-  group_range(p, blockIdx.y, lo, hi);
-  const float* U = p.U + j;
-  float s = 0.f;
-  uint32_t k = lo;
-  for (; k + kAhead <= hi; k += kAhead) {
-    float u[kAhead];
-#pragma unroll
-    for (int a = 0; a < kAhead; ++a) u[a] = __ldg(U + (size_t)p.applies[k + a].u_row * p.stride);
-#pragma unroll
-    for (int a = 0; a < kAhead; ++a) s = fmaf(-p.applies[k + a].eta, u[a], s);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, j = tid & (kSlice - 1), q = tid / kSlice;
+  const uint32_t lo = min(p.hi, p.lo + blockIdx.y * per), n = min(p.hi, lo + per) - lo;
+  const uint32_t col = blockIdx.x * kSlice, at = col + j;
+  for (uint32_t k = tid; k < n; k += kAggThreads) {
+    const ApplyDesc d = p.applies[lo + k];
+    sm.eta[k] = d.eta; sm.slot[k] = d.snap_slot; sm.row[k] = d.u_row;
   }
-  for (; k < hi; ++k) s = fmaf(-p.applies[k].eta, __ldg(U + (size_t)p.applies[k].u_row * p.stride), s);
-  p.totals[(size_t)blockIdx.y * p.stride + j] = s;
-}
-
-__global__ void __launch_bounds__(kAggThreads) apply_updates_kernel(ApplyLaunch p) {
-  // The round kernel that follows in the stream may be launched with programmatic stream
-  // serialisation: let its CTAs start their set-up (descriptors, first rows) while this grid
-  // runs.  They read nothing this grid writes before their own griddepcontrol.wait, which
-  // returns only once this grid has finished and its writes are visible.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const uint32_t j = blockIdx.x * kAggThreads + threadIdx.x;
-  const uint32_t g = blockIdx.y;
-  uint32_t lo, hi;
-  group_range(p, g, lo, hi);
-  if (j < p.n_params) {
-    float w = p.w_in[j];
-    for (uint32_t q = 0; q < g; ++q) w += p.totals[(size_t)q * p.stride + j];
-    const float* U = p.U + j;
-    uint32_t k = lo;
-    for (; k + kAhead <= hi; k += kAhead) {
-      float u[kAhead];
-#pragma unroll
-      ApplyDesc ds[kAhead];
-#pragma unroll
-      for (int a = 0; a < kAhead; ++a) ds[a] = p.applies[k + a];
-#pragma unroll
-      for (int a = 0; a < kAhead; ++a) u[a] = __ldcs(U + (size_t)ds[a].u_row * p.stride);
-#pragma unroll
-      for (int a = 0; a < kAhead; ++a) {
-        const ApplyDesc d = ds[a];
-        w = fmaf(-d.eta, u[a], w);
-        if (d.snap_slot >= 0) p.snaps[(size_t)d.snap_slot * p.stride + j] = w;
-      }
+  float w = at < p.n_params ? p.w[at] : 0.f;
+  if (col + 4 * lane < p.stride)   // (rows are padded to a multiple of 32 floats)
+    for (uint32_t k = warp; k < n; k += kAggThreads / 32)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                   ::"r"((uint32_t)__cvta_generic_to_shared(rows + k * kSlice + 4 * lane)), "l"(p.U + (size_t)sm.row[k] * p.stride + col + 4 * lane) : "memory");
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  const uint32_t quarter = (n + kSub - 1) / kSub, r0 = min(n, q * quarter), r1 = min(n, r0 + quarter);
+  {
+    float s = 0.f;
+    for (uint32_t k = r0; k < r1; ++k) s = fmaf(-sm.eta[k], rows[k * kSlice + j], s);
+    sm.sub[q][j] = s;
+  }
+  __syncthreads();
+  if (gridDim.y > 1) {
+    if (q == 0) sm.total[j] = (sm.sub[0][j] + sm.sub[1][j]) + (sm.sub[2][j] + sm.sub[3][j]);
+    mma::cluster_sync();
+    for (uint32_t r = 0; r < blockIdx.y; ++r) w += mma::ld_peer(mma::peer_addr((uint32_t)__cvta_generic_to_shared(&sm.total[j]), r));
+  }
+  for (int s = 0; s < q; ++s) w += sm.sub[s][j];
+  if (at < p.n_params) {
+    for (uint32_t k = r0; k < r1; ++k) {
+      w = fmaf(-sm.eta[k], rows[k * kSlice + j], w);
+      if (sm.slot[k] >= 0) p.snaps[(size_t)sm.slot[k] * p.stride + at] = w;
     }
-    for (; k < hi; ++k) {
-      const ApplyDesc d = p.applies[k];
-      w = fmaf(-d.eta, __ldcs(U + (size_t)d.u_row * p.stride), w);
-      if (d.snap_slot >= 0) p.snaps[(size_t)d.snap_slot * p.stride + j] = w;
-    }
-    if (g + 1 == p.groups) {
-      p.w_out[j] = w;
+    if (q == kSub - 1 && blockIdx.y + 1 == gridDim.y) {
+      p.w[at] = w;
       // the server model after this range: a non-finite entry (a NaN or an overflow that came in
       // through a client's rows or step size) is reported, never trapped on
       if (p.status && !isfinite(w)) atomicOr(p.status, 2u);
     }
   }
-  // history map and apply log: one thread per update of the group
+  // history map and apply log: one thread per update of the range
   if (blockIdx.x == 0)
-    for (uint32_t k = lo + threadIdx.x; k < hi; k += kAggThreads) {
-      const ApplyDesc d = p.applies[k];
+    for (uint32_t k = tid; k < n; k += kAggThreads) {
+      const ApplyDesc d = p.applies[lo + k];
       ApplyRec r;
-      r.client = d.client; r.round = d.round; r.seq = k;
+      r.client = d.client; r.round = d.round; r.seq = lo + k;
       r.h_after = atomicAdd(&p.H[d.client], 1u) + 1u;
-      p.log[k] = r;
+      p.log[lo + k] = r;
     }
+  if (gridDim.y > 1) mma::cluster_sync();   // nobody leaves while its total may still be read
 }
 
 __global__ void to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, size_t n) {
@@ -114,11 +106,12 @@ __global__ void to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __r
   for (; i < n; i += step) dst[i] = __float2bfloat16_rn(src[i]);
 }
 
+constexpr int kRingThreads = 128;
 // Peer-to-peer ring: Receive at every node (Algorithm 3: w_c = w_c - eta_k * U) for the sums that
 // reached it, preceded by the node's own sum of the round it has just finished.  One y-block per node
 // whose model moves; a thread keeps its parameter in a register and walks the node's short list.
-__global__ void __launch_bounds__(kAggThreads) ring_apply_kernel(RingApplyLaunch p) {
-  const uint32_t j = blockIdx.x * kAggThreads + threadIdx.x;
+__global__ void __launch_bounds__(kRingThreads) ring_apply_kernel(RingApplyLaunch p) {
+  const uint32_t j = blockIdx.x * kRingThreads + threadIdx.x;
   if (j >= p.n_params) return;
   const RingApplyDesc a = p.applies[p.lo + blockIdx.y];
   float* wp = p.node_w + (size_t)a.node * p.stride + j;
@@ -159,35 +152,51 @@ cudaError_t launch_validate_data(const float* x, const int32_t* y, uint32_t n, u
 
 cudaError_t launch_ring_apply(const RingApplyLaunch& p, cudaStream_t s) {
   if (p.hi <= p.lo) return cudaSuccess;
-  const uint32_t blocks = (p.n_params + kAggThreads - 1) / kAggThreads;
-  ring_apply_kernel<<<dim3(blocks, p.hi - p.lo, 1), kAggThreads, 0, s>>>(p);
+  const uint32_t blocks = (p.n_params + kRingThreads - 1) / kRingThreads;
+  ring_apply_kernel<<<dim3(blocks, p.hi - p.lo, 1), kRingThreads, 0, s>>>(p);
   return cudaGetLastError();
 }
 
-uint32_t apply_groups(uint32_t n_updates) {
-  uint32_t g = n_updates / 32;
-  return g < 1 ? 1 : (g > 32 ? 32 : g);
-}
-
-cudaError_t launch_apply_updates(const ApplyLaunch& p, cudaStream_t s) {
-  if (p.hi <= p.lo) return cudaSuccess;
-  const uint32_t blocks = (p.n_params + kAggThreads - 1) / kAggThreads;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.blockDim = dim3(kAggThreads, 1, 1);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (p.groups > 1) {
-    cfg.gridDim = dim3(blocks, p.groups - 1, 1);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, group_totals_kernel, p);
+cudaError_t launch_apply_updates(const ApplyLaunch& p0, cudaStream_t s) {
+  static bool opted_in[64] = {};   // more than 48 KB of shared memory has to be asked for once per device
+  int dev = 0;
+  cudaError_t de = cudaGetDevice(&dev);
+  if (de != cudaSuccess) return de;
+  const bool known = dev >= 0 && dev < 64;
+  if (!known || !opted_in[dev]) {
+    de = cudaFuncSetAttribute(apply_updates_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(AggSmem) + kMostRows * kSlice * sizeof(float)));
+    if (de != cudaSuccess) return de;
+    if (known) opted_in[dev] = true;
+  }
+  ApplyLaunch p = p0;
+  const uint32_t slices = (p.n_params + kSlice - 1) / kSlice;
+  for (uint32_t lo = p0.lo; lo < p0.hi; lo += kMostRows * kMostGroups) {
+    p.lo = lo;
+    p.hi = min(p0.hi, lo + kMostRows * kMostGroups);
+    const uint32_t n = p.hi - p.lo;
+    // a CTA per 64 updates: a quarter of them is a walk as long as the exchange of totals takes
+    uint32_t groups = 1;
+    while (groups < (uint32_t)kMostGroups && n > 64 * groups) groups *= 2;
+    const uint32_t per = (n + groups - 1) / groups;
+    const size_t smem = sizeof(AggSmem) + (size_t)per * kSlice * sizeof(float);
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1;
+    attr[1].val.clusterDim.y = groups;
+    attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(slices, groups, 1);
+    cfg.blockDim = dim3(kAggThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = groups > 1 ? 2 : 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, apply_updates_kernel, p, per);
     if (e != cudaSuccess) return e;
   }
-  cfg.gridDim = dim3(blocks, p.groups, 1);
-  return cudaLaunchKernelEx(&cfg, apply_updates_kernel, p);
+  return cudaSuccess;
 }
 
 cudaError_t launch_to_bf16(const float* src, void* dst, size_t n, cudaStream_t s) {
