@@ -86,6 +86,41 @@ DevicePool& pool() {
   return *p;
 }
 
+// A few pinned blocks for small read-backs, shared by all handles and threads; kept until the process ends.
+class PinnedPool {
+ public:
+  static constexpr size_t kBlock = 64 << 10;
+  void* get() {   // null: none to be had, go without
+    {
+      std::lock_guard<std::mutex> lock(mu_);
+      if (!free_.empty()) {
+        void* p = free_.back();
+        free_.pop_back();
+        return p;
+      }
+      if (made_ >= kMost) return nullptr;
+      ++made_;
+    }
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, kBlock, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    return p;
+  }
+  void put(void* p) {
+    std::lock_guard<std::mutex> lock(mu_);
+    free_.push_back(p);
+  }
+
+ private:
+  static constexpr int kMost = 16;
+  std::mutex mu_;
+  std::vector<void*> free_;
+  int made_ = 0;
+};
+PinnedPool& pinned() {
+  static PinnedPool* p = new PinnedPool;
+  return *p;
+}
+
 // Bump allocator over a few large device chunks: client data sets are many
 // small allocations of unknown count, and cudaMalloc per client is slow.
 struct Arena {
@@ -280,14 +315,45 @@ aet_status upload_clients(aet_handle* h, cudaStream_t s) {
   return AET_OK;
 }
 
-// After a synchronisation: did a bounded device-side wait give up?
-aet_status check_device_status(aet_handle* h) {
-  uint32_t st = 0;
-  AET_CUDA(h, cudaMemcpy(&st, h->d_status.p, sizeof(st), cudaMemcpyDeviceToHost));
+// What a status word read from the device says.
+aet_status judge_status(aet_handle* h, uint32_t st) {
   if (st) cudaMemset(h->d_status.p, 0, sizeof(uint32_t));
   if (st & 1u) return fail(h, AET_ERR_TIMEOUT, "a bounded wait for an asynchronous row copy gave up; results are invalid");
   if (st & 4u) return fail(h, AET_ERR_STATE, "a debug check failed on the device: a label, row number or slot was out of range; results are invalid");
   if (st & 2u) return fail(h, AET_ERR_NUMERIC, "a non-finite value reached the server model (or, with debug checks, sits in a client's rows); results are invalid");
+  return AET_OK;
+}
+// After a synchronisation: did a bounded device-side wait give up?
+aet_status check_device_status(aet_handle* h) {
+  uint32_t st = 0;
+  AET_CUDA(h, cudaMemcpy(&st, h->d_status.p, sizeof(st), cudaMemcpyDeviceToHost));
+  return judge_status(h, st);
+}
+
+// A model out of the device, once the stream is done and the status word is clean; `out` stays untouched on error.  Small
+// models come with the status word through pinned memory: one wait instead of three.
+aet_status read_model(aet_handle* h, const float* src, float* out, cudaStream_t s) {
+  const size_t bytes = (size_t)h->P * sizeof(float);
+  cudaPointerAttributes attr{};
+  const bool known = cudaPointerGetAttributes(&attr, out) == cudaSuccess;
+  cudaGetLastError();
+  const bool to_host = known && (attr.type == cudaMemoryTypeHost || attr.type == cudaMemoryTypeUnregistered);
+  void* pin = to_host && bytes + 16 <= PinnedPool::kBlock ? pinned().get() : nullptr;
+  if (pin) {
+    uint32_t* st = reinterpret_cast<uint32_t*>(static_cast<char*>(pin) + PinnedPool::kBlock - 16);
+    cudaError_t e = cudaMemcpyAsync(pin, src, bytes, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(st, h->d_status.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    const cudaError_t w = cudaStreamSynchronize(s);   // (also before the block goes back)
+    if (e == cudaSuccess) e = w;
+    aet_status r = e == cudaSuccess ? judge_status(h, *st) : cuda_fail(h, e, "reading a model");
+    if (r == AET_OK) memcpy(out, pin, bytes);
+    pinned().put(pin);
+    return r;
+  }
+  AET_CUDA(h, cudaStreamSynchronize(s));
+  if (aet_status ds = check_device_status(h)) return ds;
+  AET_CUDA(h, cudaMemcpyAsync(out, src, bytes, cudaMemcpyDefault, s));
+  AET_CUDA(h, cudaStreamSynchronize(s));
   return AET_OK;
 }
 
@@ -500,8 +566,7 @@ aet_status aet_reset(aet_handle* h, void* cuda_stream) {
   if (!h) return AET_ERR_ARG;
   join_prepare(h);
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  AET_CUDA(h, cudaMemcpyAsync(h->w_cur(), h->w0.p, h->stride * sizeof(float), cudaMemcpyDeviceToDevice, s));
-  AET_CUDA(h, cudaMemsetAsync(h->d_H.p, 0, h->cfg.n_clients * sizeof(uint32_t), s));
+  AET_CUDA(h, launch_copy_and_zero(h->w_cur(), h->w0.p, h->stride, h->d_H.p, h->cfg.n_clients, s));
   if (h->cfg.topology == 1)
     for (uint32_t c = 0; c < h->cfg.n_clients; ++c)
       AET_CUDA(h, cudaMemcpyAsync(h->node_w.p + (size_t)c * h->stride, h->w0.p, h->stride * sizeof(float), cudaMemcpyDeviceToDevice, s));
@@ -625,7 +690,7 @@ aet_status aet_run_rounds(aet_handle* h, uint32_t n_rounds, void* cuda_stream) {
     std::string err;
     if (!simulate(h->cfg, n_rounds, st, h->delays, cp.sched, err)) return fail(h, AET_ERR_CONFIG, err);
     cp.after = st;
-    build_plan(h->cfg, h->delays, cp.sched.events, (h->cfg.flags & AET_FLAG_KEEP_UPDATE_SUMS) != 0, cp.plan);
+    build_plan(h->cfg, h->delays, cp.sched, (h->cfg.flags & AET_FLAG_KEEP_UPDATE_SUMS) != 0, cp.plan);
     cp.valid = true;
   }
   const Plan& plan = cp.plan;
@@ -653,9 +718,8 @@ aet_status aet_run_rounds(aet_handle* h, uint32_t n_rounds, void* cuda_stream) {
     AET_CUDA(h, cudaMemcpyAsync(h->d_plan.p, pack.data(), plan_bytes, cudaMemcpyHostToDevice, s));
     cp.uploaded = true;
   }
-  AET_CUDA(h, cudaMemsetAsync(h->d_trig.p, 0, E * sizeof(TriggerRec), s));
-  // snapshot 0 = the server model as this call begins
-  AET_CUDA(h, cudaMemcpyAsync(h->snaps.p, h->w_cur(), h->stride * sizeof(float), cudaMemcpyDeviceToDevice, s));
+  // snapshot 0 = the server model as this call begins; no round has been triggered yet
+  AET_CUDA(h, launch_copy_and_zero(h->snaps.p, h->w_cur(), h->stride, reinterpret_cast<uint32_t*>(h->d_trig.p), E * sizeof(TriggerRec) / 4, s));
 
   RoundLaunch r{};
   r.tasks = reinterpret_cast<const TaskDesc*>(h->d_plan.p);
@@ -735,7 +799,7 @@ aet_status aet_prepare_rounds(aet_handle* h, uint32_t n_rounds) {
         SchedState st = cp.before;
         if (!simulate(h->cfg, n_rounds, st, h->prep_delays, cp.sched, err)) return;
         cp.after = st;
-        build_plan(h->cfg, h->prep_delays, cp.sched.events, keep, cp.plan);
+        build_plan(h->cfg, h->prep_delays, cp.sched, keep, cp.plan);
         cp.valid = true;
       }
       h->prep_ok = true;
@@ -750,26 +814,15 @@ aet_status aet_get_global_model(aet_handle* h, float* out, size_t n_params, void
   if (!h || !out) return h ? fail(h, AET_ERR_ARG, "null argument") : AET_ERR_ARG;
   if (n_params != h->P) return fail(h, AET_ERR_ARG, "n_params does not match the model");
   if (h->cfg.topology == 1) return fail(h, AET_ERR_STATE, "the peer-to-peer topology has no server model: use aet_get_node_model");
-  cudaStream_t s = (cudaStream_t)cuda_stream;
-  AET_CUDA(h, cudaStreamSynchronize(s));
-  if (aet_status ds = check_device_status(h)) return ds;   // `out` stays untouched on error
-  AET_CUDA(h, cudaMemcpyAsync(out, h->w_cur(), (size_t)h->P * sizeof(float), cudaMemcpyDefault, s));
-  AET_CUDA(h, cudaStreamSynchronize(s));
-  return AET_OK;
+  return read_model(h, h->w_cur(), out, (cudaStream_t)cuda_stream);
 }
 
 aet_status aet_get_node_model(aet_handle* h, uint32_t node, float* out, size_t n_params, void* cuda_stream) {
   if (!h || !out) return h ? fail(h, AET_ERR_ARG, "null argument") : AET_ERR_ARG;
   if (n_params != h->P) return fail(h, AET_ERR_ARG, "n_params does not match the model");
   if (node >= h->cfg.n_clients) return fail(h, AET_ERR_ARG, "node index out of range");
-  cudaStream_t s = (cudaStream_t)cuda_stream;
-  AET_CUDA(h, cudaStreamSynchronize(s));
-  if (aet_status ds = check_device_status(h)) return ds;
   // client-server: at quiescence every client slot equals the server model
-  const float* src = h->cfg.topology == 1 ? h->node_w.p + (size_t)node * h->stride : h->w_cur();
-  AET_CUDA(h, cudaMemcpyAsync(out, src, (size_t)h->P * sizeof(float), cudaMemcpyDefault, s));
-  AET_CUDA(h, cudaStreamSynchronize(s));
-  return AET_OK;
+  return read_model(h, h->cfg.topology == 1 ? h->node_w.p + (size_t)node * h->stride : h->w_cur(), out, (cudaStream_t)cuda_stream);
 }
 
 aet_status aet_get_update_sum(aet_handle* h, uint32_t seq, float* out, size_t n_params, void* cuda_stream) {
@@ -970,7 +1023,7 @@ uint32_t aet_debug_plan_waves(const aet_config* cfg, uint32_t n_rounds) {
   SchedResult res;
   if (!simulate(*cfg, n_rounds, st, cache, res, err)) return 0;
   Plan plan;
-  build_plan(*cfg, cache, res.events, (cfg->flags & AET_FLAG_KEEP_UPDATE_SUMS) != 0, plan);
+  build_plan(*cfg, cache, res, (cfg->flags & AET_FLAG_KEEP_UPDATE_SUMS) != 0, plan);
   return (uint32_t)plan.apply_upto.size();
 }
 
@@ -987,7 +1040,7 @@ aet_status aet_debug_plan_layout(const aet_config* cfg, uint32_t n_rounds, uint3
   SchedResult res;
   if (!simulate(*cfg, n_rounds, st, cache, res, err)) return fail(nullptr, AET_ERR_CONFIG, err);
   Plan plan;
-  build_plan(*cfg, cache, res.events, (cfg->flags & AET_FLAG_KEEP_UPDATE_SUMS) != 0, plan);
+  build_plan(*cfg, cache, res, (cfg->flags & AET_FLAG_KEEP_UPDATE_SUMS) != 0, plan);
   const uint32_t n_waves = (uint32_t)plan.apply_upto.size();
   for (uint32_t L = 0; L < n_waves; ++L) {
     apply_upto[L] = plan.apply_upto[L];

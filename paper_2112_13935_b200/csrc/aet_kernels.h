@@ -184,6 +184,9 @@ __device__ __forceinline__ void publish_empty_round(const RoundLaunch& p, const 
 }
 #endif
 
+// dst[0, n) = src (n a multiple of 4), zero[0, nz) = 0 (nz words): what a run or a reset sets up, in one launch
+cudaError_t launch_copy_and_zero(float* dst, const float* src, size_t n, uint32_t* zero, size_t nz, cudaStream_t s);
+
 // bf16 conversion of a client's rows at load time (precision 1).
 cudaError_t launch_to_bf16(const float* src, void* dst, size_t n, cudaStream_t s);
 

@@ -278,8 +278,16 @@ bool simulate(const aet_config& c, uint32_t n_rounds, SchedState& st, DelayCache
     if (round + 1 < last) q.push({e.t_trigger, kStart, cl, round + 1});
   }
   if (n_blocked || seq != out.events.size()) { err = "schedule did not reach quiescence"; return false; }
-  std::sort(out.events.begin(), out.events.end(),
-            [](const aet_event& a, const aet_event& b) { return a.seq < b.seq; });
+  // Events were made as their rounds started, that is in (t_start, client, round) order; seq is a permutation of them.
+  out.by_start.resize(out.events.size());
+  {
+    std::vector<aet_event> made(out.events.size());
+    made.swap(out.events);
+    for (size_t k = 0; k < made.size(); ++k) {
+      out.by_start[k] = made[k].seq;
+      out.events[made[k].seq] = made[k];
+    }
+  }
 
   aet_summary& s = out.summary;
   s = aet_summary{};
@@ -296,23 +304,17 @@ bool simulate(const aet_config& c, uint32_t n_rounds, SchedState& st, DelayCache
   return true;
 }
 
-void build_plan(const aet_config& c, const DelayCache& cache, const std::vector<aet_event>& events, bool keep_all, Plan& plan) {
+void build_plan(const aet_config& c, const DelayCache& cache, const SchedResult& sched, bool keep_all, Plan& plan) {
+  const std::vector<aet_event>& events = sched.events;
   const size_t E = events.size();
   plan = Plan{};
   plan.applies.resize(E);
   plan.u_row_of.assign(E, 0);
   // Level of a task = 1 + max(level of every update it starts from, level of
   // the client's previous round).  Tasks of one level are mutually independent.
-  std::vector<uint32_t> order(E);
-  for (size_t k = 0; k < E; ++k) order[k] = (uint32_t)k;
-  std::sort(order.begin(), order.end(), [&](uint32_t a, uint32_t b) {
-    // an empty round starts and ends on the same tick as the client's next one: keep round order
-    return std::tie(events[a].t_start, events[a].client, events[a].round) <
-           std::tie(events[b].t_start, events[b].client, events[b].round);
-  });
   std::vector<uint32_t> level(E, 0), prev_level(c.n_clients, 0);
   uint32_t pref = 0, pref_max = 0, n_waves = 0;
-  for (uint32_t k : order) {
+  for (uint32_t k : sched.by_start) {   // (of rounds starting on one tick, an empty one and its client's next among them, the earlier first)
     const aet_event& e = events[k];
     while (pref < e.seen) { pref_max = std::max(pref_max, level[pref]); ++pref; }
     uint32_t lv = 1 + std::max(pref_max, prev_level[e.client]);
@@ -322,12 +324,13 @@ void build_plan(const aet_config& c, const DelayCache& cache, const std::vector<
   }
   // Tasks grouped by wave, longest first.
   std::vector<uint32_t> by_wave(E);
-  for (size_t k = 0; k < E; ++k) by_wave[k] = (uint32_t)k;
-  std::sort(by_wave.begin(), by_wave.end(), [&](uint32_t a, uint32_t b) {
-    if (level[a] != level[b]) return level[a] < level[b];
-    if (events[a].samples != events[b].samples) return events[a].samples > events[b].samples;
-    return a < b;
-  });
+  {
+    struct Key { uint64_t wave_size; uint32_t seq; };   // wave, then ~samples
+    std::vector<Key> keys(E);
+    for (size_t k = 0; k < E; ++k) keys[k] = {(uint64_t)level[k] << 32 | (uint32_t)~events[k].samples, (uint32_t)k};
+    std::sort(keys.begin(), keys.end(), [](const Key& a, const Key& b) { return a.wave_size != b.wave_size ? a.wave_size < b.wave_size : a.seq < b.seq; });
+    for (size_t k = 0; k < E; ++k) by_wave[k] = keys[k].seq;
+  }
   plan.wave_off.assign(n_waves + 1, 0);
   plan.apply_upto.assign(n_waves, 0);
   for (uint32_t k : by_wave) plan.wave_off[level[k]] += 1;   // size of wave level-1, shifted by one
@@ -345,11 +348,15 @@ void build_plan(const aet_config& c, const DelayCache& cache, const std::vector<
     plan.apply_upto[L] = std::max(upto, L ? plan.apply_upto[L - 1] : 0u);
   }
   // A client's update sums still in flight when one of its rounds starts.
-  std::vector<std::vector<uint32_t>> mine(c.n_clients);
-  for (size_t k = 0; k < E; ++k) mine[events[k].client].push_back((uint32_t)k);
+  std::vector<uint32_t> mine_off(c.n_clients + 2, 0), mine(E);   // every client's updates in seq order
+  for (size_t k = 0; k < E; ++k) mine_off[events[k].client + 2] += 1;
+  for (uint32_t cl = 2; cl <= c.n_clients; ++cl) mine_off[cl] += mine_off[cl - 1];
+  for (size_t k = 0; k < E; ++k) mine[mine_off[events[k].client + 1]++] = (uint32_t)k;
   auto for_each_inflight = [&](const aet_event& e, auto&& fn) {
-    for (uint32_t j : mine[e.client])
+    for (uint32_t i = mine_off[e.client]; i < mine_off[e.client + 1]; ++i) {
+      const uint32_t j = mine[i];
       if (events[j].round < e.round && events[j].seq >= e.seen) fn(j);
+    }
   };
 
   // ---- rows of the update-sum array and snapshot slots ----

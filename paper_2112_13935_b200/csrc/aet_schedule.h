@@ -29,6 +29,7 @@ struct DelayCache {
 
 struct SchedResult {
   std::vector<aet_event> events;  // ordered by seq
+  std::vector<uint32_t> by_start; // their seqs in (t_start, client, round) order
   aet_summary summary;
 };
 
@@ -78,7 +79,7 @@ struct Plan {
 // keep_all: one row per event and one slot per distinct start position, never reused
 // (row = seq), so that every update sum can be read back after the run.  Otherwise rows
 // and slots are recycled as soon as nothing later in the launch order reads them.
-void build_plan(const aet_config& c, const DelayCache& cache, const std::vector<aet_event>& events, bool keep_all, Plan& plan);
+void build_plan(const aet_config& c, const DelayCache& cache, const SchedResult& sched, bool keep_all, Plan& plan);
 
 // ---- peer-to-peer ring (Section 1, Fig. 1b) ------------------------------
 // Every node keeps its own model and history map; a round's sum goes to the two ring neighbours
