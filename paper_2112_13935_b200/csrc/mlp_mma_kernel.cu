@@ -14,6 +14,9 @@
 //   3  every CTA runs the narrow layers, the softmax and the backward pass down to dZ_0 redundantly (same inputs, same
 //      order: the same bits in every CTA);
 //   4  dW_0^T = dZ_0^T X over the CTA's inputs: the accumulator fragment is the thread's own piece of W_0^T - update in place.
+//      With bf16 operands the next iteration's step 1 rides along: an entry of W_0 is read and written once per iteration
+//      (3.4 -> 3.1 ms at 12 clients of 3072-128-32-10).  fp32 keeps two passes: cross terms and split dZ_0 together do not
+//      fit the registers without giving up the loads in flight (32.9 instead of 32.5 ms).
 // The hand-overs need no cluster barrier: a CTA sends its part of Z_0 for the next iteration only after it has all of A_0
 // of this one, which the owners sent after taking everybody's part.
 //
@@ -56,7 +59,7 @@ struct MmaPlan {
   int CL, units, upc, upw;          // 16-input units: all, per CTA, per warp
   int MT, WM, WK;                   // hidden tiles of 16; warps over tiles, over input parts
   int rgs;                          // hidden rows owned per CTA, in groups of 8
-  int xpitch, xbufs;                // minibatch columns: elements per row, buffers
+  int xpitch;                       // minibatch columns (two buffers): elements per row
   int ap[kMaxL], zp[kMaxL], wp[kMaxL], np[kMaxL];   // pitches of A_l, dZ_l, W_l (l >= 1), padded rows of W_l
   int ext;                          // words per thread beyond tensor memory
   // offsets in floats
@@ -94,10 +97,9 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
   auto take = [&](int floats) { const int at = o; o += up(floats, 4); return at; };
   const int elems = bf ? 2 : 1;      // elements per float
   p.xpitch = 16 * p.upc + 8;         // 8 mod 16 elements: fragment loads hit different banks
-  p.xbufs = 2;
   p.o_bar = take(16);
   p.o_idx = take(4 * 64);
-  p.o_x = take(p.xbufs * p.Bp * p.xpitch / elems);
+  p.o_x = take(2 * p.Bp * p.xpitch / elems);
   p.o_in = take(cl * p.rgs * 8 * p.Bp);
   const int part = (p.WK - 1) * p.WM * p.bt * 128;
   for (int l = 0; l < p.nl; ++l) {
@@ -395,7 +397,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   constexpr int kChunk = 16 / (int)sizeof(T);
   const bool whole = (D0 * sizeof(T)) % 16 == 0;
   auto copy_rows = [&](uint32_t it) {
-    T* x = xb0 + (it % m.xbufs) * Bp * m.xpitch;
+    T* x = xb0 + (it & 1) * Bp * m.xpitch;
     const T* src = reinterpret_cast<const T*>(cd.x) + x0;
 #pragma unroll 1
     for (int r = warp; r < B; r += kWarps) {
@@ -513,50 +515,54 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   }
   const int own_q = tid / Bp, own_b = tid - own_q * Bp;   // this thread's four owned rows and sample in step 2
 
+  float acc[BT][4], crs[BT][4];   // this warp's part of Z_0^T; (fp32) the cross terms
+  auto clear = [&]() {
+#pragma unroll
+    for (int b = 0; b < BT; ++b)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) { acc[b][c] = 0.f; crs[b][c] = 0.f; }
+  };
+  auto forward = [&](const T* xu, const float (&w)[8]) {   // one unit of inputs
+#pragma unroll
+    for (int h = 0; h < 16 / kStep; ++h) {
+      FragA<BF> a;
+      FragB<BF> f[BT];
+      if constexpr (BF) {
+        a.v[0] = pack_bf16(w[0], w[1]); a.v[1] = pack_bf16(w[2], w[3]);
+        a.v[2] = pack_bf16(w[4], w[5]); a.v[3] = pack_bf16(w[6], w[7]);
+      } else {
+        a.v[0] = split(w[4 * h]); a.v[1] = split(w[4 * h + 2]);
+        a.v[2] = split(w[4 * h + 1]); a.v[3] = split(w[4 * h + 3]);
+      }
+#pragma unroll
+      for (int b = 0; b < BT; ++b) load_s(f[b], xu + 8 * b * m.xpitch + 8 * h, m.xpitch, g, tt);
+      products(acc, crs, crs, a, f);
+    }
+  };
+  auto forward_all = [&](const T* X) {
+    clear();
+#pragma unroll 1
+    for (int u = 0; u < wn; ++u) {
+      uint32_t r[8];
+      float w[8];
+      own.issue(u, r);
+      own.wait(r, w);
+      forward(X + 16 * (w0 + u), w);
+    }
+  };
+  auto rows_of = [&](uint32_t it) { return xb0 + (it & 1) * Bp * m.xpitch; };
+
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();   // the first rows are in
+  if (BF) forward_all(rows_of(0));
+
 #pragma unroll 1
   for (uint32_t it = 0; it < t.steps; ++it) {
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (it + 1 < t.steps) draw_rows(it + 1);
-    __syncthreads();   // this iteration's rows are in, the next one's numbers too; everybody is done with the last one
-    const T* X = xb0 + (it % m.xbufs) * Bp * m.xpitch;
-    if (it + 1 < t.steps) copy_rows(it + 1);
-
     // ================= 1: this CTA's part of Z_0^T =================
+    if (!BF) forward_all(rows_of(it));
     {
-      float acc[BT][4], crs[BT][4];
-#pragma unroll
-      for (int b = 0; b < BT; ++b)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) { acc[b][c] = 0.f; crs[b][c] = 0.f; }
-#pragma unroll 1
-      for (int u = 0; u < wn; ++u) {
-        const T* xu = X + 16 * (w0 + u);
-        uint32_t r[8];
-        float w[8];
-        own.issue(u, r);
-        FragB<BF> f[BT];
-#pragma unroll
-        for (int b = 0; b < BT; ++b)
-          load_s(f[b], xu + 8 * b * m.xpitch, m.xpitch, g, tt);
-        own.wait(r, w);
-#pragma unroll
-        for (int h = 0; h < 16 / kStep; ++h) {
-          FragA<BF> a;
-          if constexpr (BF) {
-            a.v[0] = pack_bf16(w[0], w[1]); a.v[1] = pack_bf16(w[2], w[3]);
-            a.v[2] = pack_bf16(w[4], w[5]); a.v[3] = pack_bf16(w[6], w[7]);
-          } else {
-            a.v[0] = split(w[4 * h]); a.v[1] = split(w[4 * h + 2]);
-            a.v[2] = split(w[4 * h + 1]); a.v[3] = split(w[4 * h + 3]);
-          }
-          if (h) {
-#pragma unroll
-            for (int b = 0; b < BT; ++b)
-              load_s(f[b], xu + 8 * b * m.xpitch + 8 * h, m.xpitch, g, tt);
-          }
-          products(acc, crs, crs, a, f);
-        }
-      }
+      if (it + 1 < t.steps) draw_rows(it + 1);
+      __syncthreads();   // everybody is out of the last pass: the buffer of its rows and the area of dZ_0 are free
       if (!BF) {
 #pragma unroll
         for (int b = 0; b < BT; ++b)
@@ -591,6 +597,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         }
       }
     }
+
+    if (it + 1 < t.steps) copy_rows(it + 1);
 
     // ================= 2: owned rows: sum over the CTAs, bias, ReLU; A_0 (or the logits) to every CTA =================
     if (nrg > 0) {
@@ -756,6 +764,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           gb[0] = s0; gb[8] = s1;
         }
       }
+      if (l == 1) asm volatile("cp.async.wait_group 0;" ::: "memory");   // the next rows, for everybody behind this barrier
       __syncthreads();
       // dW_l^T = dZ_l^T A_{l-1}, update
       const int mt = m.np[l] / 16, ni = up(m.d[l], 16) / 8;
@@ -795,7 +804,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       }
     }
     // biases: every layer's gradient is in (the barriers above lie between)
-    if (nl == 1) __syncthreads();
+    if (nl == 1) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+    }
 #pragma unroll 1
     for (int e = tid; e < m.nb; e += kThreads) {
       const float gb = gbias[e] + smem[m.o_gb2 + e];
@@ -803,8 +815,12 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       ubias[e] += gb;
     }
 
-    // ================= 4: dW_0^T over this CTA's inputs, update in place =================
+    // ================= 4: dW_0^T over this CTA's inputs, update in place; bf16: the next Z_0 in the same pass =================
     if (wn > 0) {
+      const bool more = it + 1 < t.steps;
+      const T* X = rows_of(it);
+      const T* Xn = rows_of(it + 1);
+      if (BF) clear();
       constexpr int kBk = 8 * BT / kStep;   // k-steps over the samples at most
       constexpr bool kHold = BF || BT <= 4;   // room for all of dZ_0's fragments
       FragA<BF> a[kHold ? kBk : 1];
@@ -819,19 +835,19 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         uint32_t r[8], rs[8];
         own.issue(u, r);
         if (!BF) own.issue(ug + u, rs);
-        float acc[2][4] = {}, x1[2][4] = {}, x2[2][4] = {};
+        float d[2][4] = {}, x1[2][4] = {}, x2[2][4] = {};
 #pragma unroll
         for (int k = 0; k < kBk; ++k) {
-            if (!kHold) load_zt(a[0], Z(0) + k * kStep * m.zp[0] + 16 * wm, m.zp[0], lane);
-            FragB<BF> f[2];
-            load_st2(f, xu + k * kStep * m.xpitch, m.xpitch, lane);
-            products(acc, x1, x2, a[kHold ? k : 0], f);
-          }
+          if (!kHold) load_zt(a[0], Z(0) + k * kStep * m.zp[0] + 16 * wm, m.zp[0], lane);
+          FragB<BF> f[2];
+          load_st2(f, xu + k * kStep * m.xpitch, m.xpitch, lane);
+          products(d, x1, x2, a[kHold ? k : 0], f);
+        }
         float w[8], us[8];
         own.wait(r, w);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          us[i] = fmaf(lambda, w[i], term<BF>(acc[i >> 2][i & 3], x1[i >> 2][i & 3], x2[i >> 2][i & 3]));   // the gradient
+          us[i] = fmaf(lambda, w[i], term<BF>(d[i >> 2][i & 3], x1[i >> 2][i & 3], x2[i >> 2][i & 3]));   // the gradient
           w[i] = fmaf(-eta, us[i], w[i]);
         }
         own.store(u, w);
@@ -842,6 +858,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           for (int i = 0; i < 8; ++i) us[i] += v[i];
           own.store(ug + u, us);
         }
+        if (BF && more) forward(Xn + 16 * (w0 + u), w);
       }
       own.store_wait();
     }
