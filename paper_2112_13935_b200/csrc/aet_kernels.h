@@ -53,17 +53,13 @@ struct RoundLaunch {
 // One CTA waits (at most max_polls polls) on a barrier nobody signals, then sets bit 0 of *status.
 cudaError_t launch_wait_probe(uint32_t* status, uint32_t max_polls, cudaStream_t s);
 
-// Softmax regression 784 -> 10, batch 1: one CTA per round-task; the kernel is picked by lambda and by
-// how many round-tasks the launch holds.  Asynchronous on s; may start under the tail of the previous kernel in s
+// Softmax regression 784 -> 10, batch 1; the kernel is picked by how many round-tasks the launch holds.  Asynchronous on s; may start under the tail of the previous kernel in s
 // (programmatic stream serialisation) and waits on the device before reading that kernel's output.
 cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s);
 // at most one round-task per SM: a cluster of up to four CTAs per round-task (see lr_chain_kernel.cu)
 cudaError_t launch_lr_chain_rounds(const RoundLaunch& p, uint32_t sms, cudaStream_t s);
 // one CTA per round-task; crowded: two CTAs per SM (see lr_block_kernel.cu)
 cudaError_t launch_lr_block_rounds(const RoundLaunch& p, bool crowded, cudaStream_t s);
-// lambda = 0, more round-tasks than SMs: update sum in tensor memory, accumulated by tcgen05.mma (tf32 x 3)
-bool lr_tc_eligible(const RoundLaunch& p);
-cudaError_t launch_lr_tc_rounds(const RoundLaunch& p, cudaStream_t s);
 
 struct MlpShape {
   uint32_t n_layers, dims[8], batch, precision;
@@ -87,13 +83,6 @@ cudaError_t launch_mlp_wide_rounds(const MlpLaunch& p, cudaStream_t s);
 // spread over a cluster (see mlp_mma_kernel.cu)
 bool mlp_mma_eligible(const MlpShape& shape);
 cudaError_t launch_mlp_mma_rounds(const MlpLaunch& p, cudaStream_t s);
-// fp32 784-128-C models, batch 32: the model stays on-chip for the whole round (4-CTA cluster)
-bool mlp_res_eligible(const MlpLaunch& p);
-cudaError_t launch_mlp_res_rounds(const MlpLaunch& p, cudaStream_t s);
-// bf16 D0-256-128-C models, batch 64: one CTA per round-task streams the first layer through a
-// warp-specialised tcgen05 pipeline (see mlp_stream_kernel.cu)
-bool mlp_stream_eligible(const MlpShape& shape);
-cudaError_t launch_mlp_stream_rounds(const MlpLaunch& p, cudaStream_t s);
 // bf16 models whose first layer fits the tensor-core kernel (tcgen05 + TMEM)
 bool mlp_tc_eligible(const MlpShape& shape);
 cudaError_t launch_mlp_tc_rounds(const MlpLaunch& p, cudaStream_t s);

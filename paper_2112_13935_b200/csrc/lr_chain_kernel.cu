@@ -16,9 +16,9 @@
 //                with the model that gives;
 //   Gram warps   the products of the rows of a block with one another and with those of the block before;
 //   producer     row copies and labels, as soon as a block has left its slot;
-//   (clusters)   one warp adds the CTAs' parts of the couplings.
+//   sum warp     adds the CTAs' parts of the couplings.
 // Partial sums over warps and CTAs are added in a fixed order.
-// Few round-tasks leave SMs idle, so a round-task takes a cluster of 4, 2 or 1 CTAs, each with its range of the
+// Few round-tasks leave SMs idle, so a round-task takes a cluster of 4 or 2 CTAs, each with its range of the
 // inputs (98 k-steps of 8); the recurrence is repeated in every CTA (same inputs, same order: the same bits).
 //
 // The products are m16n8k8 tf32 with split operands (mma_common.cuh).  U^T[class][pixel] accumulates in the fragment
@@ -74,8 +74,8 @@ struct Shape {
   static constexpr int kPitch = kCols % 16 == 8 ? kCols : kCols + 8;
   // Rings of what CTAs send one another.  A CTA that has the deltas of block k knows that its peers have taken what
   // belongs to block k - 2; it may itself be sending logits of block k + 2 and couplings of block k + NS.
-  static constexpr int kInZ = CL > 1 ? 4 : 2, kInG = CL > 1 ? NS + 2 : NS;
-  static constexpr int kWarps = QUIET ? (NM + NG + 2) / 3 * 4 : NM + NG + (CL > 1 ? 3 : 2);
+  static constexpr int kInZ = 4, kInG = NS + 2;
+  static constexpr int kWarps = QUIET ? (NM + NG + 2) / 3 * 4 : NM + NG + 3;
   static constexpr int kThreads = kWarps * 32;
   static constexpr bool kCarry = KG <= 7;   // Gram warps keep the split rows of the block before in registers
   static_assert(!QUIET || (NM + NG > 6 && NM + NG <= 12), "three schedulers for the products, the fourth for the rest");
@@ -87,10 +87,10 @@ struct Shape {
     float gpart[2][NG][kCoup];
     float zin[kInZ][CL][kZ];        // per CTA of the cluster
     float gin[kInG][CL][kCoup];
-    float coup[CL > 1 ? 2 : 1][CL > 1 ? kCoup : 4];   // summed over the cluster
-    float zsum[CL > 1 ? 2 : 1][CL > 1 ? kZ : 4];
+    float coup[2][kCoup];   // summed over the cluster
+    float zsum[2][kZ];
     float dbuf[2][2][kB * kCh];     // deltas by parity of the block and class half: [sample][five classes]
-    uint32_t amax[kInG][16];        // largest coupling, as bits: per Gram warp (one CTA), or [0] (cluster)
+    uint32_t amax[2];               // largest coupling, as bits
     float qp[32];                   // powers of q
     int ys[8][kB];
     uint64_t full[NS], freed[NS];
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
 
   const TaskDesc t = p.by_value ? p.one_task : p.tasks[p.task_begin + blockIdx.x / CL];
   if (!debug_task_ok(p, t)) return;
-  const uint32_t rank = CL > 1 ? mma::cluster_rank() : 0;
+  const uint32_t rank = mma::cluster_rank();
   if (t.n_samples == 0) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (rank == 0) publish_empty_round(p, t, kParams);
@@ -125,7 +125,6 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
     if (id < NM) { role = kModel; warp = id; }
     else if (id < NM + NG) { role = kGram; warp = id - NM; }
     else { role = min(kRec + (id - NM - NG), (int)kIdle); warp = 0; }
-    if (CL == 1 && role == kSum) role = kIdle;
   }
   const uint32_t n = t.n_samples, nblk = (n + kB - 1) / kB;
   const float eta = t.eta, neta = -t.eta;
@@ -136,8 +135,8 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) { mbar_init(&sm.full[s], 1); mbar_init(&sm.freed[s], NM + NG); }
-    for (int s = 0; s < S::kInZ; ++s) mbar_init(&sm.bz[s], CL > 1 ? 1 : 2);
-    for (int s = 0; s < S::kInG; ++s) mbar_init(&sm.bg[s], CL > 1 ? 1 : NG);
+    for (int s = 0; s < S::kInZ; ++s) mbar_init(&sm.bz[s], 1);
+    for (int s = 0; s < S::kInG; ++s) mbar_init(&sm.bg[s], 1);
     for (int s = 0; s < 2; ++s) { mbar_init(&sm.ready[s], 1); mbar_init(&sm.delta[s], 1); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     double q = 1.0 - (double)eta * (double)p.l2, v = 1.0;
@@ -146,7 +145,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
   for (int i = threadIdx.x; i < 2 * kDbuf; i += S::kThreads) (&sm.dbuf[0][0][0])[i] = 0.f;
   for (int i = threadIdx.x; i < NS * kB; i += S::kThreads)   // columns no copy writes: inputs that add nothing
     for (int c = 8 * cnt; c < S::kCols; ++c) sm.rows[i / kB][i % kB][c] = 0.f;
-  if (CL > 1) mma::cluster_sync(); else __syncthreads();   // a peer's barriers exist before anything is sent to it
+  mma::cluster_sync();   // a peer's barriers exist before anything is sent to it
 
   // After a wait has given up nothing waits any more: the round runs through on whatever is there, the status
   // word is set, and every CTA of the cluster reaches the end.
@@ -166,16 +165,11 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
     const int s_mine = lane & 15, h = lane >> 4;
     const float* dall0 = &sm.dbuf[0][h][0];
     for (uint32_t k = 0; k < nblk; ++k) {
-      const int b = k & 1, ig = k % S::kInG, iz = k % S::kInZ;
+      const int b = k & 1;
       const uint32_t nv = min((uint32_t)kB, n - k * kB);
-      if (CL > 1) {
-        wait(&sm.ready[b], (k >> 1) & 1);
-      } else {
-        wait(&sm.bg[ig], (k / S::kInG) & 1);
-        wait(&sm.bz[iz], (k / S::kInZ) & 1);
-      }
-      const float* in = CL > 1 ? sm.coup[b] : sm.gin[ig][0];
-      const float* zi = CL > 1 ? sm.zsum[b] : sm.zin[iz][0];
+      wait(&sm.ready[b], (k >> 1) & 1);
+      const float* in = sm.coup[b];
+      const float* zi = sm.zsum[b];
       float z0[kCh], L[kB];
 #pragma unroll
       for (int c = 0; c < kCh; ++c) z0[c] = zi[(h * kCh + c) * kB + s_mine];
@@ -185,7 +179,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
         const float4 v = lr4[i];
         L[4 * i] = v.x; L[4 * i + 1] = v.y; L[4 * i + 2] = v.z; L[4 * i + 3] = v.w;
       }
-      const float amax = __uint_as_float(CL > 1 ? sm.amax[b][0] : warp_max(lane < NG ? sm.amax[ig][lane] : 0u));
+      const float amax = __uint_as_float(sm.amax[b]);
       const int y = sm.ys[k & 7][s_mine];
       // acc[c] += sum over s < cnt of f[s] delta[s][c]; deltas lie [sample][class] in a class half, five apart
       auto add_deltas = [&](const float* d, const float (&f)[kB], float (&acc)[kCh]) {
@@ -292,7 +286,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.full[sb]);
     }
-  } else if (CL > 1 && role == kSum) {
+  } else if (role == kSum) {
     // ================= the CTAs' parts, summed in rank order =================
     if (lane == 0) {
       mbar_expect_tx(&sm.bg[0], CL * kSendG0);
@@ -318,7 +312,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
         if (k) out[kOffC + at] = c;
       }
       const uint32_t m = warp_max(__float_as_uint(big));
-      if (lane == 0) sm.amax[b][0] = m;
+      if (lane == 0) sm.amax[b] = m;
       wait_cluster(&sm.bz[iz], (k / S::kInZ) & 1);
 #pragma unroll
       for (int i = 0; i < kZ / 32; ++i) {
@@ -390,7 +384,6 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
       // CTA of the cluster
       const int ig = kb % S::kInG;
       const float one = rank == 0 ? scale : 0.f;   // the bias input's part of a coupling
-      uint32_t big = 0;
       const int e = warp * 32 + lane;
       const bool own = e < 64;
       const int tr = (e & 63) >> 2, s0 = 4 * (e & 3);
@@ -413,27 +406,12 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
           float f = scale;
           if (decay) f *= sm.qp[own ? max(tr - 1 - s0 - i, 0) : tr + kB - 1 - s0 - i];
           v[i] = fmaf(v[i], f, one);
-          if (own) {
-            if (s0 + i >= tr) v[i] = 0.f;
-            if (CL == 1) big = max(big, __float_as_uint(fabsf(v[i])));
-          }
+          if (own && s0 + i >= tr) v[i] = 0.f;
         }
         const float4 out = make_float4(v[0], v[1], v[2], v[3]);
-        if (CL == 1) {
-          *reinterpret_cast<float4*>(&sm.gin[ig][0][at]) = out;
-        } else {
-          const uint32_t to = smem_addr(&sm.gin[ig][rank][at]), bar = smem_addr(&sm.bg[ig]);
+        const uint32_t to = smem_addr(&sm.gin[ig][rank][at]), bar = smem_addr(&sm.bg[ig]);
 #pragma unroll
-          for (uint32_t r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(to, r), out, mma::peer_addr(bar, r));
-        }
-      } else if (CL == 1 && own) {   // on or above the diagonal
-        *reinterpret_cast<float4*>(&sm.gin[ig][0][tr * kGp + s0]) = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      if (CL == 1) {
-        big = warp_max(big);
-        if (lane == 0) sm.amax[ig][warp] = big;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.bg[ig]);
+        for (uint32_t r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(to, r), out, mma::peer_addr(bar, r));
       }
     }
   } else if (role == kModel) {
@@ -610,17 +588,9 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
               const float4 x = *reinterpret_cast<const float4*>(&sm.zpart[kb & 1][w][4 * e]);
               v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
             }
-            if (CL == 1) {
-              *reinterpret_cast<float4*>(&sm.zin[iz][0][4 * e]) = v;
-            } else {
-              const uint32_t to = smem_addr(&sm.zin[iz][rank][4 * e]), bar = smem_addr(&sm.bz[iz]);
+            const uint32_t to = smem_addr(&sm.zin[iz][rank][4 * e]), bar = smem_addr(&sm.bz[iz]);
 #pragma unroll
-              for (uint32_t r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(to, r), v, mma::peer_addr(bar, r));
-            }
-          }
-          if (CL == 1) {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.bz[iz]);
+            for (uint32_t r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(to, r), v, mma::peer_addr(bar, r));
           }
         }
       }
@@ -664,7 +634,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
     }
   }
   if (!ok && p.status && lane == 0) atomicOr(p.status, 1u);
-  if (CL > 1) mma::cluster_sync(); else __syncthreads();   // no CTA leaves while a peer may still send to it
+  mma::cluster_sync();   // no CTA leaves while a peer may still send to it
   if (!ok && role == kProd)   // copies still in flight target this CTA's shared memory: a bounded chance to land
     for (int s = 0; s < NS; ++s) {
       mbar_wait_limit(&sm.full[s], 0, 1u << 16);
@@ -677,7 +647,6 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
   }
 }
 
-typedef Shape<1, 10, 10, 4, 25, 3, false> One;
 typedef Shape<2, 7, 7, 6, 9, 4, false> Two;
 typedef Shape<4, 5, 5, 4, 7, 4, true> Four;
 
@@ -695,7 +664,7 @@ cudaError_t launch(const RoundLaunch& p, cudaStream_t s) {
   attr[1].val.clusterDim.x = S::kCl;
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = S::kCl > 1 ? 2 : 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, lr_chain_kernel<S>, p);
 }
 
@@ -708,9 +677,7 @@ cudaError_t launch_lr_chain_rounds(const RoundLaunch& p, uint32_t sms, cudaStrea
   if (e != cudaSuccess) return e;
   const bool known = dev >= 0 && dev < 64;
   if (!known || !opted_in[dev]) {
-    e = cudaFuncSetAttribute(lr_chain_kernel<One>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(One::Smem));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(lr_chain_kernel<Two>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Two::Smem));
+    e = cudaFuncSetAttribute(lr_chain_kernel<Two>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Two::Smem));
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(lr_chain_kernel<Four>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Four::Smem));
     if (e != cudaSuccess) return e;
@@ -718,8 +685,7 @@ cudaError_t launch_lr_chain_rounds(const RoundLaunch& p, uint32_t sms, cudaStrea
   }
   // As many CTAs per round-task as the SMs hold at once; clusters do not straddle GPCs, so a few SMs stay unused.
   if (p.n_tasks * 4 <= sms - sms / 8) return launch<Four>(p, s);
-  if (p.n_tasks * 2 <= sms - sms / 16) return launch<Two>(p, s);
-  return launch<One>(p, s);
+  return launch<Two>(p, s);   // (the caller has checked that two fit)
 }
 
 }  // namespace aet

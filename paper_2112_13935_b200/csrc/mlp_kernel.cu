@@ -412,10 +412,8 @@ uint32_t mlp_pick_cluster(const MlpShape& shape, uint32_t n_clients) {
 cudaError_t launch_mlp_rounds(const MlpLaunch& p, cudaStream_t s) {
   if (p.r.n_tasks == 0) return cudaSuccess;
   if (mlp_wide_eligible(p.shape)) return launch_mlp_wide_rounds(p, s);
-  if (mlp_stream_eligible(p.shape)) return launch_mlp_stream_rounds(p, s);
   if (p.r.stride && mlp_mma_eligible(p.shape)) return launch_mlp_mma_rounds(p, s);
   if (mlp_tc_eligible(p.shape)) return launch_mlp_tc_rounds(p, s);
-  if (mlp_res_eligible(p)) return launch_mlp_res_rounds(p, s);
   const Smem m = make_smem(p.shape);
   const size_t smem = (size_t)m.total * sizeof(float);
   // The shared-memory opt-in is a per-device attribute of the kernel and cheap to set: set it on

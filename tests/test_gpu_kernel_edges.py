@@ -1,0 +1,115 @@
+"""Every round kernel and aggregation shape at the edges of its tiles, blocks and launch rules, against the CPU checker.
+
+A client's first round starts from w_0 on both sides, so its update sum is held to the per-round bar; which kernel and
+cluster width runs it is set by how many clients the launch holds.  Later rounds start from models that differ by
+round-off and are held to the end-to-end bars."""
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import sim
+from paper_2112_13935_b200 import api, workloads
+from gpu_helpers import U_TOL, check_against_oracle, make, rel_err, run_gpu, to_device
+
+pytestmark = pytest.mark.gpu
+
+BF16_TOL, BF16_FLIP_FRAC, BF16_FLIP_TOL = 3e-4, 1e-2, 3e-2   # a bf16 rounding or a ReLU mask may fall the other way
+
+
+def check(cfg, w_tol=2e-5, bf16=False):
+    data, w0 = make(cfg)
+    ref = sim.run(cfg, data, w0)
+    gpu = run_gpu(cfg, data, w0)
+    check_against_oracle(cfg, data, w0, gpu, ref)
+    assert rel_err(gpu["w"], ref["w"]) <= (1e-3 if bf16 else w_tol)
+    for e in ref["events"]:
+        k = e["seq"]
+        want = np.asarray(ref["U"][k])
+        d = np.abs(gpu["U"][k] - want) / max(np.abs(want).max(), 1e-300)
+        if not bf16:
+            assert d.max() <= (U_TOL if e["round"] == 0 else 1e-4), (e["client"], e["round"], d.max())
+        elif e["round"] == 0:
+            assert (d > BF16_TOL).mean() <= BF16_FLIP_FRAC and d.max() <= BF16_FLIP_TOL, (e["client"], d.max())
+
+
+@pytest.mark.parametrize("l2", [0.0, 1e-3])
+@pytest.mark.parametrize("n_clients", [3, 50, 100, 200])    # clusters of four, of two; one CTA; two CTAs per SM
+@pytest.mark.parametrize("first", [1, 7, 15, 31])           # rounds of first, first + 1, first + 2 samples: around blocks of 8 and 16
+def test_regression_rounds_around_whole_blocks(n_clients, first, l2):
+    check(workloads.get_config("cfg5", n_clients=n_clients, n_rounds=3, sched_a=1, sched_b=first, l2=l2, lr=0.002 if n_clients < 10 else 1e-4,
+                               data=dict(per_client=40)))
+
+
+@pytest.mark.parametrize("dims,batch,n_clients", [
+    ([784, 128, 10], 32, 4), ([784, 128, 10], 32, 20), ([784, 128, 10], 32, 40), ([784, 128, 10], 32, 80),   # clusters of 8, 4, 2, 1
+    ([784, 128, 32], 64, 4),          # most samples and classes
+    ([50, 17, 10], 7, 3),             # one hidden tile and a bit, minibatch inside a tile, rows not a multiple of 16 bytes
+    ([100, 16, 10], 9, 3), ([100, 112, 33, 12], 17, 3), ([272, 20, 20, 20, 15], 33, 3), ([64, 100, 10], 41, 3), ([64, 30, 10], 50, 3),
+])
+def test_fp32_mlp_rounds(dims, batch, n_clients):
+    check(workloads.get_config("cfg3", n_clients=n_clients, n_rounds=2, dims=dims, batch=batch, sched_a=batch, sched_b=2 * batch, l2=1e-3,
+                               data=dict(total=70 * n_clients, dim=dims[0])))
+
+
+@pytest.mark.parametrize("dims,batch,n_clients", [
+    ([512, 256, 10], 16, 4), ([520, 100, 30, 10], 48, 4), ([200, 17, 10], 33, 20), ([1024, 64, 16], 64, 80),   # first layer on the chip
+    ([1024, 256, 128, 10], 64, 4), ([512, 256, 128, 10], 64, 20), ([512, 256, 128, 10], 64, 50), ([160, 256, 128, 16], 64, 90),
+    ([1024, 256, 128, 10], 32, 50), ([1024, 256, 10], 64, 4), ([512, 256, 10], 32, 50), ([128, 256, 11], 64, 90),   # ... streamed: clusters of 8, 4, 2, 1
+])
+def test_bf16_mlp_rounds(dims, batch, n_clients):
+    check(workloads.get_config("cfg4", n_clients=n_clients, n_rounds=2, dims=dims, batch=batch, sched_a=batch, sched_b=2 * batch, l2=1e-3,
+                               n_stragglers=0, data=dict(kind="iid", total=70 * n_clients, dim=dims[0])), bf16=True)
+
+
+@pytest.mark.parametrize("batch,n_clients", [(1, 3), (8, 3), (9, 3), (16, 20), (17, 3), (24, 3), (24, 20), (25, 3)])   # (the last two: the general kernel)
+def test_conv_rounds(batch, n_clients):
+    check(workloads.get_config("cfg7", n_clients=n_clients, n_rounds=2, batch=batch, sched_a=batch, sched_b=batch, l2=1e-3,
+                               data=dict(total=60 * n_clients)))
+
+
+@pytest.mark.parametrize("n_clients", [1, 64, 65, 3100])   # updates between two waves: one, around a sub-range, more than a cluster holds at once
+def test_aggregation_of_short_and_long_ranges(n_clients):
+    cfg = workloads.get_config("cfg5", n_clients=n_clients, n_rounds=2, sched_a=0, sched_b=1, lr=1e-4, data=dict(per_client=4))
+    data, w0 = make(cfg)
+    ref = sim.run(cfg, data, w0)
+    gpu = run_gpu(cfg, data, w0)
+    check_against_oracle(cfg, data, w0, gpu, ref)
+    acc = w0.astype(np.float64)
+    for e in ref["events"]:
+        acc -= sim.step_size(cfg, e["round"]) * gpu["U"][e["seq"]].astype(np.float64)
+    assert np.abs(acc - gpu["w"]).max() <= 2e-6 * max(1.0, np.abs(acc).max())
+
+
+def test_handles_of_several_threads_share_released_memory():
+    cfgs = [workloads.get_config("cfg5", n_clients=n, n_rounds=3, data=dict(per_client=32)) for n in (5, 70, 170)]
+    made = [make(c) for c in cfgs]
+    want = [run_gpu(c, d, w, want_U=False)["w"].tobytes() for c, (d, w) in zip(cfgs, made)]
+    got = [[] for _ in range(4)]
+
+    def work(i):
+        for j in range(6):
+            k = (i + j) % 3
+            got[i].append((k, run_gpu(cfgs[k], *made[k], want_U=False)["w"].tobytes()))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert all(len(g) == 6 and all(w == want[k] for k, w in g) for g in got)
+
+
+@pytest.mark.parametrize("shift", [0, 1])   # floats off a 16-byte boundary: the specialised kernel, the general one
+def test_one_round_without_allocation_on_any_alignment(shift):
+    cfg = workloads.get_config("cfg1", data=dict(per_client=100))
+    data, w0 = make(cfg)
+    buf = torch.zeros(3, w0.size + 4, dtype=torch.float32, device="cuda")
+    w, U, w_end = (buf.view(-1)[i * (w0.size + 4 - (w0.size % 4)) + shift:][:w0.size] for i in range(3))
+    w.copy_(torch.from_numpy(w0))
+    x, y = to_device(data)[1]
+    api.aet_round_no_alloc(cfg, 1, 2, x, y, w, U, w_end)
+    torch.cuda.synchronize()
+    U_ref, w_ref = sim.run_task(cfg, data[1], 1, 2, w0.astype(np.float64))
+    assert rel_err(U.cpu().numpy(), U_ref) <= U_TOL and rel_err(w_end.cpu().numpy(), w_ref) <= U_TOL
