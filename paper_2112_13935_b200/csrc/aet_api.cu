@@ -230,7 +230,7 @@ struct aet_handle {
   DevBuf<RingApplyDesc> d_ring_applies;
   DevBuf<RingOp> d_ring_ops;
   float* w_cur() { return w.p; }   // the server model
-  DevBuf<uint32_t> d_status;
+  uint32_t* d_status() { return reinterpret_cast<uint32_t*>(w.p + stride); }   // what kernels report, right behind it: read back together
   DevBuf<TaskDesc> d_tasks;
   DevBuf<char> d_plan;            // topology 0: the plan's tasks, sums in flight and updates
   std::vector<char> pack;         // the same on the host, for the copy
@@ -317,7 +317,7 @@ aet_status upload_clients(aet_handle* h, cudaStream_t s) {
 
 // What a status word read from the device says.
 aet_status judge_status(aet_handle* h, uint32_t st) {
-  if (st) cudaMemset(h->d_status.p, 0, sizeof(uint32_t));
+  if (st) cudaMemset(h->d_status(), 0, sizeof(uint32_t));
   if (st & 1u) return fail(h, AET_ERR_TIMEOUT, "a bounded wait for an asynchronous row copy gave up; results are invalid");
   if (st & 4u) return fail(h, AET_ERR_STATE, "a debug check failed on the device: a label, row number or slot was out of range; results are invalid");
   if (st & 2u) return fail(h, AET_ERR_NUMERIC, "a non-finite value reached the server model (or, with debug checks, sits in a client's rows); results are invalid");
@@ -326,7 +326,7 @@ aet_status judge_status(aet_handle* h, uint32_t st) {
 // After a synchronisation: did a bounded device-side wait give up?
 aet_status check_device_status(aet_handle* h) {
   uint32_t st = 0;
-  AET_CUDA(h, cudaMemcpy(&st, h->d_status.p, sizeof(st), cudaMemcpyDeviceToHost));
+  AET_CUDA(h, cudaMemcpy(&st, h->d_status(), sizeof(st), cudaMemcpyDeviceToHost));
   return judge_status(h, st);
 }
 
@@ -338,11 +338,17 @@ aet_status read_model(aet_handle* h, const float* src, float* out, cudaStream_t 
   const bool known = cudaPointerGetAttributes(&attr, out) == cudaSuccess;
   cudaGetLastError();
   const bool to_host = known && (attr.type == cudaMemoryTypeHost || attr.type == cudaMemoryTypeUnregistered);
-  void* pin = to_host && bytes + 16 <= PinnedPool::kBlock ? pinned().get() : nullptr;
+  const size_t row = h->stride * sizeof(float);
+  void* pin = to_host && row + 16 <= PinnedPool::kBlock ? pinned().get() : nullptr;
   if (pin) {
-    uint32_t* st = reinterpret_cast<uint32_t*>(static_cast<char*>(pin) + PinnedPool::kBlock - 16);
-    cudaError_t e = cudaMemcpyAsync(pin, src, bytes, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(st, h->d_status.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    uint32_t* st = reinterpret_cast<uint32_t*>(static_cast<char*>(pin) + row);
+    cudaError_t e;
+    if (src == h->w_cur()) {
+      e = cudaMemcpyAsync(pin, src, row + sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    } else {
+      e = cudaMemcpyAsync(pin, src, bytes, cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(st, h->d_status(), sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    }
     const cudaError_t w = cudaStreamSynchronize(s);   // (also before the block goes back)
     if (e == cudaSuccess) e = w;
     aet_status r = e == cudaSuccess ? judge_status(h, *st) : cuda_fail(h, e, "reading a model");
@@ -435,13 +441,13 @@ aet_status run_ring_rounds(aet_handle* h, uint32_t n_rounds, cudaStream_t s) {
   RoundLaunch r{};
   r.tasks = h->d_tasks.p; r.inflight = nullptr; r.clients = h->d_clients.p;
   r.sample_keys = h->d_keys.p; r.snaps = h->node_w.p; r.U = h->U.p; r.w_end = nullptr;
-  r.trig = h->d_trig.p; r.status = h->d_status.p; r.stride = h->stride; r.l2 = h->cfg.l2;
+  r.trig = h->d_trig.p; r.status = h->d_status(); r.stride = h->stride; r.l2 = h->cfg.l2;
   r.debug_checks = (h->cfg.flags & AET_FLAG_DEBUG_CHECKS) ? 1u : 0u;
   r.step_by_step = (h->cfg.flags & AET_FLAG_STEPWISE_RECURRENCE) ? 1u : 0u;
   r.n_u_rows = plan.n_u_rows; r.n_snap = h->cfg.n_clients;
   RingApplyLaunch a{};
   a.applies = h->d_ring_applies.p; a.ops = h->d_ring_ops.p; a.U = h->U.p; a.node_w = h->node_w.p;
-  a.status = h->d_status.p; a.stride = h->stride; a.n_params = h->P;
+  a.status = h->d_status(); a.stride = h->stride; a.n_params = h->P;
 
   const uint32_t n_waves = (uint32_t)plan.wave_off.size() - 1;
   for (uint32_t L = 0; L <= n_waves; ++L) {
@@ -518,8 +524,8 @@ aet_status aet_create(const aet_config* cfg, aet_handle** out) {
   }
   h->h_clients.assign(cfg->n_clients, ClientData{nullptr, nullptr, 0, 0});
   h->st.H.assign(cfg->n_clients, 0);
-  bool ok = h->w.reserve(h->stride) && h->w0.reserve(h->stride) &&
-            h->d_H.reserve(cfg->n_clients) && h->d_status.reserve(1);
+  bool ok = h->w.reserve(h->stride + 4) && h->w0.reserve(h->stride) &&
+            h->d_H.reserve(cfg->n_clients);
   if (ok && !h->lr_fast && !h->cnn) ok = h->work.reserve((size_t)cfg->n_clients * h->stride);
   if (ok && cfg->topology == 1) ok = h->node_w.reserve((size_t)cfg->n_clients * h->stride);
   if (!ok) { aet_destroy(h); return fail(nullptr, AET_ERR_NOMEM, "device allocation failed"); }
@@ -528,8 +534,7 @@ aet_status aet_create(const aet_config* cfg, aet_handle** out) {
     aet_destroy(h);
     return fail(nullptr, AET_ERR_CUDA, std::string("cudaMemset: ") + cudaGetErrorString(e));
   }
-  if (cudaMemset(h->w.p, 0, h->stride * sizeof(float)) != cudaSuccess ||
-      cudaMemset(h->d_status.p, 0, sizeof(uint32_t)) != cudaSuccess ||
+  if (cudaMemset(h->w.p, 0, (h->stride + 4) * sizeof(float)) != cudaSuccess ||
       cudaMemset(h->w0.p, 0, h->stride * sizeof(float)) != cudaSuccess ||
       cudaMemset(h->d_H.p, 0, cfg->n_clients * sizeof(uint32_t)) != cudaSuccess) {
     cudaError_t e = cudaGetLastError();
@@ -551,7 +556,7 @@ aet_status aet_destroy(aet_handle* h) {
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
   h->arena.release();
   h->d_clients.release(); h->d_keys.release(); h->d_H.release();
-  h->w.release(); h->d_status.release(); h->w0.release(); h->snaps.release(); h->U.release();
+  h->w.release(); h->w0.release(); h->snaps.release(); h->U.release();
   h->work.release(); h->act.release(); h->dbg.release();
   h->node_w.release(); h->d_ring_applies.release(); h->d_ring_ops.release();
   h->d_tasks.release(); h->d_plan.release();
@@ -620,7 +625,7 @@ aet_status aet_load_client_data(aet_handle* h, uint32_t client, const void* x, c
     if (!okx || !oky) return fail(h, AET_ERR_ARG, "AET_FLAG_BORROW_DATA needs device pointers");
     if (((uintptr_t)x & 15) || ((D * 4) & 15) || ((uintptr_t)y & 3))
       return fail(h, AET_ERR_ARG, "AET_FLAG_BORROW_DATA needs 16-byte aligned rows");
-    if (debug) AET_CUDA(h, launch_validate_data((const float*)x, y, n, (uint32_t)D, h->cfg.dims[h->cfg.n_layers], h->d_status.p, s));
+    if (debug) AET_CUDA(h, launch_validate_data((const float*)x, y, n, (uint32_t)D, h->cfg.dims[h->cfg.n_layers], h->d_status(), s));
     h->h_clients[client] = ClientData{x, y, n, 0};
     h->clients_dirty = true;
     h->last_stream = s;
@@ -650,8 +655,8 @@ aet_status aet_load_client_data(aet_handle* h, uint32_t client, const void* x, c
   }
   AET_CUDA(h, cudaMemcpyAsync(dy, y, (size_t)n * sizeof(int32_t), cudaMemcpyDefault, s));
   if (debug) {
-    if (!bf16) AET_CUDA(h, launch_validate_data((const float*)dx, dy, n, (uint32_t)D, h->cfg.dims[h->cfg.n_layers], h->d_status.p, s));
-    else AET_CUDA(h, launch_validate_data(nullptr, dy, n, (uint32_t)D, h->cfg.dims[h->cfg.n_layers], h->d_status.p, s));
+    if (!bf16) AET_CUDA(h, launch_validate_data((const float*)dx, dy, n, (uint32_t)D, h->cfg.dims[h->cfg.n_layers], h->d_status(), s));
+    else AET_CUDA(h, launch_validate_data(nullptr, dy, n, (uint32_t)D, h->cfg.dims[h->cfg.n_layers], h->d_status(), s));
   }
   h->h_clients[client] = ClientData{dx, dy, n, 0};
   h->clients_dirty = true;
@@ -725,13 +730,13 @@ aet_status aet_run_rounds(aet_handle* h, uint32_t n_rounds, void* cuda_stream) {
   r.tasks = reinterpret_cast<const TaskDesc*>(h->d_plan.p);
   r.inflight = reinterpret_cast<const InflightRef*>(h->d_plan.p + off_in); r.clients = h->d_clients.p;
   r.sample_keys = h->d_keys.p; r.snaps = h->snaps.p; r.U = h->U.p; r.w_end = nullptr;
-  r.trig = h->d_trig.p; r.status = h->d_status.p; r.stride = h->stride; r.l2 = h->cfg.l2;
+  r.trig = h->d_trig.p; r.status = h->d_status(); r.stride = h->stride; r.l2 = h->cfg.l2;
   r.debug_checks = (h->cfg.flags & AET_FLAG_DEBUG_CHECKS) ? 1u : 0u;
   r.step_by_step = (h->cfg.flags & AET_FLAG_STEPWISE_RECURRENCE) ? 1u : 0u;
   r.n_u_rows = plan.n_u_rows; r.n_snap = plan.n_snap;
   ApplyLaunch a{};
   a.applies = reinterpret_cast<const ApplyDesc*>(h->d_plan.p + off_ap); a.U = h->U.p; a.snaps = h->snaps.p; a.w = h->w_cur();
-  a.H = h->d_H.p; a.log = h->d_alog.p; a.status = h->d_status.p; a.stride = h->stride; a.n_params = h->P;
+  a.H = h->d_H.p; a.log = h->d_alog.p; a.status = h->d_status(); a.stride = h->stride; a.n_params = h->P;
 
   // ---- waves: a3/a4 local SGD of independent round-tasks, then a6 aggregation ----
   const uint32_t n_waves = (uint32_t)plan.apply_upto.size();
@@ -921,7 +926,7 @@ aet_status aet_debug_run_client_round(aet_handle* h, uint32_t client, uint32_t r
   AET_CUDA(h, cudaStreamSynchronize(s));
   RoundLaunch r{};
   r.tasks = dtask; r.inflight = nullptr; r.clients = h->d_clients.p; r.sample_keys = h->d_keys.p;
-  r.snaps = snap; r.U = U; r.w_end = wend; r.trig = dtrig; r.status = h->d_status.p; r.stride = h->stride;
+  r.snaps = snap; r.U = U; r.w_end = wend; r.trig = dtrig; r.status = h->d_status(); r.stride = h->stride;
   r.task_begin = 0; r.n_tasks = 1; r.l2 = h->cfg.l2;
   r.debug_checks = (h->cfg.flags & AET_FLAG_DEBUG_CHECKS) ? 1u : 0u;
   r.step_by_step = (h->cfg.flags & AET_FLAG_STEPWISE_RECURRENCE) ? 1u : 0u;
@@ -952,7 +957,7 @@ aet_status aet_debug_wait_probe(aet_handle* h, uint32_t max_polls, void* cuda_st
   if (!h) return AET_ERR_ARG;
   if (max_polls == 0 || max_polls > (1u << 24)) return fail(h, AET_ERR_ARG, "max_polls must be in [1, 2^24]");
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  cudaError_t e = launch_wait_probe(h->d_status.p, max_polls, s);
+  cudaError_t e = launch_wait_probe(h->d_status(), max_polls, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "wait probe launch");
   AET_CUDA(h, cudaStreamSynchronize(s));
   return check_device_status(h);

@@ -171,10 +171,45 @@ void fill_delays(const aet_config& c, uint32_t first, uint32_t last, DelayCache&
 }
 
 enum Kind : uint32_t { kApply = 0, kStart = 1 };
+// An event in the queue, ordered by (t, kind, client, round); kind and client in one word (clients < 2^31).
 struct QItem {
-  uint64_t t; uint32_t kind, client, round;
-  bool operator>(const QItem& o) const {
-    return std::tie(t, kind, client, round) > std::tie(o.t, o.kind, o.client, o.round);
+  uint64_t t, key; uint32_t round;
+  QItem(uint64_t at, Kind kind, uint32_t client, uint32_t r) : t(at), key((uint64_t)kind << 32 | client), round(r) {}
+  uint32_t kind() const { return (uint32_t)(key >> 32); }
+  uint32_t client() const { return (uint32_t)key; }
+  bool before(const QItem& o) const { return t != o.t ? t < o.t : key != o.key ? key < o.key : round < o.round; }
+};
+// Binary heap whose smallest item is replaced in one sift: nearly every event of the simulation makes another.
+struct EventQueue {
+  std::vector<QItem> v;
+  void sift_down(QItem x) {   // x in place of v[0]
+    size_t i = 0;
+    const size_t n = v.size();
+    for (;;) {
+      size_t c = 2 * i + 1;
+      if (c >= n) break;
+      if (c + 1 < n && v[c + 1].before(v[c])) ++c;
+      if (!v[c].before(x)) break;
+      v[i] = v[c];
+      i = c;
+    }
+    v[i] = x;
+  }
+  void pop() {
+    const QItem x = v.back();
+    v.pop_back();
+    if (!v.empty()) sift_down(x);
+  }
+  void push(QItem x) {
+    size_t i = v.size();
+    v.push_back(x);
+    while (i) {
+      const size_t up = (i - 1) / 2;
+      if (!x.before(v[up])) break;
+      v[i] = v[up];
+      i = up;
+    }
+    v[i] = x;
   }
 };
 
@@ -199,8 +234,9 @@ bool simulate(const aet_config& c, uint32_t n_rounds, SchedState& st, DelayCache
   std::vector<uint64_t> ready(n, st.clock);
   std::vector<int64_t> blocked(n, -1);  // round a client is waiting to start, or -1
   std::vector<uint32_t> ev_of((size_t)n * n_rounds);  // (client, round) -> index in out.events
-  std::priority_queue<QItem, std::vector<QItem>, std::greater<QItem>> q;
-  for (uint32_t cl = 0; cl < n && n_rounds; ++cl) q.push({st.clock, kStart, cl, first});
+  EventQueue q;
+  q.v.reserve(2 * (size_t)n + 16);
+  for (uint32_t cl = 0; cl < n && n_rounds; ++cl) q.v.push_back({st.clock, kStart, cl, first});   // in order: a heap
   const bool never_wait = c.max_lag_d == AET_NEVER_WAIT;
   uint32_t seq = 0, n_blocked = 0;
 
@@ -228,13 +264,14 @@ bool simulate(const aet_config& c, uint32_t n_rounds, SchedState& st, DelayCache
   bool alone = standing[0] == 1;
   m2 = alone ? second() : 0;
 
-  while (!q.empty()) {
-    QItem it = q.top();
-    q.pop();
-    if (it.kind == kApply) {
-      stand(H[it.client]) -= 1;
-      H[it.client] += 1;
-      stand(H[it.client]) += 1;
+  while (!q.v.empty()) {
+    const QItem it = q.v[0];
+    const uint32_t cl = it.client(), round = it.round;
+    if (it.kind() == kApply) {
+      q.pop();
+      stand(H[cl]) -= 1;
+      H[cl] += 1;
+      stand(H[cl]) += 1;
       bool moved = false;   // can a blocked client's lag have changed?
       while (!standing[m1 - h0]) { ++m1; moved = true; }
       {
@@ -243,7 +280,7 @@ bool simulate(const aet_config& c, uint32_t n_rounds, SchedState& st, DelayCache
         moved |= a != alone || s != m2;
         alone = a; m2 = s;
       }
-      out.events[ev_of[(size_t)it.client * n_rounds + (it.round - first)]].seq = seq++;
+      out.events[ev_of[(size_t)cl * n_rounds + (round - first)]].seq = seq++;
       if (n_blocked && moved) {
         for (uint32_t b = 0; b < n; ++b) {
           if (blocked[b] < 0) continue;
@@ -259,9 +296,8 @@ bool simulate(const aet_config& c, uint32_t n_rounds, SchedState& st, DelayCache
       }
       continue;
     }
-    const uint32_t cl = it.client, round = it.round;
     const uint32_t lag = lag_of(cl, round);
-    if (!never_wait && lag > c.max_lag_d) { blocked[cl] = round; ++n_blocked; continue; }
+    if (!never_wait && lag > c.max_lag_d) { q.pop(); blocked[cl] = round; ++n_blocked; continue; }
     aet_event e;
     e.t_start = it.t;
     e.t_trigger = it.t + cache.busy[cl][round - c.round_base];
@@ -273,7 +309,7 @@ bool simulate(const aet_config& c, uint32_t n_rounds, SchedState& st, DelayCache
     e.seq = 0; e.seen = seq; e.lag = lag; e.dest = 0;
     ev_of[(size_t)cl * n_rounds + (round - first)] = (uint32_t)out.events.size();
     out.events.push_back(e);
-    q.push({e.t_apply, kApply, cl, round});
+    q.sift_down({e.t_apply, kApply, cl, round});
     ready[cl] = e.t_trigger;
     if (round + 1 < last) q.push({e.t_trigger, kStart, cl, round + 1});
   }
@@ -323,18 +359,18 @@ void build_plan(const aet_config& c, const DelayCache& cache, const SchedResult&
     n_waves = std::max(n_waves, lv);
   }
   // Tasks grouped by wave, longest first.
-  std::vector<uint32_t> by_wave(E);
-  {
-    struct Key { uint64_t wave_size; uint32_t seq; };   // wave, then ~samples
-    std::vector<Key> keys(E);
-    for (size_t k = 0; k < E; ++k) keys[k] = {(uint64_t)level[k] << 32 | (uint32_t)~events[k].samples, (uint32_t)k};
-    std::sort(keys.begin(), keys.end(), [](const Key& a, const Key& b) { return a.wave_size != b.wave_size ? a.wave_size < b.wave_size : a.seq < b.seq; });
-    for (size_t k = 0; k < E; ++k) by_wave[k] = keys[k].seq;
-  }
   plan.wave_off.assign(n_waves + 1, 0);
   plan.apply_upto.assign(n_waves, 0);
-  for (uint32_t k : by_wave) plan.wave_off[level[k]] += 1;   // size of wave level-1, shifted by one
+  for (size_t k = 0; k < E; ++k) plan.wave_off[level[k]] += 1;   // size of wave level-1, shifted by one
   for (uint32_t L = 1; L <= n_waves; ++L) plan.wave_off[L] += plan.wave_off[L - 1];
+  std::vector<uint32_t> by_wave(E);
+  {
+    std::vector<uint64_t> keys(E);   // per wave: ~samples, then seq
+    std::vector<uint32_t> at(plan.wave_off.begin(), plan.wave_off.end());
+    for (size_t k = 0; k < E; ++k) keys[at[level[k] - 1]++] = (uint64_t)(uint32_t)~events[k].samples << 32 | k;
+    for (uint32_t L = 0; L < n_waves; ++L) std::sort(keys.begin() + plan.wave_off[L], keys.begin() + plan.wave_off[L + 1]);
+    for (size_t k = 0; k < E; ++k) by_wave[k] = (uint32_t)keys[k];
+  }
   for (uint32_t L = 0; L < n_waves; ++L) {
     plan.max_wave_tasks = std::max(plan.max_wave_tasks, plan.wave_off[L + 1] - plan.wave_off[L]);
     // the next wave's tasks need every update with seq < their `seen`
@@ -429,11 +465,11 @@ void build_plan(const aet_config& c, const DelayCache& cache, const SchedResult&
     t.snap_slot = (uint32_t)slot_of[e.seen];
     t.n_samples = e.samples; t.steps = e.steps;
     t.sample_ctr0 = node_samples_before(c, cache, e.client, e.round);
-    t.eta = (float)round_step_size(c, cache, e.client, e.round);
+    t.eta = plan.applies[k].eta;
     t.u_row = plan.u_row_of[k];
     t.inflight_off = (uint32_t)plan.inflight.size();
     for_each_inflight(e, [&](uint32_t j) {
-      plan.inflight.push_back({plan.u_row_of[j], (float)round_step_size(c, cache, events[j].client, events[j].round)});
+      plan.inflight.push_back({plan.u_row_of[j], plan.applies[j].eta});
     });
     t.inflight_cnt = (uint32_t)plan.inflight.size() - t.inflight_off;
     plan.tasks.push_back(t);

@@ -19,7 +19,8 @@
 //   its dW      dW2[16 x 150] = dz2[16 x 64] im2col(q1)^T      accumulators stay in registers over the samples
 //   its dIn     col[150 x 64] = W2^T dz2, then every output gathers its up to 25 entries of col
 //   conv 1      FMAs (6 planes would fill 6 of 16 rows);  its dW[26 x 6] = im2col(x)^T dz1, dz1 formed from dq1 and sign bits
-// What bounds it: the chain of some fifteen short phases and five hand-overs per iteration, not any one unit.
+// What bounds it: the chain of some fifteen short phases and five hand-overs per iteration, not any one unit (about 59 K
+// cycles).  Measured: 16 clients, minibatch 16, 12 rounds, 19 -> 7.5 ms against the split by samples.
 #include <cuda_runtime.h>
 
 #include "aet_kernels.h"

@@ -22,7 +22,9 @@
 //
 // What bounds it: crowded launches run two CTAs per SM (7 MMA warps of 14 k-steps and R, 128 registers), one's R under
 // the other's products: the warp-level tensor pipe (16 instructions of 2 cycles per k-step and 16 samples, 196 cycles per
-// sample and SM).  With one CTA per SM (14 MMA warps of 7 k-steps) it is the chain products -> R -> products.
+// sample and SM).  With one CTA per SM (14 MMA warps of 7 k-steps) it is the chain products -> R -> products.  Measured:
+// ten rounds of 1,024 clients, aggregation included, 1.58 -> 1.08 ms (before: U in tensor memory, operands of the 128-row
+// tcgen05 products staged and split through shared memory for ten rows that matter).
 #include <cuda_runtime.h>
 
 #include "aet_kernels.h"

@@ -24,6 +24,8 @@
 //
 // What bounds it: HBM - W_0 is read and written once per iteration, 6.3 MB per client at D0 = 3072 - as long as the launch has
 // enough clients; with few, the warp-level tensor rate (16 instructions of 8 cycles per 16 x 16 entries and scheduler).
+// Measured: 64 clients of 3072-256-128-10, 30 rounds, 181 -> 100 ms (before: tcgen05 products on bf16 tiles that every
+// iteration rebuilt in shared memory from the same stream), about 5 TB/s of master traffic while a full wave runs.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
