@@ -634,7 +634,23 @@ aet_status aet_load_client_data(aet_handle* h, uint32_t client, const void* x, c
   void* dx = h->arena.alloc(elems * (bf16 ? 2 : 4));
   int32_t* dy = (int32_t*)h->arena.alloc((size_t)n * sizeof(int32_t));
   if (!dx || !dy) return fail(h, AET_ERR_NOMEM, "device allocation failed");
-  if (!bf16) {
+  // Page-locked host arrays: the GPU fetches rows and labels itself.  A copy costs 5 us beside its bytes, two of them as much
+  // as 500 KB; from 2.5 MB on (measured) the copy engine's higher rate wins, except that bf16 would need an fp32 copy first.
+  constexpr size_t kFetchMost = 2 << 20;
+  const void *px = nullptr, *py = nullptr;   // the arrays as the device sees them
+  if ((bf16 || elems * 4 <= kFetchMost) && elems % 4 == 0) {
+    cudaPointerAttributes ax{}, ay{};
+    if (cudaPointerGetAttributes(&ax, x) == cudaSuccess && ax.type == cudaMemoryTypeHost && cudaPointerGetAttributes(&ay, y) == cudaSuccess &&
+        ay.type == cudaMemoryTypeHost && ax.devicePointer && ay.devicePointer && !((uintptr_t)ax.devicePointer & 15) &&
+        !((uintptr_t)ay.devicePointer & 3)) {
+      px = ax.devicePointer;
+      py = ay.devicePointer;
+    }
+    cudaGetLastError();
+  }
+  if (px) {
+    AET_CUDA(h, launch_fetch_client(static_cast<const float*>(px), dx, bf16, elems / 4, static_cast<const int32_t*>(py), dy, n, s));
+  } else if (!bf16) {
     AET_CUDA(h, cudaMemcpyAsync(dx, x, elems * 4, cudaMemcpyDefault, s));
   } else {
     cudaPointerAttributes attr{};
@@ -653,7 +669,7 @@ aet_status aet_load_client_data(aet_handle* h, uint32_t client, const void* x, c
       if (e != cudaSuccess) return cuda_fail(h, e, "bf16 conversion of client data");
     }
   }
-  AET_CUDA(h, cudaMemcpyAsync(dy, y, (size_t)n * sizeof(int32_t), cudaMemcpyDefault, s));
+  if (!py) AET_CUDA(h, cudaMemcpyAsync(dy, y, (size_t)n * sizeof(int32_t), cudaMemcpyDefault, s));
   if (debug) {
     if (!bf16) AET_CUDA(h, launch_validate_data((const float*)dx, dy, n, (uint32_t)D, h->cfg.dims[h->cfg.n_layers], h->d_status(), s));
     else AET_CUDA(h, launch_validate_data(nullptr, dy, n, (uint32_t)D, h->cfg.dims[h->cfg.n_layers], h->d_status(), s));

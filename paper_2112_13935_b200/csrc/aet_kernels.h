@@ -176,6 +176,10 @@ __device__ __forceinline__ void publish_empty_round(const RoundLaunch& p, const 
 // dst[0, n) = src (n a multiple of 4), zero[0, nz) = 0 (nz words): what a run or a reset sets up, in one launch
 cudaError_t launch_copy_and_zero(float* dst, const float* src, size_t n, uint32_t* zero, size_t nz, cudaStream_t s);
 
+// A client's rows (4 n4 values from a 16-byte boundary on; bf16: rounded on the way) and labels out of page-locked host
+// memory the device can address, in one launch.
+cudaError_t launch_fetch_client(const float* x, void* dx, bool bf16, size_t n4, const int32_t* y, int32_t* dy, uint32_t n, cudaStream_t s);
+
 // bf16 conversion of a client's rows at load time (precision 1).
 cudaError_t launch_to_bf16(const float* src, void* dst, size_t n, cudaStream_t s);
 

@@ -106,6 +106,31 @@ __global__ void copy_and_zero_kernel(float4* dst, const float4* src, size_t n4, 
   for (size_t i = i0; i < nz; i += step) zero[i] = 0;
 }
 
+// What bounds it: the host link, 50 GB/s read from here against 55 by the copy engine, but nothing is paid per array: a
+// client of 627 KB takes 19 us instead of 26, and a bf16 client needs no fp32 copy on the device.
+template <bool BF>
+__global__ void __launch_bounds__(256) fetch_client_kernel(const float4* __restrict__ x, void* __restrict__ dx, size_t n4, const int32_t* __restrict__ y,
+                                                            int32_t* __restrict__ dy, uint32_t n) {
+  const size_t step = (size_t)gridDim.x * blockDim.x, i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (size_t i = i0; i < n; i += step) dy[i] = y[i];
+  for (size_t i = i0; i < n4; i += 4 * step) {
+    float4 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i + q * step < n4) v[q] = x[i + q * step];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (i + q * step >= n4) continue;
+      if (BF) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v[q].x, v[q].y), b = __floats2bfloat162_rn(v[q].z, v[q].w);
+        static_cast<uint2*>(dx)[i + q * step] = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+      } else {
+        static_cast<float4*>(dx)[i + q * step] = v[q];
+      }
+    }
+  }
+}
+
 __global__ void to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst, size_t n) {
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const size_t step = (size_t)gridDim.x * blockDim.x;
@@ -209,6 +234,16 @@ cudaError_t launch_copy_and_zero(float* dst, const float* src, size_t n, uint32_
   size_t blocks = (n / 4 + nz + 255) / 256;
   if (blocks > 148 * 4) blocks = 148 * 4;
   copy_and_zero_kernel<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<float4*>(dst), reinterpret_cast<const float4*>(src), n / 4, zero, nz);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fetch_client(const float* x, void* dx, bool bf16, size_t n4, const int32_t* y, int32_t* dy, uint32_t n, cudaStream_t s) {
+  size_t blocks = (n4 + 4 * 256 - 1) / (4 * 256);
+  if (blocks > 148) blocks = 148;
+  if (!blocks) blocks = 1;
+  const float4* x4 = reinterpret_cast<const float4*>(x);
+  if (bf16) fetch_client_kernel<true><<<(unsigned)blocks, 256, 0, s>>>(x4, dx, n4, y, dy, n);
+  else fetch_client_kernel<false><<<(unsigned)blocks, 256, 0, s>>>(x4, dx, n4, y, dy, n);
   return cudaGetLastError();
 }
 

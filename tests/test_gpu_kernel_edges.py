@@ -113,3 +113,21 @@ def test_one_round_without_allocation_on_any_alignment(shift):
     torch.cuda.synchronize()
     U_ref, w_ref = sim.run_task(cfg, data[1], 1, 2, w0.astype(np.float64))
     assert rel_err(U.cpu().numpy(), U_ref) <= U_TOL and rel_err(w_end.cpu().numpy(), w_ref) <= U_TOL
+
+
+@pytest.mark.parametrize("name,over", [
+    ("cfg5", dict(n_clients=5, data=dict(per_client=1))), ("cfg5", dict(n_clients=3, data=dict(per_client=668))),
+    ("cfg5", dict(n_clients=3, data=dict(per_client=669))),                       # the last size fetched by a kernel, the first copied
+    ("cfg3", dict(n_clients=3, dims=[50, 17, 10], data=dict(total=301, dim=50))),   # rows that are not whole 16-byte pieces
+    ("cfg4", dict(n_clients=3, n_stragglers=0, dims=[200, 64, 10], data=dict(kind="iid", total=500, dim=200))),   # bf16
+])
+def test_client_data_from_page_locked_pageable_and_device_memory(name, over):
+    cfg = workloads.get_config(name, n_rounds=2, **over)
+    data, w0 = make(cfg)
+    cpu = [(torch.from_numpy(x), torch.from_numpy(y)) for x, y in data]
+    got = []
+    for place in (lambda t: t, lambda t: t.pin_memory(), lambda t: t.cuda()):
+        with api.Session(cfg, [(place(x), place(y)) for x, y in cpu], torch.from_numpy(w0).cuda()) as s:
+            s.run()
+            got.append(s.model().tobytes())
+    assert got[0] == got[1] == got[2]
