@@ -835,19 +835,19 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         uint32_t r[8], rs[8];
         own.issue(u, r);
         if (!BF) own.issue(ug + u, rs);
-        float d[2][4] = {}, x1[2][4] = {}, x2[2][4] = {};
+        float d[2][4] = {}, x1[2][4] = {};
 #pragma unroll
         for (int k = 0; k < kBk; ++k) {
           if (!kHold) load_zt(a[0], Z(0) + k * kStep * m.zp[0] + 16 * wm, m.zp[0], lane);
           FragB<BF> f[2];
           load_st2(f, xu + k * kStep * m.xpitch, m.xpitch, lane);
-          products(d, x1, x2, a[kHold ? k : 0], f);
+          products(d, x1, x1, a[kHold ? k : 0], f);
         }
         float w[8], us[8];
         own.wait(r, w);
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          us[i] = fmaf(lambda, w[i], term<BF>(d[i >> 2][i & 3], x1[i >> 2][i & 3], x2[i >> 2][i & 3]));   // the gradient
+          us[i] = fmaf(lambda, w[i], (BF ? d[i >> 2][i & 3] : d[i >> 2][i & 3] + x1[i >> 2][i & 3]));   // the gradient
           w[i] = fmaf(-eta, us[i], w[i]);
         }
         own.store(u, w);
