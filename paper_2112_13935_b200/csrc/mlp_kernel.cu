@@ -411,6 +411,10 @@ uint32_t mlp_pick_cluster(const MlpShape& shape, uint32_t n_clients) {
 
 cudaError_t launch_mlp_rounds(const MlpLaunch& p, cudaStream_t s) {
   if (p.r.n_tasks == 0) return cudaSuccess;
+  // Streamed where the first layer is too large for any cluster's tensor memory (64 clients of 3072-256-128-10: 100 ms, 346 on
+  // tcgen05 operand tiles); on the chip wherever a cluster of up to eight holds it (784-100-37-10: 3.0 ms, 9.0 on the general
+  // kernel) - except for calls without a handle (stride 0), whose rows need not lie on 16-byte boundaries; then operand tiles
+  // for tcgen05, then the general kernel.
   if (mlp_wide_eligible(p.shape)) return launch_mlp_wide_rounds(p, s);
   if (p.r.stride && mlp_mma_eligible(p.shape)) return launch_mlp_mma_rounds(p, s);
   if (mlp_tc_eligible(p.shape)) return launch_mlp_tc_rounds(p, s);
