@@ -14,7 +14,8 @@
 // Nothing is reused before its readers are done because each step needs the one before from all CTAs.  All weights stay in
 // shared memory, all update sums in the registers of the threads that own the parameters, for the whole round.
 //
-// Products are m16n8k8 tf32 on split fp32 operands (mma_common.cuh), convolutions as implicit GEMMs:
+// Products are m16n8k8 tf32 on split fp32 operands (mma_common.cuh; both heads rounded: rms error of a round 1.9e-7, as plain
+// FMAs), convolutions as implicit GEMMs:
 //   conv 2      Z[16 x 64] = W2[16 x 150] im2col(q1)           M = output planes exactly; the bias is tap 150 with input 1
 //   its dW      dW2[16 x 150] = dz2[16 x 64] im2col(q1)^T      accumulators stay in registers over the samples
 //   its dIn     col[150 x 64] = W2^T dz2, then every output gathers its up to 25 entries of col
@@ -37,7 +38,6 @@ using lr::mbar_init;
 using lr::smem_addr;
 using mma::Split;
 using mma::split;
-using mma::split_t;
 
 constexpr int kWarps = 16, kThreads = kWarps * 32;
 constexpr int kS = 28, kC1 = 6, kP1 = 12, kC2 = 16, kFlat = 256, kF1 = 120, kF2 = 84, kN = 10;
@@ -68,11 +68,11 @@ __device__ __forceinline__ FA a_cols_k(const float* w, int pitch, int g, int tt)
 }
 __device__ __forceinline__ FB b_rows(const float* x, int pitch, int g, int tt) {   // [column][k]
   const float2 a = *reinterpret_cast<const float2*>(x + g * pitch + 2 * tt);
-  return {split_t(a.x), split_t(a.y)};
+  return {split(a.x), split(a.y)};
 }
 __device__ __forceinline__ FB b_cols_k(const float* x, int pitch, int g, int tt) {   // [k][column], k = tt | tt + 4
   const float* p = x + tt * pitch + g;
-  return {split_t(p[0]), split_t(p[4 * pitch])};
+  return {split(p[0]), split(p[4 * pitch])};
 }
 __device__ __forceinline__ void mul(float (&d)[4], float (&x)[4], const FA& a, const FB& b) {
   mma::tf32(d, a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].hi, b.v[1].hi);
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
         const bool last = s == kPw2 / 8 - 1 && tt == 3;   // taps 150 (the bias input) and 151
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-          const FB f = {split_t(last ? 1.f : i0[kP1 * r]), split_t(last ? 0.f : i1[kP1 * r])};
+          const FB f = {split(last ? 1.f : i0[kP1 * r]), split(last ? 0.f : i1[kP1 * r])};
           mul(acc[r], crs[r], a, f);
         }
       }
@@ -635,10 +635,10 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
         for (int h = 0; h < 2; ++h) {
           const FB f = {split(bits & (1u << (2 * h)) ? v : 0.f), split(bits & (2u << (2 * h)) ? v : 0.f)};
           const float* xi = xp + (2 * py + h) * kS;
-          mul(a1[0], x1[0], {split_t(xi[oa]), split_t(xi[ob]), split_t(xi[oa + 1]), split_t(xi[ob + 1])}, f);
+          mul(a1[0], x1[0], {split(xi[oa]), split(xi[ob]), split(xi[oa + 1]), split(xi[ob + 1])}, f);
           // taps 16 .. 23, then 24, the bias (an input of 1) and none
           const float t0 = g == 0 ? xi[od] : (g == 1 ? 1.f : 0.f), t1 = g == 0 ? xi[od + 1] : (g == 1 ? 1.f : 0.f);
-          mul(a1[1], x1[1], {split_t(xi[oc]), split_t(t0), split_t(xi[oc + 1]), split_t(t1)}, f);
+          mul(a1[1], x1[1], {split(xi[oc]), split(t0), split(xi[oc + 1]), split(t1)}, f);
         }
       }
     };
@@ -679,7 +679,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
             const float* in = q1 + o2[i] + 2 * tt;
             float v0 = in[(y0 + y) * kP1], v1 = in[(y0 + y) * kP1 + 1];
             if (n >= 150) v0 = v1 = n == 150 ? 1.f : 0.f;   // the bias
-            mul(a2[i], x2[i], f, {split_t(v0), split_t(v1)});
+            mul(a2[i], x2[i], f, {split(v0), split(v1)});
           }
         }
       }
