@@ -286,7 +286,9 @@ const char* aet_last_error(const aet_handle* h);
  * 10 x batch x sum of layer widths); larger requests return AET_ERR_CONFIG
  * with the sizes in aet_last_error(NULL).  The call is asynchronous on
  * `cuda_stream`, launches at most two kernels and calls neither cudaMalloc nor
- * cudaFree.  Its first call on a device looks the array's device address up
+ * cudaFree.  Its kernels read x, y and w_in only when all earlier work of the
+ * stream is complete, also behind a kernel that lets its dependents start early
+ * (programmatic dependent launch).  Its first call on a device looks the array's device address up
  * (cudaGetSymbolAddress); make that first call outside any stream capture.
  * All calls share the one array and what the last call left in it (the entry
  * point clears what must start at zero), so two calls whose kernels could

@@ -41,7 +41,7 @@ struct RoundLaunch {
   uint32_t crowded_hint;         // non-zero: pick the kernel a full wave of this run's clients would get,
                                  // however few tasks this launch holds (single-task parity runs)
   // One round-task with its descriptors in the launch itself (n_tasks 1, no sums in flight; lr_chain_kernel only):
-  // nothing has to be in device memory beforehand.
+  // nothing has to be in device memory beforehand, and rows and labels are read behind the device-side wait too.
   uint32_t by_value;
   TaskDesc one_task;
   ClientData one_client;

@@ -267,6 +267,9 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
     }
   } else if (role == kProd) {
     // ================= producer: rows and labels =================
+    // Inside a handle rows and labels are older than the set-up launch of the run, which lets nothing start early; without
+    // one they are the caller's, whose kernel ahead in the stream may still be writing them.
+    if (p.by_value) asm volatile("griddepcontrol.wait;" ::: "memory");
     const ClientData cd = p.by_value ? p.one_client : p.clients[t.client];
     const uint64_t key = p.by_value ? p.one_key : p.sample_keys[t.client];
     const float* xrows = reinterpret_cast<const float*>(cd.x) + 8 * ks0;
