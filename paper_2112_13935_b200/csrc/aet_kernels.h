@@ -76,6 +76,11 @@ cudaError_t launch_mlp_rounds(const MlpLaunch& p, cudaStream_t s);
 size_t mlp_act_floats(const MlpShape& shape);
 uint32_t mlp_pick_cluster(const MlpShape& shape, uint32_t n_clients);
 const char* mlp_check_shape(const MlpShape& shape);  // null if the kernel can run it
+// bf16 shapes whose update sum of W_0 is (W_start - W_end) / eta instead of a sum over the iterations: large first layers with
+// whole 128-row chunks per CTA, where a second fp32 array of W_0's size would have to be streamed or kept on the chip beside it.
+// The quotient is only as good as 2^-24 |w| / eta (1e-3 of U's rms at eta 5e-4 and one iteration, a sum 5e-8): no other shape
+// is given to a kernel that derives.
+bool mlp_derives_w0(const MlpShape& shape);
 // bf16 D0-256-(128-)C models, batch 32 or 64: the first layer streams through a cluster (see mlp_wide_kernel.cu)
 bool mlp_wide_eligible(const MlpShape& shape);
 cudaError_t launch_mlp_wide_rounds(const MlpLaunch& p, cudaStream_t s);

@@ -402,6 +402,12 @@ const char* mlp_check_shape(const MlpShape& shape) {
   return nullptr;
 }
 
+bool mlp_derives_w0(const MlpShape& s) {
+  const bool streamed = s.precision == 1 && s.n_layers == 3 && s.dims[1] == 256 && s.dims[2] == 128 && s.dims[3] <= 16 && s.batch == 64 &&
+                        s.dims[0] % 256 == 0;
+  return streamed || mlp_tc_eligible(s);
+}
+
 uint32_t mlp_pick_cluster(const MlpShape& shape, uint32_t n_clients) {
   uint32_t c = 8;
   while (c > 1 && (uint64_t)n_clients * c > 148) c >>= 1;
@@ -411,7 +417,7 @@ uint32_t mlp_pick_cluster(const MlpShape& shape, uint32_t n_clients) {
 
 cudaError_t launch_mlp_rounds(const MlpLaunch& p, cudaStream_t s) {
   if (p.r.n_tasks == 0) return cudaSuccess;
-  // Streamed where the first layer is too large for any cluster's tensor memory (64 clients of 3072-256-128-10: 100 ms, 346 on
+  // Streamed where the first layer is 256 wide (64 clients of 3072-256-128-10: 100 ms, 346 on
   // tcgen05 operand tiles); on the chip wherever a cluster of up to eight holds it (784-100-37-10: 3.0 ms, 9.0 on the general
   // kernel) - except for calls without a handle (stride 0), whose rows need not lie on 16-byte boundaries; then operand tiles
   // for tcgen05, then the general kernel.

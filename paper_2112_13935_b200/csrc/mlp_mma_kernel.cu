@@ -26,8 +26,9 @@
 // tiles; at 16-64 samples per iteration the warp-level instructions' rate (1,024 bf16 / 512 tf32 multiply-adds per clock
 // and SM) is not what limits a round: hand-overs, updates and the narrow layers are.
 //
-// precision 1: the update sum of W_0 is (W_start - W_end) / eta; everything else accumulates U (the narrow layers' sums
-// beside W_0 in tensor memory).
+// Update sums are accumulated beside the weights (W_0's in the thread's own words, the narrow layers' in shared memory).
+// bf16 shapes that mlp_derives_w0 names have no room for W_0's: theirs is (W_start - W_end) / eta, and the narrow layers' lie
+// in the tensor memory that frees.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -64,7 +65,7 @@ struct MmaPlan {
   int ext;                          // words per thread beyond tensor memory
   // offsets in floats
   int o_x, o_in, o_part, o_a[kMaxL], o_z[kMaxL], o_w[kMaxL], o_u[kMaxL], o_b, o_ub, o_gb, o_gb2, nb, o_logit, o_ext, o_idx, o_bar, total;
-  int useg, us[kMaxL];              // bf16: first 4-word piece of the narrow layers' update sums, of layer l's
+  int useg, us[kMaxL];              // W_0's sum derived: first 4-word piece of the narrow layers' update sums, of layer l's
   int imt[kMaxL], iitems[kMaxL], kp[kMaxL];   // ceil(2^20 / tiles of outputs | items); parts of the inputs
   int boff[kMaxL];                  // of layer l's biases in the bias arrays
 };
@@ -89,7 +90,8 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
   p.upc = (p.units + cl - 1) / cl;
   p.upw = (p.upc + p.WK - 1) / p.WK;
   if (cl > 1 && p.upc * (cl - 1) >= p.units) return p;   // the last CTA would have nothing
-  const int words = p.upw * 8 * (bf ? 1 : 2);
+  const bool derive = bf && mlp_derives_w0(s);
+  const int words = p.upw * 8 * (derive ? 1 : 2);
   p.useg = words / 4;
   p.ext = words > kTmemWords ? words - kTmemWords : 0;
   p.rgs = (2 * p.MT + cl - 1) / cl;
@@ -112,7 +114,7 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
       p.wp[l] = up(p.d[l], 16) + 8;
       p.np[l] = n;
       p.o_w[l] = take(n * p.wp[l]);
-      if (!bf) p.o_u[l] = take(n * p.wp[l]);
+      if (!derive) p.o_u[l] = take(n * p.wp[l]);
     }
   }
   // dZ_0 and the partial products of the input parts are never needed at the same time
@@ -124,7 +126,7 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
     p.imt[l] = inv(mt); p.iitems[l] = inv(items);
     p.kp[l] = items >= kWarps ? 1 : (kWarps / items < ks ? kWarps / items : ks);
   }
-  if (bf) {   // the narrow layers' update sums beside W_0 in tensor memory, a piece per tile of 16 x 8
+  if (derive) {   // the narrow layers' update sums beside W_0 in tensor memory, a piece per tile of 16 x 8
     int at = p.useg;
     for (int l = 1; l < p.nl; ++l) {
       p.us[l] = at;
@@ -304,7 +306,8 @@ struct MmaLaunch {
   MmaPlan m;
 };
 
-template <bool BF, int BT>
+// SUM: W_0's update sum is accumulated
+template <bool BF, int BT, bool SUM>
 __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_constant__ MmaLaunch p) {
   typedef typename Elem<BF>::T T;
   constexpr int kStep = Elem<BF>::kStep;
@@ -372,7 +375,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   Own own;
   own.tmem = *tmem_at + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * kTmemWords;
   own.ext = smem + m.o_ext + tid;
-  const int ug = m.upw;   // first group of the update sum (fp32)
+  const int ug = m.upw;   // first group of W_0's update sum
 
   bool ok = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) {
@@ -469,10 +472,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     for (int q = 0; q < kChunkG; ++q)
       if (q < n) {
         own.store(g0 + q, v[q]);
-        if (!BF) own.store(ug + g0 + q, zero);
+        if (SUM) own.store(ug + g0 + q, zero);
       }
   }
-  if (BF) {
+  if (!SUM) {
     const float zero[4] = {};
 #pragma unroll 1
     for (int q = m.useg; q < m.us[0]; ++q) own.store4(q, zero);
@@ -781,7 +784,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           products(acc, x1, x2, fa, fb);
         }
         float uq[4];
-        if (BF) own.load4(m.us[l] + (e >> 4), uq);
+        if (!SUM) own.load4(m.us[l] + (e >> 4), uq);
 #pragma unroll
         for (int r2 = 0; r2 < 2; ++r2) {
           const int at = (16 * i + g + 8 * r2) * m.wp[l] + 8 * j + 2 * tt, c = 2 * r2;
@@ -791,7 +794,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           const float g1 = fmaf(lambda, wv.y, term<BF>(acc[0][c + 1], x1[0][c + 1], x2[0][c + 1]));
           wv.x = fmaf(-eta, g0, wv.x); wv.y = fmaf(-eta, g1, wv.y);
           *w = wv;
-          if (BF) {
+          if (!SUM) {
             uq[c] += g0; uq[c + 1] += g1;
           } else {
             float2* u = reinterpret_cast<float2*>(smem + m.o_u[l] + at);
@@ -800,7 +803,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
             *u = uv;
           }
         }
-        if (BF) own.store4(m.us[l] + (e >> 4), uq);
+        if (!SUM) own.store4(m.us[l] + (e >> 4), uq);
       }
     }
     // biases: every layer's gradient is in (the barriers above lie between)
@@ -834,7 +837,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         const T* xu = X + 16 * (w0 + u);
         uint32_t r[8], rs[8];
         own.issue(u, r);
-        if (!BF) own.issue(ug + u, rs);
+        if (SUM) own.issue(ug + u, rs);
         float d[2][4] = {}, x1[2][4] = {};
 #pragma unroll
         for (int k = 0; k < kBk; ++k) {
@@ -851,7 +854,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           w[i] = fmaf(-eta, us[i], w[i]);
         }
         own.store(u, w);
-        if (!BF) {
+        if (SUM) {
           float v[8];
           own.wait(rs, v);
 #pragma unroll
@@ -876,7 +879,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     for (int g0 = 0; g0 < wn; g0 += kChunkG) {
       const int n = min(kChunkG, wn - g0);
       float us[kChunkG][8];
-      if (BF) start_groups(g0, n, us);
+      if (!SUM) start_groups(g0, n, us);
 #pragma unroll
       for (int q = 0; q < kChunkG; ++q)
         if (q < n) {
@@ -884,7 +887,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           uint32_t r[8];
           own.issue(g0 + q, r);
           own.wait(r, w);
-          if (!BF) {
+          if (SUM) {
             own.issue(ug + g0 + q, r);
             own.wait(r, us[q]);
           } else {
@@ -909,10 +912,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
 #pragma unroll 1
           for (int e = tid; e < K * N; e += kThreads) {
             const int at = (e % N) * m.wp[l] + e / N;
-            if (!BF) Urow[o + e] = smem[m.o_u[l] + at] + bad;
+            if (SUM) Urow[o + e] = smem[m.o_u[l] + at] + bad;
             if (wrow) wrow[o + e] = smem[m.o_w[l] + at] + bad;
           }
-          if (BF) {
+          if (!SUM) {
             const int mt = m.np[l] / 16, tiles = mt * (up(K, 16) / 8);
 #pragma unroll 1
             for (int e = warp; e < tiles; e += kWarps) {
@@ -948,10 +951,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(*tmem_at) : "memory");
 }
 
-template <bool BF, int BT>
+template <bool BF, int BT, bool SUM>
 cudaError_t launch(const MmaLaunch& p, cudaStream_t s) {
   const size_t smem = (size_t)p.m.total * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(mlp_mma_kernel<BF, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(mlp_mma_kernel<BF, BT, SUM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(p.r.n_tasks * p.m.CL, 1, 1);
@@ -964,7 +967,7 @@ cudaError_t launch(const MmaLaunch& p, cudaStream_t s) {
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = p.m.CL > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, mlp_mma_kernel<BF, BT>, p);
+  return cudaLaunchKernelEx(&cfg, mlp_mma_kernel<BF, BT, SUM>, p);
 }
 
 // The widest cluster that leaves every round-task of the launch its own SMs; where none does, the smallest that holds
@@ -1001,21 +1004,22 @@ cudaError_t launch_mlp_mma_rounds(const MlpLaunch& p, cudaStream_t s) {
   if (!q.m.total) return cudaErrorInvalidConfiguration;
   if (p.shape.precision == 0) {
     switch (q.m.bt) {
-      case 1: return launch<false, 1>(q, s);
-      case 2: return launch<false, 2>(q, s);
-      case 3: return launch<false, 3>(q, s);
-      case 4: return launch<false, 4>(q, s);
-      case 5: return launch<false, 5>(q, s);
-      case 6: return launch<false, 6>(q, s);
-      case 7: return launch<false, 7>(q, s);
-      default: return launch<false, 8>(q, s);
+      case 1: return launch<false, 1, true>(q, s);
+      case 2: return launch<false, 2, true>(q, s);
+      case 3: return launch<false, 3, true>(q, s);
+      case 4: return launch<false, 4, true>(q, s);
+      case 5: return launch<false, 5, true>(q, s);
+      case 6: return launch<false, 6, true>(q, s);
+      case 7: return launch<false, 7, true>(q, s);
+      default: return launch<false, 8, true>(q, s);
     }
   }
+  const bool sum = !mlp_derives_w0(p.shape);
   switch (q.m.bt) {
-    case 2: return launch<true, 2>(q, s);
-    case 4: return launch<true, 4>(q, s);
-    case 6: return launch<true, 6>(q, s);
-    default: return launch<true, 8>(q, s);
+    case 2: return sum ? launch<true, 2, true>(q, s) : launch<true, 2, false>(q, s);
+    case 4: return sum ? launch<true, 4, true>(q, s) : launch<true, 4, false>(q, s);
+    case 6: return sum ? launch<true, 6, true>(q, s) : launch<true, 6, false>(q, s);
+    default: return sum ? launch<true, 8, true>(q, s) : launch<true, 8, false>(q, s);
   }
 }
 

@@ -19,8 +19,9 @@
 // same order: the same bits).  Memory is reused without cluster barriers: parts are sent only after every peer's warps have
 // said that they are done with what lies there.
 //
-// The update sums of the two wide layers are (W_start - W_end) / eta (w -= eta g and U += g in the same step); the class
-// layer's and the biases' are accumulated.
+// The update sum of W_0 is (W_start - W_end) / eta (w -= eta g and U += g in the same step; mlp_derives_w0 says for which
+// shapes), W_1's likewise at minibatch 64; at 32 tensor memory holds it, and W_0 streams from its first unit on.  The class layer's and the
+// biases' are accumulated.
 //
 // What bounds it: HBM - W_0 is read and written once per iteration, 6.3 MB per client at D0 = 3072 - as long as the launch has
 // enough clients; with few, the warp-level tensor rate (16 instructions of 8 cycles per 16 x 16 entries and scheduler).
@@ -88,8 +89,10 @@ struct Lay {   // shared memory, in bytes
   static constexpr int w2 = dead_end > in_end ? dead_end : in_end, logit = w2 + 16 * kPw2 * 4, z2 = logit + Bp * 17 * 4;
   static constexpr int bias = z2 + Bp * kPz * 2, ub = bias + kNb * 4, gb = ub + kNb * 4, gb2 = gb + kNb * 4;
   static constexpr int kStage = 2 * Bp * kPx * 2;
-  static constexpr int ring = (gb2 + kNb * 4 + 15) / 16 * 16, idx = ring + kRing * kStage, bars = idx + 4 * 64 * 4, total = bars + 128;
-  static constexpr int kRes = MID ? 6 : 14;    // units of W_0 in tensor memory (a group each); then W_1's 8 groups, W_2's update sum
+  static constexpr bool kSum1 = MID && BT == 4;   // W_1's update sum is accumulated (tensor memory), W_2's lies here
+  static constexpr int u2 = (gb2 + kNb * 4 + 15) / 16 * 16, ring = u2 + (kSum1 ? kH1 / 16 * 32 * 32 : 0), idx = ring + kRing * kStage, bars = idx + 4 * 64 * 4, total = bars + 128;
+  // units of W_0 in tensor memory (a group each); then W_1's 8 groups; then W_2's update sum, or W_1's 8 groups
+  static constexpr int kRes = kSum1 ? 0 : MID ? 6 : 14;
   static_assert(z0 % 16 == 0 && z1 % 16 == 0 && a1 % 16 == 0 && w2 % 16 == 0 && logit % 16 == 0 && z2 % 16 == 0 && bias % 16 == 0 && idx % 16 == 0 && bars % 8 == 0, "alignment");
   static_assert(total <= 227 * 1024, "fits an SM");
 };
@@ -240,9 +243,29 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
     *reinterpret_cast<uint32_t*>(d + 8) = pack_bf16(w[4], w[5]);
     *reinterpret_cast<uint32_t*>(d + 8 * kP0 + 8) = pack_bf16(w[6], w[7]);
   };
+  constexpr bool kSum1 = M::kSum1;
+  float* const us2 = reinterpret_cast<float*>(smem + M::u2) + tid * 8;   // kSum1: W_2's update sum, a thread's own words
+  auto load_u2 = [&](float (&v)[8]) {
+    if (!kSum1) { own.load(kU2, v); return; }
+#pragma unroll
+    for (int i = 0; i < 8; i += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(us2 + i);
+      v[i] = x.x; v[i + 1] = x.y; v[i + 2] = x.z; v[i + 3] = x.w;
+    }
+  };
+  auto store_u2 = [&](const float (&v)[8]) {
+    if (!kSum1) { own.store(kU2, v); own.store_wait(); return; }
+#pragma unroll
+    for (int i = 0; i < 8; i += 4) *reinterpret_cast<float4*>(us2 + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+  };
   {
     const float zero[8] = {};
-    own.store(kU2, zero);
+    if (kSum1) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) own.store(kU2 + q, zero);
+    } else {
+      own.store(kU2, zero);
+    }
     own.store_wait();
   }
   draw_rows(0);
@@ -270,13 +293,13 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
   float* const Urow = p.r.U + (size_t)t.u_row * p.r.stride;
   float* const wrow = p.r.w_end ? p.r.w_end + (size_t)t.u_row * p.r.stride : nullptr;
   const float inv_eta = 1.f / eta;
-  auto publish_words = [&](size_t at, int pitch, const float (&s)[8], const float (&w)[8]) {
+  auto publish_words = [&](size_t at, int pitch, const float (&s)[8], const float (&w)[8]) {   // update sums, weights
     // a round whose copies or hand-overs gave up leaves NaN behind as well as the status bit
     const float bad = ok ? 0.f : __int_as_float(0x7FFFFFFF);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const size_t a = at + (size_t)((i & 1) + ((i & 4) ? 8 : 0)) * pitch + ((i & 2) ? 8 : 0);
-      Urow[a] = (s[i] - w[i]) * inv_eta + bad;
+      Urow[a] = s[i] + bad;
       if (wrow) wrow[a] = w[i] + bad;
     }
   };
@@ -386,7 +409,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
             mma_bf16(acc[LOOK ? b + 1 : 0], f, x[2], x[3]);
           }
         } else {
-          publish_words(nat + (size_t)u * (16 * kH0), kH0, sv[GRAD && LOOK ? 0 : j], w);
+          float (&s)[8] = sv[GRAD && LOOK ? 0 : j];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) s[i] = (s[i] - w[i]) * inv_eta;
+          publish_words(nat + (size_t)u * (16 * kH0), kH0, s, w);
         }
       }
       ++qc;
@@ -583,7 +609,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
         mma_bf16(acc[1], f, x[2], x[3]);
       }
       float us[8];
-      own.load(kU2, us);
+      load_u2(us);
 #pragma unroll
       for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -596,8 +622,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
           *w = v;
           us[4 * h + 2 * q] += g0; us[4 * h + 2 * q + 1] += g1;
         }
-      own.store(kU2, us);
-      own.store_wait();
+      store_u2(us);
     }
     if (MID) {
       {   // dZ_0 = relu' (W_1 dZ_1): a warp has 16 hidden units of layer 0, all samples
@@ -644,8 +669,20 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
           mma_bf16(acc[1], f[k], x[2], x[3]);
         }
         own.load(kRes + q, w);
+        if (kSum1) {
+          float us[8];
+          own.load(kU2 + q, us);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) w[i] = fmaf(-eta, fmaf(lambda, w[i], acc[i >> 2][i & 3]), w[i]);
+          for (int i = 0; i < 8; ++i) {
+            const float gr = fmaf(lambda, w[i], acc[i >> 2][i & 3]);
+            w[i] = fmaf(-eta, gr, w[i]);
+            us[i] += gr;
+          }
+          own.store(kU2 + q, us);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) w[i] = fmaf(-eta, fmaf(lambda, w[i], acc[i >> 2][i & 3]), w[i]);
+        }
         own.store(kRes + q, w);
         put_w1(q, w);
       }
@@ -669,8 +706,14 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
 #pragma unroll 1
     for (int q = rank; q < 8; q += CL) {
       float s[8], w[8];
-      start_words(w1_at(q), kH1, s);
       own.load(kRes + q, w);
+      if (kSum1) {
+        own.load(kU2 + q, s);
+      } else {
+        start_words(w1_at(q), kH1, s);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] = (s[i] - w[i]) * inv_eta;
+      }
       publish_words(w1_at(q), kH1, s, w);
     }
   }
@@ -678,7 +721,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
     const float bad = ok ? 0.f : __int_as_float(0x7FFFFFFF);
     if (warp < K2 / 16) {
       float us[8];
-      own.load(kU2, us);
+      load_u2(us);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int k = 16 * warp + 2 * tt + (i & 1) + ((i & 4) ? 8 : 0), c = g + ((i & 2) ? 8 : 0);
@@ -733,7 +776,7 @@ bool splits(uint32_t d0, uint32_t cl) { return d0 % (kChunk * cl) == 0 && d0 / (
 bool mlp_wide_eligible(const MlpShape& s) {
   const bool mid = s.n_layers == 3 && s.dims[2] == (uint32_t)kH1;
   return s.precision == 1 && s.dims[1] == (uint32_t)kH0 && (mid || s.n_layers == 2) && s.dims[s.n_layers] <= (uint32_t)kMaxC &&
-         (s.batch == 32 || s.batch == 64) && splits(s.dims[0], 1);
+         (s.batch == 32 || s.batch == 64) && splits(s.dims[0], 1) && mlp_derives_w0(s);
 }
 
 cudaError_t launch_mlp_wide_rounds(const MlpLaunch& p, cudaStream_t s) {

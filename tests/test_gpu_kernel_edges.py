@@ -63,6 +63,33 @@ def test_bf16_mlp_rounds(dims, batch, n_clients):
                                n_stragglers=0, data=dict(kind="iid", total=70 * n_clients, dim=dims[0])), bf16=True)
 
 
+# One iteration from the start model: a sum holds W_0's gradient to fp32 rounding (1e-7 of its rms); a bf16 rounding of an
+# activation that falls the other way moves dZ, and with it W_0's gradient, by at most some 1e-5; (W_start - W_end) / eta would be
+# off by 2^-25 |w| / eta, 2e-4 and more of the gradient's rms at this step size.
+@pytest.mark.parametrize("dims,batch,n_clients,layers", [
+    ([784, 100, 10], 32, 8, (0, 1)), ([200, 17, 10], 33, 20, (0, 1)), ([520, 100, 30, 10], 48, 4, (0, 1, 2)), ([1024, 64, 16], 64, 80, (0, 1)),
+    ([512, 256, 10], 64, 4, (0,)), ([160, 256, 128, 16], 64, 4, (0, 1)), ([784, 128, 10], 32, 40, (0, 1)),
+    ([1024, 256, 128, 10], 32, 50, (1,)),    # W_0 streams, W_1's sum is kept
+])
+def test_bf16_update_sums_are_sums(dims, batch, n_clients, layers):
+    cfg = workloads.get_config("cfg4", n_clients=n_clients, n_rounds=1, dims=dims, batch=batch, sched_a=batch, sched_b=batch, n_stragglers=0,
+                               lr=0.0005, data=dict(kind="iid", total=70 * n_clients, dim=dims[0]))
+    data, w0 = make(cfg)
+    gpu = run_gpu(cfg, data, w0)
+    with api.Session(cfg, to_device(data), torch.from_numpy(w0).cuda()) as s:
+        s.run()
+        events, _ = s.log()
+    for k in (0, len(events) - 1):
+        want, _ = sim.run_task(cfg, data[events[k]["client"]], events[k]["client"], 0, w0.astype(np.float64))
+        at = 0
+        for l in range(len(dims) - 1):
+            n = dims[l] * dims[l + 1]
+            d, ref = gpu["U"][k][at:at + n] - want[at:at + n], want[at:at + n]
+            if l in layers:
+                assert np.sqrt((d * d).mean() / (ref * ref).mean()) <= 2e-5, (events[k]["client"], l)
+            at += n + dims[l + 1]
+
+
 @pytest.mark.parametrize("batch,n_clients", [(1, 3), (8, 3), (9, 3), (16, 20), (17, 3), (24, 3), (24, 20), (25, 3)])   # (the last two: the general kernel)
 def test_conv_rounds(batch, n_clients):
     check(workloads.get_config("cfg7", n_clients=n_clients, n_rounds=2, batch=batch, sched_a=batch, sched_b=batch, l2=1e-3,
