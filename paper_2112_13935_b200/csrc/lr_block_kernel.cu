@@ -9,7 +9,8 @@
 //   Z^T = W^T X^T, partial sums to shared memory;            R warp: z, then sweeps z <- z0 + L delta(z) over the eight
 //   the next block's Gram matrix, under R;                   samples at once until they no longer move; delta out;
 //   U^T = q^8 U^T + sum_s q^(7-s) delta_s x_s^T.             biases; row copies two blocks ahead.
-// All products are m16n8k8 tf32 with split operands (mma_common.cuh).  With the ten classes on the M side eight samples
+// Products are m16n8k8 tf32 with split operands (mma_common.cuh); with one CTA per SM the update takes operands in three bf16
+// parts instead (a round of 50 samples 1.5e-7 -> 0.6e-7 off fp64, fp32 FMAs 0.7e-7), two pairs of parts per instruction.  With the ten classes on the M side eight samples
 // fill an n-tile of the logits and a k-step of the update exactly, and the accumulator fragment of U^T is the operand
 // fragment of the next logits product when the k index of a step is read as pixel (2t | 2t + 1): U never leaves
 // registers, W = q^n W_start - eta U is formed in place, W_start waits in shared memory in fragment order.  A block's
@@ -36,6 +37,8 @@ namespace aet {
 namespace {
 
 using namespace lr;
+using mma::Parts;
+using mma::parts_t;
 using mma::Split;
 using mma::split;
 using mma::split_t;
@@ -52,6 +55,7 @@ struct Shape {
   static constexpr bool kDecay = DECAY;
   static constexpr int kThreads = (NW + 1) * 32;
   static constexpr int kCtas = NW <= 7 ? 2 : 1;
+  static constexpr bool kParts = kCtas == 1;   // the update's operands in three bf16 parts; otherwise in two tf32 parts
   static_assert(NW * KS == kSteps8, "every warp has the same number of k-steps");
   struct __align__(128) Smem {
     float rows[kRing][kBk][kPitch];
@@ -60,7 +64,7 @@ struct Shape {
     float zpart[NW][16 * kBk];      // per warp: rows 0-9 logits [class][sample], rows 10-15 x_(row - 10) . x_sample
     float pair[NW];                 // per warp: x_6 . x_7
     float4 zsum[32];                // the same summed over the warps
-    float4 dfrag[2][32];            // delta as first operand of the update: heads and remainders in fragment order
+    float4 dfrag[2][32];            // delta as first operand of the update, in fragment order: heads and remainders, or (kParts) as it is
     float dbuf[kBk][16];            // deltas between sweeps: [sample][4 q + i] = class q + 4 i
     float qp[16];                   // powers of q
     int ys[4][kBk];
@@ -226,8 +230,8 @@ __global__ void __launch_bounds__(S::kThreads, S::kCtas) lr_block_kernel(RoundLa
         if (!__any_sync(0xffffffffu, live && !(change * gain <= kTol)) && !p.step_by_step) left = 0;
         __syncwarp();
       }
-      // delta as the update's first operand: (row class, column sample); lane 4 g + tt of a fragment holds rows g, g + 8
-      // and columns tt, tt + 4
+      // delta as the update's first operand: (row class, column sample); lane 4 g + tt of a fragment holds rows g, g + 8,
+      // and columns tt and tt + 4 (as its pair)
       float sum[kOwn];
 #pragma unroll
       for (int i = 0; i < kOwn; ++i) {
@@ -235,10 +239,14 @@ __global__ void __launch_bounds__(S::kThreads, S::kCtas) lr_block_kernel(RoundLa
         sum[i] = live && c < kC ? d[i] : 0.f;
         if (c < kC) {
           const float v = decay && live ? sum[i] * sm.qp[nv - 1 - j] : sum[i];
-          const Split sp = split(v);
           const int at = 4 * (c & 7) + (j & 3), comp = (c >> 3) + 2 * (j >> 2);
-          reinterpret_cast<uint32_t*>(&sm.dfrag[0][at])[comp] = sp.hi;
-          reinterpret_cast<uint32_t*>(&sm.dfrag[1][at])[comp] = sp.lo;
+          if (S::kParts) {
+            reinterpret_cast<float*>(&sm.dfrag[0][at])[comp] = v;
+          } else {
+            const Split sp = split(v);
+            reinterpret_cast<uint32_t*>(&sm.dfrag[0][at])[comp] = sp.hi;
+            reinterpret_cast<uint32_t*>(&sm.dfrag[1][at])[comp] = sp.lo;
+          }
         }
       }
       __syncwarp();
@@ -358,18 +366,37 @@ __global__ void __launch_bounds__(S::kThreads, S::kCtas) lr_block_kernel(RoundLa
       asm volatile("bar.sync 3, %0;" ::"n"((NW + 1) * 32) : "memory");
       {
         // ---- U^T += sum_s q^(nv-1-s) delta_s x_s^T ----
-        float4 h4 = sm.dfrag[0][lane], l4 = sm.dfrag[1][lane];
-        const uint32_t h0 = __float_as_uint(h4.x), h1 = __float_as_uint(h4.y), h2 = __float_as_uint(h4.z), h3 = __float_as_uint(h4.w);
-        const uint32_t l0 = __float_as_uint(l4.x), l1 = __float_as_uint(l4.y), l2 = __float_as_uint(l4.z), l3 = __float_as_uint(l4.w);
+        if (S::kParts) {
+          const float4 dv = sm.dfrag[0][lane];
+          const Parts p0 = mma::parts(dv.x, dv.z), p1 = mma::parts(dv.y, dv.w);   // classes g, g + 8
+          const uint32_t ba[4] = {p0.b, p1.b, p0.a, p1.a};
 #pragma unroll
-        for (int j = 0; j < KS; ++j) {
-          const Split v0 = split_t(xb[8 * j]), v1 = split_t(xb[4 * kPitch + 8 * j]);
-          float d[4] = {};
-          mma::tf32(d, l0, l1, l2, l3, v0.hi, v1.hi);
-          mma::tf32(d, h0, h1, h2, h3, v0.lo, v1.lo);
-          mma::tf32(d, h0, h1, h2, h3, v0.hi, v1.hi);
+          for (int j = 0; j < KS; ++j) {
+            const Parts x = parts_t(xb[8 * j], xb[4 * kPitch + 8 * j]);
+            // k index of 16: the eight samples with one pair of parts, then with another; the leading parts by themselves (beside
+            // the small ones their sum would be cut further up)
+            float d[4] = {}, e[4] = {};
+            mma::mma_bf16_k8(e, p0.c, p1.c, x.a);
+            mma::mma_bf16_k8(d, p0.a, p1.a, x.a);
+            mma::mma_bf16(e, ba, x.b, x.c);
+            mma::mma_bf16(e, ba, x.a, x.b);
 #pragma unroll
-          for (int c = 0; c < 4; ++c) U[j][c] += d[c];
+            for (int c = 0; c < 4; ++c) U[j][c] += d[c] + e[c];
+          }
+        } else {
+          float4 h4 = sm.dfrag[0][lane], l4 = sm.dfrag[1][lane];
+          const uint32_t h0 = __float_as_uint(h4.x), h1 = __float_as_uint(h4.y), h2 = __float_as_uint(h4.z), h3 = __float_as_uint(h4.w);
+          const uint32_t l0 = __float_as_uint(l4.x), l1 = __float_as_uint(l4.y), l2 = __float_as_uint(l4.z), l3 = __float_as_uint(l4.w);
+#pragma unroll
+          for (int j = 0; j < KS; ++j) {
+            const Split v0 = split_t(xb[8 * j]), v1 = split_t(xb[4 * kPitch + 8 * j]);
+            float d[4] = {};
+            mma::tf32(d, l0, l1, l2, l3, v0.hi, v1.hi);
+            mma::tf32(d, h0, h1, h2, h3, v0.lo, v1.lo);
+            mma::tf32(d, h0, h1, h2, h3, v0.hi, v1.hi);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) U[j][c] += d[c];
+          }
         }
       }
     }

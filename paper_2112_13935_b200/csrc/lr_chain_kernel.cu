@@ -21,7 +21,9 @@
 // Few round-tasks leave SMs idle, so a round-task takes a cluster of 4 or 2 CTAs, each with its range of the
 // inputs (98 k-steps of 8); the recurrence is repeated in every CTA (same inputs, same order: the same bits).
 //
-// The products are m16n8k8 tf32 with split operands (mma_common.cuh).  U^T[class][pixel] accumulates in the fragment
+// Logits and Gram matrices are m16n8k8 tf32 products on split operands, the update m16n8k16 bf16 products on operands in three
+// parts (mma_common.cuh): what it loses stays in U, and with tf32 a round of 50 samples was 1.5e-7 off fp64 instead of 0.6e-7
+// (fp32 FMAs 0.7e-7), for 1 to 3 % of the time of few long chains.  U^T[class][pixel] accumulates in the fragment
 // (class g, pixels 2t, 2t + 1), which is the A fragment of the logits product Z^T = W^T X^T when the k index of a step
 // is read as pixel (2t | 2t + 1): W = q^n W_start - eta U is formed in place.  A block's sum starts from zero and is
 // added to U by an fp32 add, so that the tensor cores' own rounding never accumulates over a round.
@@ -48,8 +50,10 @@ namespace aet {
 namespace {
 
 using namespace lr;
+using mma::Parts;
+using mma::parts;
+using mma::parts_t;
 using mma::Split;
-using mma::split;
 using mma::split_t;
 
 constexpr int kB = 16;                       // samples per block
@@ -467,45 +471,34 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
     for (uint32_t kb = 0; kb < nblk + 2; ++kb) {
       const bool update = kb >= 2, look = kb < nblk;
       const uint32_t k = update ? kb - 2 : 0, nv = min((uint32_t)kB, n - k * kB);
-      // What does not depend on the deltas comes before the wait for them: the rows of block k as the update's second
-      // operand ([sample][pixel], pixel g of the warp's k-steps), split, and those of block kb.
+      // the rows of block k as the update's second operand ([sample][pixel], pixel g of the warp's k-steps), and those of block kb
       const float* xb = &sm.rows[k % NS][tt][8 * warp + g];
       const float* xr = &sm.rows[kb % NS][g][8 * warp + 2 * tt];
-      constexpr bool kEarly = KM <= 4;   // room for them in registers
-      Split x[kEarly ? KM : 2][4];
-      float2 r0[kEarly ? KM : 1], r1[kEarly ? KM : 1];
       if (look) wait(&sm.full[kb % NS], (kb / NS) & 1);
-      if (kEarly) {
-#pragma unroll
-        for (int j = 0; j < (kEarly ? KM : 1); ++j) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) x[j][i] = split_t(xb[4 * i * S::kPitch + 8 * NM * j]);
-          r0[j] = *reinterpret_cast<const float2*>(xr + 8 * NM * j);
-          r1[j] = *reinterpret_cast<const float2*>(xr + 8 * S::kPitch + 8 * NM * j);
-        }
-      }
       if (update) {
-        // ---- U^T = q^nv U^T + sum_s q^(nv-1-s) delta_s x_s ----
+        // ---- U^T = q^nv U^T + sum_s q^(nv-1-s) delta_s x_s; the k index of the product is read as samples t, t + 4, t + 8, t + 12 ----
         wait(&sm.delta[k & 1], (k >> 1) & 1);
-        Split a[2][4];
+        Parts a[2][2];   // [eight samples][classes g, g + 8]
         {
           const float* d0 = &sm.dbuf[k & 1][g / kCh][g % kCh];
           const float* d1 = &sm.dbuf[k & 1][1][two ? g + 3 : 0];   // classes 8, 9
           float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-          for (int m = 0; m < 2; ++m)
+          for (int m = 0; m < 2; ++m) {
+            float v0[2], v1[2];
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
               const int s = 8 * m + tt + 4 * i;
-              float v0 = d0[s * kCh], v1 = two ? d1[s * kCh] : 0.f;
-              if (biases) { s0 += v0; s1 += v1; }
+              v0[i] = d0[s * kCh]; v1[i] = two ? d1[s * kCh] : 0.f;
+              if (biases) { s0 += v0[i]; s1 += v1[i]; }
               if (decay) {
                 const float f = (uint32_t)s < nv ? sm.qp[nv - 1 - s] : 0.f;
-                v0 *= f; v1 *= f;
+                v0[i] *= f; v1[i] *= f;
               }
-              a[m][2 * i] = split(v0);
-              a[m][2 * i + 1] = split(v1);
             }
+            a[m][0] = parts(v0[0], v0[1]);
+            a[m][1] = parts(v1[0], v1[1]);
+          }
           if (biases) {
             s0 += shx(s0, 1); s1 += shx(s1, 1);
             ub0 += s0 + shx(s0, 2); ub1 += s1 + shx(s1, 2);
@@ -522,33 +515,41 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
           for (uint32_t i = 0; i < nv; ++i) qwd *= qd;
           qw = (float)qwd;
         }
-        // the six products of a k-step depend on one another: several k-steps side by side
-        constexpr int kSide = kEarly ? KM : 2;
+        const uint32_t aa[4] = {a[0][0].a, a[0][1].a, a[1][0].a, a[1][1].a}, ab[4] = {a[0][0].b, a[0][1].b, a[1][0].b, a[1][1].b};
+        const uint32_t ac[4] = {a[0][0].c, a[0][1].c, a[1][0].c, a[1][1].c};
+        // k-steps side by side, as many as there are registers for: the products of one depend on one another.  (Rows fetched and
+        // split before the wait for the deltas: 5 clients on the ring 8.84 instead of 8.19 ms.)
+        constexpr int kSide = S::kThreads <= 384 ? KM : 2;
 #pragma unroll
         for (int j0 = 0; j0 < KM; j0 += kSide) {
-          float d[kSide][4] = {};
-          if (!kEarly) {
+          float d[kSide][4] = {}, e[kSide][4] = {};
+          Parts x[kSide][2];
 #pragma unroll
-            for (int jj = 0; jj < kSide; ++jj)
+          for (int jj = 0; jj < kSide; ++jj)
 #pragma unroll
-              for (int i = 0; i < 4; ++i)
-                if (j0 + jj < KM) x[jj][i] = split_t(xb[4 * i * S::kPitch + 8 * NM * (j0 + jj)]);
-          }
+            for (int m = 0; m < 2; ++m)
+              if (j0 + jj < KM) {
+                const float* at = xb + 8 * m * S::kPitch + 8 * NM * (j0 + jj);
+                x[jj][m] = parts_t(at[0], at[4 * S::kPitch]);
+              }
 #pragma unroll
           for (int term = 0; term < 6; ++term)
 #pragma unroll
             for (int jj = 0; jj < kSide; ++jj) {
               if (j0 + jj >= KM) continue;
-              const int m = term & 1, i = 2 * m;   // which eight samples
-              if (term < 2) mma::tf32(d[jj], a[m][0].lo, a[m][1].lo, a[m][2].lo, a[m][3].lo, x[jj][i].hi, x[jj][i + 1].hi);
-              else if (term < 4) mma::tf32(d[jj], a[m][0].hi, a[m][1].hi, a[m][2].hi, a[m][3].hi, x[jj][i].lo, x[jj][i + 1].lo);
-              else mma::tf32(d[jj], a[m][0].hi, a[m][1].hi, a[m][2].hi, a[m][3].hi, x[jj][i].hi, x[jj][i + 1].hi);
+              const Parts &x0 = x[jj][0], &x1 = x[jj][1];
+              if (term == 0) mma::mma_bf16(e[jj], ac, x0.a, x1.a);
+              if (term == 1) mma::mma_bf16(d[jj], aa, x0.a, x1.a);
+              if (term == 2) mma::mma_bf16(e[jj], aa, x0.c, x1.c);
+              if (term == 3) mma::mma_bf16(e[jj], ab, x0.b, x1.b);
+              if (term == 4) mma::mma_bf16(e[jj], ab, x0.a, x1.a);
+              if (term == 5) mma::mma_bf16(e[jj], aa, x0.b, x1.b);
             }
 #pragma unroll
           for (int jj = 0; jj < kSide; ++jj)
 #pragma unroll
             for (int c = 0; c < 4; ++c)
-              if (j0 + jj < KM) U[j0 + jj][c] += d[jj][c];
+              if (j0 + jj < KM) U[j0 + jj][c] += d[jj][c] + e[jj][c];
         }
       }
       if (look) {
@@ -556,11 +557,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
         float zm[2][4] = {}, zx[2][4] = {};
 #pragma unroll
         for (int j = 0; j < KM; ++j) {
-          if (!kEarly) {
-            r0[0] = *reinterpret_cast<const float2*>(xr + 8 * NM * j);
-            r1[0] = *reinterpret_cast<const float2*>(xr + 8 * S::kPitch + 8 * NM * j);
-          }
-          const float2 x0 = r0[kEarly ? j : 0], x1 = r1[kEarly ? j : 0];
+          const float2 x0 = *reinterpret_cast<const float2*>(xr + 8 * NM * j), x1 = *reinterpret_cast<const float2*>(xr + 8 * S::kPitch + 8 * NM * j);
           const Split a = split_t(x0.x), b = split_t(x0.y), c = split_t(x1.x), d = split_t(x1.y);
           const Split w0 = split_t(fmaf(neta, U[j][0], qw * ws[j][0])), w2 = split_t(fmaf(neta, U[j][1], qw * ws[j][1]));
           const Split w1 = split_t(fmaf(neta, U[j][2], qw * ws[j][2])), w3 = split_t(fmaf(neta, U[j][3], qw * ws[j][3]));

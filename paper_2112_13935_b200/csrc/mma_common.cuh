@@ -52,6 +52,39 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
   asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
+// Two fp32 values as three bf16 each, a + b + c, exactly: 8 + 8 + 8 bits of significand, pairs in one register.
+//   parts    nearest at each step (remainders of either sign)
+//   parts_t  cut at each step: no conversions, only logic and two subtractions per value
+// aa + (ab + ba) + (ac + bb + ca) leaves 2^-25 of a product out, of random sign where at least one side is rounded.  Against
+// sums of fp32 FMAs (0.5e-7 to 1.0e-7 rms for 32 terms, 2.3e-7 to 5.0e-7 for 784; two tf32 parts: 0.9e-7 to 1.3e-7, cut 2.0e-7
+// to 2.3e-7): 0.3e-7 to 0.5e-7 for 32, and the leading products of 8 x 8 bits barely feel that the tensor cores cut instead
+// of rounding, so that 128 terms in one accumulator are still below FMAs (0.5e-7 to 1.2e-7 against 1.0e-7 to 2.0e-7).  The
+// tensor work is that of three tf32 products.
+struct Parts { uint32_t a, b, c; };
+__device__ __forceinline__ float lo_of(uint32_t pair) { return __uint_as_float(pair << 16); }
+__device__ __forceinline__ float hi_of(uint32_t pair) { return __uint_as_float(pair & 0xFFFF0000u); }
+__device__ __forceinline__ Parts parts(float x, float y) {
+  Parts p;
+  p.a = pack_bf16(x, y);
+  x -= lo_of(p.a); y -= hi_of(p.a);
+  p.b = pack_bf16(x, y);
+  p.c = pack_bf16(x - lo_of(p.b), y - hi_of(p.b));
+  return p;
+}
+__device__ __forceinline__ Parts parts_t(float x, float y) {
+  Parts p;
+  p.a = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
+  x -= hi_of(__float_as_uint(x)); y -= hi_of(__float_as_uint(y));
+  p.b = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
+  x -= hi_of(__float_as_uint(x)); y -= hi_of(__float_as_uint(y));
+  p.c = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
+  return p;
+}
+// m16n8k8: a0 (row g, k 2t | 2t + 1), a1 (g + 8, the same); b0 (k 2t | 2t + 1, col g)
+__device__ __forceinline__ void mma_bf16_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(b0));
+}
 __device__ __forceinline__ void ldmatrix4t(uint32_t (&r)[4], uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");

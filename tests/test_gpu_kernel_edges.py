@@ -42,6 +42,31 @@ def test_regression_rounds_around_whole_blocks(n_clients, first, l2):
                                data=dict(per_client=40)))
 
 
+def round_rms(cfg, w0, clients):
+    """rms error of the first round's update sums over the rms of the sums, all parameters of `clients` together."""
+    data = workloads.make_client_data(cfg)
+    got = run_gpu(cfg, data, w0)
+    with api.Session(cfg, to_device(data), torch.from_numpy(w0).cuda()) as s:
+        s.run()
+        seq = {e["client"]: e["seq"] for e in s.log()[0]}
+    err = ref = 0.0
+    for c in clients:
+        want, _ = sim.run_task(cfg, data[c], c, 0, w0.astype(np.float64))
+        err += ((got["U"][seq[c]] - want) ** 2).sum()
+        ref += (want ** 2).sum()
+    return float(np.sqrt(err / ref))
+
+
+# What sums of fp32 FMAs in this order leave: 0.67e-7 at 50 samples, 2.0e-7 at 600 (measured against fp64); operands of 22 bits
+# instead of 24 would show at 50 (1.5e-7).
+@pytest.mark.parametrize("n_clients", [3, 50, 100])   # clusters of four, of two; one CTA
+@pytest.mark.parametrize("samples,bar", [(50, 0.9e-7), (600, 2.2e-7)])
+def test_regression_rounds_are_as_good_as_fp32_sums(n_clients, samples, bar):
+    cfg = workloads.get_config("cfg5", n_clients=n_clients, n_rounds=1, sched_a=1, sched_b=samples, l2=0.0, lr=0.002, data=dict(per_client=64))
+    w0 = np.random.default_rng(0).normal(0, 0.05, workloads.n_params(cfg["dims"])).astype(np.float32)
+    assert round_rms(cfg, w0, range(3)) <= bar
+
+
 @pytest.mark.parametrize("dims,batch,n_clients", [
     ([784, 128, 10], 32, 4), ([784, 128, 10], 32, 20), ([784, 128, 10], 32, 40), ([784, 128, 10], 32, 80),   # clusters of 8, 4, 2, 1
     ([784, 128, 32], 64, 4),          # most samples and classes
