@@ -20,10 +20,13 @@
 // The hand-overs need no cluster barrier: a CTA sends its part of Z_0 for the next iteration only after it has all of A_0
 // of this one, which the owners sent after taking everybody's part.
 //
-// Products are m16n8k16 bf16, or m16n8k8 tf32 on split fp32 operands (mma_common.cuh).  The transposed orientation puts
+// Products are m16n8k16 bf16.  fp32 operands go in as three bf16 parts each, six products in place of one (mma_common.cuh):
+// rows and dZ lie in shared memory as three planes, split once where they are written (rows when an iteration begins); weights and
+// activations are split on every read (three planes of A_0 for every peer: 37.3 instead of 31 ms for 32 clients).  One round's update sums are then as close to fp64 as sums of fp32 FMAs (0.7e-7 to
+// 1e-7 rms; 2.5e-7 with two tf32 parts) and no slower: a split row is read by every hidden tile, forward and backward.  The transposed orientation puts
 // hidden units on M, samples (forward) or inputs (gradient) on N: the fragment of a thread is the same in both products.
 // tcgen05 would need W_0 as an operand in shared memory (bf16 image or hi/lo pair) rewritten every iteration and 64-row
-// tiles; at 16-64 samples per iteration the warp-level instructions' rate (1,024 bf16 / 512 tf32 multiply-adds per clock
+// tiles; at 16-64 samples per iteration the warp-level instructions' rate (1,024 bf16 multiply-adds per clock
 // and SM) is not what limits a round: hand-overs, updates and the narrow layers are.
 //
 // Update sums are accumulated beside the weights (W_0's in the thread's own words, the narrow layers' in shared memory).
@@ -31,6 +34,8 @@
 // in the tensor memory that frees.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "aet_kernels.h"
 #include "aet_rng.h"
@@ -44,12 +49,13 @@ using lr::kWaitLimit;
 using lr::mbar_expect_tx;
 using lr::mbar_init;
 using lr::smem_addr;
+using mma::ldmatrix4;
 using mma::ldmatrix4t;
 using mma::mma_bf16;
 using mma::pack_bf16;
-using mma::Split;
-using mma::split;
-using mma::split_t;
+using mma::Parts;
+using mma::parts;
+using mma::parts_t;
 
 constexpr int kWarps = 16, kThreads = kWarps * 32;
 constexpr int kTmemWords = 128;     // per thread: 512 columns over the four warps that share 32 lanes
@@ -60,7 +66,7 @@ struct MmaPlan {
   int CL, units, upc, upw;          // 16-input units: all, per CTA, per warp
   int MT, WM, WK;                   // hidden tiles of 16; warps over tiles, over input parts
   int rgs;                          // hidden rows owned per CTA, in groups of 8
-  int xpitch;                       // minibatch columns (two buffers): elements per row
+  int bufs, xpitch;                 // minibatch columns: buffers (two; fp32 one if no more fit) of planes; elements per row
   int ap[kMaxL], zp[kMaxL], wp[kMaxL], np[kMaxL];   // pitches of A_l, dZ_l, W_l (l >= 1), padded rows of W_l
   int ext;                          // words per thread beyond tensor memory
   // offsets in floats
@@ -72,8 +78,8 @@ struct MmaPlan {
 
 __host__ __device__ inline int up(int v, int m) { return (v + m - 1) / m * m; }
 
-// Whether and how a shape runs on clusters of cl CTAs; total == 0: it does not.
-MmaPlan make_plan(const MlpShape& s, int cl) {
+// Whether and how a shape runs on clusters of cl CTAs with `bufs` buffers for minibatch columns; total == 0: it does not.
+MmaPlan lay_out(const MlpShape& s, int cl, int bufs) {
   MmaPlan p{};
   const bool bf = s.precision == 1;
   p.nl = (int)s.n_layers;
@@ -97,20 +103,22 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
   p.rgs = (2 * p.MT + cl - 1) / cl;
   int o = 0;
   auto take = [&](int floats) { const int at = o; o += up(floats, 4); return at; };
-  const int elems = bf ? 2 : 1;      // elements per float
+  const int planes = bf ? 1 : 3;     // of bf16
   p.xpitch = 16 * p.upc + 8;         // 8 mod 16 elements: fragment loads hit different banks
   p.o_bar = take(16);
   p.o_idx = take(4 * 64);
-  p.o_x = take(2 * p.Bp * p.xpitch / elems);
+  p.bufs = bufs;
+  p.o_x = take(bufs * planes * p.Bp * p.xpitch / 2);
   p.o_in = take(cl * p.rgs * 8 * p.Bp);
   const int part = (p.WK - 1) * p.WM * p.bt * 128;
   for (int l = 0; l < p.nl; ++l) {
     const int n = up(p.d[l + 1], 16);
-    p.ap[l] = p.zp[l] = n + 8;
-    if (l + 1 < p.nl) p.o_a[l] = take(p.Bp * p.ap[l] / elems);
+    p.ap[l] = n + 8;
+    p.zp[l] = bf ? n + 8 : 8 * (p.bt | 1);   // dZ: bf16 [sample][n], fp32 [n][sample] (an odd number of 16-byte pieces)
+    if (l + 1 < p.nl) p.o_a[l] = take(p.Bp * p.ap[l] / (bf ? 2 : 1));
     else if (l == 0) p.o_a[0] = take(p.Bp * p.ap[0]);   // no hidden layer: the logits, fp32
     if (l > 0) {
-      p.o_z[l] = take(p.Bp * p.zp[l] / elems);
+      p.o_z[l] = take(bf ? p.Bp * p.zp[l] / 2 : planes * n * p.zp[l] / 2);
       p.wp[l] = up(p.d[l], 16) + 8;
       p.np[l] = n;
       p.o_w[l] = take(n * p.wp[l]);
@@ -118,11 +126,12 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
     }
   }
   // dZ_0 and the partial products of the input parts are never needed at the same time
-  const int z0 = up(p.Bp * p.zp[0], elems) / elems, least = kWarps * 128;
-  p.o_part = p.o_z[0] = take(part > z0 ? (part > least ? part : least) : (z0 > least ? z0 : least));
+  const int z0 = bf ? p.Bp * p.zp[0] / 2 : planes * 16 * p.MT * p.zp[0] / 2, least = kWarps * 128;
+  const int area = part > z0 ? (part > least ? part : least) : (z0 > least ? z0 : least);
+  p.o_part = p.o_z[0] = take(area);
   for (int l = 1; l < p.nl; ++l) {
     auto inv = [](int d) { return ((1 << 20) + d - 1) / d; };
-    const int mt = p.np[l] / 16, items = mt * p.bt, ks = up(p.d[l], bf ? 16 : 8) / (bf ? 16 : 8);
+    const int mt = p.np[l] / 16, items = mt * p.bt, ks = up(p.d[l], 16) / 16;
     p.imt[l] = inv(mt); p.iitems[l] = inv(items);
     p.kp[l] = items >= kWarps ? 1 : (kWarps / items < ks ? kWarps / items : ks);
   }
@@ -139,11 +148,16 @@ MmaPlan make_plan(const MlpShape& s, int cl) {
   for (int l = 0; l < p.nl; ++l) { p.boff[l] = nb; nb += up(p.d[l + 1], 16); }
   p.nb = nb;
   p.o_b = take(nb); p.o_ub = take(nb); p.o_gb = take(nb); p.o_gb2 = take(nb);
-  p.o_logit = take(p.Bp * 33);
+  // with two hidden layers a barrier lies between the last use of the logits and dZ_0: they share its area
+  p.o_logit = !bf && p.nl > 2 && least + p.Bp * 33 <= area ? p.o_part + least : take(p.Bp * 33);
   p.o_ext = take(p.ext * kThreads);
   p.total = o;
   if ((size_t)o * 4 > 227 * 1024) p.total = 0;
   return p;
+}
+MmaPlan make_plan(const MlpShape& s, int cl) {
+  const MmaPlan p = lay_out(s, cl, 2);
+  return p.total || s.precision == 1 ? p : lay_out(s, cl, 1);
 }
 
 // ---- fragments -----------------------------------------------------------------------------------------------------
@@ -151,101 +165,218 @@ __device__ __forceinline__ void ldmatrix2t(uint32_t (&r)[2], uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr) : "memory");
 }
 
-// One operand fragment set of a k-step (fp32: 8 wide, head and remainder; bf16: 16 wide).
-template <bool BF> struct FragA;
-template <> struct FragA<false> { Split v[4]; };
-template <> struct FragA<true> { uint32_t v[4]; };
-template <bool BF> struct FragB;
-template <> struct FragB<false> { Split v[2]; };
-template <> struct FragB<true> { uint32_t v[2]; };
+typedef __nv_bfloat16 T;
+__device__ __forceinline__ void ldmatrix2(uint32_t (&r)[2], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr) : "memory");
+}
 
-// d[i] += a b[i] for N column tiles; fp32: the two cross terms into x1 and x2.  Term by term, so that no
+// Operand fragments of a k-step of 16 in NP parts (bf16 operands one, fp32 three); arrays in shared memory are NP planes,
+// `plane` elements apart.
+template <int NP> struct FragA { uint32_t v[NP][4]; };
+template <int NP> struct FragB { uint32_t v[NP][2]; };
+template <int NP> __device__ __forceinline__ void set_pair(FragA<NP>& f, int i, float lo, float hi) {   // weights
+  if constexpr (NP == 1) {
+    f.v[0][i] = pack_bf16(lo, hi);
+  } else {
+    const Parts p = parts(lo, hi);
+    f.v[0][i] = p.a; f.v[1][i] = p.b; f.v[2][i] = p.c;
+  }
+}
+
+// d[i] += a b[i] for N column tiles; three parts: all but the leading product into x1 and x2.  Term by term, so that no
 // instruction waits for the one before it.
 template <int N>
-__device__ __forceinline__ void products(float (&d)[N][4], float (&x1)[N][4], float (&x2)[N][4], const FragA<false>& a, const FragB<false> (&b)[N]) {
+__device__ __forceinline__ void products(float (&d)[N][4], float (&x1)[N][4], float (&x2)[N][4], const FragA<3>& a, const FragB<3> (&b)[N]) {
 #pragma unroll
-  for (int i = 0; i < N; ++i) mma::tf32(d[i], a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b[i].v[0].hi, b[i].v[1].hi);
+  for (int i = 0; i < N; ++i) mma_bf16(x1[i], a.v[2], b[i].v[0][0], b[i].v[0][1]);
 #pragma unroll
-  for (int i = 0; i < N; ++i) mma::tf32(x1[i], a.v[0].lo, a.v[1].lo, a.v[2].lo, a.v[3].lo, b[i].v[0].hi, b[i].v[1].hi);
+  for (int i = 0; i < N; ++i) mma_bf16(x2[i], a.v[0], b[i].v[2][0], b[i].v[2][1]);
 #pragma unroll
-  for (int i = 0; i < N; ++i) mma::tf32(x2[i], a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b[i].v[0].lo, b[i].v[1].lo);
+  for (int i = 0; i < N; ++i) mma_bf16(d[i], a.v[0], b[i].v[0][0], b[i].v[0][1]);
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma_bf16(x1[i], a.v[1], b[i].v[1][0], b[i].v[1][1]);
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma_bf16(x2[i], a.v[1], b[i].v[0][0], b[i].v[0][1]);
+#pragma unroll
+  for (int i = 0; i < N; ++i) mma_bf16(x1[i], a.v[0], b[i].v[1][0], b[i].v[1][1]);
 }
 template <int N>
-__device__ __forceinline__ void products(float (&d)[N][4], float (&)[N][4], float (&)[N][4], const FragA<true>& a, const FragB<true> (&b)[N]) {
+__device__ __forceinline__ void products(float (&d)[N][4], float (&)[N][4], float (&)[N][4], const FragA<1>& a, const FragB<1> (&b)[N]) {
 #pragma unroll
-  for (int i = 0; i < N; ++i) mma_bf16(d[i], a.v, b[i].v[0], b[i].v[1]);
+  for (int i = 0; i < N; ++i) mma_bf16(d[i], a.v[0], b[i].v[0][0], b[i].v[0][1]);
 }
-// the sum over the terms of one entry
-template <bool BF> __device__ __forceinline__ float term(float d, float x1, float x2) { return BF ? d : d + (x1 + x2); }
-
-template <bool BF> struct Elem { typedef float T; static constexpr int kStep = 8; };
-template <> struct Elem<true> { typedef __nv_bfloat16 T; static constexpr int kStep = 16; };
+// ... over eight k (an odd number of sample tiles as k): the first halves of the fragments, two pairs of parts as one k index of 16
+__device__ __forceinline__ void product_k8(float (&d)[4], float (&x1)[4], float (&x2)[4], const FragA<3>& a, const FragB<3>& b) {
+  const uint32_t a20[4] = {a.v[2][0], a.v[2][1], a.v[0][0], a.v[0][1]}, a11[4] = {a.v[1][0], a.v[1][1], a.v[1][0], a.v[1][1]};
+  mma_bf16(x1, a20, b.v[0][0], b.v[2][0]);
+  mma_bf16(x2, a11, b.v[1][0], b.v[0][0]);
+  mma::mma_bf16_k8(d, a.v[0][0], a.v[0][1], b.v[0][0]);
+  mma::mma_bf16_k8(x1, a.v[0][0], a.v[0][1], b.v[1][0]);
+}
+// One tile by itself: an accumulator per product, so that none waits for another of its k-step
+template <int NP> struct Acc { float v[NP == 1 ? 1 : 6][4] = {}; };
+__device__ __forceinline__ void product(Acc<1>& d, const FragA<1>& a, const FragB<1>& b) { mma_bf16(d.v[0], a.v[0], b.v[0][0], b.v[0][1]); }
+__device__ __forceinline__ void product(Acc<3>& d, const FragA<3>& a, const FragB<3>& b) {
+  mma_bf16(d.v[0], a.v[0], b.v[0][0], b.v[0][1]);
+  mma_bf16(d.v[1], a.v[1], b.v[0][0], b.v[0][1]);
+  mma_bf16(d.v[2], a.v[0], b.v[1][0], b.v[1][1]);
+  mma_bf16(d.v[3], a.v[1], b.v[1][0], b.v[1][1]);
+  mma_bf16(d.v[4], a.v[2], b.v[0][0], b.v[0][1]);
+  mma_bf16(d.v[5], a.v[0], b.v[2][0], b.v[2][1]);
+}
+__device__ __forceinline__ void product_k8(Acc<3>& d, const FragA<3>& a, const FragB<3>& b) { product_k8(d.v[0], d.v[4], d.v[3], a, b); }
+__device__ __forceinline__ float value(const Acc<1>& d, int c) { return d.v[0][c]; }
+__device__ __forceinline__ float value(const Acc<3>& d, int c) { return d.v[0][c] + ((d.v[1][c] + d.v[2][c]) + (d.v[3][c] + (d.v[4][c] + d.v[5][c]))); }
 
 // First operand from an fp32 weight array [row][k] (rows g, g + 8; the k index of a step is read as pairs 2t | 2t + 1)
-__device__ __forceinline__ void load_w(FragA<false>& f, const float* w, int pitch, int g, int tt) {
-  const float2 a = *reinterpret_cast<const float2*>(w + g * pitch + 2 * tt), b = *reinterpret_cast<const float2*>(w + (g + 8) * pitch + 2 * tt);
-  f.v[0] = split(a.x); f.v[1] = split(b.x); f.v[2] = split(a.y); f.v[3] = split(b.y);
-}
-__device__ __forceinline__ void load_w(FragA<true>& f, const float* w, int pitch, int g, int tt) {
+template <int NP> __device__ __forceinline__ void load_w(FragA<NP>& f, const float* w, int pitch, int g, int tt) {
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const float2 a = *reinterpret_cast<const float2*>(w + g * pitch + 8 * h + 2 * tt), b = *reinterpret_cast<const float2*>(w + (g + 8) * pitch + 8 * h + 2 * tt);
-    f.v[2 * h] = pack_bf16(a.x, a.y); f.v[2 * h + 1] = pack_bf16(b.x, b.y);
+    set_pair(f, 2 * h, a.x, a.y); set_pair(f, 2 * h + 1, b.x, b.y);
   }
 }
 // First operand W^T: rows are the k index of an fp32 array [n][row], k = n in pairs
-__device__ __forceinline__ void load_wt(FragA<false>& f, const float* w, int pitch, int g, int tt) {
-  const float* p = w + 2 * tt * pitch + g;
-  f.v[0] = split(p[0]); f.v[1] = split(p[8]); f.v[2] = split(p[pitch]); f.v[3] = split(p[pitch + 8]);
-}
-__device__ __forceinline__ void load_wt(FragA<true>& f, const float* w, int pitch, int g, int tt) {
+template <int NP> __device__ __forceinline__ void load_wt(FragA<NP>& f, const float* w, int pitch, int g, int tt) {
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const float* p = w + (8 * h + 2 * tt) * pitch + g;
-    f.v[2 * h] = pack_bf16(p[0], p[pitch]); f.v[2 * h + 1] = pack_bf16(p[8], p[pitch + 8]);
+    set_pair(f, 2 * h, p[0], p[pitch]); set_pair(f, 2 * h + 1, p[8], p[pitch + 8]);
   }
 }
 // Second operand from samples [sample][k], column = sample g
-__device__ __forceinline__ void load_s(FragB<false>& f, const float* x, int pitch, int g, int tt) {
-  const float2 a = *reinterpret_cast<const float2*>(x + g * pitch + 2 * tt);
-  f.v[0] = split_t(a.x); f.v[1] = split_t(a.y);
+template <int NP> __device__ __forceinline__ void load_s(FragB<NP>& f, const T* x, int plane, int pitch, int lane) {
+  if constexpr (NP == 1) {
+    const T* p = x + (lane >> 2) * pitch + 2 * (lane & 3);
+    f.v[0][0] = *reinterpret_cast<const uint32_t*>(p);
+    f.v[0][1] = *reinterpret_cast<const uint32_t*>(p + 8);
+  } else {
+    const uint32_t at = smem_addr(x + (lane & 7) * pitch + (lane & 8));
+#pragma unroll
+    for (int q = 0; q < NP; ++q) ldmatrix2(f.v[q], at + 2u * q * plane);
+  }
 }
-__device__ __forceinline__ void load_s(FragB<true>& f, const __nv_bfloat16* x, int pitch, int g, int tt) {
-  f.v[0] = *reinterpret_cast<const uint32_t*>(x + g * pitch + 2 * tt);
-  f.v[1] = *reinterpret_cast<const uint32_t*>(x + g * pitch + 8 + 2 * tt);
-}
-// First operand dZ^T: rows are columns of an array [sample][n], k = sample
-__device__ __forceinline__ void load_zt(FragA<false>& f, const float* z, int pitch, int lane) {
-  const float* p = z + (lane & 3) * pitch + (lane >> 2);
-  f.v[0] = split(p[0]); f.v[1] = split(p[8]); f.v[2] = split(p[4 * pitch]); f.v[3] = split(p[4 * pitch + 8]);
-}
-__device__ __forceinline__ void load_zt(FragA<true>& f, const __nv_bfloat16* z, int pitch, int lane) {
-  const int i = lane >> 3, r = lane & 7;
-  ldmatrix4t(f.v, smem_addr(z + ((i >> 1) * 8 + r) * pitch + (i & 1) * 8));
+// ... N tiles of eight samples
+template <int NP, int N> __device__ __forceinline__ void load_sn(FragB<NP> (&f)[N], const T* x, int plane, int pitch, int lane) {
+  if constexpr (NP == 1) {
+#pragma unroll
+    for (int b = 0; b < N; ++b) load_s(f[b], x + 8 * b * pitch, plane, pitch, lane);
+  } else {
+#pragma unroll
+    for (int b = 0; b + 1 < N; b += 2) {
+      const uint32_t at = smem_addr(x + (8 * b + (lane >> 4) * 8 + (lane & 7)) * pitch + (lane & 8));
+#pragma unroll
+      for (int q = 0; q < NP; ++q) {
+        uint32_t r[4];
+        ldmatrix4(r, at + 2u * q * plane);
+        f[b].v[q][0] = r[0]; f[b].v[q][1] = r[1]; f[b + 1].v[q][0] = r[2]; f[b + 1].v[q][1] = r[3];
+      }
+    }
+    if (N % 2) load_s(f[N - 1], x + 8 * (N - 1) * pitch, plane, pitch, lane);
+  }
 }
 // Second operand from an array [sample][n], k = sample, column = n
-__device__ __forceinline__ void load_st(FragB<false>& f, const float* x, int pitch, int lane) {
-  const float* p = x + (lane & 3) * pitch + (lane >> 2);
-  f.v[0] = split_t(p[0]); f.v[1] = split_t(p[4 * pitch]);
+template <int NP> __device__ __forceinline__ void load_st(FragB<NP>& f, const T* x, int plane, int pitch, int lane) {
+  const uint32_t at = smem_addr(x + (lane & 15) * pitch);
+#pragma unroll
+  for (int q = 0; q < NP; ++q) ldmatrix2t(f.v[q], at + 2u * q * plane);
 }
-__device__ __forceinline__ void load_st(FragB<true>& f, const __nv_bfloat16* x, int pitch, int lane) {
-  const int r = lane & 15;
-  ldmatrix2t(f.v, smem_addr(x + r * pitch));
+// dZ_l: bf16 [sample][n], fp32 [n][sample] in planes - there the two samples of an accumulator fragment are one word of a plane.
+// As first operand dZ^T: rows n, k = sample
+__device__ __forceinline__ void load_zt(FragA<1>& f, const T* z, int k, int n, int, int pitch, int lane) {
+  const int i = lane >> 3, r = lane & 7;
+  ldmatrix4t(f.v[0], smem_addr(z + (k + (i >> 1) * 8 + r) * pitch + n + (i & 1) * 8));
+}
+__device__ __forceinline__ void load_zt(FragA<3>& f, const T* z, int k, int n, int plane, int pitch, int lane) {
+  const uint32_t at = smem_addr(z + (n + (lane & 15)) * pitch + k + (lane >> 4) * 8);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) ldmatrix4(f.v[q], at + 2u * q * plane);
+}
+__device__ __forceinline__ void load_zt_k8(FragA<3>& f, const T* z, int k, int n, int plane, int pitch, int lane) {
+  const uint32_t at = smem_addr(z + (n + (lane & 15)) * pitch + k);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    uint32_t r[2];
+    ldmatrix2(r, at + 2u * q * plane);
+    f.v[q][0] = r[0]; f.v[q][1] = r[1];
+  }
+}
+// ... as second operand: k = n, columns the N tiles of eight samples from s on
+template <int N> __device__ __forceinline__ void load_zb(FragB<1> (&f)[N], const T* z, int k, int s, int, int pitch, int lane) {
+  load_sn(f, z + s * pitch + k, 0, pitch, lane);
+}
+template <int N> __device__ __forceinline__ void load_zb(FragB<3> (&f)[N], const T* z, int k, int s, int plane, int pitch, int lane) {
+#pragma unroll
+  for (int b = 0; b + 1 < N; b += 2) {
+    const uint32_t at = smem_addr(z + (k + (lane & 15)) * pitch + s + 8 * b + (lane >> 4) * 8);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      uint32_t r[4];
+      ldmatrix4t(r, at + 2u * q * plane);
+      f[b].v[q][0] = r[0]; f[b].v[q][1] = r[1]; f[b + 1].v[q][0] = r[2]; f[b + 1].v[q][1] = r[3];
+    }
+  }
+  if (N % 2) load_st(f[N - 1], z + k * pitch + s + 8 * (N - 1), plane, pitch, lane);
+}
+// two samples s, s + 1 (s even) of column n
+__device__ __forceinline__ void put_z(FragA<1>, T* z, int s, int n, int, int pitch, float v0, float v1) {
+  z[s * pitch + n] = __float2bfloat16_rn(v0);
+  z[(s + 1) * pitch + n] = __float2bfloat16_rn(v1);
+}
+__device__ __forceinline__ void put_z(FragA<3>, T* z, int s, int n, int plane, int pitch, float v0, float v1) {
+  const Parts p = parts(v0, v1);
+  T* at = z + n * pitch + s;
+  *reinterpret_cast<uint32_t*>(at) = p.a;
+  *reinterpret_cast<uint32_t*>(at + plane) = p.b;
+  *reinterpret_cast<uint32_t*>(at + 2 * plane) = p.c;
 }
 // ... two column tiles side by side
-__device__ __forceinline__ void load_st2(FragB<false> (&f)[2], const float* x, int pitch, int lane) {
-  load_st(f[0], x, pitch, lane);
-  load_st(f[1], x + 8, pitch, lane);
+template <int NP> __device__ __forceinline__ void load_st2(FragB<NP> (&f)[2], const T* x, int plane, int pitch, int lane) {
+  const uint32_t at = smem_addr(x + (lane & 15) * pitch + (lane >> 4) * 8);
+#pragma unroll
+  for (int q = 0; q < NP; ++q) {
+    uint32_t r[4];
+    ldmatrix4t(r, at + 2u * q * plane);
+    f[0].v[q][0] = r[0]; f[0].v[q][1] = r[1]; f[1].v[q][0] = r[2]; f[1].v[q][1] = r[3];
+  }
 }
-__device__ __forceinline__ void load_st2(FragB<true> (&f)[2], const __nv_bfloat16* x, int pitch, int lane) {
-  uint32_t r[4];
-  ldmatrix4t(r, smem_addr(x + (lane & 15) * pitch + (lane >> 4) * 8));
-  f[0].v[0] = r[0]; f[0].v[1] = r[1]; f[1].v[0] = r[2]; f[1].v[1] = r[3];
+template <int NP> __device__ __forceinline__ void load_st2_k8(FragB<NP> (&f)[2], const T* x, int plane, int pitch, int lane) {
+  const uint32_t at = smem_addr(x + (lane & 7) * pitch + (lane & 8));
+#pragma unroll
+  for (int q = 0; q < NP; ++q) {
+    uint32_t r[2];
+    ldmatrix2t(r, at + 2u * q * plane);
+    f[0].v[q][0] = r[0]; f[1].v[q][0] = r[1];
+  }
 }
-__device__ __forceinline__ void put(float* p, float v) { *p = v; }
-__device__ __forceinline__ void put(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+// Weights and dZ are split by rounding, rows and activations by cutting: of the terms that the products leave out one side
+// always has a random sign.
+// Activations: bf16, or fp32 as they are; second operands from them, split (cut) on the way
+__device__ __forceinline__ void put_a(T* p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ void put_a(float* p, float v) { *p = v; }
+__device__ __forceinline__ void set_pair(FragB<3>& f, int i, float lo, float hi) {
+  const Parts p = parts_t(lo, hi);
+  f.v[0][i] = p.a; f.v[1][i] = p.b; f.v[2][i] = p.c;
+}
+__device__ __forceinline__ void load_a(FragB<1>& f, const T* x, int pitch, int lane) { load_s(f, x, 0, pitch, lane); }
+__device__ __forceinline__ void load_a(FragB<3>& f, const float* x, int pitch, int lane) {   // [sample][k], column = sample g
+  const float* p = x + (lane >> 2) * pitch + 2 * (lane & 3);
+  const float2 a = *reinterpret_cast<const float2*>(p), b = *reinterpret_cast<const float2*>(p + 8);
+  set_pair(f, 0, a.x, a.y);
+  set_pair(f, 1, b.x, b.y);
+}
+__device__ __forceinline__ void load_at(FragB<1>& f, const T* x, int pitch, int lane) { load_st(f, x, 0, pitch, lane); }
+__device__ __forceinline__ void load_at(FragB<3>& f, const float* x, int pitch, int lane) {   // [sample][n], k = sample, column = n
+  const float* p = x + 2 * (lane & 3) * pitch + (lane >> 2);
+  set_pair(f, 0, p[0], p[pitch]);
+  set_pair(f, 1, p[8 * pitch], p[9 * pitch]);
+}
+__device__ __forceinline__ void load_at_k8(FragB<3>& f, const float* x, int pitch, int lane) {
+  const float* p = x + 2 * (lane & 3) * pitch + (lane >> 2);
+  set_pair(f, 0, p[0], p[pitch]);
+}
 __device__ __forceinline__ float get(const float* p) { return *p; }
-__device__ __forceinline__ float get(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+__device__ __forceinline__ float get(const T* p) { return __bfloat162float(*p); }
 
 // ---- a thread's own words: tensor memory, then shared memory ----------------------------------------------------------
 struct Own {
@@ -309,8 +440,7 @@ struct MmaLaunch {
 // SUM: W_0's update sum is accumulated
 template <bool BF, int BT, bool SUM>
 __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_constant__ MmaLaunch p) {
-  typedef typename Elem<BF>::T T;
-  constexpr int kStep = Elem<BF>::kStep;
+  constexpr int NP = BF ? 1 : 3, kStep = 16;
   extern __shared__ __align__(128) float smem[];
   const MmaPlan& m = p.m;
   // the number of sample tiles is a constant: run-time guards around single instructions cut the code into blocks of
@@ -332,6 +462,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   const float eta = t.eta, lambda = p.r.l2;
 
   T* const xb0 = reinterpret_cast<T*>(smem + m.o_x);
+  const int xpl = Bp * m.xpitch;   // distance of the planes
   float* const inbox = smem + m.o_in;
   float* const part = smem + m.o_part;
   float* const bias = smem + m.o_b;
@@ -341,8 +472,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   int* const idx = reinterpret_cast<int*>(smem + m.o_idx);        // [2][64] row numbers, then [2][64] labels
   uint64_t* const bars = reinterpret_cast<uint64_t*>(smem + m.o_bar);   // [0] parts of Z_0, [1] A_0
   uint32_t* const tmem_at = reinterpret_cast<uint32_t*>(bars + 2);
-  auto A = [&](int l) { return reinterpret_cast<T*>(smem + m.o_a[l]); };
+  typedef typename std::conditional<BF, T, float>::type In;   // a client's values, and activations
+  auto A = [&](int l) { return reinterpret_cast<In*>(smem + m.o_a[l]); };
   auto Z = [&](int l) { return reinterpret_cast<T*>(smem + m.o_z[l]); };
+  auto zplane = [&](int l) { return up(m.d[l + 1], 16) * m.zp[l]; };   // (fp32)
 
   const int u0 = min(m.units, (int)rank * m.upc), nu = min(m.units, u0 + m.upc) - u0;   // this CTA's input units
   const int x0 = 16 * u0, nx = min(D0, x0 + 16 * nu) - x0;                              // ... and columns
@@ -366,7 +499,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   if (CL > 1) mma::cluster_sync(); else __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t in_bytes = (uint32_t)(CL * nrg * 8 * Bp * 4), a_bytes = (uint32_t)(16 * m.MT * Bp * (nl > 1 ? sizeof(T) : sizeof(float)));
+  const uint32_t in_bytes = (uint32_t)(CL * nrg * 8 * Bp * 4), a_bytes = (uint32_t)(16 * m.MT * Bp * (nl > 1 ? sizeof(In) : sizeof(float)));
   if (tid == 0) {
     if (nrg > 0) mbar_expect_tx(&bars[0], in_bytes);
     mbar_expect_tx(&bars[1], a_bytes);
@@ -397,15 +530,19 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(idx + 128 + (it & 1) * 64 + tid)), "l"(cd.y + id) : "memory");
     }
   };
-  constexpr int kChunk = 16 / (int)sizeof(T);
-  const bool whole = (D0 * sizeof(T)) % 16 == 0;
+  constexpr int kChunk = 16 / (int)sizeof(In);
+  const bool whole = (D0 * sizeof(In)) % 16 == 0;
+  auto rows_of = [&](uint32_t it) { return xb0 + (m.bufs > 1 ? (it & 1) : 0) * NP * xpl; };
+  // bf16: into their buffer (asynchronous copies); fp32: into L2, to be fetched and split when there is time
   auto copy_rows = [&](uint32_t it) {
-    T* x = xb0 + (it & 1) * Bp * m.xpitch;
-    const T* src = reinterpret_cast<const T*>(cd.x) + x0;
+    T* x = rows_of(it);
+    const In* src = reinterpret_cast<const In*>(cd.x) + x0;
 #pragma unroll 1
     for (int r = warp; r < B; r += kWarps) {
-      const T* row = src + (size_t)idx[(it & 1) * 64 + r] * D0;
-      if (whole) {
+      const In* row = src + (size_t)idx[(it & 1) * 64 + r] * D0;
+      if (!BF) {
+        for (int c = 32 * lane; c < nx; c += 1024) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + c));
+      } else if (whole) {
 #pragma unroll 1
         for (int c = lane * kChunk; c < nx; c += 32 * kChunk)
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(x + r * m.xpitch + c)), "l"(row + c) : "memory");
@@ -415,6 +552,45 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // fp32: the columns of iteration it, split into their planes
+  const int quads = 4 * nu;
+  const uint32_t iquads = quads ? 0xFFFFFFFFu / (uint32_t)quads + 1 : 0;   // e / quads = high word of e iquads (e quads < 2^32)
+  auto split_rows = [&](uint32_t it) {
+    T* const X = rows_of(it);
+    const float* src = reinterpret_cast<const float*>(cd.x) + x0;
+    constexpr int kTrip = 4;
+#pragma unroll 1
+    for (int e0 = tid; e0 < B * quads; e0 += kTrip * kThreads) {   // kTrip loads on their way before the first is split
+      float4 v[kTrip];
+      int at[kTrip];
+#pragma unroll
+      for (int q = 0; q < kTrip; ++q) {
+        const int e = e0 + q * kThreads, r = (int)__umulhi((uint32_t)e, iquads), c = 4 * (e - r * quads);
+        v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        at[q] = e < B * quads ? r * m.xpitch + c : -1;
+        if (at[q] >= 0) {
+          const float* from = src + (size_t)idx[(it & 1) * 64 + r] * D0 + c;
+          if (whole) {
+            if (c < nx) v[q] = __ldg(reinterpret_cast<const float4*>(from));
+          } else {
+            if (c < nx) v[q].x = __ldg(from);
+            if (c + 1 < nx) v[q].y = __ldg(from + 1);
+            if (c + 2 < nx) v[q].z = __ldg(from + 2);
+            if (c + 3 < nx) v[q].w = __ldg(from + 3);
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kTrip; ++q)
+        if (at[q] >= 0) {
+          const Parts a = parts_t(v[q].x, v[q].y), b = parts_t(v[q].z, v[q].w);
+          T* x = X + at[q];
+          *reinterpret_cast<uint2*>(x) = make_uint2(a.a, b.a);
+          *reinterpret_cast<uint2*>(x + xpl) = make_uint2(a.b, b.b);
+          *reinterpret_cast<uint2*>(x + 2 * xpl) = make_uint2(a.c, b.c);
+        }
+    }
   };
 
   // ---- start model: snapshot minus own update sums still in flight ----
@@ -506,7 +682,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     }
   }
   __syncthreads();
-  copy_rows(0);
+  if (BF) copy_rows(0);
+  else if (m.bufs > 1) split_rows(0);
 
   // Where this lane's row of Z_0 (g, or g + 8 for odd lanes) goes: its owner's inbox and barrier (warps of the first part).
   uint32_t row_at, row_bar;
@@ -526,20 +703,26 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       for (int c = 0; c < 4; ++c) { acc[b][c] = 0.f; crs[b][c] = 0.f; }
   };
   auto forward = [&](const T* xu, const float (&w)[8]) {   // one unit of inputs
+    FragA<NP> a;
 #pragma unroll
-    for (int h = 0; h < 16 / kStep; ++h) {
-      FragA<BF> a;
-      FragB<BF> f[BT];
-      if constexpr (BF) {
-        a.v[0] = pack_bf16(w[0], w[1]); a.v[1] = pack_bf16(w[2], w[3]);
-        a.v[2] = pack_bf16(w[4], w[5]); a.v[3] = pack_bf16(w[6], w[7]);
-      } else {
-        a.v[0] = split(w[4 * h]); a.v[1] = split(w[4 * h + 2]);
-        a.v[2] = split(w[4 * h + 1]); a.v[3] = split(w[4 * h + 3]);
-      }
-#pragma unroll
-      for (int b = 0; b < BT; ++b) load_s(f[b], xu + 8 * b * m.xpitch + 8 * h, m.xpitch, g, tt);
+    for (int i = 0; i < 4; ++i) set_pair(a, i, w[2 * i], w[2 * i + 1]);
+    if constexpr (BF) {
+      FragB<NP> f[BT];
+      load_sn(f, xu, xpl, m.xpitch, lane);
       products(acc, crs, crs, a, f);
+    } else {   // sample tiles two at a time: room for their three parts
+#pragma unroll
+      for (int b = 0; b < BT; b += 2) {
+        if (b + 1 < BT) {
+          FragB<NP> f[2];
+          load_sn(f, xu + 8 * b * m.xpitch, xpl, m.xpitch, lane);
+          products(reinterpret_cast<float (&)[2][4]>(acc[b]), reinterpret_cast<float (&)[2][4]>(crs[b]), reinterpret_cast<float (&)[2][4]>(crs[b]), a, f);
+        } else {
+          FragB<NP> f[1];
+          load_sn(f, xu + 8 * b * m.xpitch, xpl, m.xpitch, lane);
+          products(reinterpret_cast<float (&)[1][4]>(acc[b]), reinterpret_cast<float (&)[1][4]>(crs[b]), reinterpret_cast<float (&)[1][4]>(crs[b]), a, f);
+        }
+      }
     }
   };
   auto forward_all = [&](const T* X) {
@@ -553,19 +736,25 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       forward(X + 16 * (w0 + u), w);
     }
   };
-  auto rows_of = [&](uint32_t it) { return xb0 + (it & 1) * Bp * m.xpitch; };
 
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();   // the first rows are in
   if (BF) forward_all(rows_of(0));
 
 #pragma unroll 1
   for (uint32_t it = 0; it < t.steps; ++it) {
     // ================= 1: this CTA's part of Z_0^T =================
-    if (!BF) forward_all(rows_of(it));
+    if (it + 1 < t.steps) draw_rows(it + 1);
+    __syncthreads();   // everybody is out of the last pass: the buffer of its rows and the area of dZ_0 are free
+    if (!BF) {
+      if (it + 1 < t.steps) copy_rows(it + 1);
+      if (m.bufs == 1) {   // no second buffer: the rows come in now
+        split_rows(it);
+        __syncthreads();
+      }
+      forward_all(rows_of(it));
+    }
     {
-      if (it + 1 < t.steps) draw_rows(it + 1);
-      __syncthreads();   // everybody is out of the last pass: the buffer of its rows and the area of dZ_0 are free
       if (!BF) {
 #pragma unroll
         for (int b = 0; b < BT; ++b)
@@ -601,7 +790,10 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       }
     }
 
-    if (it + 1 < t.steps) copy_rows(it + 1);
+    if (it + 1 < t.steps) {   // the next rows, under the hand-over
+      if (BF) copy_rows(it + 1);
+      else if (m.bufs > 1) split_rows(it + 1);
+    }
 
     // ================= 2: owned rows: sum over the CTAs, bias, ReLU; A_0 (or the logits) to every CTA =================
     if (nrg > 0) {
@@ -626,7 +818,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         // (without hidden layers these are the logits: fp32 whatever the operands)
         const uint32_t bar = smem_addr(&bars[1]);
         if (BF && nl > 1) {
-          const uint32_t at = smem_addr(reinterpret_cast<__nv_bfloat16*>(A(0)) + b * m.ap[0] + n), lo = pack_bf16(v[0], v[1]), hi = pack_bf16(v[2], v[3]);
+          const uint32_t at = smem_addr(A(0) + b * m.ap[0] + n), lo = pack_bf16(v[0], v[1]), hi = pack_bf16(v[2], v[3]);
 #pragma unroll 1
           for (int r = 0; r < CL; ++r) send2(mma::peer_addr(at, r), lo, hi, mma::peer_addr(bar, r));
         } else {
@@ -650,28 +842,28 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
 #pragma unroll 1
       for (int e = warp; e < items * kp; e += kWarps) {
         const int part_k = kp > 1 ? div20(e, m.iitems[l]) : 0, item = e - part_k * items, b = div20(item, m.imt[l]), i = item - b * mt;
-        float acc[1][4] = {}, x1[1][4] = {}, x2[1][4] = {};
+        Acc<NP> acc;
         const float* w = smem + m.o_w[l] + 16 * i * m.wp[l];
-        const T* a = A(l - 1) + 8 * b * m.ap[l - 1];
+        const In* a = A(l - 1) + 8 * b * m.ap[l - 1];
         const int per = (ks + kp - 1) / kp, k1 = min(ks, per * (part_k + 1));
 #pragma unroll 4
         for (int k = per * part_k; k < k1; ++k) {
-          FragA<BF> fa;
-          FragB<BF> fb[1];
+          FragA<NP> fa;
+          FragB<NP> fb;
           load_w(fa, w + k * kStep, m.wp[l], g, tt);
-          load_s(fb[0], a + k * kStep, m.ap[l - 1], g, tt);
-          products(acc, x1, x2, fa, fb);
+          load_a(fb, a + k * kStep, m.ap[l - 1], lane);
+          product(acc, fa, fb);
         }
         if (kp > 1) {
 #pragma unroll
-          for (int c = 0; c < 4; ++c) part[e * 128 + c * 32 + lane] = term<BF>(acc[0][c], x1[0][c], x2[0][c]);
+          for (int c = 0; c < 4; ++c) part[e * 128 + c * 32 + lane] = value(acc, c);
           continue;
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
-          const float v = term<BF>(acc[0][c], x1[0][c], x2[0][c]) + bias[m.boff[l] + n];
-          if (!last) put(A(l) + s * m.ap[l] + n, fmaxf(v, 0.f));
+          const float v = value(acc, c) + bias[m.boff[l] + n];
+          if (!last) put_a(A(l) + s * m.ap[l] + n, fmaxf(v, 0.f));
           else if (n < m.d[nl]) logit[s * 33 + n] = v;
         }
       }
@@ -684,7 +876,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           float v = bias[m.boff[l] + n];
 #pragma unroll 1
           for (int k = 0; k < kp; ++k) v += part[k * items * 128 + e];
-          if (!last) put(A(l) + s * m.ap[l] + n, fmaxf(v, 0.f));
+          if (!last) put_a(A(l) + s * m.ap[l] + n, fmaxf(v, 0.f));
           else if (n < m.d[nl]) logit[s * 33 + n] = v;
         }
         __syncthreads();
@@ -694,7 +886,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       const int C = m.d[nl], s = tid >> 2, q = tid & 3;
       if (s < Bp) {
         const float* z = nl > 1 ? logit + s * 33 : smem + m.o_a[0] + s * m.ap[0];
-        T* dz = Z(nl - 1) + s * m.zp[nl - 1];
+        T* dz = BF ? Z(nl - 1) + s * m.zp[nl - 1] : Z(nl - 1) + s;
+        const int zpl = zplane(nl - 1);
         float v[8], mx = -3e38f, sum = 0.f;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -715,7 +908,15 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           const int c = q + 4 * i;
           if (4 * i >= up(C, 16)) continue;
           const float d = c < C ? (v[i] * inv - (c == y ? 1.f : 0.f)) * fb : 0.f;
-          put(dz + c, d);
+          if constexpr (BF) {
+            dz[c] = __float2bfloat16_rn(d);
+          } else {
+            const Parts p = parts(d, 0.f);
+            T* at = dz + c * m.zp[nl - 1];
+            at[0] = __ushort_as_bfloat16((unsigned short)p.a);
+            at[zpl] = __ushort_as_bfloat16((unsigned short)p.b);
+            at[2 * zpl] = __ushort_as_bfloat16((unsigned short)p.c);
+          }
           if (c < C) logit[s * 33 + c] = d;   // unrounded, for the bias gradient (the four lanes have read the sample's logits)
         }
       }
@@ -741,24 +942,27 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       for (int e = warp; e < mi * halves; e += kWarps) {
         const int half = halves > 1 && e >= mi ? 1 : 0, i = e - half * mi, b0 = half * kHalf;
         float s0 = 0.f, s1 = 0.f;
-        float acc[kHalf][4] = {}, crs[kHalf][4] = {};
+        constexpr int kX = BF || kHalf > 4 ? 1 : 2;   // accumulators of the small terms
+        float acc[kHalf][4] = {}, crs[kX][kHalf][4] = {};
 #pragma unroll 1
         for (int k = 0; k < K; k += kStep) {
-          FragA<BF> fa;
-          FragB<BF> fb[kHalf];
+          FragA<NP> fa;
+          FragB<NP> fb[kHalf];
           load_wt(fa, smem + m.o_w[l] + k * m.wp[l] + 16 * i, m.wp[l], g, tt);
-#pragma unroll
-          for (int b = 0; b < kHalf; ++b) load_s(fb[b], Z(l) + 8 * (b0 + b) * m.zp[l] + k, m.zp[l], g, tt);
-          products(acc, crs, crs, fa, fb);
+          load_zb(fb, Z(l), k, 8 * b0, zplane(l), m.zp[l], lane);
+          products(acc, crs[0], crs[kX - 1], fa, fb);
         }
 #pragma unroll
         for (int b = 0; b < kHalf; ++b)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * (b0 + b) + 2 * tt + (c & 1);
-            const float v = get(A(l - 1) + s * m.ap[l - 1] + n) > 0.f ? acc[b][c] + (BF ? 0.f : crs[b][c]) : 0.f;
-            put(Z(l - 1) + s * m.zp[l - 1] + n, v);
-            if (c & 2) s1 += v; else s0 += v;
+          for (int c = 0; c < 4; c += 2) {
+            const int n = 16 * i + g + (c ? 8 : 0), s = 8 * (b0 + b) + 2 * tt;
+            float v[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+              v[q] = get(A(l - 1) + (s + q) * m.ap[l - 1] + n) > 0.f ? acc[b][c + q] + (BF ? 0.f : kX > 1 ? crs[0][b][c + q] + crs[kX - 1][b][c + q] : crs[0][b][c + q]) : 0.f;
+            put_z(FragA<NP>(), Z(l - 1), s, n, zplane(l - 1), m.zp[l - 1], v[0], v[1]);
+            if (c) s1 += v[0] + v[1]; else s0 += v[0] + v[1];
           }
         s0 += __shfl_xor_sync(0xffffffffu, s0, 1); s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
         s0 += __shfl_xor_sync(0xffffffffu, s0, 2); s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
@@ -774,14 +978,20 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
 #pragma unroll 1
       for (int e = warp; e < mt * ni; e += kWarps) {
         const int j = div20(e, m.imt[l]), i = e - j * mt;
-        float acc[1][4] = {}, x1[1][4] = {}, x2[1][4] = {};
+        Acc<NP> acc;
+        FragA<NP> fa;
+        FragB<NP> fb;
 #pragma unroll 2
-        for (int k = 0; k < Bp; k += kStep) {
-          FragA<BF> fa;
-          FragB<BF> fb[1];
-          load_zt(fa, Z(l) + k * m.zp[l] + 16 * i, m.zp[l], lane);
-          load_st(fb[0], A(l - 1) + k * m.ap[l - 1] + 8 * j, m.ap[l - 1], lane);
-          products(acc, x1, x2, fa, fb);
+        for (int k = 0; k + kStep <= Bp; k += kStep) {
+          load_zt(fa, Z(l), k, 16 * i, zplane(l), m.zp[l], lane);
+          load_at(fb, A(l - 1) + k * m.ap[l - 1] + 8 * j, m.ap[l - 1], lane);
+          product(acc, fa, fb);
+        }
+        if constexpr (BT % 2 != 0) {
+          constexpr int k = Bp - 8;
+          load_zt_k8(fa, Z(l), k, 16 * i, zplane(l), m.zp[l], lane);
+          load_at_k8(fb, A(l - 1) + k * m.ap[l - 1] + 8 * j, m.ap[l - 1], lane);
+          product_k8(acc, fa, fb);
         }
         float uq[4];
         if (!SUM) own.load4(m.us[l] + (e >> 4), uq);
@@ -790,8 +1000,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           const int at = (16 * i + g + 8 * r2) * m.wp[l] + 8 * j + 2 * tt, c = 2 * r2;
           float2* w = reinterpret_cast<float2*>(smem + m.o_w[l] + at);
           float2 wv = *w;
-          const float g0 = fmaf(lambda, wv.x, term<BF>(acc[0][c], x1[0][c], x2[0][c]));
-          const float g1 = fmaf(lambda, wv.y, term<BF>(acc[0][c + 1], x1[0][c + 1], x2[0][c + 1]));
+          const float g0 = fmaf(lambda, wv.x, value(acc, c)), g1 = fmaf(lambda, wv.y, value(acc, c + 1));
           wv.x = fmaf(-eta, g0, wv.x); wv.y = fmaf(-eta, g1, wv.y);
           *w = wv;
           if (!SUM) {
@@ -824,13 +1033,14 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
       const T* X = rows_of(it);
       const T* Xn = rows_of(it + 1);
       if (BF) clear();
-      constexpr int kBk = 8 * BT / kStep;   // k-steps over the samples at most
+      constexpr int kBk = BT / 2;   // whole k-steps over the samples; an odd tile goes by itself
       constexpr bool kHold = BF || BT <= 4;   // room for all of dZ_0's fragments
-      FragA<BF> a[kHold ? kBk : 1];
+      const int zpl = zplane(0);
+      FragA<NP> a[kHold ? (BT + 1) / 2 : 1];
       if (kHold) {
 #pragma unroll
-        for (int k = 0; k < kBk; ++k)
-          load_zt(a[kHold ? k : 0], Z(0) + k * kStep * m.zp[0] + 16 * wm, m.zp[0], lane);
+        for (int k = 0; k < kBk; ++k) load_zt(a[kHold ? k : 0], Z(0), k * kStep, 16 * wm, zpl, m.zp[0], lane);
+        if constexpr (BT % 2 != 0) load_zt_k8(a[kHold ? kBk : 0], Z(0), kBk * kStep, 16 * wm, zpl, m.zp[0], lane);
       }
 #pragma unroll 1
       for (int u = 0; u < wn; ++u) {
@@ -841,10 +1051,17 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
         float d[2][4] = {}, x1[2][4] = {};
 #pragma unroll
         for (int k = 0; k < kBk; ++k) {
-          if (!kHold) load_zt(a[0], Z(0) + k * kStep * m.zp[0] + 16 * wm, m.zp[0], lane);
-          FragB<BF> f[2];
-          load_st2(f, xu + k * kStep * m.xpitch, m.xpitch, lane);
+          if (!kHold) load_zt(a[0], Z(0), k * kStep, 16 * wm, zpl, m.zp[0], lane);
+          FragB<NP> f[2];
+          load_st2(f, xu + k * kStep * m.xpitch, xpl, m.xpitch, lane);
           products(d, x1, x1, a[kHold ? k : 0], f);
+        }
+        if constexpr (BT % 2 != 0) {
+          if (!kHold) load_zt_k8(a[0], Z(0), kBk * kStep, 16 * wm, zpl, m.zp[0], lane);
+          FragB<NP> f[2];
+          load_st2_k8(f, xu + kBk * kStep * m.xpitch, xpl, m.xpitch, lane);
+          product_k8(d[0], x1[0], x1[0], a[kHold ? kBk : 0], f[0]);
+          product_k8(d[1], x1[1], x1[1], a[kHold ? kBk : 0], f[1]);
         }
         float w[8], us[8];
         own.wait(r, w);

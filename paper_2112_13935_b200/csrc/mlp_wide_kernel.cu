@@ -246,17 +246,24 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
   constexpr bool kSum1 = M::kSum1;
   float* const us2 = reinterpret_cast<float*>(smem + M::u2) + tid * 8;   // kSum1: W_2's update sum, a thread's own words
   auto load_u2 = [&](float (&v)[8]) {
-    if (!kSum1) { own.load(kU2, v); return; }
+    if constexpr (!kSum1) {
+      own.load(kU2, v);
+    } else {
 #pragma unroll
-    for (int i = 0; i < 8; i += 4) {
-      const float4 x = *reinterpret_cast<const float4*>(us2 + i);
-      v[i] = x.x; v[i + 1] = x.y; v[i + 2] = x.z; v[i + 3] = x.w;
+      for (int i = 0; i < 8; i += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(us2 + i);
+        v[i] = x.x; v[i + 1] = x.y; v[i + 2] = x.z; v[i + 3] = x.w;
+      }
     }
   };
   auto store_u2 = [&](const float (&v)[8]) {
-    if (!kSum1) { own.store(kU2, v); own.store_wait(); return; }
+    if constexpr (!kSum1) {
+      own.store(kU2, v);
+      own.store_wait();
+    } else {
 #pragma unroll
-    for (int i = 0; i < 8; i += 4) *reinterpret_cast<float4*>(us2 + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+      for (int i = 0; i < 8; i += 4) *reinterpret_cast<float4*>(us2 + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    }
   };
   {
     const float zero[8] = {};
