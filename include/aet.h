@@ -163,8 +163,18 @@ typedef struct {
 aet_status aet_create(const aet_config* cfg, aet_handle** out);
 
 /* End of the run of Algorithm 3's loop "for round i": free everything the
- * handle owns (synchronises the device first). */
+ * handle owns (synchronises the device first).  Its device memory stays with
+ * the library for the next handle, as far as what is kept so stays within 512 MB
+ * and 128 blocks for the whole process; the library gives it back by itself only
+ * when one of its own allocations fails. */
 aet_status aet_destroy(aet_handle* h);
+
+/* Give back to the driver what destroyed handles have left with the library:
+ * device memory (see aet_destroy) and the pinned blocks of small read-backs (at
+ * most 1 MB).  For a process whose other parts need the memory (the paper has no
+ * counterpart).  Handles that are alive, of any thread, keep theirs and stay
+ * usable; freeing waits for the device, as cudaFree does.  Errors: AET_ERR_CUDA. */
+aet_status aet_release_memory(void);
 
 /* Back to the state right after aet_create + aet_set_global_model + data load:
  * global model = the last model set (zeros if none), no rounds done, clock 0,

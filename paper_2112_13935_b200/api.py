@@ -81,6 +81,11 @@ def aet_destroy(h):
     _check(h, _lib.load().aet_destroy(h))
 
 
+def aet_release_memory():
+    """Device memory kept from destroyed handles, and pinned blocks, back to the driver."""
+    _check(None, _lib.load().aet_release_memory())
+
+
 def aet_reset(h, stream=None):
     _check(h, _lib.load().aet_reset(h, _stream(stream)))
 

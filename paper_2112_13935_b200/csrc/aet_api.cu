@@ -25,8 +25,8 @@ thread_local std::string g_create_error;
 
 // Device memory of destroyed handles, kept for the next one: cudaMalloc and cudaFree of a handle's dozen arrays cost a
 // short job (create, load, run, destroy) more than its run - milliseconds, at times tens of them.  Bounded per process,
-// given back to the driver whenever an allocation fails or the bound is reached; blocks come back only after the device
-// has been synchronised, so any stream may use them next.
+// given back to the driver by aet_release_memory and whenever an allocation fails, never grown past the bound; blocks come
+// back only after the device has been synchronised, so any stream may use them next.
 class DevicePool {
  public:
   void* get(size_t bytes) {
@@ -67,6 +67,10 @@ class DevicePool {
     held_ += b.bytes;
     free_.push_back(b);
   }
+  void release() {   // everything no handle holds, back to the driver
+    std::lock_guard<std::mutex> lock(mu_);
+    flush();
+  }
 
  private:
   struct Block { void* p; size_t bytes; int dev; };
@@ -86,7 +90,7 @@ DevicePool& pool() {
   return *p;
 }
 
-// A few pinned blocks for small read-backs, shared by all handles and threads; kept until the process ends.
+// A few pinned blocks for small read-backs, shared by all handles and threads; kept until aet_release_memory.
 class PinnedPool {
  public:
   static constexpr size_t kBlock = 64 << 10;
@@ -102,12 +106,23 @@ class PinnedPool {
       ++made_;
     }
     void* p = nullptr;
-    if (cudaHostAlloc(&p, kBlock, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (cudaHostAlloc(&p, kBlock, cudaHostAllocPortable) != cudaSuccess) {
+      cudaGetLastError();
+      std::lock_guard<std::mutex> lock(mu_);
+      --made_;
+      return nullptr;
+    }
     return p;
   }
   void put(void* p) {
     std::lock_guard<std::mutex> lock(mu_);
     free_.push_back(p);
+  }
+  void release() {
+    std::lock_guard<std::mutex> lock(mu_);
+    for (void* p : free_) cudaFreeHost(p);
+    made_ -= (int)free_.size();
+    free_.clear();
   }
 
  private:
@@ -564,6 +579,14 @@ aet_status aet_destroy(aet_handle* h) {
   cudaGetLastError();
   if (before != h->device) cudaSetDevice(before);
   delete h;
+  return AET_OK;
+}
+
+aet_status aet_release_memory(void) {
+  pool().release();
+  pinned().release();
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(nullptr, AET_ERR_CUDA, std::string("releasing memory: ") + cudaGetErrorString(e));
   return AET_OK;
 }
 

@@ -14,6 +14,27 @@ def _small(**kw):
     return workloads.get_config("cfg1", n_rounds=3, data=dict(per_client=200), **kw)
 
 
+def test_memory_left_by_destroyed_handles_goes_back_on_request():
+    cfg = workloads.get_config("cfg5", n_clients=40, n_rounds=2, data=dict(per_client=800))     # 100 MB of rows
+    data, w0 = make(cfg)
+    dev, start = to_device(data), torch.from_numpy(w0).cuda()
+    api.aet_release_memory()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    models = []
+    for _ in range(2):
+        with api.Session(cfg, dev, start) as s:
+            s.run()
+            models.append(s.model().tobytes())
+            assert torch.cuda.mem_get_info()[0] < free
+            api.aet_release_memory()                                    # a living handle keeps its memory
+            models.append(s.model().tobytes())
+    assert free - torch.cuda.mem_get_info()[0] <= 512 << 20
+    api.aet_release_memory()
+    assert torch.cuda.mem_get_info()[0] >= free
+    assert len(set(models)) == 1
+
+
 @pytest.mark.parametrize("l2", [1e-4, 0.0])
 def test_a_nan_pixel_is_reported_as_numeric_and_the_handle_stays_usable(l2):
     cfg = _small(l2=l2)
