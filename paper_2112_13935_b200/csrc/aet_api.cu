@@ -63,7 +63,17 @@ class DevicePool {
     if (it == live_.end()) return;
     const Block b = it->second;
     live_.erase(it);
-    if (held_ + b.bytes > kMost || free_.size() >= kMostBlocks) { cudaFree(p); return; }
+    // Over the bound the largest go: a large block costs least beside the copies that fill it.
+    while (held_ + b.bytes > kMost || free_.size() >= kMostBlocks) {
+      size_t most = free_.size();
+      for (size_t i = 0; i < free_.size(); ++i)
+        if (free_[i].bytes > b.bytes && (most == free_.size() || free_[i].bytes > free_[most].bytes)) most = i;
+      if (most == free_.size()) { cudaFree(p); return; }
+      cudaFree(free_[most].p);
+      held_ -= free_[most].bytes;
+      free_[most] = free_.back();
+      free_.pop_back();
+    }
     held_ += b.bytes;
     free_.push_back(b);
   }
@@ -142,12 +152,18 @@ struct Arena {
   std::vector<void*> chunks;
   char* cur = nullptr;
   size_t left = 0;
-  size_t next = 8ull << 20;   // chunks grow from 8 MB to 256 MB: a small job takes a small one
+  // Chunks of 8 to 256 MB: the first as large as the first client's arrays say that all of them will be, so that neither a small
+  // job takes much nor a large one many (a chunk costs 0.3 to 0.6 ms), the next ones growing if that was too little.
+  static constexpr size_t kLeast = 8ull << 20, kMost = 256ull << 20;
+  size_t next = kLeast;
+  void expect(size_t bytes) {
+    if (chunks.empty()) next = bytes < kLeast ? kLeast : bytes > kMost ? kMost : (bytes + kLeast - 1) / kLeast * kLeast;
+  }
   void* alloc(size_t bytes) {
     bytes = (bytes + 255) & ~(size_t)255;
     if (bytes > left) {
       size_t want = bytes > next ? bytes : next;
-      if (next < (256ull << 20)) next = next * 4 < (256ull << 20) ? next * 4 : 256ull << 20;
+      if (next < kMost) next = next * 4 < kMost ? next * 4 : kMost;
       void* p = pool().get(want);
       if (!p) return nullptr;
       chunks.push_back(p);
@@ -654,6 +670,7 @@ aet_status aet_load_client_data(aet_handle* h, uint32_t client, const void* x, c
     h->last_stream = s;
     return AET_OK;
   }
+  h->arena.expect((elems * (bf16 ? 2 : 4) + (size_t)n * sizeof(int32_t) + 512) * h->cfg.n_clients);
   void* dx = h->arena.alloc(elems * (bf16 ? 2 : 4));
   int32_t* dy = (int32_t*)h->arena.alloc((size_t)n * sizeof(int32_t));
   if (!dx || !dy) return fail(h, AET_ERR_NOMEM, "device allocation failed");
