@@ -50,14 +50,17 @@ struct RoundLaunch {
   float l2;
 };
 
+// How many clusters of 1, 2, 4 or 8 CTAs with an SM each the current device runs at once (see device_info.cu).
+cudaError_t clusters_at_once(uint32_t cluster, uint32_t* out);
+
 // One CTA waits (at most max_polls polls) on a barrier nobody signals, then sets bit 0 of *status.
 cudaError_t launch_wait_probe(uint32_t* status, uint32_t max_polls, cudaStream_t s);
 
 // Softmax regression 784 -> 10, batch 1; the kernel is picked by how many round-tasks the launch holds.  Asynchronous on s; may start under the tail of the previous kernel in s
 // (programmatic stream serialisation) and waits on the device before reading that kernel's output.
 cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s);
-// at most one round-task per SM: a cluster of up to four CTAs per round-task (see lr_chain_kernel.cu)
-cudaError_t launch_lr_chain_rounds(const RoundLaunch& p, uint32_t sms, cudaStream_t s);
+// a cluster of four or two CTAs per round-task (see lr_chain_kernel.cu)
+cudaError_t launch_lr_chain_rounds(const RoundLaunch& p, uint32_t cluster, cudaStream_t s);
 // one CTA per round-task; crowded: two CTAs per SM (see lr_block_kernel.cu)
 cudaError_t launch_lr_block_rounds(const RoundLaunch& p, bool crowded, cudaStream_t s);
 
@@ -108,7 +111,7 @@ size_t cnn_act_floats(const CnnShape& s);
 const char* cnn_check_shape(const CnnShape& s);   // null if the kernel can run it
 cudaError_t launch_cnn_rounds(const CnnLaunch& p, cudaStream_t s);
 // The LeNet shape, minibatches of up to 24 samples, on clusters of 8 or 4 CTAs (see cnn_mma_kernel.cu); 0: not eligible
-uint32_t cnn_mma_cluster(const CnnShape& s, uint32_t n_tasks, uint32_t sms);
+cudaError_t cnn_mma_cluster(const CnnShape& s, uint32_t n_tasks, uint32_t* cluster);
 cudaError_t launch_cnn_mma_rounds(const CnnLaunch& p, uint32_t cluster, cudaStream_t s);
 
 // Ordered aggregation: for seq in [lo, hi): w -= eta_seq * U[seq]; keep a copy

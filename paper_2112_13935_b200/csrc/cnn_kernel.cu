@@ -547,24 +547,25 @@ const char* cnn_check_shape(const CnnShape& s) {
 
 cudaError_t launch_cnn_rounds(const CnnLaunch& p0, cudaStream_t s) {
   if (p0.r.n_tasks == 0) return cudaSuccess;
-  int sms = 0;   // asked of the current device at every launch: cheap, and right on any device of the process
-  {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
-  if (const uint32_t c = cnn_mma_cluster(p0.shape, p0.r.n_tasks, (uint32_t)sms)) return launch_cnn_mma_rounds(p0, c, s);
-  // CTAs per round-task: as many as the minibatch has samples and the launch leaves SMs for
+  uint32_t mma = 0;
+  cudaError_t e = cnn_mma_cluster(p0.shape, p0.r.n_tasks, &mma);
+  if (e != cudaSuccess) return e;
+  if (mma) return launch_cnn_mma_rounds(p0, mma, s);
+  // CTAs per round-task: as many as the minibatch has samples and the device runs at once for every round-task
   uint32_t cl = kMaxCl;
-  while (cl > 1 && (cl > p0.shape.batch || p0.r.n_tasks * cl > (uint32_t)sms)) cl >>= 1;
+  for (; cl > 1; cl >>= 1) {
+    uint32_t fit = 0;
+    e = clusters_at_once(cl, &fit);
+    if (e != cudaSuccess) return e;
+    if (cl <= p0.shape.batch && p0.r.n_tasks <= fit) break;
+  }
   CnnLaunch p = p0;
   size_t smem = cnn_smem_bytes_staged(p.shape, cl, true);
   p.stage_acts = smem != 0;
   if (!smem) smem = cnn_smem_bytes_staged(p.shape, cl, false);
   p.stage_rows = smem != 0;
   if (!smem) smem = cnn_smem_bytes(p.shape);
-  cudaError_t e = cudaFuncSetAttribute(cnn_round_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(cnn_round_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(p.r.n_tasks * cl, 1, 1);

@@ -672,7 +672,7 @@ cudaError_t launch(const RoundLaunch& p, cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_lr_chain_rounds(const RoundLaunch& p, uint32_t sms, cudaStream_t s) {
+cudaError_t launch_lr_chain_rounds(const RoundLaunch& p, uint32_t cluster, cudaStream_t s) {
   static bool opted_in[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -685,9 +685,7 @@ cudaError_t launch_lr_chain_rounds(const RoundLaunch& p, uint32_t sms, cudaStrea
     if (e != cudaSuccess) return e;
     if (known) opted_in[dev] = true;
   }
-  // As many CTAs per round-task as the SMs hold at once; clusters do not straddle GPCs, so a few SMs stay unused.
-  if (p.n_tasks * 4 <= sms - sms / 8) return launch<Four>(p, s);
-  return launch<Two>(p, s);   // (the caller has checked that two fit)
+  return cluster == 4 ? launch<Four>(p, s) : launch<Two>(p, s);
 }
 
 }  // namespace aet

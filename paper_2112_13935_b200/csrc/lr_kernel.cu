@@ -1,8 +1,9 @@
 // Softmax regression 784 -> 10, batch 1: which kernel runs a launch of round-tasks.
 //
-// Up to about half an SM's share of the launch per round-task, the round's serial chain sets the time: a cluster of two or
-// four CTAs per round-task (lr_chain_kernel.cu).  With more round-tasks than that, a cluster would leave some of them
-// waiting for SMs: one CTA each (lr_block_kernel.cu), and with more round-tasks than SMs its two-per-SM shape.
+// As long as the device runs a cluster for every round-task at once, the round's serial chain sets the time: four or two CTAs per
+// round-task (lr_chain_kernel.cu).  With more round-tasks than that, a cluster would leave some of them
+// waiting for SMs: one CTA each (lr_block_kernel.cu), and with more round-tasks than SMs its two-per-SM shape.  Rounds of 400
+// samples: 33 clients 88 us on four CTAs, 98 on two; 74 clients 113 us on two, 161 on one.
 #include <cuda_runtime.h>
 
 #include "aet_kernels.h"
@@ -36,22 +37,14 @@ cudaError_t launch_wait_probe(uint32_t* status, uint32_t max_polls, cudaStream_t
 
 cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s) {
   if (p.n_tasks == 0) return cudaSuccess;
-  static int sm_count[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  uint32_t ones = 0, pairs = 0, fours = 0;
+  cudaError_t e = clusters_at_once(1, &ones);
+  if (e == cudaSuccess) e = clusters_at_once(2, &pairs);
+  if (e == cudaSuccess) e = clusters_at_once(4, &fours);
   if (e != cudaSuccess) return e;
-  const bool known = dev >= 0 && dev < 64;
-  int sms = known ? sm_count[dev] : 0;
-  if (!sms) {
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    if (known) sm_count[dev] = sms;
-  }
-  const bool crowded = p.n_tasks > (uint32_t)sms || p.crowded_hint;
-  if (crowded) return launch_lr_block_rounds(p, true, s);
-  // (clusters do not straddle GPCs: one SM in sixteen is not counted on)
-  if (p.n_tasks * 2 > (uint32_t)(sms - sms / 16)) return launch_lr_block_rounds(p, false, s);
-  return launch_lr_chain_rounds(p, (uint32_t)sms, s);
+  if (p.n_tasks > ones || p.crowded_hint) return launch_lr_block_rounds(p, true, s);
+  if (p.n_tasks > pairs) return launch_lr_block_rounds(p, false, s);
+  return launch_lr_chain_rounds(p, p.n_tasks > fours ? 2 : 4, s);
 }
 
 }  // namespace aet

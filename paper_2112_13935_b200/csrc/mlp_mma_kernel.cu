@@ -1187,18 +1187,20 @@ cudaError_t launch(const MmaLaunch& p, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, mlp_mma_kernel<BF, BT, SUM>, p);
 }
 
-// The widest cluster that leaves every round-task of the launch its own SMs; where none does, the smallest that holds
-// the first layer.
-MmaPlan pick_plan(const MlpShape& s, uint32_t n_tasks, uint32_t sms) {
-  MmaPlan last{};
+// The widest cluster of which the device runs one for every round-task of the launch at once; where there is none, the smallest
+// that holds the first layer.
+cudaError_t pick_plan(const MlpShape& s, uint32_t n_tasks, MmaPlan* out) {
+  *out = MmaPlan{};
 #pragma unroll 1
   for (int cl = 8; cl >= 1; cl >>= 1) {
     const MmaPlan p = make_plan(s, cl);
     if (!p.total) continue;
-    last = p;
-    if (n_tasks * cl <= sms) return p;
+    *out = p;
+    uint32_t fit = 0;
+    if (const cudaError_t e = clusters_at_once((uint32_t)cl, &fit)) return e;
+    if (n_tasks <= fit) break;
   }
-  return last;
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -1211,13 +1213,9 @@ bool mlp_mma_eligible(const MlpShape& shape) {
 }
 
 cudaError_t launch_mlp_mma_rounds(const MlpLaunch& p, cudaStream_t s) {
-  int sms = 0, dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
   MmaLaunch q;
   q.r = p.r;
-  q.m = pick_plan(p.shape, p.r.n_tasks, (uint32_t)sms);
+  if (const cudaError_t e = pick_plan(p.shape, p.r.n_tasks, &q.m)) return e;
   if (!q.m.total) return cudaErrorInvalidConfiguration;
   if (p.shape.precision == 0) {
     switch (q.m.bt) {

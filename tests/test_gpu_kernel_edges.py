@@ -35,7 +35,7 @@ def check(cfg, w_tol=2e-5, bf16=False):
 
 
 @pytest.mark.parametrize("l2", [0.0, 1e-3])
-@pytest.mark.parametrize("n_clients", [3, 50, 100, 200])    # clusters of four, of two; one CTA; two CTAs per SM
+@pytest.mark.parametrize("n_clients", [3, 33, 74, 100, 200])    # clusters of four, of two (the most of each); one CTA; two CTAs per SM
 @pytest.mark.parametrize("first", [1, 7, 15, 31])           # rounds of first, first + 1, first + 2 samples: around blocks of 8 and 16
 def test_regression_rounds_around_whole_blocks(n_clients, first, l2):
     check(workloads.get_config("cfg5", n_clients=n_clients, n_rounds=3, sched_a=1, sched_b=first, l2=l2, lr=0.002 if n_clients < 10 else 1e-4,
@@ -82,7 +82,7 @@ def test_fp32_mlp_rounds(dims, batch, n_clients):
 @pytest.mark.parametrize("dims,batch,n_clients", [
     ([512, 256, 10], 16, 4), ([520, 100, 30, 10], 48, 4), ([200, 17, 10], 33, 20), ([1024, 64, 16], 64, 80),   # first layer on the chip
     ([1024, 256, 128, 10], 64, 4), ([512, 256, 128, 10], 64, 20), ([512, 256, 128, 10], 64, 50), ([160, 256, 128, 16], 64, 90),
-    ([1024, 256, 128, 10], 32, 50), ([1024, 256, 10], 64, 4), ([512, 256, 10], 32, 50), ([128, 256, 11], 64, 90),   # ... streamed: clusters of 8, 4, 2, 1
+    ([1024, 256, 128, 10], 32, 50), ([1024, 256, 128, 10], 64, 16), ([1024, 256, 10], 64, 4), ([512, 256, 10], 32, 50), ([128, 256, 11], 64, 90),   # ... streamed: clusters of 8, 4, 2, 1
 ])
 def test_bf16_mlp_rounds(dims, batch, n_clients):
     check(workloads.get_config("cfg4", n_clients=n_clients, n_rounds=2, dims=dims, batch=batch, sched_a=batch, sched_b=2 * batch, l2=1e-3,
@@ -145,6 +145,35 @@ def test_aggregation_of_short_and_long_ranges(n_clients):
     for e in ref["events"]:
         acc -= sim.step_size(cfg, e["round"]) * gpu["U"][e["seq"]].astype(np.float64)
     assert np.abs(acc - gpu["w"]).max() <= 2e-6 * max(1.0, np.abs(acc).max())
+
+
+def wave_us(cfg):
+    """Device time of one wave: the median over passes of a one-round run."""
+    data, w0 = make(cfg)
+    times = []
+    with api.Session(cfg, to_device(data), torch.from_numpy(w0).cuda()) as s:
+        for _ in range(15):
+            s.reset()
+            begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            begin.record()
+            s.run()
+            end.record()
+            torch.cuda.synchronize()
+            times.append(begin.elapsed_time(end))
+    return float(np.median(times[3:]))
+
+
+# A wave on clusters of which the device runs too few at once is two waves; on narrower ones it is one.  So a few clients more on
+# the next narrower cluster never make the wave shorter (two waves took 1.15 to 1.45 times as long as those).
+@pytest.mark.parametrize("name,over,fewer,more", [
+    ("cfg4", dict(n_stragglers=0, sched_a=64, sched_b=1280, data=dict(kind="per_client", per_client=64)), 16, 17),
+    ("cfg4", dict(n_stragglers=0, sched_a=64, sched_b=1280, data=dict(kind="per_client", per_client=64)), 35, 38),
+    ("cfg7", dict(sched_a=16, sched_b=320, data=dict(kind="per_client", per_client=64)), 16, 17),
+    ("cfg5", dict(sched_a=1, sched_b=400, lr=1e-4, data=dict(per_client=64)), 70, 75),
+])
+def test_fewer_clients_never_take_longer(name, over, fewer, more):
+    t = [wave_us(workloads.get_config(name, n_clients=n, n_rounds=1, **over)) for n in (fewer, more)]
+    assert t[0] <= 1.08 * t[1], t
 
 
 def test_handles_of_several_threads_share_released_memory():
