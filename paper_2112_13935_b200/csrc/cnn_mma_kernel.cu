@@ -14,14 +14,14 @@
 // Nothing is reused before its readers are done because each step needs the one before from all CTAs.  All weights stay in
 // shared memory, all update sums in the registers of the threads that own the parameters, for the whole round.
 //
-// Products are m16n8k8 tf32 on split fp32 operands (mma_common.cuh; both heads rounded: rms error of a round 1.9e-7, as plain
-// FMAs), convolutions as implicit GEMMs:
+// Products are bf16 on operands in three parts (mma_common.cuh; rms error of a round 0.5e-7 to 1.1e-7 as with fp32 FMAs, 1.1e-7 to
+// 1.5e-7 with two tf32 parts), convolutions as implicit GEMMs:
 //   conv 2      Z[16 x 64] = W2[16 x 150] im2col(q1)           M = output planes exactly; the bias is tap 150 with input 1
 //   its dW      dW2[16 x 150] = dz2[16 x 64] im2col(q1)^T      accumulators stay in registers over the samples
 //   its dIn     col[150 x 64] = W2^T dz2, then every output gathers its up to 25 entries of col
 //   conv 1      FMAs (6 planes would fill 6 of 16 rows);  its dW[26 x 6] = im2col(x)^T dz1, dz1 formed from dq1 and sign bits
-// What bounds it: the chain of some fifteen short phases and five hand-overs per iteration, not any one unit (about 59 K
-// cycles).  Measured: 16 clients, minibatch 16, 12 rounds, 19 -> 7.5 ms against the split by samples.
+// What bounds it: the chain of some fifteen short phases and five hand-overs per iteration, not any one unit (about 55 K
+// cycles).  Measured: 16 clients, minibatch 16, 12 rounds, 18.9 -> 7.5 ms against the split by samples.
 #include <cuda_runtime.h>
 
 #include "aet_kernels.h"
@@ -36,8 +36,9 @@ using lr::kWaitLimit;
 using lr::mbar_expect_tx;
 using lr::mbar_init;
 using lr::smem_addr;
-using mma::Split;
-using mma::split;
+using mma::Parts;
+using mma::parts;
+using mma::parts_t;
 
 constexpr int kWarps = 16, kThreads = kWarps * 32;
 constexpr int kS = 28, kC1 = 6, kP1 = 12, kC2 = 16, kFlat = 256, kF1 = 120, kF2 = 84, kN = 10;
@@ -50,40 +51,52 @@ constexpr int kMaxPer = 4;                              // samples per CTA
 constexpr int kOW1 = 0, kOb1 = 150, kOW2 = 156, kOb2 = 2556, kOF1 = 2572, kObF1 = kOF1 + kFlat * kF1, kOF2 = kObF1 + kF1,
               kObF2 = kOF2 + kF1 * kF2, kOF3 = kObF2 + kF2, kObF3 = kOF3 + kF2 * kN, kP = kObF3 + kN;
 static_assert(kP == 44426, "the LeNet shape");
+static_assert(kF1 / 8 % 2 == 1 && kPh2 / 8 % 2 == 1, "the dense layers' last step is one of eight");
 
 // ---- fragments (lane = 4 g + tt; the k index of a step is read as pairs 2 tt | 2 tt + 1 unless said otherwise) ----------
-struct FA { Split v[4]; };
-struct FB { Split v[2]; };
+// An operand's pair of k values in three bf16 parts, split by rounding (the convolutions' gathered inputs by cutting)
+struct FA { Parts lo, hi; };   // rows g and g + 8
+struct FB { Parts v; };
 __device__ __forceinline__ FA a_rows(const float* w, int pitch, int g, int tt) {   // [row][k]
   const float2 a = *reinterpret_cast<const float2*>(w + g * pitch + 2 * tt), b = *reinterpret_cast<const float2*>(w + (g + 8) * pitch + 2 * tt);
-  return {split(a.x), split(b.x), split(a.y), split(b.y)};
+  return {parts(a.x, a.y), parts(b.x, b.y)};
 }
 __device__ __forceinline__ FA a_cols(const float* w, int pitch, int g, int tt) {   // [k][row]
   const float* p = w + 2 * tt * pitch + g;
-  return {split(p[0]), split(p[8]), split(p[pitch]), split(p[pitch + 8])};
+  return {parts(p[0], p[pitch]), parts(p[8], p[pitch + 8])};
 }
 __device__ __forceinline__ FA a_cols_k(const float* w, int pitch, int g, int tt) {   // [k][row], k = tt | tt + 4
   const float* p = w + tt * pitch + g;
-  return {split(p[0]), split(p[8]), split(p[4 * pitch]), split(p[4 * pitch + 8])};
+  return {parts(p[0], p[4 * pitch]), parts(p[8], p[4 * pitch + 8])};
 }
 __device__ __forceinline__ FB b_rows(const float* x, int pitch, int g, int tt) {   // [column][k]
   const float2 a = *reinterpret_cast<const float2*>(x + g * pitch + 2 * tt);
-  return {split(a.x), split(a.y)};
+  return {parts(a.x, a.y)};
 }
 __device__ __forceinline__ FB b_cols_k(const float* x, int pitch, int g, int tt) {   // [k][column], k = tt | tt + 4
   const float* p = x + tt * pitch + g;
-  return {split(p[0]), split(p[4 * pitch])};
+  return {parts(p[0], p[4 * pitch])};
 }
-__device__ __forceinline__ void mul(float (&d)[4], float (&x)[4], const FA& a, const FB& b) {
-  mma::tf32(d, a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].hi, b.v[1].hi);
-  mma::tf32(x, a.v[0].lo, a.v[1].lo, a.v[2].lo, a.v[3].lo, b.v[0].hi, b.v[1].hi);
-  mma::tf32(x, a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].lo, b.v[1].lo);
+// Eight k: the leading parts by themselves, two pairs of the small ones as one k index of 16
+__device__ __forceinline__ void mul3(float (&d)[4], float (&x)[4], float (&y)[4], const FA& a, const FB& b) {
+  const uint32_t ca[4] = {a.lo.c, a.hi.c, a.lo.a, a.hi.a}, bb[4] = {a.lo.b, a.hi.b, a.lo.b, a.hi.b};
+  mma::mma_bf16_k8(d, a.lo.a, a.hi.a, b.v.a);
+  mma::mma_bf16(x, ca, b.v.a, b.v.c);
+  mma::mma_bf16(y, bb, b.v.b, b.v.a);
+  mma::mma_bf16_k8(x, a.lo.a, a.hi.a, b.v.b);
 }
-__device__ __forceinline__ void mul3(float (&d)[3][4], const FA& a, const FB& b) {   // a term an accumulator: three short chains
-  mma::tf32(d[0], a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].hi, b.v[1].hi);
-  mma::tf32(d[1], a.v[0].lo, a.v[1].lo, a.v[2].lo, a.v[3].lo, b.v[0].hi, b.v[1].hi);
-  mma::tf32(d[2], a.v[0].hi, a.v[1].hi, a.v[2].hi, a.v[3].hi, b.v[0].lo, b.v[1].lo);
+__device__ __forceinline__ void mul(float (&d)[4], float (&x)[4], const FA& a, const FB& b) { mul3(d, x, x, a, b); }
+// Sixteen k: two steps of eight as one
+__device__ __forceinline__ void mul6(float (&d)[4], float (&x)[4], float (&y)[4], const FA& a0, const FB& b0, const FA& a1, const FB& b1) {
+  const uint32_t a[4] = {a0.lo.a, a0.hi.a, a1.lo.a, a1.hi.a}, b[4] = {a0.lo.b, a0.hi.b, a1.lo.b, a1.hi.b}, c[4] = {a0.lo.c, a0.hi.c, a1.lo.c, a1.hi.c};
+  mma::mma_bf16(x, c, b0.v.a, b1.v.a);
+  mma::mma_bf16(d, a, b0.v.a, b1.v.a);
+  mma::mma_bf16(y, a, b0.v.c, b1.v.c);
+  mma::mma_bf16(x, b, b0.v.b, b1.v.b);
+  mma::mma_bf16(y, b, b0.v.a, b1.v.a);
+  mma::mma_bf16(x, a, b0.v.b, b1.v.b);
 }
+__device__ __forceinline__ void mul2(float (&d)[4], float (&x)[4], const FA& a0, const FB& b0, const FA& a1, const FB& b1) { mul6(d, x, x, a0, b0, a1, b1); }
 __device__ __forceinline__ void send1(uint32_t addr, float v, uint32_t bar) {   // 4 bytes to a peer
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(__float_as_uint(v)), "r"(bar) : "memory");
 }
@@ -298,25 +311,40 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     const int e_half = kShare ? warp >> 3 : 0;
     auto conv2 = [&](int b, int yp, int s0, int s1, float (&acc)[2][4], float (&crs)[2][4]) {
       const float* q = sm + M::q1 + b * kQ1 + 2 * yp * kP1 + g;
-#pragma unroll 5
-      for (int s = s0; s < s1; ++s) {
-        const FA a = a_rows(sm + M::wc + 8 * s, kPw2, g, tt);
+      auto taps = [&](int s, FA& a, FB (&f)[2]) {
+        a = a_rows(sm + M::wc + 8 * s, kPw2, g, tt);
         const uint32_t o2 = *reinterpret_cast<const uint32_t*>(off + 8 * s + 2 * tt);
         const float* i0 = q + (o2 & 0xFFFF);
         const float* i1 = q + (o2 >> 16);
         const bool last = s == kPw2 / 8 - 1 && tt == 3;   // taps 150 (the bias input) and 151
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const FB f = {split(last ? 1.f : i0[kP1 * r]), split(last ? 0.f : i1[kP1 * r])};
-          mul(acc[r], crs[r], a, f);
+        for (int r = 0; r < 2; ++r) f[r] = {parts_t(last ? 1.f : i0[kP1 * r], last ? 0.f : i1[kP1 * r])};
+      };
+      FA a0, a1;
+      FB f0[2], f1[2];
+#pragma unroll 3
+      for (int s = s0; s + 1 < s1; s += 2) {
+        taps(s, a0, f0);
+        taps(s + 1, a1, f1);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {   // added up in fp32: the tensor cores would cut a sum of positive inputs always the same way
+          float d[4] = {};
+          mul2(d, crs[r], a0, f0[r], a1, f1[r]);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[r][c] += d[c];
         }
+      }
+      if ((s1 - s0) & 1) {
+        taps(s1 - 1, a0, f0);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) mul(acc[r], crs[r], a0, f0[r]);
       }
     };
     if (kShare) {
       const int e = warp & 7;
       if (e < 4 * nb) {
-        if (e_half == 0) conv2(e >> 2, e & 3, 0, 9, acc2, crs2);
-        else conv2(e >> 2, e & 3, 9, kPw2 / 8, acc2, crs2);
+        if (e_half == 0) conv2(e >> 2, e & 3, 0, 10, acc2, crs2);
+        else conv2(e >> 2, e & 3, 10, kPw2 / 8, acc2, crs2);
         if (e_half) {
           float* d = sm + M::col + kWarps * 64 + e * 256 + lane;
 #pragma unroll
@@ -362,18 +390,17 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[0], bytes[0]);
     {
       float acc[MT1][BT][4] = {}, crs[MT1][BT][4] = {};
+      const int k = 16 * warp;
+      FA a[MT1][2];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int k = 16 * warp + 8 * h;
-        FA a[MT1];
+      for (int i = 0; i < MT1; ++i)
 #pragma unroll
-        for (int i = 0; i < MT1; ++i) a[i] = a_rows(sm + M::w1 + 16 * i * kPq2 + k, kPq2, g, tt);
+        for (int h = 0; h < 2; ++h) a[i][h] = a_rows(sm + M::w1 + 16 * i * kPq2 + k + 8 * h, kPq2, g, tt);
 #pragma unroll
-        for (int b = 0; b < BT; ++b) {
-          const FB f = b_rows(sm + M::q2 + 8 * b * kPq2 + k, kPq2, g, tt);
+      for (int b = 0; b < BT; ++b) {
+        const FB f0 = b_rows(sm + M::q2 + 8 * b * kPq2 + k, kPq2, g, tt), f1 = b_rows(sm + M::q2 + 8 * b * kPq2 + k + 8, kPq2, g, tt);
 #pragma unroll
-          for (int i = 0; i < MT1; ++i) mul(acc[i][b], crs[i][b], a[i], f);
-        }
+        for (int i = 0; i < MT1; ++i) mul2(acc[i][b], crs[i][b], a[i][0], f0, a[i][1], f1);
       }
       __syncthreads();   // staged pooled maps have left the area the parts go to
       float* part = sm + M::col + warp * 16 * MT1 * Bp;
@@ -406,9 +433,11 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     for (int e = warp; e < 6 * BT; e += kWarps) {
       const int i = e % 6, b = e / 6;
       float acc[3][4] = {};
+      auto w_at = [&](int s) { return a_rows(sm + M::w2 + 16 * i * kPh1 + 8 * s, kPh1, g, tt); };
+      auto h_at = [&](int s) { return b_rows(sm + M::h1 + 8 * b * kPh1 + 8 * s, kPh1, g, tt); };
 #pragma unroll
-      for (int s = 0; s < kF1 / 8; ++s)
-        mul3(acc, a_rows(sm + M::w2 + 16 * i * kPh1 + 8 * s, kPh1, g, tt), b_rows(sm + M::h1 + 8 * b * kPh1 + 8 * s, kPh1, g, tt));
+      for (int s = 0; s + 1 < kF1 / 8; s += 2) mul6(acc[0], acc[1], acc[2], w_at(s), h_at(s), w_at(s + 1), h_at(s + 1));
+      mul3(acc[0], acc[1], acc[2], w_at(kF1 / 8 - 1), h_at(kF1 / 8 - 1));
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
@@ -444,7 +473,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
       for (int i = 0; i < 3; ++i) { v[i] = lr::ex2((v[i] - mx) * lr::kLog2e); sum += v[i]; }
       sum += lr::shx(sum, 1);
       sum += lr::shx(sum, 2);
-      const float fb = s < B ? 1.f / (float)B : 0.f, inv = lr::rcp(sum);
+      const float fb = s < B ? 1.f / (float)B : 0.f, inv = 1.f / sum;
       const int y = idx[(it & 1) * 64 + 32 + s];
 #pragma unroll
       for (int i = 0; i < 3; ++i)
@@ -471,9 +500,11 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
       for (int e = warp; e < MT1 * BT; e += 4) {
         const int i = e / BT, b = e % BT;
         float acc[3][4] = {};
+        auto w_at = [&](int s) { return a_cols(sm + M::w2 + 8 * s * kPh1 + rank * N1 + 16 * i, kPh1, g, tt); };
+        auto d_at = [&](int s) { return b_rows(sm + M::dh2 + 8 * b * kPh2 + 8 * s, kPh2, g, tt); };
 #pragma unroll
-        for (int s = 0; s < kPh2 / 8; ++s)
-          mul3(acc, a_cols(sm + M::w2 + 8 * s * kPh1 + rank * N1 + 16 * i, kPh1, g, tt), b_rows(sm + M::dh2 + 8 * b * kPh2 + 8 * s, kPh2, g, tt));
+        for (int s = 0; s + 1 < kPh2 / 8; s += 2) mul6(acc[0], acc[1], acc[2], w_at(s), d_at(s), w_at(s + 1), d_at(s + 1));
+        mul3(acc[0], acc[1], acc[2], w_at(kPh2 / 8 - 1), d_at(kPh2 / 8 - 1));
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const int n = 16 * i + g + ((c & 2) ? 8 : 0), s = 8 * b + 2 * tt + (c & 1);
@@ -487,8 +518,10 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
         float gr = 0.f;
         if (e < kF2 * kN) {
           const int i = e / kN, c = e % kN;
-#pragma unroll 8
-          for (int b = 0; b < Bp; ++b) gr = fmaf(sm[M::h2 + b * kPh2 + i], sm[M::z3 + b * 12 + c], gr);
+          float g4[4] = {};   // four short sums: fewer roundings on a long one
+#pragma unroll
+          for (int b = 0; b < Bp; ++b) g4[b & 3] = fmaf(sm[M::h2 + b * kPh2 + i], sm[M::z3 + b * 12 + c], g4[b & 3]);
+          gr = (g4[0] + g4[1]) + (g4[2] + g4[3]);
           const float w = sm[M::w3 + e];
           gr = fmaf(lambda, w, gr);
           sm[M::w3 + e] = fmaf(-eta, gr, w);
@@ -496,8 +529,10 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
           const int q = e - kF2 * kN;
           const float* d = q < kF2 ? sm + M::dh2 + q : sm + M::z3 + q - kF2;
           const int pitch = q < kF2 ? kPh2 : 12;
-#pragma unroll 8
-          for (int b = 0; b < Bp; ++b) gr += d[b * pitch];
+          float g4[4] = {};
+#pragma unroll
+          for (int b = 0; b < Bp; ++b) g4[b & 3] += d[b * pitch];
+          gr = (g4[0] + g4[1]) + (g4[2] + g4[3]);
           float* w = q < kF2 ? sm + M::b2 + q : sm + M::b3 + q - kF2;
           *w = fmaf(-eta, gr, *w);
         }
@@ -508,10 +543,11 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     {   // this CTA's part of dq2, 16 inputs per warp, to the samples' CTAs
       float acc[BT][4] = {}, crs[BT][4] = {};
 #pragma unroll
-      for (int s = 0; s < 2 * MT1; ++s) {
-        const FA a = a_cols(sm + M::w1 + 8 * s * kPq2 + 16 * warp, kPq2, g, tt);
+      for (int s = 0; s < 2 * MT1; s += 2) {
+        const FA a0 = a_cols(sm + M::w1 + 8 * s * kPq2 + 16 * warp, kPq2, g, tt), a1 = a_cols(sm + M::w1 + 8 * (s + 1) * kPq2 + 16 * warp, kPq2, g, tt);
 #pragma unroll
-        for (int b = 0; b < BT; ++b) mul(acc[b], crs[b], a, b_rows(sm + M::dh1 + 8 * b * kPd1 + 8 * s, kPd1, g, tt));
+        for (int b = 0; b < BT; ++b)
+          mul2(acc[b], crs[b], a0, b_rows(sm + M::dh1 + 8 * b * kPd1 + 8 * s, kPd1, g, tt), a1, b_rows(sm + M::dh1 + 8 * b * kPd1 + 8 * (s + 1), kPd1, g, tt));
       }
       const uint32_t inv = (1u << 16) / (uint32_t)per + 1;
 #pragma unroll
@@ -532,11 +568,18 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
 #pragma unroll
     for (int i = 0; i < MT1; ++i) {
       float acc[2][4] = {}, crs[2][4] = {};
+      auto d_at = [&](int s) { return a_cols_k(sm + M::dh1 + 8 * s * kPd1 + 16 * i, kPd1, g, tt); };
+      auto q_at = [&](int s, int h) { return b_cols_k(sm + M::q2 + 8 * s * kPq2 + 16 * warp + 8 * h, kPq2, g, tt); };
 #pragma unroll
-      for (int s = 0; s < BT; ++s) {
-        const FA a = a_cols_k(sm + M::dh1 + 8 * s * kPd1 + 16 * i, kPd1, g, tt);
+      for (int s = 0; s + 1 < BT; s += 2) {
+        const FA a0 = d_at(s), a1 = d_at(s + 1);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) mul(acc[h], crs[h], a, b_cols_k(sm + M::q2 + 8 * s * kPq2 + 16 * warp + 8 * h, kPq2, g, tt));
+        for (int h = 0; h < 2; ++h) mul2(acc[h], crs[h], a0, q_at(s, h), a1, q_at(s + 1, h));
+      }
+      if (BT % 2) {
+        const FA a = d_at(BT - 1);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) mul(acc[h], crs[h], a, q_at(BT - 1, h));
       }
 #pragma unroll
       for (int h = 0; h < 2; ++h)
@@ -550,36 +593,40 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
           u1[i][h][2 * r] += g0; u1[i][h][2 * r + 1] += g1;
         }
     }
-    {   // dense 2: 6 x 15 tiles, all of a warp's products before its first update (stores would hold the loads back)
-      float acc[6][4] = {};
 #pragma unroll
-      for (int r = 0; r < 6; ++r) {
-        const int e = min(warp + kWarps * r, 89), j = e / 6, i = e - 6 * j;
+    for (int r0 = 0; r0 < 6; r0 += 3) {   // dense 2: 6 x 15 tiles, the products of three before their first update (stores would hold the loads back)
+      float acc[3][4] = {}, crs[3][4] = {};
 #pragma unroll
-        for (int s = 0; s < BT; ++s)
-          mul(acc[r], acc[r], a_cols_k(sm + M::dh2 + 8 * s * kPh2 + 16 * i, kPh2, g, tt), b_cols_k(sm + M::h1 + 8 * s * kPh1 + 8 * j, kPh1, g, tt));
+      for (int r = 0; r < 3; ++r) {
+        const int e = min(warp + kWarps * (r0 + r), 89), j = e / 6, i = e - 6 * j;
+        auto d_at = [&](int s) { return a_cols_k(sm + M::dh2 + 8 * s * kPh2 + 16 * i, kPh2, g, tt); };
+        auto h_at = [&](int s) { return b_cols_k(sm + M::h1 + 8 * s * kPh1 + 8 * j, kPh1, g, tt); };
+#pragma unroll
+        for (int s = 0; s + 1 < BT; s += 2) mul2(acc[r], crs[r], d_at(s), h_at(s), d_at(s + 1), h_at(s + 1));
+        if (BT % 2) mul(acc[r], crs[r], d_at(BT - 1), h_at(BT - 1));
       }
 #pragma unroll
-      for (int r = 0; r < 6; ++r) {
-        const int e = warp + kWarps * r, j = e / 6, i = e - 6 * j;
+      for (int r = 0; r < 3; ++r) {
+        const int e = warp + kWarps * (r0 + r), j = e / 6, i = e - 6 * j;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const int n = 16 * i + g + 8 * q;
           if (e < 90 && n < kF2) {
             float2* w = reinterpret_cast<float2*>(sm + M::w2 + n * kPh1 + 8 * j + 2 * tt);
             float2 v = *w;
-            const float g0 = fmaf(lambda, v.x, acc[r][2 * q]), g1 = fmaf(lambda, v.y, acc[r][2 * q + 1]);
+            const float g0 = fmaf(lambda, v.x, acc[r][2 * q] + crs[r][2 * q]), g1 = fmaf(lambda, v.y, acc[r][2 * q + 1] + crs[r][2 * q + 1]);
             v.x = fmaf(-eta, g0, v.x); v.y = fmaf(-eta, g1, v.y);
             *w = v;
-            if (r % CL == rank) { u2[r / CL][2 * q] += g0; u2[r / CL][2 * q + 1] += g1; }
+            if ((r0 + r) % CL == rank) { u2[(r0 + r) / CL][2 * q] += g0; u2[(r0 + r) / CL][2 * q + 1] += g1; }
           }
         }
       }
     }
     if (tid < N1) {
-      float gr = 0.f;
-#pragma unroll 8
-      for (int b = 0; b < Bp; ++b) gr += sm[M::dh1 + b * kPd1 + tid];
+      float g4[4] = {};
+#pragma unroll
+      for (int b = 0; b < Bp; ++b) g4[b & 3] += sm[M::dh1 + b * kPd1 + tid];
+      const float gr = (g4[0] + g4[1]) + (g4[2] + g4[3]);
       sm[M::b1 + tid] = fmaf(-eta, gr, sm[M::b1 + tid]);
       ub1 += gr;
     }
@@ -631,15 +678,18 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
         const int at = (plane ? g : 0) * 144 + py * kP1 + px;
         const float v = plane ? 0.25f * sm[M::dq1 + hi * kQ1 + at] : 0.f;
         const uint32_t bits = m1[(s0 + hi) * kQ1 + at];
+        FA lo[2], up[2];   // taps 0 .. 15; taps 16 .. 23, then 24, the bias (an input of 1) and none
+        FB f[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          const FB f = {split(bits & (1u << (2 * h)) ? v : 0.f), split(bits & (2u << (2 * h)) ? v : 0.f)};
           const float* xi = xp + (2 * py + h) * kS;
-          mul(a1[0], x1[0], {split(xi[oa]), split(xi[ob]), split(xi[oa + 1]), split(xi[ob + 1])}, f);
-          // taps 16 .. 23, then 24, the bias (an input of 1) and none
+          f[h] = {parts(bits & (1u << (2 * h)) ? v : 0.f, bits & (2u << (2 * h)) ? v : 0.f)};
+          lo[h] = {parts_t(xi[oa], xi[oa + 1]), parts_t(xi[ob], xi[ob + 1])};
           const float t0 = g == 0 ? xi[od] : (g == 1 ? 1.f : 0.f), t1 = g == 0 ? xi[od + 1] : (g == 1 ? 1.f : 0.f);
-          mul(a1[1], x1[1], {split(xi[oc]), split(t0), split(xi[oc + 1]), split(t1)}, f);
+          up[h] = {parts_t(xi[oc], xi[oc + 1]), parts_t(t0, t1)};
         }
+        mul2(a1[0], x1[0], lo[0], f[0], lo[1], f[1]);
+        mul2(a1[1], x1[1], up[0], f[0], up[1], f[1]);
       }
     };
     __syncthreads();   // dq2's parts have been read: col may take their place
@@ -658,8 +708,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             float acc[4] = {}, crs[4] = {};
-            mul(acc, crs, f0, b_cols_k(sm + M::dz2 + 8 * (y + h), kPdz, g, tt));
-            mul(acc, crs, f1, b_cols_k(sm + M::dz2 + 8 * kPdz + 8 * (y + h), kPdz, g, tt));
+            mul2(acc, crs, f0, b_cols_k(sm + M::dz2 + 8 * (y + h), kPdz, g, tt), f1, b_cols_k(sm + M::dz2 + 8 * kPdz + 8 * (y + h), kPdz, g, tt));
             float* d = sm + M::col + (16 * i + g) * kPcol + 8 * (y + h) + 2 * tt;
             if (16 * i + g < 150) *reinterpret_cast<float2*>(d) = make_float2(acc[0] + crs[0], acc[1] + crs[1]);
             if (16 * i + g + 8 < 150) *reinterpret_cast<float2*>(d + 8 * kPcol) = make_float2(acc[2] + crs[2], acc[3] + crs[3]);
@@ -669,17 +718,17 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
       // dW2[plane x tap] += dz2 im2col(q1)^T over four rows of outputs
       const int y0 = 4 * (warp & 1);   // (the same half for all of a warp's tiles)
 #pragma unroll
-      for (int y = 0; y < 4; ++y) {
-        const FA f = a_rows(sm + M::dz2 + 8 * (y0 + y), kPdz, g, tt);
+      for (int y = 0; y < 4; y += 2) {
+        const FA f0 = a_rows(sm + M::dz2 + 8 * (y0 + y), kPdz, g, tt), f1 = a_rows(sm + M::dz2 + 8 * (y0 + y + 1), kPdz, g, tt);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
           const int q = warp + kWarps * i;
           if (q < 38) {
             const int n = 8 * (q >> 1) + g;
-            const float* in = q1 + o2[i] + 2 * tt;
-            float v0 = in[(y0 + y) * kP1], v1 = in[(y0 + y) * kP1 + 1];
-            if (n >= 150) v0 = v1 = n == 150 ? 1.f : 0.f;   // the bias
-            mul(a2[i], x2[i], f, {split(v0), split(v1)});
+            const float* in = q1 + o2[i] + 2 * tt + (y0 + y) * kP1;
+            float v0 = in[0], v1 = in[1], v2 = in[kP1], v3 = in[kP1 + 1];
+            if (n >= 150) v0 = v1 = v2 = v3 = n == 150 ? 1.f : 0.f;   // the bias
+            mul2(a2[i], x2[i], f0, {parts_t(v0, v1)}, f1, {parts_t(v2, v3)});
           }
         }
       }

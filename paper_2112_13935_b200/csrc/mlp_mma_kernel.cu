@@ -901,7 +901,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           if (4 * i < C) { v[i] = lr::ex2((v[i] - mx) * lr::kLog2e); sum += v[i]; }
         sum += __shfl_xor_sync(0xffffffffu, sum, 1);
         sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-        const float fb = s < B ? 1.f / (float)B : 0.f, inv = lr::rcp(sum);
+        const float fb = s < B ? 1.f / (float)B : 0.f, inv = 1.f / sum;
         const int y = idx[128 + (it & 1) * 64 + s];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
