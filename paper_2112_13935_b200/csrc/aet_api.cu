@@ -679,14 +679,22 @@ aet_status aet_load_client_data(aet_handle* h, uint32_t client, const void* x, c
   constexpr size_t kFetchMost = 2 << 20;
   const void *px = nullptr, *py = nullptr;   // the arrays as the device sees them
   if ((bf16 || elems * 4 <= kFetchMost) && elems % 4 == 0) {
-    cudaPointerAttributes ax{}, ay{};
-    if (cudaPointerGetAttributes(&ax, x) == cudaSuccess && ax.type == cudaMemoryTypeHost && cudaPointerGetAttributes(&ay, y) == cudaSuccess &&
-        ay.type == cudaMemoryTypeHost && ax.devicePointer && ay.devicePointer && !((uintptr_t)ax.devicePointer & 15) &&
-        !((uintptr_t)ay.devicePointer & 3)) {
-      px = ax.devicePointer;
-      py = ay.devicePointer;
+    // the whole array page-locked and in one piece as the device sees it: its last byte as far from the first there as here
+    auto seen = [](const void* from, size_t bytes) -> const void* {
+      cudaPointerAttributes first{}, last{};
+      const char* end = static_cast<const char*>(from) + bytes - 1;
+      const bool ok = cudaPointerGetAttributes(&first, from) == cudaSuccess && cudaPointerGetAttributes(&last, end) == cudaSuccess &&
+                      first.type == cudaMemoryTypeHost && last.type == cudaMemoryTypeHost && first.devicePointer && last.devicePointer &&
+                      static_cast<const char*>(last.devicePointer) - static_cast<const char*>(first.devicePointer) == (ptrdiff_t)bytes - 1;
+      cudaGetLastError();
+      return ok ? first.devicePointer : nullptr;
+    };
+    const void* sx = seen(x, elems * 4);
+    const void* sy = sx ? seen(y, (size_t)n * sizeof(int32_t)) : nullptr;
+    if (sx && sy && !((uintptr_t)sx & 15) && !((uintptr_t)sy & 3)) {
+      px = sx;
+      py = sy;
     }
-    cudaGetLastError();
   }
   if (px) {
     AET_CUDA(h, launch_fetch_client(static_cast<const float*>(px), dx, bf16, elems / 4, static_cast<const int32_t*>(py), dy, n, s));
