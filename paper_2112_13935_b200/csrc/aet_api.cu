@@ -40,8 +40,7 @@ class DevicePool {
           (best == free_.size() || free_[i].bytes < free_[best].bytes)) best = i;
     if (best < free_.size()) {
       const Block b = free_[best];
-      free_[best] = free_.back();
-      free_.pop_back();
+      free_.erase(free_.begin() + best);
       held_ -= b.bytes;
       live_[b.p] = b;
       return b.p;
@@ -63,16 +62,11 @@ class DevicePool {
     if (it == live_.end()) return;
     const Block b = it->second;
     live_.erase(it);
-    // Over the bound the largest go: a large block costs least beside the copies that fill it.
-    while (held_ + b.bytes > kMost || free_.size() >= kMostBlocks) {
-      size_t most = free_.size();
-      for (size_t i = 0; i < free_.size(); ++i)
-        if (free_[i].bytes > b.bytes && (most == free_.size() || free_[i].bytes > free_[most].bytes)) most = i;
-      if (most == free_.size()) { cudaFree(p); return; }
-      cudaFree(free_[most].p);
-      held_ -= free_[most].bytes;
-      free_[most] = free_.back();
-      free_.pop_back();
+    if (b.bytes > kMost) { cudaFree(p); return; }
+    while (held_ + b.bytes > kMost || free_.size() >= kMostBlocks) {   // over the bound the oldest go: the next handle is most like the last
+      cudaFree(free_.front().p);
+      held_ -= free_.front().bytes;
+      free_.erase(free_.begin());
     }
     held_ += b.bytes;
     free_.push_back(b);
@@ -91,7 +85,7 @@ class DevicePool {
     held_ = 0;
   }
   std::mutex mu_;
-  std::vector<Block> free_;
+  std::vector<Block> free_;   // in the order they came back
   std::unordered_map<void*, Block> live_;
   size_t held_ = 0;
 };
@@ -683,8 +677,8 @@ aet_status aet_load_client_data(aet_handle* h, uint32_t client, const void* x, c
     auto seen = [](const void* from, size_t bytes) -> const void* {
       cudaPointerAttributes first{}, last{};
       const char* end = static_cast<const char*>(from) + bytes - 1;
-      const bool ok = cudaPointerGetAttributes(&first, from) == cudaSuccess && cudaPointerGetAttributes(&last, end) == cudaSuccess &&
-                      first.type == cudaMemoryTypeHost && last.type == cudaMemoryTypeHost && first.devicePointer && last.devicePointer &&
+      const bool ok = cudaPointerGetAttributes(&first, from) == cudaSuccess && first.type == cudaMemoryTypeHost && first.devicePointer &&
+                      cudaPointerGetAttributes(&last, end) == cudaSuccess && last.type == cudaMemoryTypeHost && last.devicePointer &&
                       static_cast<const char*>(last.devicePointer) - static_cast<const char*>(first.devicePointer) == (ptrdiff_t)bytes - 1;
       cudaGetLastError();
       return ok ? first.devicePointer : nullptr;
