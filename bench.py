@@ -105,21 +105,8 @@ def algorithmic_flops(cfg, samples):
     return per_sample * samples
 
 
-def fp32_fma_peak_tflops():
-    """Plain fp32 FMA peak from the unit counts and the maximum SM clock:
-    148 SMs x 128 fp32 lanes x 2 flops x clock (a register-only FMA loop measured 126 of the
-    128 lanes per clock on this part)."""
-    mhz = 1965.0
-    try:
-        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
-            mhz = float(json.load(f).get("sm_max_mhz", mhz))
-    except Exception:
-        pass
-    return 148 * 128 * 2 * mhz * 1e6 / 1e12, f"derived: 148 SMs x 128 fp32 lanes x 2 x {mhz:.0f} MHz"
-
-
 def regression_flops(cfg, samples):
-    """Softmax regression, batch 1: logits, model update and update sum are one FMA per
+    """Softmax regression, batch 1: logits, model update and update sum are one multiply-add per
     parameter and sample each (the l2 term adds two more per weight)."""
     from paper_2112_13935_b200 import workloads
     P = workloads.n_params(cfg["dims"])
@@ -352,17 +339,16 @@ def measure_device(cfg, steps, warmup, passes_per_step=None, clock_index=None):
         if cfg["precision"] == 1:     # bf16 operands: the dense contraction runs on the tensor cores
             tpeak, tkind = measured_peak_tflops()
             bound = "tensor"
-        else:                         # fp32 model: plain FMAs
-            tpeak, tkind = fp32_fma_peak_tflops()
-            bound = "alu"
+        else:                         # fp32 operands in three bf16 parts: six products on the tensor cores for one
+            tpeak, tkind = measured_peak_tflops()
+            tpeak, tkind = tpeak / 6, tkind + " / 6 (six bf16 products for one of fp32)"
+            bound = "tensor"
         roof = {"bound": bound, "kernel": "local-SGD rounds (MLP)" if cfg["model"] == 1 else "local-SGD rounds (conv)", "achieved": tf, "peak": tpeak,
                 "unit": "TFLOP/s", "frac": tf / tpeak, "traffic": None, "peak_kind": tkind,
                 "hbm_gbs_algorithmic": achieved}
     else:
-        # the batch-1 regression kernel sits on the FMA / HBM ridge: its fp32 FMA rate beside the HBM figure
-        apeak, akind = fp32_fma_peak_tflops()
-        atf = regression_flops(cfg, samples) / (sgd_ms * 1e-3) / 1e12
-        roof.update(alu_tflops=atf, alu_peak=apeak, alu_frac=atf / apeak, alu_peak_kind=akind)
+        # the algorithm's fp32 operations beside the HBM figure (they run on the tensor cores, in two or three parts per operand)
+        roof.update(fp32_tflops=regression_flops(cfg, samples) / (sgd_ms * 1e-3) / 1e12)
     roof.update(launches_per_step=n_sgd_launches, kernel_ms_per_step=sgd_ms,
                 kernel_ms_mode="separate passes with events around every launch: no overlap between a kernel "
                                "and its neighbours, so the sum can exceed the pass it belongs to",

@@ -4,8 +4,9 @@
 // random compute / network delays (Section 3.3.2) without fixing a generator.
 // Here every random quantity is a pure function of (seed, stream, client,
 // counter): the SplitMix64 output function (Steele, Lea, Flood 2014) applied to
-// golden-ratio-spaced inputs.  Delays are integer ticks computed without
-// floating point, so the event order is identical on every machine.
+// golden-ratio-spaced inputs.  Delays are integer ticks defined without
+// floating point, so the event order is identical on every machine; the host's
+// log2 only stands in where its error cannot reach the result (neg_log2_q32).
 #pragma once
 #include <math.h>
 #include <stdint.h>
@@ -47,9 +48,10 @@ AET_HD uint32_t sample_index(uint64_t r, uint32_t n) {
 // -log2(x / 2^64) in Q32, x = r (1 when r == 0): integer part from the leading
 // bit, 32 fraction bits by squaring the Q1.63 mantissa and watching for >= 2.
 //
-// The squaring truncates, so its 32 bits are floor(2^32 (log2 m - d)) with 0 <= d < 2^-61.  A double-precision log2 is
-// within 2^-50 of log2 m, so the same bits follow from it unless 2^32 log2 m lies within 2^-17 of an integer (one draw
-// in 2^16), where the squaring decides.  (About 10 ns instead of 60 ns; the delay draws were most of a first run.)
+// The squaring truncates, so its 32 bits are floor(2^32 (log2 m - d)) with 0 <= d < 2^-61.  A double-precision log2 of m rounded to
+// double is within 2^-50 of log2 m if the libm is within five units of the last place (of values below one, 2^-53; the rounding of m
+// takes 2^-52.4; common libms stay within one), so the same bits follow from it unless 2^32 log2 m lies within 2^-17 of an
+// integer (one draw in 2^16), where the squaring decides.  (About 10 ns instead of 60 ns; the delay draws were most of a first run.)
 inline uint64_t neg_log2_q32(uint64_t r) {
   uint64_t x = r ? r : 1;
   int e = 63 - __builtin_clzll(x);

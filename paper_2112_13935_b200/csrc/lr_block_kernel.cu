@@ -21,11 +21,11 @@
 // most d leaves it within (1 + a)^7 (r / 2) d of the solution, a = max |L| / 2, r = max_t sum_s |L[t][s]|; seven sweeps are
 // always enough.
 //
-// What bounds it: crowded launches run two CTAs per SM (7 MMA warps of 14 k-steps and R, 128 registers), one's R under
-// the other's products: the warp-level tensor pipe (16 instructions of 2 cycles per k-step and 16 samples, 196 cycles per
-// sample and SM).  With one CTA per SM (14 MMA warps of 7 k-steps) it is the chain products -> R -> products.  Measured:
-// ten rounds of 1,024 clients, aggregation included, 1.58 -> 1.08 ms (before: U in tensor memory, operands of the 128-row
-// tcgen05 products staged and split through shared memory for ten rows that matter).
+// What bounds it: latency.  Crowded launches run two CTAs per SM (7 MMA warps of 14 k-steps and R, 128 registers), one's R under
+// the other's products, and rounds of one to ten blocks: start model, first rows and trigger are a third to a half of a launch; the
+// tensor pipe is active 20 to 23 % of it, issue slots 30 %, DRAM at 34 % of the copy rate.  With one CTA per SM (14 MMA warps of 7
+// k-steps) it is the chain products -> R -> products.  Measured: ten rounds of 1,024 clients, aggregation included, 1.58 -> 1.07
+// ms (before: U in tensor memory, operands of the 128-row tcgen05 products staged and split through shared memory for ten rows that matter).
 #include <cuda_runtime.h>
 
 #include "aet_kernels.h"

@@ -37,8 +37,8 @@
 // makes the first i samples exact, so at most fifteen are needed whatever the coupling.
 //
 // What bounds it: the latency of the recurrence, about 330 cycles a sweep.  Measured against eight steps at a time on one
-// CTA, products and recurrence in turn: 16 clients of 29,760 samples in all the rounds 3.40 -> 1.35 ms, 5 clients for 110
-// rounds 20.3 -> 8.1 ms.  Clusters of eight are slower (2.5 ms instead of 1.5: more parts to add, later hand-overs).
+// CTA, products and recurrence in turn: 16 clients of 29,760 samples in all the rounds 3.40 -> 1.39 ms, 5 clients for 110
+// rounds 20.3 -> 8.2 ms.  Clusters of eight are slower (2.5 ms instead of 1.5: more parts to add, later hand-overs).
 #include <cuda_runtime.h>
 
 #include "aet_kernels.h"

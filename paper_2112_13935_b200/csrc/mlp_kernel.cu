@@ -417,10 +417,11 @@ uint32_t mlp_pick_cluster(const MlpShape& shape, uint32_t n_clients) {
 
 cudaError_t launch_mlp_rounds(const MlpLaunch& p, cudaStream_t s) {
   if (p.r.n_tasks == 0) return cudaSuccess;
-  // Streamed where the first layer is 256 wide (64 clients of 3072-256-128-10: 100 ms, 346 on
-  // tcgen05 operand tiles); on the chip wherever a cluster of up to eight holds it (784-100-37-10: 3.0 ms, 9.0 on the general
-  // kernel) - except for calls without a handle (stride 0), whose rows need not lie on 16-byte boundaries; then operand tiles
-  // for tcgen05, then the general kernel.
+  // Streamed where the first layer is 256 wide and its update sum may be derived (64 clients of 3072-256-128-10: 100 ms, 346 on
+  // tcgen05 operand tiles), also where a cluster would hold it (20 iterations of 1024-256-10 at minibatch 64, 8 / 32 / 80 clients:
+  // 0.29 / 0.39 / 1.06 ms, on the chip 0.41 / 1.21 / 2.43; with a second hidden layer 4 to 7 times); on the chip wherever a cluster of up to
+  // eight holds it (784-100-37-10: 3.3 ms, 9.0 on the general kernel) - except for calls without a handle (stride 0), whose rows
+  // need not lie on 16-byte boundaries; then operand tiles for tcgen05, then the general kernel.
   if (mlp_wide_eligible(p.shape)) return launch_mlp_wide_rounds(p, s);
   if (p.r.stride && mlp_mma_eligible(p.shape)) return launch_mlp_mma_rounds(p, s);
   if (mlp_tc_eligible(p.shape)) return launch_mlp_tc_rounds(p, s);

@@ -1,5 +1,6 @@
-// Warp-level tensor-core products of fp32 operands for the round kernels: m16n8k8 tf32 instructions on split
-// operands, and the cluster-scope barrier wrappers the kernels that split one round-task over CTAs use.
+// Warp-level tensor-core products of fp32 operands for the round kernels: m16n8k16 bf16 instructions on operands in three parts,
+// m16n8k8 tf32 instructions on operands in two, and the cluster-scope barrier wrappers the kernels that split one round-task over
+// CTAs use.
 //
 // Why mma.sync here and not tcgen05: the contractions of a batch-1 regression block are 16 samples x 10 classes
 // (and 16 x 16 Gram matrices).  tcgen05 needs M >= 64, its operands in shared memory in both orientations and its
@@ -18,7 +19,8 @@ namespace mma {
 //   split    hi = nearest tf32, lo = the remainder (signed): hi.hi + hi.lo + lo.hi keeps a product to about 2^-22
 //   split_t  hi = v as it stands (its top 19 bits are read), lo = what that leaves out: one logic operation and one
 //            subtraction.  What the product loses of v is below 2^-21 and 2^-23 on average, an fp32 unit in the last place;
-//            used where at most one side of a product is cut this way, or where the result is only a small correction.
+//            used where at most one side of a product is cut this way, or where the result is only a small correction.  The
+//            regression's logits and Gram matrices run on these: errors there move a softmax, not a sum that is kept.
 // Measured: cvt.rna.tf32 costs a scheduler 4 cycles, the logic operation 2; crowded regression rounds spent 45 % of
 // the integer pipe and 44 % of their instructions on the former.
 struct Split { uint32_t hi, lo; };
