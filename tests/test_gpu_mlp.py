@@ -98,9 +98,9 @@ def test_mlp_bf16_tensor_core_path(over):
     print("tensor-core path per-round U errors:", ["%.1e" % v for v in errs])
 
 
-def test_stream_kernel_one_cta_and_pair_instances_agree():
-    # 80 round-tasks in the first wave: more than half the SMs, so the run takes the one-CTA instance of the
-    # streaming kernel; a round restarted on its own takes the pair.  Round 0 starts from w0 on both paths.
+def test_wide_kernel_on_one_cta_and_on_a_cluster_agree():
+    # 80 round-tasks in the first wave: more than half the SMs, so the run takes mlp_wide_kernel with one CTA each; a
+    # round restarted on its own takes a cluster of four.  Round 0 starts from w0 on both paths.
     cfg = workloads.get_config("cfg4", n_clients=80, n_rounds=2, dims=[512, 256, 128, 10], n_stragglers=2,
                                data=dict(kind="iid", total=8000, dim=512))
     data, w0 = make(cfg)
@@ -111,14 +111,14 @@ def test_stream_kernel_one_cta_and_pair_instances_agree():
     first = [e for e in ref["events"] if e["round"] == 0][::16]
     with api.Session(cfg, to_device(data), torch.from_numpy(w0).cuda()) as s:
         for e in first:
-            U_pair, _ = api.aet_debug_run_client_round(s.h, e["client"], 0, w0)
-            assert rel_err(U_pair, gpu["U"][e["seq"]]) <= 2e-6   # same arithmetic; only the first bias gradient is summed in another order
+            U_cluster, _ = api.aet_debug_run_client_round(s.h, e["client"], 0, w0)
+            assert rel_err(U_cluster, gpu["U"][e["seq"]]) <= 2e-6   # same arithmetic; only the first bias gradient is summed in another order
             check_round_U(cfg, data, s.h, e["client"], 0, w0, BF16_U_TOL, **BF16_FLIPS)
 
 
-def test_stream_kernel_runs_are_bit_identical():
-    # pairs of CTAs exchange activations and weights over distributed shared memory under cluster barriers:
-    # a missing barrier would show as run-to-run differences
+def test_wide_kernel_runs_are_bit_identical():
+    # the CTAs of a cluster exchange parts of Z_0 and activations over distributed shared memory, counted by mbarriers: a
+    # missing wait would show as run-to-run differences
     cfg = workloads.get_config("cfg4", n_clients=24, n_rounds=3, dims=[512, 256, 128, 10], n_stragglers=2,
                                data=dict(kind="iid", total=4800, dim=512))
     data, w0 = make(cfg)
