@@ -9,8 +9,10 @@
 //   Z^T = W^T X^T, partial sums to shared memory;            R warp: z, then sweeps z <- z0 + L delta(z) over the eight
 //   the next block's Gram matrix, under R;                   samples at once until they no longer move; delta out;
 //   U^T = q^8 U^T + sum_s q^(7-s) delta_s x_s^T.             biases; row copies two blocks ahead.
-// Products are m16n8k8 tf32 with split operands (mma_common.cuh); with one CTA per SM the update takes operands in three bf16
-// parts instead (a round of 50 samples 1.5e-7 -> 0.6e-7 off fp64, fp32 FMAs 0.7e-7), two pairs of parts per instruction.  With the ten classes on the M side eight samples
+// Products are m16n8k8 tf32 with split operands (mma_common.cuh).  What the update loses stays in U: with one CTA per SM, or with lambda, it
+// takes operands in three bf16 parts instead, two pairs of parts per instruction (a round of 50 samples 1.5e-7 -> 0.6e-7 off
+// fp64, fp32 FMAs 0.7e-7); crowded without lambda both tf32 heads are rounded (0.9e-7; the kernel before 1.1e-7 to 20e-7 by the length
+// of the round; three bf16 parts 0.6e-7, but 1.19 instead of 1.08 ms for 1,024 clients).  With the ten classes on the M side eight samples
 // fill an n-tile of the logits and a k-step of the update exactly, and the accumulator fragment of U^T is the operand
 // fragment of the next logits product when the k index of a step is read as pixel (2t | 2t + 1): U never leaves
 // registers, W = q^n W_start - eta U is formed in place, W_start waits in shared memory in fragment order.  A block's
@@ -23,8 +25,8 @@
 //
 // What bounds it: latency.  Crowded launches run two CTAs per SM (7 MMA warps of 14 k-steps and R, 128 registers), one's R under
 // the other's products, and rounds of one to ten blocks: start model, first rows and trigger are a third to a half of a launch; the
-// tensor pipe is active 20 to 23 % of it, issue slots 30 %, DRAM at 34 % of the copy rate.  With one CTA per SM (14 MMA warps of 7
-// k-steps) it is the chain products -> R -> products.  Measured: ten rounds of 1,024 clients, aggregation included, 1.58 -> 1.07
+// tensor pipe is active 20 to 23 % of it, issue slots 30 %, DRAM at 33 % of the copy rate.  With one CTA per SM (14 MMA warps of 7
+// k-steps) it is the chain products -> R -> products.  Measured: ten rounds of 1,024 clients, aggregation included, 1.58 -> 1.09
 // ms (before: U in tensor memory, operands of the 128-row tcgen05 products staged and split through shared memory for ten rows that matter).
 #include <cuda_runtime.h>
 
@@ -41,6 +43,7 @@ using mma::Parts;
 using mma::parts_t;
 using mma::Split;
 using mma::split;
+using mma::split_r;
 using mma::split_t;
 
 constexpr int kBk = 8;                       // samples per block
@@ -55,7 +58,7 @@ struct Shape {
   static constexpr bool kDecay = DECAY;
   static constexpr int kThreads = (NW + 1) * 32;
   static constexpr int kCtas = NW <= 7 ? 2 : 1;
-  static constexpr bool kParts = kCtas == 1;   // the update's operands in three bf16 parts; otherwise in two tf32 parts
+  static constexpr bool kParts = kCtas == 1 || DECAY;   // the update's operands in three bf16 parts; otherwise in two tf32 parts
   static_assert(NW * KS == kSteps8, "every warp has the same number of k-steps");
   struct __align__(128) Smem {
     float rows[kRing][kBk][kPitch];
@@ -320,15 +323,16 @@ __global__ void __launch_bounds__(S::kThreads, S::kCtas) lr_block_kernel(RoundLa
         const float* xr = &sm.rows[k % kRing][g][8 * k0 + 2 * tt];
         const float* second = two ? reinterpret_cast<const float*>(&sm.ws23[g][k0][tt]) : &sm.rows[k % kRing][g - 2][8 * k0 + 2 * tt];
         const float qs = two ? qw : 1.f;
+        auto sp = [](float v) { return S::kCtas == 1 ? split_r(v) : split_t(v); };   // (5 samples 4.8e-8 -> 4.1e-8 off fp64)
         float zm[4] = {}, zx[4] = {};
 #pragma unroll
         for (int j = 0; j < KS; ++j) {
           const float2 x = *reinterpret_cast<const float2*>(xr + 8 * j);
           const float2 wa = w01[32 * j];
           const float2 wb = *reinterpret_cast<const float2*>(second + 8 * j);
-          const Split a = split_t(x.x), b = split_t(x.y);
-          const Split v0 = split_t(fmaf(neta, U[j][0], decay ? qw * wa.x : wa.x)), v2 = split_t(fmaf(neta, U[j][1], decay ? qw * wa.y : wa.y));
-          const Split v1 = split_t(fmaf(neta, U[j][2], decay ? qs * wb.x : wb.x)), v3 = split_t(fmaf(neta, U[j][3], decay ? qs * wb.y : wb.y));
+          const Split a = sp(x.x), b = sp(x.y);
+          const Split v0 = sp(fmaf(neta, U[j][0], decay ? qw * wa.x : wa.x)), v2 = sp(fmaf(neta, U[j][1], decay ? qw * wa.y : wa.y));
+          const Split v1 = sp(fmaf(neta, U[j][2], decay ? qs * wb.x : wb.x)), v3 = sp(fmaf(neta, U[j][3], decay ? qs * wb.y : wb.y));
           mma::tf32(zm, v0.hi, v1.hi, v2.hi, v3.hi, a.hi, b.hi);
           mma::tf32(zx, v0.lo, v1.lo, v2.lo, v3.lo, a.hi, b.hi);
           mma::tf32(zx, v0.hi, v1.hi, v2.hi, v3.hi, a.lo, b.lo);
@@ -389,7 +393,7 @@ __global__ void __launch_bounds__(S::kThreads, S::kCtas) lr_block_kernel(RoundLa
           const uint32_t l0 = __float_as_uint(l4.x), l1 = __float_as_uint(l4.y), l2 = __float_as_uint(l4.z), l3 = __float_as_uint(l4.w);
 #pragma unroll
           for (int j = 0; j < KS; ++j) {
-            const Split v0 = split_t(xb[8 * j]), v1 = split_t(xb[4 * kPitch + 8 * j]);
+            const Split v0 = split_r(xb[8 * j]), v1 = split_r(xb[4 * kPitch + 8 * j]);
             float d[4] = {};
             mma::tf32(d, l0, l1, l2, l3, v0.hi, v1.hi);
             mma::tf32(d, h0, h1, h2, h3, v0.lo, v1.lo);

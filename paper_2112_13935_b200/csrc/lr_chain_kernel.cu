@@ -23,7 +23,8 @@
 //
 // Logits and Gram matrices are m16n8k8 tf32 products on split operands, the update m16n8k16 bf16 products on operands in three
 // parts (mma_common.cuh): what it loses stays in U, and with tf32 a round of 50 samples was 1.5e-7 off fp64 instead of 0.6e-7
-// (fp32 FMAs 0.7e-7), for 1 to 3 % of the time of few long chains.  U^T[class][pixel] accumulates in the fragment
+// (fp32 FMAs 0.7e-7), for 1 to 3 % of the time of few long chains.  The logits' heads are rounded, not cut: a round of 5 samples
+// 5.1e-8 -> 4.0e-8 (FMAs 4.0e-8 to 4.3e-8), for another percent.  U^T[class][pixel] accumulates in the fragment
 // (class g, pixels 2t, 2t + 1), which is the A fragment of the logits product Z^T = W^T X^T when the k index of a step
 // is read as pixel (2t | 2t + 1): W = q^n W_start - eta U is formed in place.  A block's sum starts from zero and is
 // added to U by an fp32 add, so that the tensor cores' own rounding never accumulates over a round.
@@ -38,7 +39,7 @@
 //
 // What bounds it: the latency of the recurrence, about 330 cycles a sweep.  Measured against eight steps at a time on one
 // CTA, products and recurrence in turn: 16 clients of 29,760 samples in all the rounds 3.40 -> 1.39 ms, 5 clients for 110
-// rounds 20.3 -> 8.2 ms.  Clusters of eight are slower (2.5 ms instead of 1.5: more parts to add, later hand-overs).
+// rounds 20.3 -> 8.3 ms.  Clusters of eight are slower (2.5 ms instead of 1.5: more parts to add, later hand-overs).
 #include <cuda_runtime.h>
 
 #include "aet_kernels.h"
@@ -54,6 +55,7 @@ using mma::Parts;
 using mma::parts;
 using mma::parts_t;
 using mma::Split;
+using mma::split_r;
 using mma::split_t;
 
 constexpr int kB = 16;                       // samples per block
@@ -558,9 +560,9 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
 #pragma unroll
         for (int j = 0; j < KM; ++j) {
           const float2 x0 = *reinterpret_cast<const float2*>(xr + 8 * NM * j), x1 = *reinterpret_cast<const float2*>(xr + 8 * S::kPitch + 8 * NM * j);
-          const Split a = split_t(x0.x), b = split_t(x0.y), c = split_t(x1.x), d = split_t(x1.y);
-          const Split w0 = split_t(fmaf(neta, U[j][0], qw * ws[j][0])), w2 = split_t(fmaf(neta, U[j][1], qw * ws[j][1]));
-          const Split w1 = split_t(fmaf(neta, U[j][2], qw * ws[j][2])), w3 = split_t(fmaf(neta, U[j][3], qw * ws[j][3]));
+          const Split a = split_r(x0.x), b = split_r(x0.y), c = split_r(x1.x), d = split_r(x1.y);
+          const Split w0 = split_r(fmaf(neta, U[j][0], qw * ws[j][0])), w2 = split_r(fmaf(neta, U[j][1], qw * ws[j][1]));
+          const Split w1 = split_r(fmaf(neta, U[j][2], qw * ws[j][2])), w3 = split_r(fmaf(neta, U[j][3], qw * ws[j][3]));
           mma::tf32(zm[0], w0.hi, w1.hi, w2.hi, w3.hi, a.hi, b.hi);
           mma::tf32(zm[1], w0.hi, w1.hi, w2.hi, w3.hi, c.hi, d.hi);
           mma::tf32(zx[0], w0.lo, w1.lo, w2.lo, w3.lo, a.hi, b.hi);

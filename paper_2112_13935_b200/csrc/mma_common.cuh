@@ -19,8 +19,8 @@ namespace mma {
 //   split    hi = nearest tf32, lo = the remainder (signed): hi.hi + hi.lo + lo.hi keeps a product to about 2^-22
 //   split_t  hi = v as it stands (its top 19 bits are read), lo = what that leaves out: one logic operation and one
 //            subtraction.  What the product loses of v is below 2^-21 and 2^-23 on average, an fp32 unit in the last place;
-//            used where at most one side of a product is cut this way, or where the result is only a small correction.  The
-//            regression's logits and Gram matrices run on these: errors there move a softmax, not a sum that is kept.
+//            used for the Gram matrices (small corrections) and the crowded regression's logits: errors there move a softmax, not a
+//            sum that is kept.
 // Measured: cvt.rna.tf32 costs a scheduler 4 cycles, the logic operation 2; crowded regression rounds spent 45 % of
 // the integer pipe and 44 % of their instructions on the former.
 struct Split { uint32_t hi, lo; };
@@ -34,6 +34,13 @@ __device__ __forceinline__ Split split_t(float v) {
   Split s;
   s.hi = __float_as_uint(v);
   s.lo = __float_as_uint(v - __uint_as_float(s.hi & 0xFFFFE000u));
+  return s;
+}
+// as split (ties away from zero), by an addition on the bits: half of the cost of the conversion
+__device__ __forceinline__ Split split_r(float v) {
+  Split s;
+  s.hi = (__float_as_uint(v) + 0x1000u) & 0xFFFFE000u;
+  s.lo = __float_as_uint(v - __uint_as_float(s.hi));
   return s;
 }
 // d[16 x 8] += a[16 x 8] b[8 x 8]; lane = 4 g + t.  a0 (row g, k t), a1 (g + 8, t), a2 (g, t + 4), a3 (g + 8, t + 4);
