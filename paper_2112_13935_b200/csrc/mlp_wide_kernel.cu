@@ -7,7 +7,7 @@
 //
 // A cluster of CL CTAs of 16 warps per round-task; a CTA has a range of the inputs, warp w the hidden units 16 w .. 16 w + 15.
 // One pass over the CTA's inputs, 16 at a time, does the backward product of an iteration and the forward product of the
-// next: the thread fetches its 8 entries of W_0 (two units ahead), forms their gradient dZ_0^T X (m16n8k16, the accumulator
+// next: the thread fetches its 8 entries of W_0 (four units ahead), forms their gradient dZ_0^T X (m16n8k16, the accumulator
 // fragment is the thread's own entries), updates, writes them back and multiplies the new bf16 values - already the operand
 // fragment - with the next minibatch.  No thread waits for another inside a pass but for the input columns: chunks of 32
 // columns of both minibatches come through a ring of three (cp.async, counted by mbarriers).  The master lies in
@@ -23,10 +23,14 @@
 // shapes), W_1's likewise at minibatch 64; at 32 tensor memory holds it, and W_0 streams from its first unit on.  The class layer's and the
 // biases' are accumulated.
 //
-// What bounds it: HBM - W_0 is read and written once per iteration, 6.3 MB per client at D0 = 3072 - as long as the launch has
-// enough clients; with few, the warp-level tensor rate (16 instructions of 8 cycles per 16 x 16 entries and scheduler).
-// Measured: 64 clients of 3072-256-128-10, 30 rounds, 181 -> 100 ms (before: tcgen05 products on bf16 tiles that every
-// iteration rebuilt in shared memory from the same stream), about 5 TB/s of master traffic while a full wave runs.
+// What bounds it: with enough clients the shared memory pipe, busy nine cycles of ten during a pass (every warp reads the fragments of
+// both minibatches' columns: 32 wavefronts per unit; the stream itself takes 16), 1,150 cycles per unit; with few, the warp-level
+// tensor rate (16 instructions of 8 cycles per 16 x 16 entries and scheduler) and the narrow layers.
+// A pass is not bound by HBM any more: W_0 is read and written once per iteration, 6.3 MB per client at D0 = 3072, and since every pass
+// goes the other way round than the one before it a quarter of that stays in L2 (DRAM traffic of two waves 938 -> 706 MB).
+// Measured, 64 clients of 3072-256-128-10, 30 rounds: 103.3 -> 95.8 ms with units four ahead in shared memory for all cluster widths
+// (before: two in registers, fed from two in shared memory, which a unit's wait emptied); tcgen05 products on bf16 tiles
+// that every iteration rebuilt in shared memory from the same stream took 181 ms.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -84,9 +88,10 @@ struct Lay {   // shared memory, in bytes
   // dZ_0, dZ_1, A_1: dead during a pass, whose parts of Z_0 come in there: up to 7 / 8 of 16 tiles of 16 x Bp
   static constexpr int z0 = a0 + Bp * kP0 * 2, z1 = z0 + Bp * kP0 * 2, a1 = z1 + (MID ? Bp * kP1 * 2 : 0), dead_end = a1 + (MID ? Bp * kP1 * 2 : 0);
   static constexpr int in_end = z0 + 14 * BT * 512;
-  static_assert(!MID || BT != 8 || dead_end - z1 >= kWarps * 2048, "two units per warp");
+  static constexpr int kSlots = 4, stage_end = z0 + kSlots * kWarps * 1024;   // units of W_0 on their way in, from z0 on
   static constexpr int part = MID ? z1 : z0;   // the class layer's partial sums: before dZ of the layer below is written
-  static constexpr int w2 = dead_end > in_end ? dead_end : in_end, logit = w2 + 16 * kPw2 * 4, z2 = logit + Bp * 17 * 4;
+  static constexpr int top = dead_end > in_end ? dead_end : in_end;
+  static constexpr int w2 = top > stage_end ? top : stage_end, logit = w2 + 16 * kPw2 * 4, z2 = logit + Bp * 17 * 4;
   static constexpr int bias = z2 + Bp * kPz * 2, ub = bias + kNb * 4, gb = ub + kNb * 4, gb2 = gb + kNb * 4;
   static constexpr int kStage = 2 * Bp * kPx * 2;
   static constexpr bool kSum1 = MID && BT == 4;   // W_1's update sum is accumulated (tensor memory), W_2's lies here
@@ -311,9 +316,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
     }
   };
 
-  // With at most two CTAs the parts of Z_0 leave dZ_1's and A_1's place free during a pass: 2 KB per warp
-  const bool deep = MID && BT == 8 && CL <= 2;
-  float* const deep_at = reinterpret_cast<float*>(smem + M::z1) + warp * 512 + lane * 4;
+  constexpr int kSlots = M::kSlots;
+  float* const slot = reinterpret_cast<float*>(smem + M::z0) + warp * 256 + lane * 4;   // + 4096 per slot
   // One pass over the CTA's inputs.  GRAD: the gradient of iteration itc and the update (otherwise the start model comes
   // in); LOOK: the forward product of iteration itc + 1 and its hand-over (otherwise the update sums go out).
   auto pass = [&](auto grad_, auto look_, int itc) {
@@ -325,49 +329,39 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
       for (int k = 0; k < (GRAD ? KS : 0); ++k)
         ldmatrix4t(a[k], smem_addr(Z0 + (16 * k + (lane >> 4) * 8 + (lane & 7)) * kP0 + 16 * warp + ((lane >> 3) & 1) * 8));
     }
-    if (LOOK && CL > 1) {   // this warp needs nothing any more of what the peers' parts will overwrite
-      __syncwarp();
-      if (lane < CL && lane != rank) mma::arrive_peer(mma::peer_addr(smem_addr(b_free), lane));
-    }
-    // The master two units ahead in registers; with `deep` the two units behind those are on their way into shared memory
-    // (each lane copies and reads its own 32 bytes of a unit).  A group of copies per unit.
-    float4 wb[2][2];
-    auto fetch = [&](int u, float4 (&d)[2]) {
-      const float4* s = reinterpret_cast<const float4*>(master + (size_t)u * (kWarps * 256));
-      d[0] = __ldcg(s);
-      d[1] = __ldcg(s + 32);
-    };
-    auto stage = [&](int u) {
-      const float* s = master + (size_t)u * (kWarps * 256);
-      const uint32_t d = smem_addr(deep_at + (u & 1) * 256);
-      if (u < nu) {
+    // Units of the master on their way into shared memory, kSlots ahead: each lane copies and reads its own 32 bytes of a
+    // unit, a group of copies per unit.
+    // Every pass walks the inputs the other way round than the pass before it: what that one touched last is still in L2.
+    const bool back = GRAD && !(itc & 1);
+    const int lo = back ? 0 : kRes, hi = back ? nu - kRes : nu;   // places in that order whose units stream
+    auto unit = [&](int i) { return back ? nu - 1 - i : i; };
+    auto stage = [&](int i) {
+      const float* s = master + (size_t)unit(i) * (kWarps * 256);
+      const uint32_t d = smem_addr(slot + (i % kSlots) * 4096);
+      if (i < hi) {
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(s) : "memory");
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 512), "l"(s + 128) : "memory");
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    if (GRAD) {
+    if (GRAD) {   // (what the slots lie in)
+      __syncthreads();   // every warp has its fragments of dZ_0 and is done with dZ_1 and A_1
 #pragma unroll
-      for (int j = 0; j < 2; ++j)
-        if (kRes + j < nu) fetch(kRes + j, wb[j]);
-      if (deep) {
-        stage(kRes + 2);
-        stage(kRes + 3);
-      }
+      for (int i = 0; i < kSlots; ++i) stage(lo + i);
     }
 #pragma unroll 1
     for (int c = 0; c < nch; ++c) {
       float sv[GRAD && LOOK ? 1 : 2][8];
       if (!(GRAD && LOOK)) {
 #pragma unroll
-        for (int j = 0; j < 2; ++j) start_words(nat + (size_t)(2 * c + j) * (16 * kH0), kH0, sv[GRAD && LOOK ? 0 : j]);
+        for (int j = 0; j < 2; ++j) start_words(nat + (size_t)unit(2 * c + j) * (16 * kH0), kH0, sv[GRAD && LOOK ? 0 : j]);
       }
       wait(&full[qc % kRing], (qc / kRing) & 1);
       const bf16* xc = ring + (qc % kRing) * 2 * Bp * kPx;
       const bf16* xn = xc + Bp * kPx;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        const int u = 2 * c + j;
+        const int i2 = 2 * c + j, u = unit(i2), col = 16 * (u & 1);
         float w[8];
         if (!GRAD) {
 #pragma unroll
@@ -375,24 +369,19 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
         } else if (u < kRes) {
           own.load(u, w);
         } else {
-          w[0] = wb[j][0].x; w[1] = wb[j][0].y; w[2] = wb[j][0].z; w[3] = wb[j][0].w;
-          w[4] = wb[j][1].x; w[5] = wb[j][1].y; w[6] = wb[j][1].z; w[7] = wb[j][1].w;
-          if (deep) {
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-            const float4* s = reinterpret_cast<const float4*>(deep_at + (u & 1) * 256);
-            wb[j][0] = s[0];
-            wb[j][1] = s[32];
-            stage(u + 4);
-          } else if (u + 2 < nu) {
-            fetch(u + 2, wb[j]);
-          }
+          asm volatile("cp.async.wait_group %0;" ::"n"(kSlots - 1) : "memory");
+          const float4* s = reinterpret_cast<const float4*>(slot + (i2 % kSlots) * 4096);
+          const float4 v0 = s[0], v1 = s[32];
+          w[0] = v0.x; w[1] = v0.y; w[2] = v0.z; w[3] = v0.w;
+          w[4] = v1.x; w[5] = v1.y; w[6] = v1.z; w[7] = v1.w;
+          stage(i2 + kSlots);
         }
         if (GRAD) {
           float gr[2][4] = {};
 #pragma unroll
           for (int k = 0; k < KS; ++k) {
             uint32_t f[4];   // the columns of this unit as second operand, 16 samples
-            ldmatrix4t(f, smem_addr(xc + (16 * k + (lane & 15)) * kPx + 16 * j + (lane >> 4) * 8));
+            ldmatrix4t(f, smem_addr(xc + (16 * k + (lane & 15)) * kPx + col + (lane >> 4) * 8));
             mma_bf16(gr[0], a[GRAD ? k : 0], f[0], f[1]);
             mma_bf16(gr[1], a[GRAD ? k : 0], f[2], f[3]);
           }
@@ -411,7 +400,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
 #pragma unroll
           for (int b = 0; b < BT; b += 2) {
             uint32_t x[4];   // two groups of eight samples
-            ldmatrix4(x, smem_addr(xn + (8 * b + (lane >> 4) * 8 + (lane & 7)) * kPx + 16 * j + ((lane >> 3) & 1) * 8));
+            ldmatrix4(x, smem_addr(xn + (8 * b + (lane >> 4) * 8 + (lane & 7)) * kPx + col + ((lane >> 3) & 1) * 8));
             mma_bf16(acc[LOOK ? b : 0], f, x[0], x[1]);
             mma_bf16(acc[LOOK ? b + 1 : 0], f, x[2], x[3]);
           }
@@ -426,10 +415,14 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
       __syncwarp();
       if (lane == 0) mbar_arrive(&freed[(qc - 1) % kRing]);
       // at the end of a chunk the slot of the one before is free without a wait: every warp is about as far
-      if (c + 2 < nch) issue(c + 2, itc, GRAD, LOOK);
+      if (c + 2 < nch) issue(back ? nch - 3 - c : c + 2, itc, GRAD, LOOK);
     }
     if (!LOOK) return;
     own.store_wait();
+    if (CL > 1) {   // this warp needs nothing any more of what the peers' parts will overwrite
+      __syncwarp();
+      if (lane < CL && lane != rank) mma::arrive_peer(mma::peer_addr(smem_addr(b_free), lane));
+    }
     const uint32_t par = (uint32_t)(itc + 1) & 1;
     if (owner != rank) {
       wait_cluster(b_free, par);
@@ -483,8 +476,9 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
       if (tid == 0 && more) mbar_expect_tx(b_a0, a0_bytes);
     }
     __syncthreads();   // A_0 is complete, the parts of Z_0 have been read
-    issue(0, (int)it, true, more);
-    issue(1, (int)it, true, more);
+    const bool back = !(it & 1);
+    issue(back ? nch - 1 : 0, (int)it, true, more);
+    issue(back ? nch - 2 : 1, (int)it, true, more);
 
     if (MID) {   // A_1 = relu(A_0 W_1 + b_1): a warp has 16 outputs and half of the samples
       float acc[BT / 2][4] = {};
@@ -702,7 +696,6 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
       bias[tid] = fmaf(-eta, gr, bias[tid]);
       ubias[tid] += gr;
     }
-    if (MID) __syncthreads();   // dZ_1 and A_1 have been read
     if (more) pass(Yes(), Yes(), (int)it);
     else pass(Yes(), No(), (int)it);
   }
