@@ -145,14 +145,17 @@ constexpr int kRingThreads = 128;
 // reached it, preceded by the node's own sum of the round it has just finished.  One y-block per node
 // whose model moves; a thread keeps its parameter in a register and walks the node's short list.
 __global__ void __launch_bounds__(kRingThreads) ring_apply_kernel(RingApplyLaunch p) {
+  // (launched as apply_updates_kernel is, and for the same reasons)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const uint32_t j = blockIdx.x * kRingThreads + threadIdx.x;
   if (j >= p.n_params) return;
   const RingApplyDesc a = p.applies[p.lo + blockIdx.y];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   float* wp = p.node_w + (size_t)a.node * p.stride + j;
   float w = *wp;
   for (uint32_t k = 0; k < a.op_cnt; ++k) {
     const RingOp op = p.ops[a.op_off + k];
-    w = fmaf(-op.eta, __ldg(p.U + (size_t)op.u_row * p.stride + j), w);
+    w = fmaf(-op.eta, p.U[(size_t)op.u_row * p.stride + j], w);
   }
   *wp = w;
   if (p.status && !isfinite(w)) atomicOr(p.status, 2u);
@@ -187,8 +190,16 @@ cudaError_t launch_validate_data(const float* x, const int32_t* y, uint32_t n, u
 cudaError_t launch_ring_apply(const RingApplyLaunch& p, cudaStream_t s) {
   if (p.hi <= p.lo) return cudaSuccess;
   const uint32_t blocks = (p.n_params + kRingThreads - 1) / kRingThreads;
-  ring_apply_kernel<<<dim3(blocks, p.hi - p.lo, 1), kRingThreads, 0, s>>>(p);
-  return cudaGetLastError();
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(blocks, p.hi - p.lo, 1);
+  cfg.blockDim = dim3(kRingThreads, 1, 1);
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, ring_apply_kernel, p);
 }
 
 cudaError_t launch_apply_updates(const ApplyLaunch& p0, cudaStream_t s) {

@@ -1,5 +1,5 @@
-// Local-SGD round of one client for softmax regression 784 -> 10, batch 1, for launches with at most one round-task
-// per SM: what counts is the length of a round's chain of dependent steps.
+// Local-SGD round of one client for softmax regression 784 -> 10, batch 1, for launches of 23 to 74 round-tasks, for which there are
+// clusters of four or two but no more: what counts is the length of a round's chain of dependent steps.
 //
 // Algorithm 3, MainComputeNode, inner loop (g = grad f(w_c, xi) + lambda W; w_c -= eta g; U_i += g; h++) sixteen
 // steps at a time.  With q = 1 - eta lambda, W_k, b_k the model at the start of block k and
@@ -37,9 +37,8 @@
 // a = max |L| / 2, r = max_t sum_s |L[t][s]| (the inverse of a unit triangular matrix with entries below a).  Sweep i
 // makes the first i samples exact, so at most fifteen are needed whatever the coupling.
 //
-// What bounds it: the latency of the recurrence, about 330 cycles a sweep.  Measured against eight steps at a time on one
-// CTA, products and recurrence in turn: 16 clients of 29,760 samples in all the rounds 3.40 -> 1.39 ms, 5 clients for 110
-// rounds 20.3 -> 8.3 ms.  Clusters of eight are slower (2.5 ms instead of 1.5: more parts to add, later hand-overs).
+// What bounds it: the latency of the recurrence, about 400 cycles a sweep, and the products' (the two in turn on one SM).  Measured
+// against eight steps at a time on one CTA: rounds of 400 samples, 33 clients 88 instead of 161 us.
 #include <cuda_runtime.h>
 
 #include "aet_kernels.h"
@@ -115,7 +114,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   typename S::Smem& sm = *reinterpret_cast<typename S::Smem*>(smem_raw);
 
-  const TaskDesc t = p.by_value ? p.one_task : p.tasks[p.task_begin + blockIdx.x / CL];
+  const TaskDesc t = p.tasks[p.task_begin + blockIdx.x / CL];
   if (!debug_task_ok(p, t)) return;
   const uint32_t rank = mma::cluster_rank();
   if (t.n_samples == 0) {
@@ -273,11 +272,9 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
     }
   } else if (role == kProd) {
     // ================= producer: rows and labels =================
-    // Inside a handle rows and labels are older than the set-up launch of the run, which lets nothing start early; without
-    // one they are the caller's, whose kernel ahead in the stream may still be writing them.
-    if (p.by_value) asm volatile("griddepcontrol.wait;" ::: "memory");
-    const ClientData cd = p.by_value ? p.one_client : p.clients[t.client];
-    const uint64_t key = p.by_value ? p.one_key : p.sample_keys[t.client];
+    // Rows and labels are older than the set-up launch of the run, which lets nothing start early.
+    const ClientData cd = p.clients[t.client];
+    const uint64_t key = p.sample_keys[t.client];
     const float* xrows = reinterpret_cast<const float*>(cd.x) + 8 * ks0;
     const uint32_t bytes = 32u * cnt;
     for (uint32_t kb = 0; kb < nblk; ++kb) {

@@ -1,8 +1,9 @@
 // Softmax regression 784 -> 10, batch 1: which kernel runs a launch of round-tasks.
 //
-// As long as the device runs a cluster for every round-task at once, the round's serial chain sets the time: four or two CTAs per
-// round-task (lr_chain_kernel.cu).  With more round-tasks than that, a cluster would leave some of them
-// waiting for SMs: one CTA each (lr_block_kernel.cu), and with more round-tasks than SMs its two-per-SM shape.  Rounds of 400
+// As long as the device runs a cluster for every round-task at once, the round's serial chain sets the time: eight or six CTAs per
+// round-task, one of which does nothing but walk it (lr_relay_kernel.cu; up to 22 round-tasks); four or two that do everything
+// alike (lr_chain_kernel.cu; up to 74).  With more round-tasks than that, a cluster would leave some of them waiting for SMs: one CTA each
+// (lr_block_kernel.cu), and with more round-tasks than SMs its two-per-SM shape.  Rounds of 400
 // samples: 33 clients 88 us on four CTAs, 98 on two; 74 clients 113 us on two, 161 on one.
 #include <cuda_runtime.h>
 
@@ -37,14 +38,17 @@ cudaError_t launch_wait_probe(uint32_t* status, uint32_t max_polls, cudaStream_t
 
 cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s) {
   if (p.n_tasks == 0) return cudaSuccess;
-  uint32_t ones = 0, pairs = 0, fours = 0;
+  uint32_t ones = 0, pairs = 0, fours = 0, sixes = 0, eights = 0;
   cudaError_t e = clusters_at_once(1, &ones);
   if (e == cudaSuccess) e = clusters_at_once(2, &pairs);
   if (e == cudaSuccess) e = clusters_at_once(4, &fours);
+  if (e == cudaSuccess) e = clusters_at_once(6, &sixes);
+  if (e == cudaSuccess) e = clusters_at_once(8, &eights);
   if (e != cudaSuccess) return e;
   if (p.n_tasks > ones || p.crowded_hint) return launch_lr_block_rounds(p, true, s);
   if (p.n_tasks > pairs) return launch_lr_block_rounds(p, false, s);
-  return launch_lr_chain_rounds(p, p.n_tasks > fours ? 2 : 4, s);
+  if (p.n_tasks > sixes) return launch_lr_chain_rounds(p, p.n_tasks > fours ? 2 : 4, s);
+  return launch_lr_relay_rounds(p, p.n_tasks > eights ? 6 : 8, s);
 }
 
 }  // namespace aet

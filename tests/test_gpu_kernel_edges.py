@@ -42,6 +42,20 @@ def test_regression_rounds_around_whole_blocks(n_clients, first, l2):
                                data=dict(per_client=40)))
 
 
+# Clusters of eight (up to 15 round-tasks on this part) and of six (up to 22); blocks of sixteen, rings of three and four blocks.
+@pytest.mark.parametrize("n_clients,first,l2", [(1, 16, 0.0), (15, 33, 1e-3), (16, 1, 1e-3), (16, 48, 0.0), (22, 17, 1e-3), (22, 79, 0.0)])
+def test_regression_rounds_of_few_clients(n_clients, first, l2):
+    check(workloads.get_config("cfg5", n_clients=n_clients, n_rounds=3, sched_a=15, sched_b=first, l2=l2, lr=0.03 / n_clients, data=dict(per_client=40)))
+
+
+# A step moves a sample's own logits by eta (|x|^2 + 1), 16 eta and more here: 33 samples carry corrections far beyond the exponential's
+# range, which the walk has to shift out.  The bar: one fp32 rounding (2^-24) per step, each amplified by no more than the softmax's
+# 1/2 x 16 eta per later step that shares its class.
+@pytest.mark.parametrize("n_clients,lr", [(3, 0.2), (3, 2.0), (18, 2.0)])   # (from 20 on the checker's own loss overflows)
+def test_regression_rounds_with_steps_that_swing(n_clients, lr):
+    check(workloads.get_config("cfg5", n_clients=n_clients, n_rounds=1, sched_a=1, sched_b=33, lr=lr, data=dict(per_client=40)))
+
+
 def round_rms(cfg, w0, clients):
     """rms error of the first round's update sums over the rms of the sums, all parameters of `clients` together."""
     data = workloads.make_client_data(cfg)
