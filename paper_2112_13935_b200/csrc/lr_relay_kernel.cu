@@ -25,9 +25,12 @@
 // lr_chain_kernel.cu, where the fragments are the same).  With lambda the kernel carries D = sum_s q^(n-1-s) delta_s x_s;
 // U = D + W_start (1 - q^n) / eta.
 //
-// What bounds it: R, 1,970 of 2,340 cycles a block of sixteen in rounds of hundreds of samples; in short rounds the start (5 us from launch
-// to the first step).  Measured against four CTAs that did everything alike: 5 clients for 110 rounds on the ring 8.27 -> 6.22 ms, 16
-// skewed clients 1.39 -> 1.28 ms, one round of 50 samples 13.1 -> 11.2 us.
+// What bounds it: R, 1,970 of 2,340 cycles a block of sixteen in rounds of hundreds of samples; in short rounds the way from one wave to the
+// next (from R's last step to the next wave's first 9 us: end of the round 2, server's kernel 5, start model and first logits 2).  The
+// next kernel may come up four blocks before a round's end, so that its rows and Gram matrices are ready when the model is (from then to
+// the first step 3.0 -> 1.5 us; 16 clients 1.28 -> 1.20 ms, ring 6.22 -> 6.12).
+// Measured against four CTAs that did everything alike: 5 clients for 110 rounds on the ring 8.27 -> 6.12 ms, 16 skewed clients
+// 1.39 -> 1.20 ms, 4 clients with l2 92 -> 82 us, one round of 50 samples 13.1 -> 10.9 us.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -63,6 +66,7 @@ constexpr int kNg = 11;                      // Gram warps of a CTA
 constexpr int kNgEven = kNg / 2;             // the first of them add up the parts of even blocks, the others those of odd ones
 constexpr int kNs = 4;                       // blocks of rows
 constexpr int kInZ = 4, kInG = 4, kCoups = 3;   // rings: logits, couplings as they come in; couplings summed
+constexpr uint32_t kEarly = 4;               // blocks before a round's end at which the next kernel may come up
 constexpr int kWarps = 12, kThreads = kWarps * 32;
 // Corrections move a logit by at most 31 max |L|; below this they cannot leave the range of the exponential.
 constexpr float kTame = 1.9f;
@@ -203,6 +207,10 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
   bool ok = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok) ok = mbar_wait(bar, parity); };
   const float scale = neta * kLog2e;
+  // The kernel behind this one may come up while the last blocks are walked: what it does before its own wait, it does with what the
+  // host wrote (and the kernel behind it, in turn: a round's rows, their Gram matrices).
+  auto launch_next = []() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); };
+  const uint32_t early = nblk > kEarly ? nblk - kEarly : 0;
 
   if (walks && warp == 0) {
     // ================= R: the recurrence, step by step; lane = (half, class) =================
@@ -216,6 +224,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       const int b = k & 1;
       const uint32_t nv = min((uint32_t)kB, n - k * kB);
       const bool mine = half == b, tells = mine && c < kC;   // (the lanes without a class keep zeros)
+      if (k == early) launch_next();
       if (k == 0) wait(&sm.rg[0], 0);
       const bool next = k + 1 < nblk;
       if (next) wait(&sm.rg[(k + 1) & 3], ((k + 1) >> 2) & 1);
@@ -295,7 +304,6 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       if (lane == 0) mbar_arrive(&sm.done[b]);
       others();
     }
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   } else if (walks && warp == 1) {
     // ================= the block's deltas, from R's exponentials, to the CTAs with the model; lane = (class half, sample) =================
     const int s = lane & 15, h = lane >> 4;
@@ -492,6 +500,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
     const int g = lane >> 2, tt = lane & 3;
     float* const gpart = &sm.g.part[0][0][0];
     const uint32_t grank = rank - MC;
+    launch_next();
     Split pv[KG][4];   // the rows of the block before, split
     for (uint32_t kb = 0; kb < nblk; ++kb) {
       wait(&sm.full[kb % NS], (kb / NS) & 1);
@@ -578,7 +587,6 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
                   mma::peer_addr(smem_addr(&sm.bg[ig]), kWalker));
       }
     }
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   } else if (models && warp < NM) {
     // ================= model warps; lane = 4 g + tt =================
     const int g = lane >> 2, tt = lane & 3;
@@ -618,6 +626,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
 
     // block kb's logits follow the update by block kb - 2: everything R needs is one block ahead of it
     for (uint32_t kb = 0; kb < nblk + 2; ++kb) {
+      if (kb == early) launch_next();
       const bool update = kb >= 2, look = kb < nblk;
       const uint32_t k = update ? kb - 2 : 0, nv = min((uint32_t)kB, n - k * kB);
       // the rows of block k as the update's second operand ([sample][pixel], pixel g of the warp's k-steps), and those of block kb
@@ -736,7 +745,6 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
     }
 
     // ---- event trigger: h reached s_{i,c}; publish U_i (and the end model) ----
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     {
       // a round whose copies never came leaves NaN behind, for callers that have no status word to look at
       const float bad = ok ? 0.f : __int_as_float(0x7FFFFFFF);
