@@ -50,7 +50,7 @@ struct RoundLaunch {
   float l2;
 };
 
-// How many clusters of 1, 2, 4, 6 or 8 CTAs with an SM each the current device runs at once (see device_info.cu).
+// How many clusters of 1 to 8 CTAs with an SM each the current device runs at once (see device_info.cu).
 cudaError_t clusters_at_once(uint32_t cluster, uint32_t* out);
 
 // One CTA waits (at most max_polls polls) on a barrier nobody signals, then sets bit 0 of *status.

@@ -1,6 +1,6 @@
 // What the launch rules need to know about the current device: how many SMs it has, and how many clusters of one CTA per SM
 // it runs at once.  Clusters do not straddle GPCs, and GPCs differ in the SMs they have left, so the second does not follow from the
-// first: 148 SMs hold 74 clusters of two, 33 of four (not 37), 22 of six and 15 of eight (not 18); a launch of one more runs as two waves.
+// first: 148 SMs hold 74 clusters of two, 45 of three, 33 of four (not 37), 26 of five, 22 of six, and 15 of seven or eight (not 21 and 18); a launch of one more runs as two waves.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -17,8 +17,8 @@ __global__ void __launch_bounds__(kThreads, 1) whole_sm_kernel(float* p) {   // 
   if (p) p[threadIdx.x] = s[threadIdx.x];
 }
 
-// [device][1, 2, 4, 6 or 8 CTAs]; 0: not asked yet.  Two host threads may ask at once and store the same value.
-std::atomic<uint32_t> g_fit[kMaxDevices][5] = {};
+// [device][CTAs]; 0: not asked yet.  Two host threads may ask at once and store the same value.
+std::atomic<uint32_t> g_fit[kMaxDevices][9] = {};
 
 }  // namespace
 
@@ -26,8 +26,8 @@ cudaError_t clusters_at_once(uint32_t cluster, uint32_t* out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const int slot = cluster == 1 ? 0 : cluster == 2 ? 1 : cluster == 4 ? 2 : cluster == 6 ? 3 : 4;
-  std::atomic<uint32_t>* known = dev >= 0 && dev < kMaxDevices ? &g_fit[dev][slot] : nullptr;
+  if (cluster < 1 || cluster > 8) return cudaErrorInvalidValue;
+  std::atomic<uint32_t>* known = dev >= 0 && dev < kMaxDevices ? &g_fit[dev][cluster] : nullptr;
   uint32_t n = known ? known->load(std::memory_order_relaxed) : 0;
   if (!n) {
     int v = 0;

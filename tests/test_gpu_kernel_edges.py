@@ -96,6 +96,16 @@ def test_fp32_mlp_rounds(dims, batch, n_clients):
                                data=dict(total=70 * n_clients, dim=dims[0])))
 
 
+# Clusters of seven, six, five and three: units of inputs, and groups of hidden rows, that do not come out even.
+@pytest.mark.parametrize("dims,batch,n_clients,bf16", [
+    ([784, 112, 10], 24, 12, False), ([784, 128, 10], 32, 20, False), ([770, 17, 10], 8, 24, False), ([784, 128, 10], 16, 44, False),
+    ([200, 100, 10], 32, 12, True), ([112, 64, 10], 32, 24, True), ([784, 128, 10], 32, 44, True),
+])
+def test_mlp_rounds_on_clusters_that_are_no_powers_of_two(dims, batch, n_clients, bf16):
+    check(workloads.get_config("cfg4" if bf16 else "cfg3", n_clients=n_clients, n_rounds=2, dims=dims, batch=batch, sched_a=batch, sched_b=batch, l2=1e-3,
+                               n_stragglers=0, data=dict(kind="iid", total=70 * n_clients, dim=dims[0])), bf16=bf16)
+
+
 @pytest.mark.parametrize("dims,batch,n_clients", [
     ([512, 256, 10], 16, 4), ([520, 100, 30, 10], 48, 4), ([200, 17, 10], 33, 20), ([1024, 64, 16], 64, 80),   # first layer on the chip
     ([1024, 256, 128, 10], 64, 4), ([512, 256, 128, 10], 64, 20), ([512, 256, 128, 10], 64, 50), ([160, 256, 128, 16], 64, 90),
