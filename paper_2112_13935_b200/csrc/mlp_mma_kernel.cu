@@ -246,34 +246,23 @@ template <int NP> __device__ __forceinline__ void load_wt(FragA<NP>& f, const fl
 }
 // Second operand from samples [sample][k], column = sample g
 template <int NP> __device__ __forceinline__ void load_s(FragB<NP>& f, const T* x, int plane, int pitch, int lane) {
-  if constexpr (NP == 1) {
-    const T* p = x + (lane >> 2) * pitch + 2 * (lane & 3);
-    f.v[0][0] = *reinterpret_cast<const uint32_t*>(p);
-    f.v[0][1] = *reinterpret_cast<const uint32_t*>(p + 8);
-  } else {
-    const uint32_t at = smem_addr(x + (lane & 7) * pitch + (lane & 8));
+  const uint32_t at = smem_addr(x + (lane & 7) * pitch + (lane & 8));
 #pragma unroll
-    for (int q = 0; q < NP; ++q) ldmatrix2(f.v[q], at + 2u * q * plane);
-  }
+  for (int q = 0; q < NP; ++q) ldmatrix2(f.v[q], at + 2u * q * plane);
 }
 // ... N tiles of eight samples
 template <int NP, int N> __device__ __forceinline__ void load_sn(FragB<NP> (&f)[N], const T* x, int plane, int pitch, int lane) {
-  if constexpr (NP == 1) {
 #pragma unroll
-    for (int b = 0; b < N; ++b) load_s(f[b], x + 8 * b * pitch, plane, pitch, lane);
-  } else {
+  for (int b = 0; b + 1 < N; b += 2) {
+    const uint32_t at = smem_addr(x + (8 * b + (lane >> 4) * 8 + (lane & 7)) * pitch + (lane & 8));
 #pragma unroll
-    for (int b = 0; b + 1 < N; b += 2) {
-      const uint32_t at = smem_addr(x + (8 * b + (lane >> 4) * 8 + (lane & 7)) * pitch + (lane & 8));
-#pragma unroll
-      for (int q = 0; q < NP; ++q) {
-        uint32_t r[4];
-        ldmatrix4(r, at + 2u * q * plane);
-        f[b].v[q][0] = r[0]; f[b].v[q][1] = r[1]; f[b + 1].v[q][0] = r[2]; f[b + 1].v[q][1] = r[3];
-      }
+    for (int q = 0; q < NP; ++q) {
+      uint32_t r[4];
+      ldmatrix4(r, at + 2u * q * plane);
+      f[b].v[q][0] = r[0]; f[b].v[q][1] = r[1]; f[b + 1].v[q][0] = r[2]; f[b + 1].v[q][1] = r[3];
     }
-    if (N % 2) load_s(f[N - 1], x + 8 * (N - 1) * pitch, plane, pitch, lane);
   }
+  if (N % 2) load_s(f[N - 1], x + 8 * (N - 1) * pitch, plane, pitch, lane);
 }
 // Second operand from an array [sample][n], k = sample, column = n
 template <int NP> __device__ __forceinline__ void load_st(FragB<NP>& f, const T* x, int plane, int pitch, int lane) {
