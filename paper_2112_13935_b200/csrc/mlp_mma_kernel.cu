@@ -412,11 +412,6 @@ struct Own {
   __device__ __forceinline__ void store_wait() const { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 };
 
-__device__ __forceinline__ void send2(uint32_t addr, uint32_t a, uint32_t b, uint32_t bar) {   // 8 bytes to a peer
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
-               ::"r"(addr), "r"(a), "r"(b), "r"(bar) : "memory");
-}
-
 // n / d for 0 <= n < 2^13 by a multiplication with ceil(2^20 / d) (d <= 128: exact); a hardware division of integers is
 // some twenty dependent instructions, and every phase of the narrow layers needs a few
 __device__ __forceinline__ int div20(int n, int inv) { return (int)(((uint32_t)n * (uint32_t)inv) >> 20); }
@@ -682,7 +677,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     row_at = mma::peer_addr(smem_addr(inbox + ((int)rank * m.rgs * 8 + (rg % m.rgs) * 8 + g) * Bp + 4 * (tt >> 1)), to);
     row_bar = mma::peer_addr(smem_addr(&bars[0]), to);
   }
-  const int own_q = tid / Bp, own_b = tid - own_q * Bp;   // this thread's four owned rows and sample in step 2
+  const int own_q = tid / Bp, own_b = tid - own_q * Bp;   // this thread's owned rows and sample in step 2
 
   float acc[BT][4], crs[BT][4];   // this warp's part of Z_0^T; (fp32) the cross terms
   auto clear = [&]() {
@@ -788,32 +783,45 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     if (nrg > 0) {
       wait(&bars[0], it & 1);
       if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[0], in_bytes);
+      // (without hidden layers these are the logits: fp32 whatever the operands.)  A lane's words are a packet to each peer, and
+      // packets are what a hand-over takes its time for: 16 bytes each, four rows of a sample or eight in bf16.
+      constexpr int kRows = BF ? 8 : 4;
+      const uint32_t bar = smem_addr(&bars[1]);
       int q = own_q, b = own_b;
 #pragma unroll 1
-      for (int e = tid; e < nrg * 2 * Bp; e += kThreads) {
+      for (int e = tid; e < nrg * (8 / kRows) * Bp; e += kThreads) {
         if (e >= kThreads) { q = e / Bp; b = e - q * Bp; }
-        const int n = 8 * rg0 + 4 * q;
-        const float4 b4 = *reinterpret_cast<const float4*>(bias + n);
-        float v[4] = {b4.x, b4.y, b4.z, b4.w};
-        const float* in = inbox + 4 * q * Bp + b;
+        const int n = 8 * rg0 + kRows * q;
+        float v[kRows];
+#pragma unroll
+        for (int i = 0; i < kRows; i += 4) {
+          const float4 b4 = *reinterpret_cast<const float4*>(bias + n + i);
+          v[i] = b4.x; v[i + 1] = b4.y; v[i + 2] = b4.z; v[i + 3] = b4.w;
+        }
+        const float* in = inbox + kRows * q * Bp + b;
 #pragma unroll 4
         for (int r = 0; r < CL; ++r, in += m.rgs * 8 * Bp)
 #pragma unroll
-          for (int i = 0; i < 4; ++i) v[i] += in[i * Bp];
+          for (int i = 0; i < kRows; ++i) v[i] += in[i * Bp];
         if (nl > 1) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) v[i] = fmaxf(v[i], 0.f);
+          for (int i = 0; i < kRows; ++i) v[i] = fmaxf(v[i], 0.f);
         }
-        // (without hidden layers these are the logits: fp32 whatever the operands)
-        const uint32_t bar = smem_addr(&bars[1]);
         if (BF && nl > 1) {
-          const uint32_t at = smem_addr(A(0) + b * m.ap[0] + n), lo = pack_bf16(v[0], v[1]), hi = pack_bf16(v[2], v[3]);
+          const uint32_t at = smem_addr(A(0) + b * m.ap[0] + n);
+          uint32_t w[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) w[i] = pack_bf16(v[(2 * i) % kRows], v[(2 * i + 1) % kRows]);
 #pragma unroll 1
-          for (int r = 0; r < CL; ++r) send2(mma::peer_addr(at, r), lo, hi, mma::peer_addr(bar, r));
+          for (int r = 0; r < CL; ++r)
+            mma::send_peer(mma::peer_addr(at, r), make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3])), mma::peer_addr(bar, r));
         } else {
-          const uint32_t at = smem_addr(smem + m.o_a[0] + b * m.ap[0] + n);
+#pragma unroll
+          for (int i = 0; i < kRows; i += 4) {
+            const uint32_t at = smem_addr(smem + m.o_a[0] + b * m.ap[0] + n + i);
 #pragma unroll 1
-          for (int r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(at, r), make_float4(v[0], v[1], v[2], v[3]), mma::peer_addr(bar, r));
+            for (int r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(at, r), make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]), mma::peer_addr(bar, r));
+          }
         }
       }
     }
