@@ -388,6 +388,12 @@ aet_status read_model(aet_handle* h, const float* src, float* out, cudaStream_t 
   return AET_OK;
 }
 
+uint32_t longest_round(const TaskDesc* t, uint32_t n) {   // (the kernels' choice asks for it where there are few)
+  uint32_t most = 0;
+  for (uint32_t i = 0; n <= 32 && i < n; ++i) most = std::max(most, t[i].n_samples);
+  return most;
+}
+
 aet_status launch_rounds(aet_handle* h, const RoundLaunch& r, cudaStream_t s) {
   KernelTimer kt(h, s, 0);
   cudaError_t e;
@@ -485,6 +491,7 @@ aet_status run_ring_rounds(aet_handle* h, uint32_t n_rounds, cudaStream_t s) {
     if (L == n_waves) break;
     r.task_begin = plan.wave_off[L];
     r.n_tasks = plan.wave_off[L + 1] - plan.wave_off[L];
+    r.longest = longest_round(plan.tasks.data() + r.task_begin, r.n_tasks);
     aet_status rs = launch_rounds(h, r, s);
     if (rs != AET_OK) return rs;
   }
@@ -802,6 +809,7 @@ aet_status aet_run_rounds(aet_handle* h, uint32_t n_rounds, void* cuda_stream) {
   for (uint32_t L = 0; L < n_waves; ++L) {
     r.task_begin = plan.wave_off[L];
     r.n_tasks = plan.wave_off[L + 1] - plan.wave_off[L];
+    r.longest = longest_round(plan.tasks.data() + r.task_begin, r.n_tasks);
     aet_status rs = launch_rounds(h, r, s);
     if (rs != AET_OK) return rs;
     if (plan.apply_upto[L] > applied) {

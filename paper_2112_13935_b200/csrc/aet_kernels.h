@@ -37,6 +37,7 @@ struct RoundLaunch {
   uint32_t debug_checks;         // non-zero: sample indices and row numbers are range-checked before use
   size_t stride;
   uint32_t task_begin, n_tasks;
+  uint32_t longest;              // samples of the longest round-task of a launch of few (0: many, or not known)
   uint32_t n_u_rows, n_snap;     // extents of U and snaps (for the debug checks)
   uint32_t crowded_hint;         // non-zero: pick the kernel a full wave of this run's clients would get,
                                  // however few tasks this launch holds (single-task parity runs)

@@ -1,5 +1,5 @@
-// Local-SGD round of one client for softmax regression 784 -> 10, batch 1, for launches of 23 to 74 round-tasks, for which there are
-// clusters of four or two but no more: what counts is the length of a round's chain of dependent steps.
+// Local-SGD round of one client for softmax regression 784 -> 10, batch 1, for launches of 16 to 74 round-tasks that lr_relay_kernel.cu
+// does not take: what counts is the length of a round's chain of dependent steps.
 //
 // Algorithm 3, MainComputeNode, inner loop (g = grad f(w_c, xi) + lambda W; w_c -= eta g; U_i += g; h++) sixteen
 // steps at a time.  With q = 1 - eta lambda, W_k, b_k the model at the start of block k and

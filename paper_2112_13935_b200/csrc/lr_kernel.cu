@@ -1,8 +1,9 @@
 // Softmax regression 784 -> 10, batch 1: which kernel runs a launch of round-tasks.
 //
 // As long as the device runs a cluster for every round-task at once, the round's serial chain sets the time: eight or six CTAs per
-// round-task, one of which does nothing but walk it (lr_relay_kernel.cu; up to 22 round-tasks); four or two that do everything
-// alike (lr_chain_kernel.cu; up to 74).  With more round-tasks than that, a cluster would leave some of them waiting for SMs: one CTA each
+// round-task, one of which does nothing but walk it (lr_relay_kernel.cu; up to 15 round-tasks, and up to 22 with rounds above 64 samples:
+// 16 clients, three rounds of 32 / 64 / 128 / 400 samples each 54 / 63 / 66 / 142 us on six, 45 to 53 / 59 to 72 / 70 to 84 / 164 to 195 on four, by
+// the step size); four or two that do everything alike (lr_chain_kernel.cu; up to 74).  With more round-tasks than that, a cluster would leave some of them waiting for SMs: one CTA each
 // (lr_block_kernel.cu), and with more round-tasks than SMs its two-per-SM shape.  Rounds of 400
 // samples: 33 clients 88 us on four CTAs, 98 on two; 74 clients 113 us on two, 161 on one.
 #include <cuda_runtime.h>
@@ -47,8 +48,9 @@ cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   if (p.n_tasks > ones || p.crowded_hint) return launch_lr_block_rounds(p, true, s);
   if (p.n_tasks > pairs) return launch_lr_block_rounds(p, false, s);
-  if (p.n_tasks > sixes) return launch_lr_chain_rounds(p, p.n_tasks > fours ? 2 : 4, s);
-  return launch_lr_relay_rounds(p, p.n_tasks > eights ? 6 : 8, s);
+  const bool six = p.n_tasks > eights && p.n_tasks <= sixes && p.longest > 64;
+  if (p.n_tasks > eights && !six) return launch_lr_chain_rounds(p, p.n_tasks > fours ? 2 : 4, s);
+  return launch_lr_relay_rounds(p, six ? 6 : 8, s);
 }
 
 }  // namespace aet
