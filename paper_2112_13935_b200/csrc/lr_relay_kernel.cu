@@ -64,6 +64,7 @@ constexpr uint32_t kSendG0 = 8 * 64, kSendG = kSendG0 + 8 * 128;
 constexpr uint32_t kSendD = 3 * kC * 8 * 4;  // ... and the walker about a block's deltas: three planes of [class][pair of samples]
 constexpr int kNg = 11;                      // Gram warps of a CTA
 constexpr int kNgEven = kNg / 2;             // the first of them add up the parts of even blocks, the others those of odd ones
+constexpr int kGramParts = 3;                // blocks of Gram parts not yet added up (two are too few: see where they are)
 constexpr int kNs = 4;                       // blocks of rows
 constexpr int kInZ = 4, kInG = 4, kCoups = 3;   // rings: logits, couplings as they come in; couplings summed
 constexpr uint32_t kEarly = 4;               // blocks before a round's end at which the next kernel may come up
@@ -87,7 +88,7 @@ struct Shape {
   };
   struct Gram {
     float rows[kNs][kB][kPitchG];
-    float part[2][kNg][kCoup];
+    float part[kGramParts][kNg][kCoup];
   };
   struct Walk {
     float zin[kInZ][MC][kZ], gin[kInG][GC][kCoup];   // per CTA, as they come in
@@ -529,7 +530,8 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.freed[kb % NS]);
-      float* part = gpart + ((kb & 1) * NG + warp) * kCoup;
+      float* const block = gpart + (int)(kb % kGramParts) * NG * kCoup;
+      float* part = block + warp * kCoup;
 #pragma unroll
       for (int m = 0; m < 2; ++m)
 #pragma unroll
@@ -542,7 +544,9 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
               make_float2(hh[m][2 * r2] + cx[m][2 * r2], hh[m][2 * r2 + 1] + cx[m][2 * r2 + 1]);
         }
       // Half of the warps add up a block's parts while the others are at the next block's products: they only say that theirs are
-      // there.  (A barrier per parity.  Every warp waits at one of two blocks: it overwrites no parts that are still being read.)
+      // there.  A barrier per parity.  A warp that writes block kb has waited at kb - 1 or at kb - 2, whichever its half adds up, and every
+      // warp arrives there behind its sums of block kb - 3: those have been read.  The sums of kb - 2 may not have been: warps of one half
+      // do not wait for one another between two of their blocks.  Hence three buffers, not two.
       const int first = kb & 1 ? kNgEven : 0, sums = kb & 1 ? NG - kNgEven : kNgEven;
       if (warp < first || warp >= first + sums) {
         asm volatile("bar.arrive %0, %1;" ::"r"(2 + (kb & 1)), "n"(NG * 32) : "memory");
@@ -564,7 +568,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
         } else {
           tr = (e - 64) >> 3; s0 = 2 * (e & 7);
         }
-        const float* from = gpart + (kb & 1) * NG * kCoup + (own ? 0 : kOffC) + tr * kGp + s0;
+        const float* from = block + (own ? 0 : kOffC) + tr * kGp + s0;
         float v0 = 0.f, v1 = 0.f;
 #pragma unroll
         for (int w = 0; w < NG; ++w) {
@@ -572,7 +576,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
           v0 += x.x; v1 += x.y;
         }
         if (own) {
-          const float* up = gpart + (kb & 1) * NG * kCoup + s0 * kGp + tr;
+          const float* up = block + s0 * kGp + tr;
 #pragma unroll
           for (int w = 0; w < NG; ++w) { v0 += up[w * kCoup]; v1 += up[w * kCoup + kGp]; }
         }

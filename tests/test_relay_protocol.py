@@ -1,0 +1,57 @@
+"""The hand-overs inside the regression's relay kernel, checked as a protocol on the CPU with the constants of its source."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2112_13935_b200", "csrc")
+
+
+def source(name="lr_relay_kernel.cu"):
+    return open(os.path.join(CSRC, name)).read()
+
+
+def constant(name):
+    return int(re.search(r"constexpr int (?:.*, )?%s = (\d+)" % name, source()).group(1))
+
+
+def gram_races(warps, buffers, blocks=9):
+    """(reader, writer, block) where a warp may write its part of a block over parts another one still adds up.
+
+    Per block kb a warp writes part [kb % buffers], arrives at the barrier of kb's parity and, if its half adds up blocks of that
+    parity, waits there and then reads the parts of all warps."""
+    half = warps // 2
+    sums = [[w for w in range(warps) if (w < half) == (kb % 2 == 0)] for kb in range(blocks)]
+    steps = [[(kind, kb) for kb in range(blocks) for kind in ("write", "arrive") + (("read",) if w in sums[kb] else ())]
+             for w in range(warps)]
+    before = {}    # (warp, step): the steps it must follow
+    for w in range(warps):
+        for a, b in zip(steps[w], steps[w][1:]):
+            before.setdefault((w, b), []).append((w, a))
+    for kb in range(blocks):
+        for w in sums[kb]:
+            before.setdefault((w, ("read", kb)), []).extend((v, ("arrive", kb)) for v in range(warps))
+
+    def follows(node, seen):
+        for p in before.get(node, ()):
+            if p not in seen:
+                seen.add(p)
+                follows(p, seen)
+        return seen
+
+    races = []
+    for w in range(warps):
+        for kb in range(buffers, blocks):
+            past = follows((w, ("write", kb)), set())
+            races += [(r, w, kb) for r in sums[kb - buffers] if (r, ("read", kb - buffers)) not in past and r != w]
+        for kb in range(2, blocks):   # a barrier is not entered again before the last use of it is complete
+            past = follows((w, ("arrive", kb)), set())
+            assert all((v, ("arrive", kb - 2)) in past for v in range(warps) if v != w)
+    return races
+
+
+def test_gram_parts_are_read_before_they_are_written_over():
+    warps = constant("kNg")
+    assert gram_races(warps, 2)                              # two buffers: nothing holds a warp of the half that adds up
+    assert not gram_races(warps, constant("kGramParts"))
+    assert "part[kGramParts][kNg][kCoup]" in source()
