@@ -116,11 +116,6 @@ __device__ __forceinline__ float sum_of(float4 a, float4 b, float2 c) { return (
 __device__ __forceinline__ void send_pair(uint32_t addr, float a, float b, uint32_t bar) {   // 8 bytes to a peer
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(a), "f"(b), "r"(bar) : "memory");
 }
-// Nothing but reads goes before it, and their values have been used: a release at cluster scope, which waits for all of the warp's
-// memory operations, is not needed.
-__device__ __forceinline__ void arrive_peer_relaxed(uint32_t bar) {
-  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ void send_quad(uint32_t addr, uint4 v, uint32_t bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
                ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
@@ -207,6 +202,10 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
   // word is set, and every CTA of the cluster reaches the end.
   bool ok = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok) ok = mbar_wait(bar, parity); };
+  auto wait_peer = [&](uint64_t* bar, uint32_t parity) {   // for what peers sent, or have taken
+    const uint32_t at = smem_addr(bar);
+    for (uint32_t i = 0; ok && !mma::try_wait_cluster(at, parity); ++i) ok = i < kWaitLimit;
+  };
   const float scale = neta * kLog2e;
   // The kernel behind this one may come up while the last blocks are walked: what it does before its own wait, it does with what the
   // host wrote (and the kernel behind it, in turn: a round's rows, their Gram matrices).
@@ -378,7 +377,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       if (lane < kB) sm.w.hot[k & 7][lane] = hot;
       if (k + 1 < nblk) y = label(k + 1);
       const int ig = k % kInG, s = lane & 15;
-      wait(&sm.bg[ig], (k / kInG) & 1);
+      wait_peer(&sm.bg[ig], (k / kInG) & 1);
       if (k >= kCoups) wait(&sm.done[(k - kCoups) & 1], ((k - kCoups) >> 1) & 1);   // R is done with block k - 3, whose place this is
       float* out = sm.w.coup[k % kCoups];
       const float* in = &sm.w.gin[ig][0][0];
@@ -407,7 +406,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.rg[k & 3]);
       if (lane < GC && k + kInG < nblk)   // the CTAs that sent them may send block k + 4
-        arrive_peer_relaxed(mma::peer_addr(smem_addr(&sm.gfree[ig]), MC + lane));
+        mma::arrive_peer(mma::peer_addr(smem_addr(&sm.gfree[ig]), MC + lane));
     }
   } else if (walks && warp == 3) {
     // ================= logits: the CTAs' parts in rank order, and the biases =================
@@ -436,7 +435,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
 #pragma unroll
         for (int i = 0; i < kCh; ++i) bk[i] = kLog2e * fmaf(neta, sm.w.ub[b][h * kCh + i], b0[i]);
       }
-      wait(&sm.bz[iz], (k / kInZ) & 1);
+      wait_peer(&sm.bz[iz], (k / kInZ) & 1);
       const float* in = &sm.w.zin[iz][0][h * kCh * kB + s];
       float v[kCh];   // five classes of a sample
 #pragma unroll
@@ -557,7 +556,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       const int ig = kb % kInG;
       const float one = grank == 0 ? scale : 0.f;   // the bias input's part of a coupling
       // two entries per thread: 64 pairs that reach below the diagonal, 128 of the matrix to the block before
-      if (kb >= kInG) wait(&sm.gfree[ig], (kb / kInG - 1) & 1);   // the walker has taken block kb - 4
+      if (kb >= kInG) wait_peer(&sm.gfree[ig], (kb / kInG - 1) & 1);   // the walker has taken block kb - 4
       for (int e = (warp - first) * 32 + lane; e < (kb ? 192 : 64); e += sums * 32) {
         const bool own = e < 64;
         int tr, s0;
@@ -660,7 +659,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       }
       if (update) {
         // ---- U^T = q^nv U^T + sum_s q^(nv-1-s) delta_s x_s; the k index of the product is read as samples t, t + 4, t + 8, t + 12 ----
-        wait(&sm.delta[k & 1], (k >> 1) & 1);
+        wait_peer(&sm.delta[k & 1], (k >> 1) & 1);
         if (threadIdx.x == 0 && kb < nblk) mbar_expect_tx(&sm.delta[k & 1], kSendD);   // for block k + 2
         uint32_t aa[4], ab[4], ac[4];
         {

@@ -55,3 +55,16 @@ def test_gram_parts_are_read_before_they_are_written_over():
     assert gram_races(warps, 2)                              # two buffers: nothing holds a warp of the half that adds up
     assert not gram_races(warps, constant("kGramParts"))
     assert "part[kGramParts][kNg][kCoup]" in source()
+
+
+def test_what_peers_sent_is_waited_for_at_cluster_scope():
+    # st.async and remote arrivals come from other CTAs of the cluster: whoever waits for them acquires, and whoever frees a
+    # peer's slot releases, at that scope (a CTA-scope wait orders nothing against another CTA's accesses)
+    text = source()
+    sent = set(re.findall(r"peer_addr\(smem_addr\(&sm\.(\w+)\[", text)) | set(re.findall(r"bar = smem_addr\(&sm\.(\w+)\[", text))
+    barriers = set(re.findall(r"mbar_init\(&sm\.(\w+)\[", text)) & sent
+    assert barriers == {"bz", "bg", "gfree", "delta"}
+    waits = [(how, bar) for how, bar in re.findall(r"\b(\w+)\(&sm\.(\w+)\[[^;]*?\) & 1\)", text) if how.startswith("wait")]
+    assert {bar for how, bar in waits} >= barriers | {"full", "done"}
+    assert all((how == "wait_peer") == (bar in barriers) for how, bar in waits), waits
+    assert "mbarrier.arrive.relaxed" not in text
