@@ -757,6 +757,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       for (int pass = 0; pass < (p.w_end ? 2 : 1); ++pass) {
         float* row = (pass == 0 ? p.U : p.w_end) + (size_t)t.u_row * p.stride;
         const float fw = pass == 0 ? c1 : qw, fu = pass == 0 ? 1.f : neta;
+        __syncwarp();   // the second pass starts with the buffer the first one ended with, where KM is odd
 #pragma unroll
         for (int j = 0; j < KM; ++j) {   // a k-step's 80 parameters through the warp's own buffer: whole lines out
           float* st = sm.m.zpart[j & 1][warp];

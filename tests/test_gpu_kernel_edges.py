@@ -244,6 +244,24 @@ def test_one_round_without_allocation_on_any_alignment(shift):
     assert rel_err(U.cpu().numpy(), U_ref) <= U_TOL and rel_err(w_end.cpu().numpy(), w_ref) <= U_TOL
 
 
+# The end model leaves through the buffers the update sum left through: the sum is, bit for bit, that of a run, which asks for no end model.
+@pytest.mark.parametrize("samples,l2", [(1, 0.0), (17, 1e-3), (50, 0.0), (160, 1e-3)])
+def test_update_sums_beside_end_models(samples, l2):
+    cfg = workloads.get_config("cfg5", n_clients=15, n_rounds=1, sched_a=1, sched_b=samples, l2=l2, lr=0.002, data=dict(per_client=64))
+    w0 = np.random.default_rng(1).normal(0, 0.05, workloads.n_params(cfg["dims"])).astype(np.float32)
+    data = workloads.make_client_data(cfg)
+    gpu = run_gpu(cfg, data, w0)
+    with api.Session(cfg, to_device(data), torch.from_numpy(w0).cuda()) as s:
+        s.run()
+        seq = {e["client"]: e["seq"] for e in s.log()[0]}
+        w, U, w_end = torch.from_numpy(w0).cuda(), torch.empty(w0.size, device="cuda"), torch.empty(w0.size, device="cuda")
+        for c, (x, y) in enumerate(to_device(data)):
+            for _ in range(4):
+                api.aet_round_no_alloc(cfg, c, 0, x, y, w, U, w_end)
+                assert U.cpu().numpy().tobytes() == gpu["U"][seq[c]].tobytes(), c
+            assert rel_err(w_end.cpu().numpy(), sim.run_task(cfg, data[c], c, 0, w0.astype(np.float64))[1]) <= U_TOL
+
+
 @pytest.mark.parametrize("name,over", [
     ("cfg5", dict(n_clients=5, data=dict(per_client=1))), ("cfg5", dict(n_clients=3, data=dict(per_client=668))),
     ("cfg5", dict(n_clients=3, data=dict(per_client=669))),                       # the last size fetched by a kernel, the first copied
