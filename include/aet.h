@@ -316,6 +316,11 @@ aet_status aet_round_no_alloc(const aet_config* cfg, uint32_t client, uint32_t r
 aet_status aet_schedule_only(const aet_config* cfg, uint32_t n_rounds, aet_event* out,
                              size_t capacity, size_t* n_events, aet_summary* summary);
 
+/* Which kernel a launch of n_tasks regression round-tasks takes (784 -> 10, batch 1; the longest of `longest` samples;
+ * by_value: aet_round_no_alloc) on a device that runs at_once[n] clusters of n CTAs at once, n = 1 .. 8: 16 times the kernel
+ * (0 relay, 1 chain, 2 block, 3 block crowded) plus the CTAs per round-task. */
+uint32_t aet_debug_regression_kernel(uint32_t n_tasks, uint32_t longest, uint32_t by_value, const uint32_t* at_once);
+
 /* Draw number `counter` of stream (seed, stream, client); streams: 0 sample
  * index, 1 compute delay, 2 network delay. */
 uint64_t aet_debug_draw(uint64_t seed, uint32_t stream, uint32_t client, uint64_t counter);

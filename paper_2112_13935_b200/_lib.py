@@ -77,6 +77,7 @@ PROTOTYPES = {
                                      C.c_uint32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
     "aet_schedule_only": (C.c_int, [C.POINTER(AetConfig), C.c_uint32, C.POINTER(AetEvent), C.c_size_t,
                                     C.POINTER(C.c_size_t), C.POINTER(AetSummary)]),
+    "aet_debug_regression_kernel": (C.c_uint32, [C.c_uint32, C.c_uint32, C.c_uint32, C.POINTER(C.c_uint32)]),
     "aet_debug_draw": (C.c_uint64, [C.c_uint64, C.c_uint32, C.c_uint32, C.c_uint64]),
     "aet_debug_delay_ticks": (C.c_uint64, [C.c_uint32, C.c_uint64, C.c_uint64, C.c_uint64]),
     "aet_debug_plan_waves": (C.c_uint32, [C.POINTER(AetConfig), C.c_uint32]),

@@ -210,6 +210,12 @@ def aet_schedule_only(cfg, n_rounds: int, raw: bool = False):
     return _events_from(arr, n.value), _summary_from(s)
 
 
+def aet_debug_regression_kernel(n_tasks, longest, by_value, at_once):
+    """(kernel, CTAs per round-task) of a launch of regression round-tasks; at_once[n]: clusters of n CTAs the device runs at once."""
+    got = _lib.load().aet_debug_regression_kernel(n_tasks, longest, int(by_value), (C.c_uint32 * 9)(*at_once))
+    return ("relay", "chain", "block", "crowded")[got // 16], got % 16
+
+
 def aet_debug_draw(seed, stream_id, client, counter) -> int:
     return int(_lib.load().aet_debug_draw(seed, stream_id, client, counter))
 

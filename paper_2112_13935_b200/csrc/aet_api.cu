@@ -1077,6 +1077,13 @@ aet_status aet_schedule_only(const aet_config* cfg, uint32_t n_rounds, aet_event
   return AET_OK;
 }
 
+uint32_t aet_debug_regression_kernel(uint32_t n_tasks, uint32_t longest, uint32_t by_value, const uint32_t* at_once) {
+  uint32_t n[9];
+  for (int i = 0; i < 9; ++i) n[i] = at_once[i];
+  const LrChoice c = choose_lr_kernel(n_tasks, longest, by_value != 0, n);
+  return (uint32_t)c.kernel * 16 + c.cluster;
+}
+
 uint64_t aet_debug_draw(uint64_t seed, uint32_t stream, uint32_t client, uint64_t counter) {
   return draw(stream_key(seed, stream, client), counter);
 }

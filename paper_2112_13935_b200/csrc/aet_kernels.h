@@ -41,7 +41,7 @@ struct RoundLaunch {
   uint32_t n_u_rows, n_snap;     // extents of U and snaps (for the debug checks)
   uint32_t crowded_hint;         // non-zero: pick the kernel a full wave of this run's clients would get,
                                  // however few tasks this launch holds (single-task parity runs)
-  // One round-task with its descriptors in the launch itself (n_tasks 1, no sums in flight; lr_relay_kernel only):
+  // One round-task with its descriptors in the launch itself (n_tasks 1, no sums in flight; lr_relay_kernel and lr_chain_kernel):
   // nothing has to be in device memory beforehand, and rows and labels are read behind the device-side wait too.
   uint32_t by_value;
   TaskDesc one_task;
@@ -51,7 +51,7 @@ struct RoundLaunch {
   float l2;
 };
 
-// How many clusters of 1 to 8 CTAs with an SM each the current device runs at once (see device_info.cu).
+// How many clusters of 1 to 8 CTAs with an SM each the current device runs at once, 0 where it runs none (see device_info.cu).
 cudaError_t clusters_at_once(uint32_t cluster, uint32_t* out);
 
 // One CTA waits (at most max_polls polls) on a barrier nobody signals, then sets bit 0 of *status.
@@ -60,6 +60,10 @@ cudaError_t launch_wait_probe(uint32_t* status, uint32_t max_polls, cudaStream_t
 // Softmax regression 784 -> 10, batch 1; the kernel is picked by how many round-tasks the launch holds.  Asynchronous on s; may start under the tail of the previous kernel in s
 // (programmatic stream serialisation) and waits on the device before reading that kernel's output.
 cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s);
+// ... the choice: which kernel, on how many CTAs per round-task.  at_once[n]: clusters of n CTAs the device runs at once.
+enum class LrKernel : uint32_t { kRelay, kChain, kBlock, kCrowded };
+struct LrChoice { LrKernel kernel; uint32_t cluster; };
+LrChoice choose_lr_kernel(uint32_t n_tasks, uint32_t longest, bool by_value, const uint32_t (&at_once)[9]);
 // a cluster of eight or six CTAs per round-task (see lr_relay_kernel.cu), of four or two (lr_chain_kernel.cu)
 cudaError_t launch_lr_relay_rounds(const RoundLaunch& p, uint32_t cluster, cudaStream_t s);
 cudaError_t launch_lr_chain_rounds(const RoundLaunch& p, uint32_t cluster, cudaStream_t s);

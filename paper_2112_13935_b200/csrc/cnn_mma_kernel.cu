@@ -922,7 +922,7 @@ cudaError_t cnn_mma_cluster(const CnnShape& s, uint32_t n_tasks, uint32_t* clust
   if (e != cudaSuccess) return e;
   if (kFits[0][bt - 1] && n_tasks <= eights) *cluster = 8;
   else if (kFits[1][bt - 1] && n_tasks * 4 <= sms) *cluster = 4;
-  else if (kFits[0][bt - 1] && n_tasks * 8 <= sms) *cluster = 8;
+  else if (kFits[0][bt - 1] && eights && n_tasks * 8 <= sms) *cluster = 8;
   return cudaSuccess;
 }
 

@@ -17,7 +17,7 @@ __global__ void __launch_bounds__(kThreads, 1) whole_sm_kernel(float* p) {   // 
   if (p) p[threadIdx.x] = s[threadIdx.x];
 }
 
-// [device][CTAs]; 0: not asked yet.  Two host threads may ask at once and store the same value.
+// [device][CTAs], one more than the answer; 0: not asked yet.  Two host threads may ask at once and store the same value.
 std::atomic<uint32_t> g_fit[kMaxDevices][9] = {};
 
 }  // namespace
@@ -48,10 +48,10 @@ cudaError_t clusters_at_once(uint32_t cluster, uint32_t* out) {
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&v, whole_sm_kernel, &cfg);
     }
     if (e != cudaSuccess) return e;
-    n = v > 0 ? (uint32_t)v : 1;
+    n = (uint32_t)(v > 0 ? v : 0) + 1;   // (a part of a device may have no place for a wide cluster at all)
     if (known) known->store(n, std::memory_order_relaxed);
   }
-  *out = n;
+  *out = n - 1;
   return cudaSuccess;
 }
 

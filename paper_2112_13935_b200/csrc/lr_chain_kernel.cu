@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
   extern __shared__ __align__(128) unsigned char smem_raw[];
   typename S::Smem& sm = *reinterpret_cast<typename S::Smem*>(smem_raw);
 
-  const TaskDesc t = p.tasks[p.task_begin + blockIdx.x / CL];
+  const TaskDesc t = p.by_value ? p.one_task : p.tasks[p.task_begin + blockIdx.x / CL];
   if (!debug_task_ok(p, t)) return;
   const uint32_t rank = mma::cluster_rank();
   if (t.n_samples == 0) {
@@ -272,9 +272,11 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
     }
   } else if (role == kProd) {
     // ================= producer: rows and labels =================
-    // Rows and labels are older than the set-up launch of the run, which lets nothing start early.
-    const ClientData cd = p.clients[t.client];
-    const uint64_t key = p.sample_keys[t.client];
+    // Inside a handle rows and labels are older than the set-up launch of the run, which lets nothing start early; without
+    // one they are the caller's, whose kernel ahead in the stream may still be writing them.
+    if (p.by_value) asm volatile("griddepcontrol.wait;" ::: "memory");
+    const ClientData cd = p.by_value ? p.one_client : p.clients[t.client];
+    const uint64_t key = p.by_value ? p.one_key : p.sample_keys[t.client];
     const float* xrows = reinterpret_cast<const float*>(cd.x) + 8 * ks0;
     const uint32_t bytes = 32u * cnt;
     for (uint32_t kb = 0; kb < nblk; ++kb) {

@@ -37,20 +37,24 @@ cudaError_t launch_wait_probe(uint32_t* status, uint32_t max_polls, cudaStream_t
   return cudaGetLastError();
 }
 
+LrChoice choose_lr_kernel(uint32_t n_tasks, uint32_t longest, bool by_value, const uint32_t (&at_once)[9]) {
+  const bool eights = n_tasks <= at_once[8], fours = n_tasks <= at_once[4];
+  const bool sixes = !eights && n_tasks <= at_once[6] && longest > 64;
+  if (eights || sixes) return {LrKernel::kRelay, eights ? 8u : 6u};
+  // descriptors in the launch: a kernel on clusters, whichever there is
+  if (by_value || n_tasks <= at_once[2]) return {LrKernel::kChain, fours ? 4u : 2u};
+  return {n_tasks <= at_once[1] ? LrKernel::kBlock : LrKernel::kCrowded, 1};
+}
+
 cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s) {
   if (p.n_tasks == 0) return cudaSuccess;
-  uint32_t ones = 0, pairs = 0, fours = 0, sixes = 0, eights = 0;
-  cudaError_t e = clusters_at_once(1, &ones);
-  if (e == cudaSuccess) e = clusters_at_once(2, &pairs);
-  if (e == cudaSuccess) e = clusters_at_once(4, &fours);
-  if (e == cudaSuccess) e = clusters_at_once(6, &sixes);
-  if (e == cudaSuccess) e = clusters_at_once(8, &eights);
-  if (e != cudaSuccess) return e;
-  if (p.n_tasks > ones || p.crowded_hint) return launch_lr_block_rounds(p, true, s);
-  if (p.n_tasks > pairs) return launch_lr_block_rounds(p, false, s);
-  const bool six = p.n_tasks > eights && p.n_tasks <= sixes && p.longest > 64;
-  if (p.n_tasks > eights && !six) return launch_lr_chain_rounds(p, p.n_tasks > fours ? 2 : 4, s);
-  return launch_lr_relay_rounds(p, six ? 6 : 8, s);
+  uint32_t at_once[9] = {};
+  for (uint32_t cl : {1u, 2u, 4u, 6u, 8u})
+    if (const cudaError_t e = clusters_at_once(cl, &at_once[cl])) return e;
+  const LrChoice c = p.crowded_hint ? LrChoice{LrKernel::kCrowded, 1} : choose_lr_kernel(p.n_tasks, p.longest, p.by_value != 0, at_once);
+  if (c.kernel == LrKernel::kRelay) return launch_lr_relay_rounds(p, c.cluster, s);
+  if (c.kernel == LrKernel::kChain) return launch_lr_chain_rounds(p, c.cluster, s);
+  return launch_lr_block_rounds(p, c.kernel == LrKernel::kCrowded, s);
 }
 
 }  // namespace aet

@@ -102,6 +102,32 @@ def test_schedule_rejects_bad_configs():
         assert e.value.status == status, over
 
 
+B200_CLUSTERS = [0, 148, 74, 45, 33, 26, 22, 15, 15]     # clusters of 1 .. 8 CTAs the whole device runs at once
+
+
+def test_regression_kernel_by_launch_size():
+    pick = lambda n, longest=100, by_value=False, at=B200_CLUSTERS: api.aet_debug_regression_kernel(n, longest, by_value, at)
+    for n, long_rounds, short_rounds in [(1, ("relay", 8), ("relay", 8)), (15, ("relay", 8), ("relay", 8)), (16, ("relay", 6), ("chain", 4)),
+                                         (22, ("relay", 6), ("chain", 4)), (23, ("chain", 4), ("chain", 4)), (33, ("chain", 4), ("chain", 4)),
+                                         (34, ("chain", 2), ("chain", 2)), (74, ("chain", 2), ("chain", 2)), (75, ("block", 1), ("block", 1)),
+                                         (148, ("block", 1), ("block", 1)), (149, ("crowded", 1), ("crowded", 1))]:
+        assert pick(n, 65) == long_rounds and pick(n, 64) == short_rounds, n
+    assert pick(1, 0, True) == ("relay", 8)
+
+
+def test_regression_kernels_only_on_clusters_the_device_has():
+    # a part of a device (few SMs, or none of its GPCs whole) may have no place for the wide clusters: never one of those
+    for at_once in ([0, 16, 8, 5, 4, 2, 2, 0, 0], [0, 14, 7, 4, 2, 1, 0, 0, 0], [0, 6, 3, 1, 1, 0, 0, 0, 0], [0, 4, 2, 0, 0, 0, 0, 0, 0], [0, 1] + 7 * [0]):
+        for n in range(1, 20):
+            for longest in (1, 64, 65, 400):
+                kernel, cluster = api.aet_debug_regression_kernel(n, longest, False, at_once)
+                assert at_once[cluster] >= (n if kernel != "crowded" else 1), (at_once, n, longest, kernel, cluster)
+                assert (kernel in ("relay", "chain")) == (cluster > 1)
+        if at_once[2]:      # descriptors in the launch: only the kernels on clusters take them
+            kernel, cluster = api.aet_debug_regression_kernel(1, 0, True, at_once)
+            assert kernel in ("relay", "chain") and at_once[cluster] >= 1
+
+
 def test_wave_plan_counts():
     # one client: every round depends on the previous one
     assert api.aet_debug_plan_waves(workloads.get_config("cfg1", n_clients=1), 5) == 5
