@@ -251,7 +251,8 @@ aet_status aet_get_update_sum(aet_handle* h, uint32_t seq, float* out, size_t n_
 /* Parity aid, not part of a run: one round-task (client, round) of Algorithm 3
  * started from the caller's model w_in; writes the update sum U_i and the
  * client's end-of-round model (either may be null).  Pointers: host or device,
- * n_params floats each.  Uses the same sample indices the run would use.
+ * n_params floats each.  Uses the same sample indices the run would use, and for
+ * the regression the kernel that runs this round of all clients at once.
  * Leaves the handle's state unchanged.  Synchronises `cuda_stream`. */
 aet_status aet_debug_run_client_round(aet_handle* h, uint32_t client, uint32_t round,
                                       const float* w_in, float* U_out, float* w_out,

@@ -997,13 +997,8 @@ aet_status aet_debug_run_client_round(aet_handle* h, uint32_t client, uint32_t r
   r.debug_checks = (h->cfg.flags & AET_FLAG_DEBUG_CHECKS) ? 1u : 0u;
   r.step_by_step = (h->cfg.flags & AET_FLAG_STEPWISE_RECURRENCE) ? 1u : 0u;
   r.n_u_rows = 1; r.n_snap = 1;
-  // the kernel a full wave of this handle's clients would run, so that this parity aid checks it
-  {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-      r.crowded_hint = h->cfg.n_clients > (uint32_t)sms ? 1u : 0u;
-    cudaGetLastError();
-  }
+  // (regression) the kernel a wave of this round of all clients runs, so that this parity aid checks it
+  r.wave_tasks = h->cfg.n_clients; r.longest = s_i;
   const aet_stats keep = h->stats;
   const bool timing = h->timing;
   h->timing = false;

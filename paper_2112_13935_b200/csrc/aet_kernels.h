@@ -39,8 +39,8 @@ struct RoundLaunch {
   uint32_t task_begin, n_tasks;
   uint32_t longest;              // samples of the longest round-task of a launch of few (0: many, or not known)
   uint32_t n_u_rows, n_snap;     // extents of U and snaps (for the debug checks)
-  uint32_t crowded_hint;         // non-zero: pick the kernel a full wave of this run's clients would get,
-                                 // however few tasks this launch holds (single-task parity runs)
+  uint32_t wave_tasks;           // non-zero: pick the kernel a launch of so many round-tasks would get, however few
+                                 // this one holds (single-task parity runs of the regression)
   // One round-task with its descriptors in the launch itself (n_tasks 1, no sums in flight; lr_relay_kernel and lr_chain_kernel):
   // nothing has to be in device memory beforehand, and rows and labels are read behind the device-side wait too.
   uint32_t by_value;

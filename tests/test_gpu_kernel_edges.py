@@ -262,6 +262,21 @@ def test_update_sums_beside_end_models(samples, l2):
             assert rel_err(w_end.cpu().numpy(), sim.run_task(cfg, data[c], c, 0, w0.astype(np.float64))[1]) <= U_TOL
 
 
+# A round restarted on its own runs the kernel and the cluster width that ran it among all the others: the same bits.
+@pytest.mark.parametrize("n_clients,samples,l2", [(15, 40, 0.0), (16, 40, 0.0), (16, 70, 1e-3), (22, 70, 0.0), (33, 70, 1e-3), (34, 40, 0.0),
+                                                  (74, 70, 0.0), (75, 40, 0.0), (150, 40, 1e-3)])
+def test_restarted_regression_rounds_run_the_kernel_of_the_wave(n_clients, samples, l2):
+    cfg = workloads.get_config("cfg5", n_clients=n_clients, n_rounds=1, sched_a=1, sched_b=samples, l2=l2, lr=0.001, data=dict(per_client=40))
+    data, w0 = make(cfg)
+    gpu = run_gpu(cfg, data, w0)
+    with api.Session(cfg, to_device(data), torch.from_numpy(w0).cuda()) as s:
+        s.run()
+        for e in s.log()[0][::max(1, n_clients // 5)]:
+            U, w_end = api.aet_debug_run_client_round(s.h, e["client"], 0, w0)
+            assert U.tobytes() == gpu["U"][e["seq"]].tobytes(), e["client"]
+            assert rel_err(w_end, sim.run_task(cfg, data[e["client"]], e["client"], 0, w0.astype(np.float64))[1]) <= U_TOL
+
+
 @pytest.mark.parametrize("name,over", [
     ("cfg5", dict(n_clients=5, data=dict(per_client=1))), ("cfg5", dict(n_clients=3, data=dict(per_client=668))),
     ("cfg5", dict(n_clients=3, data=dict(per_client=669))),                       # the last size fetched by a kernel, the first copied
