@@ -267,6 +267,16 @@ aet_status aet_debug_run_client_round(aet_handle* h, uint32_t client, uint32_t r
  * Section 3.3.1; this guards the library's own asynchronous copies.) */
 aet_status aet_debug_wait_probe(aet_handle* h, uint32_t max_polls, void* cuda_stream);
 
+/* Failure-detection aid: aet_debug_run_client_round of a regression handle with few
+ * clients (up to 15; up to 22 in rounds above 64 samples; no split_mode), as if the
+ * copies of one CTA of the round's cluster of 8 (6) never came.  Every wait polls at
+ * most max_polls times (1 .. 2^16).  Returns AET_ERR_TIMEOUT, with NaN among U_out,
+ * which is what a caller without a status word goes by; the handle and the CUDA
+ * context stay usable. */
+aet_status aet_debug_lost_copies(aet_handle* h, uint32_t client, uint32_t round, uint32_t cta,
+                                 uint32_t max_polls, const float* w_in, float* U_out, float* w_out,
+                                 void* cuda_stream);
+
 /* Record CUDA events around every kernel of later runs (adds a little launch
  * overhead) so that aet_get_stats can report device time per kernel. */
 aet_status aet_set_kernel_timing(aet_handle* h, int enable);

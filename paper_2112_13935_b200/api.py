@@ -282,3 +282,9 @@ class Session:
 
     def __exit__(self, *exc):
         self.close()
+
+
+def aet_debug_lost_copies(h, client: int, rnd: int, cta: int, w_in, U_out, w_out, max_polls: int = 1 << 12, stream=None):
+    """One round-task as if the copies of one CTA of its cluster never came; raises AetError(AET_ERR_TIMEOUT), with U_out written."""
+    _check(h, _lib.load().aet_debug_lost_copies(h, client, rnd, cta, max_polls, _ptr(w_in), _ptr(U_out), _ptr(w_out),
+                                                _stream(stream)))

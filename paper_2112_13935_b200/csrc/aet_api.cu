@@ -958,8 +958,8 @@ aet_status aet_get_event_log(aet_handle* h, aet_event* out, size_t capacity, siz
   return AET_OK;
 }
 
-aet_status aet_debug_run_client_round(aet_handle* h, uint32_t client, uint32_t round, const float* w_in,
-                                      float* U_out, float* w_out, void* cuda_stream) {
+static aet_status debug_round(aet_handle* h, uint32_t client, uint32_t round, uint32_t lose, uint32_t max_polls, const float* w_in,
+                              float* U_out, float* w_out, void* cuda_stream) {
   if (!h || !w_in) return h ? fail(h, AET_ERR_ARG, "null argument") : AET_ERR_ARG;
   if (client >= h->cfg.n_clients) return fail(h, AET_ERR_ARG, "client index out of range");
   if (round < h->cfg.round_base) return fail(h, AET_ERR_ARG, "round is before round_base");
@@ -997,6 +997,7 @@ aet_status aet_debug_run_client_round(aet_handle* h, uint32_t client, uint32_t r
   r.debug_checks = (h->cfg.flags & AET_FLAG_DEBUG_CHECKS) ? 1u : 0u;
   r.step_by_step = (h->cfg.flags & AET_FLAG_STEPWISE_RECURRENCE) ? 1u : 0u;
   r.n_u_rows = 1; r.n_snap = 1;
+  r.lose = lose; r.max_polls = max_polls;
   // (regression) the kernel a wave of this round of all clients runs, so that this parity aid checks it
   r.wave_tasks = h->cfg.n_clients; r.longest = s_i;
   const aet_stats keep = h->stats;
@@ -1007,11 +1008,29 @@ aet_status aet_debug_run_client_round(aet_handle* h, uint32_t client, uint32_t r
   h->stats = keep;
   if (rs != AET_OK) return rs;
   AET_CUDA(h, cudaStreamSynchronize(s));
-  if (aet_status ds = check_device_status(h)) return ds;
+  const aet_status ds = check_device_status(h);
+  if (ds && !lose) return ds;
   if (U_out) AET_CUDA(h, cudaMemcpyAsync(U_out, U, (size_t)h->P * sizeof(float), cudaMemcpyDefault, s));
   if (w_out) AET_CUDA(h, cudaMemcpyAsync(w_out, wend, (size_t)h->P * sizeof(float), cudaMemcpyDefault, s));
   AET_CUDA(h, cudaStreamSynchronize(s));
-  return AET_OK;
+  return ds;
+}
+
+aet_status aet_debug_run_client_round(aet_handle* h, uint32_t client, uint32_t round, const float* w_in,
+                                      float* U_out, float* w_out, void* cuda_stream) {
+  return debug_round(h, client, round, 0, 0, w_in, U_out, w_out, cuda_stream);
+}
+
+aet_status aet_debug_lost_copies(aet_handle* h, uint32_t client, uint32_t round, uint32_t cta, uint32_t max_polls, const float* w_in,
+                                 float* U_out, float* w_out, void* cuda_stream) {
+  if (!h) return AET_ERR_ARG;
+  if (!h->lr_fast || h->cfg.split_mode || round < h->cfg.round_base) return fail(h, AET_ERR_CONFIG, "lost copies can be played for the regression's rounds only");
+  uint32_t at_once[9] = {};
+  for (uint32_t cl = 1; cl <= 8; ++cl) AET_CUDA(h, clusters_at_once(cl, &at_once[cl]));
+  const LrChoice c = choose_lr_kernel(h->cfg.n_clients, sample_size(h->cfg, round), false, at_once);
+  if (c.kernel != LrKernel::kRelay) return fail(h, AET_ERR_CONFIG, "lost copies can be played for few clients only");
+  if (cta >= c.cluster || max_polls == 0 || max_polls > (1u << 16)) return fail(h, AET_ERR_ARG, "cta must be below the cluster's width, max_polls in [1, 2^16]");
+  return debug_round(h, client, round, cta + 1, max_polls, w_in, U_out, w_out, cuda_stream);
 }
 
 aet_status aet_debug_wait_probe(aet_handle* h, uint32_t max_polls, void* cuda_stream) {

@@ -49,6 +49,9 @@ struct RoundLaunch {
   uint64_t one_key;
   uint32_t step_by_step;         // non-zero: the recurrence of a block is always walked step by step
   float l2;
+  // Failure checks, lr_relay_kernel only (0 in every run): 1 + the CTA of the cluster whose copies are left out, or, if that is the
+  // walker, whose couplings are; and how often every wait polls then.
+  uint32_t lose, max_polls;
 };
 
 // How many clusters of 1 to 8 CTAs with an SM each the current device runs at once, 0 where it runs none (see device_info.cu).

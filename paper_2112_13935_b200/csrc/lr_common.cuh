@@ -57,6 +57,11 @@ __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, 
   return false;
 }
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) { return mbar_wait_limit(bar, parity, kWaitLimit); }
+// After a wait has given up: what peers have sent and nobody waits for any more lands while this CTA is still there (some 100 us).
+__device__ __forceinline__ void linger() {
+#pragma unroll 1
+  for (int i = 0; i < 100; ++i) __nanosleep(1000);
+}
 // One row global -> shared, 16-byte aligned on both sides, size a multiple of 16.
 __device__ __forceinline__ void bulk_load_row(float* dst, const float* src, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"

@@ -141,7 +141,8 @@ __device__ __forceinline__ float load1(uint32_t at) {
   return v;
 }
 
-template <class S>
+// LOSE: as if copies never came, with waits that end soon (RoundLaunch::lose; never part of a run).
+template <class S, bool LOSE>
 __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
   constexpr int CL = S::kCl, MC = S::kMc, NM = S::kNm, KM = S::kKm, NG = kNg, KG = S::kKg, NS = kNs, GC = S::kGc;
   constexpr int PM = S::kPitchM, PG = S::kPitchG;
@@ -198,13 +199,19 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
   }
   mma::cluster_sync();   // a peer's barriers exist before anything is sent to it
 
-  // After a wait has given up nothing waits any more: the round runs through on whatever is there, the status
-  // word is set, and every CTA of the cluster reaches the end.
+  // A thread whose wait has given up waits no more and runs through on whatever is there, but makes no other operation on a barrier
+  // and sends nothing: a second arrival on a barrier that is short of bytes would be invalid, and so would bytes without end on one
+  // that nobody arms.  Whoever depends on it gives up in turn, the model warps among them, which sets the status word and, for
+  // callers without one, leaves NaN in the update sum; every CTA of the cluster reaches the end.  (NaN among what such a thread
+  // makes, where another one would pass it on as a result.)
   bool ok = true;
-  auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok) ok = mbar_wait(bar, parity); };
+  const float kNone = __int_as_float(0x7FFFFFFF);
+  const uint32_t limit = LOSE ? p.max_polls : kWaitLimit;
+  const bool lost = LOSE && p.lose == rank + 1;
+  auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok) ok = mbar_wait_limit(bar, parity, limit); };
   auto wait_peer = [&](uint64_t* bar, uint32_t parity) {   // for what peers sent, or have taken
     const uint32_t at = smem_addr(bar);
-    for (uint32_t i = 0; ok && !mma::try_wait_cluster(at, parity); ++i) ok = i < kWaitLimit;
+    for (uint32_t i = 0; ok && !mma::try_wait_cluster(at, parity); ++i) ok = i < limit;
   };
   const float scale = neta * kLog2e;
   // The kernel behind this one may come up while the last blocks are walked: what it does before its own wait, it does with what the
@@ -246,7 +253,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       // A step uses up z[0] and moves the others down by one, round the end: after sixteen every sample is in its place again.
       // Only the next sample's logit is formed at once; the others follow while the next exponentials go round the lanes.  (A loop,
       // not sixteen copies of it: those do not fit the instruction cache, 270 cycles a step.)
-      float zc = z[0], d = 0.f;
+      float zc = ok ? z[0] : kNone, d = 0.f;   // (one sample's exponentials pass it on to all that follow)
       auto others = [&]() {
         const float end = z[0];
 #pragma unroll
@@ -301,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       if (sm.w.amax[k % kCoups] < kTame) steps(std::false_type());
       else steps(std::true_type());
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.done[b]);
+      if (ok && lane == 0) mbar_arrive(&sm.done[b]);
       others();
     }
   } else if (walks && warp == 1) {
@@ -337,7 +344,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       }
       __syncwarp();
 #pragma unroll
-      for (int j = lane; j < 3 * kC * 2; j += 32) {
+      for (int j = lane; j < 3 * kC * 2 && ok; j += 32) {   // (every lane sends some)
         const uint4 v = *reinterpret_cast<const uint4*>(&sm.w.dstage[0][0][4 * j]);
         const uint32_t to = smem_addr(&sm.m.dpart[b][j / (2 * kC)][0][4 * (j % (2 * kC))]), bar = smem_addr(&sm.delta[b]);
 #pragma unroll
@@ -354,7 +361,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
         for (int i = 0; i < kCh; ++i) sm.w.ub[b][h * kCh + i] = ub[i];
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.bsum[b]);
+      if (ok && lane == 0) mbar_arrive(&sm.bsum[b]);
     }
   } else if (walks && warp == 2) {
     // ================= couplings, summed in rank order, and labels: a block ahead of R =================
@@ -367,7 +374,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
     };
     if (lane == 0) mbar_expect_tx(&sm.bg[0], GC * kSendG0);
     int y = label(0);
-    for (uint32_t k = 0; k < nblk; ++k) {
+    for (uint32_t k = 0; k < (lost ? 0 : nblk); ++k) {
       uint32_t hot = 0;
 #pragma unroll
       for (int i = 0; i < kC; ++i) {
@@ -379,6 +386,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       const int ig = k % kInG, s = lane & 15;
       wait_peer(&sm.bg[ig], (k / kInG) & 1);
       if (k >= kCoups) wait(&sm.done[(k - kCoups) & 1], ((k - kCoups) >> 1) & 1);   // R is done with block k - 3, whose place this is
+      ok = __all_sync(0xffffffffu, ok);
       float* out = sm.w.coup[k % kCoups];
       const float* in = &sm.w.gin[ig][0][0];
       float v[8], c[8], big = 0.f;   // (all loads before the first store: the compiler cannot tell them apart)
@@ -401,11 +409,11 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       big = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(big)));
       if (lane == 0) {
         sm.w.amax[k % kCoups] = big;
-        if (k + 1 < nblk) mbar_expect_tx(&sm.bg[(k + 1) % kInG], GC * kSendG);
+        if (ok && k + 1 < nblk) mbar_expect_tx(&sm.bg[(k + 1) % kInG], GC * kSendG);
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.rg[k & 3]);
-      if (lane < GC && k + kInG < nblk)   // the CTAs that sent them may send block k + 4
+      if (ok && lane == 0) mbar_arrive(&sm.rg[k & 3]);
+      if (ok && lane < GC && k + kInG < nblk)   // the CTAs that sent them may send block k + 4
         mma::arrive_peer(mma::peer_addr(smem_addr(&sm.gfree[ig]), MC + lane));
     }
   } else if (walks && warp == 3) {
@@ -449,14 +457,15 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       m = fmaxf(m, shx(m, 16));
 #pragma unroll
       for (int i = 0; i < kCh; ++i) sm.w.zsum[b][(h * kCh + i) * kGp + s] = v[i] - m;
-      if (lane == 0 && k + 1 < nblk) mbar_expect_tx(&sm.bz[(k + 1) % kInZ], MC * kZ * 4);
+      if (!ok) sm.w.zsum[b][h * kCh * kGp + s] = kNone;
+      if (ok && lane == 0 && k + 1 < nblk) mbar_expect_tx(&sm.bz[(k + 1) % kInZ], MC * kZ * 4);
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.rz[b]);
+      if (ok && lane == 0) mbar_arrive(&sm.rz[b]);
     }
     // the biases' part of what a round leaves behind
     const int last = (nblk - 1) & 1;
     wait(&sm.bsum[last], ((nblk - 1) >> 1) & 1);
-    const float bad = ok ? 0.f : __int_as_float(0x7FFFFFFF);
+    const float bad = ok ? 0.f : kNone;
 #pragma unroll 1
     for (int pass = 0; pass < (p.w_end ? 2 : 1); ++pass) {
       float* row = (pass == 0 ? p.U : p.w_end) + (size_t)t.u_row * p.stride;
@@ -478,10 +487,10 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
     const uint64_t key = p.by_value ? p.one_key : p.sample_keys[t.client];
     const float* xrows = reinterpret_cast<const float*>(cd.x) + 8 * ks0;
     const uint32_t bytes = 32u * cnt;
-    for (uint32_t kb = 0; kb < nblk; ++kb) {
+    for (uint32_t kb = 0; kb < (lost ? 0 : nblk); ++kb) {
       const int sb = kb % NS;
       if (kb >= (uint32_t)NS) wait(&sm.freed[sb], (kb / NS - 1) & 1);   // block kb - NS has left its slot
-      if (!ok) break;
+      if (!__all_sync(0xffffffffu, ok)) break;
       const uint32_t nvb = min((uint32_t)kB, n - kb * kB);
       float* const slot = rows + sb * kB * pitch;
       for (uint32_t r = nvb; r < (uint32_t)kB; ++r)   // short last block: rows that add nothing anywhere
@@ -528,7 +537,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
         { pv[j][0] = a; pv[j][1] = b; pv[j][2] = c; pv[j][3] = d; }
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.freed[kb % NS]);
+      if (ok && lane == 0) mbar_arrive(&sm.freed[kb % NS]);
       float* const block = gpart + (int)(kb % kGramParts) * NG * kCoup;
       float* part = block + warp * kCoup;
 #pragma unroll
@@ -542,6 +551,8 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
           *reinterpret_cast<float2*>(part + kOffC + r * kGp + s) =
               make_float2(hh[m][2 * r2] + cx[m][2 * r2], hh[m][2 * r2 + 1] + cx[m][2 * r2 + 1]);
         }
+      if (!ok)
+        for (int i = 0; i < kCoup; ++i) part[i] = kNone;
       // Half of the warps add up a block's parts while the others are at the next block's products: they only say that theirs are
       // there.  A barrier per parity.  A warp that writes block kb has waited at kb - 1 or at kb - 2, whichever its half adds up, and every
       // warp arrives there behind its sums of block kb - 3: those have been read.  The sums of kb - 2 may not have been: warps of one half
@@ -557,7 +568,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       const float one = grank == 0 ? scale : 0.f;   // the bias input's part of a coupling
       // two entries per thread: 64 pairs that reach below the diagonal, 128 of the matrix to the block before
       if (kb >= kInG) wait_peer(&sm.gfree[ig], (kb / kInG - 1) & 1);   // the walker has taken block kb - 4
-      for (int e = (warp - first) * 32 + lane; e < (kb ? 192 : 64); e += sums * 32) {
+      for (int e = (warp - first) * 32 + lane; e < (kb ? 192 : 64) && ok; e += sums * 32) {
         const bool own = e < 64;
         int tr, s0;
         if (own) {   // rows 2q + 1 and 2q + 2 have q + 1 pairs each, q = 0 .. 6; row 15 eight
@@ -660,7 +671,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       if (update) {
         // ---- U^T = q^nv U^T + sum_s q^(nv-1-s) delta_s x_s; the k index of the product is read as samples t, t + 4, t + 8, t + 12 ----
         wait_peer(&sm.delta[k & 1], (k >> 1) & 1);
-        if (threadIdx.x == 0 && kb < nblk) mbar_expect_tx(&sm.delta[k & 1], kSendD);   // for block k + 2
+        if (ok && threadIdx.x == 0 && kb < nblk) mbar_expect_tx(&sm.delta[k & 1], kSendD);   // for block k + 2
         uint32_t aa[4], ab[4], ac[4];
         {
           const uint32_t* at = &sm.m.dpart[k & 1][0][g][2 * tt];
@@ -726,11 +737,12 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
           if (two)
             *reinterpret_cast<float2*>(mypart + (8 + g) * kB + s) = make_float2((zm[m][2] + zx[m][2]) * f0, (zm[m][3] + zx[m][3]) * f1);
         }
+        if (!ok) mypart[0] = kNone;   // (the first sample is one of the round's in every block)
         asm volatile("bar.sync 1, %0;" ::"n"(NM * 32) : "memory");
-        // sums over the warps, in warp order; sent to every CTA of the cluster
+        // sums over the warps, in warp order; sent to the walker
         if (warp < 2) {
           const int iz = kb % kInZ, e = warp * 32 + lane;
-          if (e < kQuadZ) {
+          if (e < kQuadZ && ok) {
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int w = 0; w < NM; ++w) {
@@ -743,14 +755,13 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       }
       if (update) {
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.freed[k % NS]);
+        if (ok && lane == 0) mbar_arrive(&sm.freed[k % NS]);
       }
     }
 
     // ---- event trigger: h reached s_{i,c}; publish U_i (and the end model) ----
     {
-      // a round whose copies never came leaves NaN behind, for callers that have no status word to look at
-      const float bad = ok ? 0.f : __int_as_float(0x7FFFFFFF);
+      const float bad = ok ? 0.f : kNone;
       const float c1 = (decay ? (float)((1.0 - qwd) / (double)eta) : 0.f) + bad;
       qw += bad;
 #pragma unroll 1
@@ -777,10 +788,11 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
   }
   if (!ok && p.status && lane == 0) atomicOr(p.status, 1u);
   mma::cluster_sync();   // no CTA leaves while a peer may still send to it
+  if (!ok) linger();
   if (!ok && !walks && warp == kWarps - 1)   // copies still in flight target this CTA's shared memory: a bounded chance to land
     for (int s = 0; s < NS; ++s) {
-      mbar_wait_limit(&sm.full[s], 0, 1u << 16);
-      mbar_wait_limit(&sm.full[s], 1, 1u << 16);
+      mbar_wait_limit(&sm.full[s], 0, min(limit, 1u << 16));
+      mbar_wait_limit(&sm.full[s], 1, min(limit, 1u << 16));
     }
   if (threadIdx.x == 0 && rank == 0) {
     TriggerRec rec;
@@ -792,7 +804,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
 typedef Shape<3, 11, 3, 2, 5> Six;
 typedef Shape<4, 9, 3, 3, 3> Eight;
 
-template <class S>
+template <class S, bool LOSE>
 cudaError_t launch(const RoundLaunch& p, cudaStream_t s) {
   static std::atomic<uint64_t> opted_in{0};   // a bit per device
   int dev = 0;
@@ -800,7 +812,7 @@ cudaError_t launch(const RoundLaunch& p, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const uint64_t bit = dev >= 0 && dev < 64 ? 1ull << dev : 0;
   if (!(opted_in.load(std::memory_order_relaxed) & bit)) {
-    e = cudaFuncSetAttribute(lr_relay_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(typename S::Smem));
+    e = cudaFuncSetAttribute(lr_relay_kernel<S, LOSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(typename S::Smem));
     if (e != cudaSuccess) return e;
     opted_in.fetch_or(bit, std::memory_order_relaxed);
   }
@@ -817,13 +829,14 @@ cudaError_t launch(const RoundLaunch& p, cudaStream_t s) {
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, lr_relay_kernel<S>, p);
+  return cudaLaunchKernelEx(&cfg, lr_relay_kernel<S, LOSE>, p);
 }
 
 }  // namespace
 
 cudaError_t launch_lr_relay_rounds(const RoundLaunch& p, uint32_t cluster, cudaStream_t s) {
-  return cluster == 8 ? launch<Eight>(p, s) : launch<Six>(p, s);
+  if (p.lose) return cluster == 8 ? launch<Eight, true>(p, s) : launch<Six, true>(p, s);
+  return cluster == 8 ? launch<Eight, false>(p, s) : launch<Six, false>(p, s);
 }
 
 }  // namespace aet

@@ -313,6 +313,26 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_handle_survives():
         assert e.value.status == 1
 
 
+# Clusters of eight: CTAs 0 to 3 hold the model, 4 to 6 the Gram matrices, 7 walks; of six: 0 to 2, 3 and 4, 5.
+@pytest.mark.parametrize("cta,rnd,over", [
+    *[(cta, rnd, {}) for cta in (0, 3, 4, 6, 7) for rnd in (0, 4)],      # one block and four
+    *[(cta, 0, dict(sched_b=100, lr=2e-3, n_rounds=1)) for cta in (0, 4, 7)],   # seven blocks: the rings go round
+    *[(cta, 0, dict(n_clients=16, sched_b=70, lr=1e-3, n_rounds=1)) for cta in (0, 2, 3, 5)],
+])
+def test_a_round_whose_copies_never_come_leaves_nan(cta, rnd, over):
+    cfg = workloads.get_config("cfg1", l2=0.0, **over)
+    data, w0 = make(cfg)
+    ref = sim.run(cfg, data, w0)
+    with api.Session(cfg, to_device(data), torch.from_numpy(w0).cuda()) as s:
+        U, w = np.zeros(w0.size, dtype=np.float32), np.zeros(w0.size, dtype=np.float32)
+        with pytest.raises(api.AetError) as e:
+            api.aet_debug_lost_copies(s.h, 1, rnd, cta, w0, U, w)
+        assert e.value.status == 6                            # AET_ERR_TIMEOUT
+        assert np.isnan(U).any() and np.isnan(w).any()
+        s.run()                                               # status was cleared; the context is intact
+        assert np.abs(s.model() - ref["w"]).max() <= 1e-5
+
+
 def test_zero_rounds_is_a_no_op():
     cfg = workloads.get_config("cfg1")
     data, w0 = make(cfg)
