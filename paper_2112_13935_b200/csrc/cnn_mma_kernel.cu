@@ -161,6 +161,9 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     for (int i = 0; i < 5; ++i)
       if (bytes[i]) mbar_expect_tx(&bars[i], bytes[i]);
   }
+  // A thread whose wait has given up waits no more and runs through on whatever is there, but neither arms a barrier (a second arrival
+  // on one that is short of bytes would be invalid) nor sends: whoever depends on it gives up in turn, the status word is set, and
+  // every CTA of the cluster reaches the end.
   bool ok = true;
   auto wait = [&](int i, uint32_t parity) {
     const uint32_t at = smem_addr(&bars[i]);
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (it) {
       wait(4, (it - 1) & 1);
-      if (tid == 0) mbar_expect_tx(&bars[4], bytes[4]);
+      if (ok && tid == 0) mbar_expect_tx(&bars[4], bytes[4]);
     }
     if (it + 1 < t.steps) draw_rows(it + 1);
     __syncthreads();
@@ -381,13 +384,14 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
       const float4 v = *reinterpret_cast<const float4*>(st + 4 * (lane & 15));
       const uint32_t at = smem_addr(sm + M::q2 + (b0 + b) * kPq2 + (lane & 15) * 16 + yp * 4);
 #pragma unroll
-      for (int r = 0; r < CL; r += 2) mma::send_peer(mma::peer_addr(at, r + (lane >> 4)), v, mma::peer_addr(smem_addr(&bars[0]), r + (lane >> 4)));
+      for (int r = 0; r < CL; r += 2)
+        if (ok) mma::send_peer(mma::peer_addr(at, r + (lane >> 4)), v, mma::peer_addr(smem_addr(&bars[0]), r + (lane >> 4)));
       __syncwarp();
     }
 
     // ================= dense 1: own outputs, all samples; the warps share the 256 inputs =================
     wait(0, it & 1);
-    if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[0], bytes[0]);
+    if (ok && tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[0], bytes[0]);
     {
       float acc[MT1][BT][4] = {}, crs[MT1][BT][4] = {};
       const int k = 16 * warp;
@@ -423,10 +427,11 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
       v = fmaxf(v, 0.f);
       const uint32_t at = smem_addr(sm + M::h1 + b * kPh1 + rank * N1 + n);
 #pragma unroll
-      for (int r = 0; r < CL; ++r) send1(mma::peer_addr(at, r), v, mma::peer_addr(smem_addr(&bars[1]), r));
+      for (int r = 0; r < CL; ++r)
+        if (ok) send1(mma::peer_addr(at, r), v, mma::peer_addr(smem_addr(&bars[1]), r));
     }
     wait(1, it & 1);
-    if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[1], bytes[1]);
+    if (ok && tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[1], bytes[1]);
 
     // ================= dense 2, dense 3, softmax, in every CTA =================
 #pragma unroll 1
@@ -559,6 +564,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
             const uint32_t to = ((uint32_t)s * inv) >> 16;
             const uint32_t at = mma::peer_addr(smem_addr(sm + M::col + (rank * kPer + s - (int)to * per) * kFlat + 16 * warp + g), to);
             const uint32_t bar = mma::peer_addr(smem_addr(&bars[2]), to);
+            if (!ok) continue;
             send1(at, acc[b][q] + crs[b][q], bar);
             send1(at + 32, acc[b][2 + q] + crs[b][2 + q], bar);
           }
@@ -635,7 +641,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     float vq[kMaxPer / 2] = {};   // dq2 / 4 of sample e / 256, input e % 256, e = tid + 512 r
     if (nb > 0) {
       wait(2, it & 1);
-      if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[2], bytes[2]);
+      if (ok && tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[2], bytes[2]);
 #pragma unroll
       for (int r = 0; r < kMaxPer / 2; ++r) {
         const int e = tid + kThreads * r;
@@ -790,11 +796,11 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
         }
       }
       const int to = e / kOwn;
-      mma::send_peer(mma::peer_addr(smem_addr(sm + M::ing + (rank * kOwn + e - to * kOwn) * 4), to), v, mma::peer_addr(smem_addr(&bars[3]), to));
+      if (ok) mma::send_peer(mma::peer_addr(smem_addr(sm + M::ing + (rank * kOwn + e - to * kOwn) * 4), to), v, mma::peer_addr(smem_addr(&bars[3]), to));
     }
     if (tid < kOwn) {
       wait(3, it & 1);
-      if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[3], bytes[3]);
+      if (ok && tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[3], bytes[3]);
       const int e0 = 4 * (rank * kOwn + tid);
       float gr[4] = {};
 #pragma unroll
@@ -814,7 +820,8 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
         const float4 v = make_float4(wcv[0], wcv[1], wcv[2], wcv[3]);
         const uint32_t at = smem_addr(sm + M::wc + e0);
 #pragma unroll
-        for (int r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(at, r), v, mma::peer_addr(smem_addr(&bars[4]), r));
+        for (int r = 0; r < CL; ++r)
+          if (ok) mma::send_peer(mma::peer_addr(at, r), v, mma::peer_addr(smem_addr(&bars[4]), r));
       }
     }
   }
@@ -876,6 +883,7 @@ __global__ void __launch_bounds__(kThreads, 1) cnn_mma_kernel(CnnLaunch p) {
     p.r.trig[t.seq] = rec;
   }
   mma::cluster_sync();   // no CTA leaves while a peer may still send to it
+  if (!ok) lr::linger();
 }
 
 template <int CL, int BT>

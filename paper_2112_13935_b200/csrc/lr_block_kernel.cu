@@ -114,6 +114,9 @@ __global__ void __launch_bounds__(S::kThreads, S::kCtas) lr_block_kernel(RoundLa
     const float* xrows = reinterpret_cast<const float*>(cd.x);
     auto produce = [&](uint32_t kb) {
       const int sb = kb % kRing;
+      // (long since here, if ever: the products of block kb - kRing are done; a barrier short of its bytes is not armed again)
+      if (kb >= (uint32_t)kRing && !mbar_try_wait(&sm.full[sb], (kb / kRing - 1) & 1)) ok = false;
+      if (!__all_sync(0xffffffffu, ok)) return;
       const uint32_t nvb = min((uint32_t)kBk, n - kb * kBk);
       for (uint32_t r = nvb; r < (uint32_t)kBk; ++r)   // short last block: rows that add nothing anywhere
         for (int i = lane; i < kD / 4; i += 32) reinterpret_cast<float4*>(sm.rows[sb][r])[i] = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -154,8 +154,9 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
     for (int c = 8 * cnt; c < S::kCols; ++c) sm.rows[i / kB][i % kB][c] = 0.f;
   mma::cluster_sync();   // a peer's barriers exist before anything is sent to it
 
-  // After a wait has given up nothing waits any more: the round runs through on whatever is there, the status
-  // word is set, and every CTA of the cluster reaches the end.
+  // A thread whose wait has given up waits no more and runs through on whatever is there, but neither arms a barrier (a second arrival
+  // on one that is short of bytes would be invalid) nor sends: whoever depends on it gives up in turn, the status word is set, and
+  // every CTA of the cluster reaches the end.
   bool ok = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok) ok = mbar_wait(bar, parity); };
   auto wait_cluster = [&](uint64_t* bar, uint32_t parity) {   // for what peers sent
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
 #pragma unroll
       for (int c = 0; c < kCh; ++c) dmine[c] = live ? d[c] : 0.f;
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.delta[b]);
+      if (ok && lane == 0) mbar_arrive(&sm.delta[b]);
     }
   } else if (role == kProd) {
     // ================= producer: rows and labels =================
@@ -282,7 +283,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
     for (uint32_t kb = 0; kb < nblk; ++kb) {
       const int sb = kb % NS;
       if (kb >= (uint32_t)NS) wait(&sm.freed[sb], (kb / NS - 1) & 1);   // block kb - NS has left its slot
-      if (!ok) break;
+      if (!__all_sync(0xffffffffu, ok)) break;
       const uint32_t nvb = min((uint32_t)kB, n - kb * kB);
       for (uint32_t r = nvb; r < (uint32_t)kB; ++r)   // short last block: rows that add nothing anywhere
         for (int i = lane; i < 8 * cnt; i += 32) sm.rows[sb][r][i] = 0.f;
@@ -331,12 +332,12 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
         for (int r = 1; r < CL; ++r) v += sm.zin[iz][r][lane + 32 * i];
         sm.zsum[b][lane + 32 * i] = v;
       }
-      if (lane == 0 && k + 1 < nblk) {
+      if (ok && lane == 0 && k + 1 < nblk) {
         mbar_expect_tx(&sm.bg[(k + 1) % S::kInG], CL * kSendG);
         mbar_expect_tx(&sm.bz[(k + 1) % S::kInZ], CL * kZ * 4);
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.ready[b]);
+      if (ok && lane == 0) mbar_arrive(&sm.ready[b]);
     }
   } else if (role == kGram) {
     // ================= Gram warps; lane = 4 g + tt =================
@@ -376,7 +377,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
       }
       // with the split rows in registers a block's slot is done with here, else one block later
       __syncwarp();
-      if (lane == 0 && (S::kCarry || kb)) mbar_arrive(&sm.freed[(S::kCarry ? kb : kb - 1) % NS]);
+      if (ok && lane == 0 && (S::kCarry || kb)) mbar_arrive(&sm.freed[(S::kCarry ? kb : kb - 1) % NS]);
       float* part = sm.gpart[kb & 1][warp];
 #pragma unroll
       for (int m = 0; m < 2; ++m)
@@ -421,7 +422,8 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
         const float4 out = make_float4(v[0], v[1], v[2], v[3]);
         const uint32_t to = smem_addr(&sm.gin[ig][rank][at]), bar = smem_addr(&sm.bg[ig]);
 #pragma unroll
-        for (uint32_t r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(to, r), out, mma::peer_addr(bar, r));
+        for (uint32_t r = 0; r < CL; ++r)
+          if (ok) mma::send_peer(mma::peer_addr(to, r), out, mma::peer_addr(bar, r));
       }
     }
   } else if (role == kModel) {
@@ -593,13 +595,14 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
             }
             const uint32_t to = smem_addr(&sm.zin[iz][rank][4 * e]), bar = smem_addr(&sm.bz[iz]);
 #pragma unroll
-            for (uint32_t r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(to, r), v, mma::peer_addr(bar, r));
+            for (uint32_t r = 0; r < CL; ++r)
+              if (ok) mma::send_peer(mma::peer_addr(to, r), v, mma::peer_addr(bar, r));
           }
         }
       }
       if (update) {
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.freed[k % NS]);
+        if (ok && lane == 0) mbar_arrive(&sm.freed[k % NS]);
       }
     }
 
@@ -639,6 +642,7 @@ __global__ void __launch_bounds__(S::kThreads, 1) lr_chain_kernel(RoundLaunch p)
   }
   if (!ok && p.status && lane == 0) atomicOr(p.status, 1u);
   mma::cluster_sync();   // no CTA leaves while a peer may still send to it
+  if (!ok) linger();
   if (!ok && role == kProd)   // copies still in flight target this CTA's shared memory: a bounded chance to land
     for (int s = 0; s < NS; ++s) {
       mbar_wait_limit(&sm.full[s], 0, 1u << 16);

@@ -494,6 +494,9 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   own.ext = smem + m.o_ext + tid;
   const int ug = m.upw;   // first group of W_0's update sum
 
+  // A thread whose wait has given up waits no more and runs through on whatever is there, but neither arms a barrier (a second arrival
+  // on one that is short of bytes would be invalid) nor sends: whoever depends on it gives up in turn, the status word is set, and
+  // every CTA of the cluster reaches the end.
   bool ok = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) {
     const uint32_t at = smem_addr(bar);
@@ -769,7 +772,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           // neighbouring lanes trade pairs: the even one then has four samples of row g, the odd one of row g + 8
           const bool odd = tt & 1;
           const float r0 = __shfl_xor_sync(0xffffffffu, odd ? acc[b][0] : acc[b][2], 1), r1 = __shfl_xor_sync(0xffffffffu, odd ? acc[b][1] : acc[b][3], 1);
-          mma::send_peer(row_at + 32u * b, odd ? make_float4(r0, r1, acc[b][2], acc[b][3]) : make_float4(acc[b][0], acc[b][1], r0, r1), row_bar);
+          if (ok) mma::send_peer(row_at + 32u * b, odd ? make_float4(r0, r1, acc[b][2], acc[b][3]) : make_float4(acc[b][0], acc[b][1], r0, r1), row_bar);
         }
       }
     }
@@ -782,7 +785,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
     // ================= 2: owned rows: sum over the CTAs, bias, ReLU; A_0 (or the logits) to every CTA =================
     if (nrg > 0) {
       wait(&bars[0], it & 1);
-      if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[0], in_bytes);
+      if (ok && tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[0], in_bytes);
       // (without hidden layers these are the logits: fp32 whatever the operands.)  A lane's words are a packet to each peer, and
       // packets are what a hand-over takes its time for: 16 bytes each, four rows of a sample or eight in bf16.
       constexpr int kRows = BF ? 8 : 4;
@@ -814,19 +817,20 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
           for (int i = 0; i < 4; ++i) w[i] = pack_bf16(v[(2 * i) % kRows], v[(2 * i + 1) % kRows]);
 #pragma unroll 1
           for (int r = 0; r < CL; ++r)
-            mma::send_peer(mma::peer_addr(at, r), make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3])), mma::peer_addr(bar, r));
+            if (ok) mma::send_peer(mma::peer_addr(at, r), make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3])), mma::peer_addr(bar, r));
         } else {
 #pragma unroll
           for (int i = 0; i < kRows; i += 4) {
             const uint32_t at = smem_addr(smem + m.o_a[0] + b * m.ap[0] + n + i);
 #pragma unroll 1
-            for (int r = 0; r < CL; ++r) mma::send_peer(mma::peer_addr(at, r), make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]), mma::peer_addr(bar, r));
+            for (int r = 0; r < CL; ++r)
+              if (ok) mma::send_peer(mma::peer_addr(at, r), make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]), mma::peer_addr(bar, r));
           }
         }
       }
     }
     wait(&bars[1], it & 1);
-    if (tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[1], a_bytes);
+    if (ok && tid == 0 && it + 1 < t.steps) mbar_expect_tx(&bars[1], a_bytes);
 
     // ================= 3: narrow layers, redundantly in every CTA =================
 #pragma unroll 1
@@ -1162,6 +1166,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_mma_kernel(const __grid_const
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   if (CL > 1) mma::cluster_sync(); else __syncthreads();   // no CTA leaves while a peer may still send to it
+  if (!ok) lr::linger();
+  __syncwarp();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(*tmem_at) : "memory");
 }
 

@@ -175,8 +175,9 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
   Own own;
   own.tmem = *tmem_at + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * 128u;
 
-  // After a wait has given up nothing waits any more: the round runs through on whatever is there, the status word is
-  // set, and every CTA of the cluster reaches the end.
+  // A thread whose wait has given up waits no more and runs through on whatever is there, but neither arms a barrier (a second arrival
+  // on one that is short of bytes would be invalid) nor sends: whoever depends on it gives up in turn, the status word is set, and
+  // every CTA of the cluster reaches the end.
   bool ok = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok) ok = mbar_wait(bar, parity); };
   auto wait_cluster = [&](uint64_t* bar, uint32_t parity) {
@@ -429,12 +430,13 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
       const int s = rank < owner ? rank : rank - 1;
       const uint32_t at = mma::peer_addr(smem_addr(inbox + (s * tpc + warp % tpc) * BT * 128 + 4 * lane), owner), bar = mma::peer_addr(smem_addr(b_in), owner);
 #pragma unroll
-      for (int b = 0; b < (LOOK ? BT : 0); ++b) mma::send_peer(at + 512u * b, make_float4(acc[b][0], acc[b][1], acc[b][2], acc[b][3]), bar);
+      for (int b = 0; b < (LOOK ? BT : 0); ++b)
+        if (ok) mma::send_peer(at + 512u * b, make_float4(acc[b][0], acc[b][1], acc[b][2], acc[b][3]), bar);
       return;
     }
     if (CL > 1) {
       wait_cluster(b_in, par);
-      if (lane == 0 && warp % tpc == 0) mbar_expect_tx(b_in, in_bytes);
+      if (ok && lane == 0 && warp % tpc == 0) mbar_expect_tx(b_in, in_bytes);
     }
 #pragma unroll 1
     for (int s = 0; s < CL - 1; ++s) {
@@ -457,7 +459,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
       const bf16* s = A0 + (q >> 1) * kP0 + 16 * warp + 8 * (q & 1);
       const float4 v = *reinterpret_cast<const float4*>(s);
       for (int r = 0; r < CL; ++r)
-        if (r != rank) mma::send_peer(mma::peer_addr(smem_addr(s), r), v, mma::peer_addr(smem_addr(b_a0), r));
+        if (ok && r != rank) mma::send_peer(mma::peer_addr(smem_addr(s), r), v, mma::peer_addr(smem_addr(b_a0), r));
     }
   };
   typedef std::true_type Yes;
@@ -473,7 +475,7 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
     if (more) draw_rows(it + 1);
     if (CL > 1) {
       wait_cluster(b_a0, it & 1);
-      if (tid == 0 && more) mbar_expect_tx(b_a0, a0_bytes);
+      if (ok && tid == 0 && more) mbar_expect_tx(b_a0, a0_bytes);
     }
     __syncthreads();   // A_0 is complete, the parts of Z_0 have been read
     const bool back = !(it & 1);
@@ -746,6 +748,8 @@ __global__ void __launch_bounds__(kThreads, 1) mlp_wide_kernel(const __grid_cons
   asm volatile("cp.async.wait_all;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   if (CL > 1) mma::cluster_sync(); else __syncthreads();   // no CTA leaves while a peer may still send to it
+  if (!ok) lr::linger();
+  __syncwarp();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(*tmem_at) : "memory");
 }
 

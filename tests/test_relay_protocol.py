@@ -1,4 +1,4 @@
-"""The hand-overs inside the regression's relay kernel, checked as a protocol on the CPU with the constants of its source."""
+"""The hand-overs between the CTAs of a cluster, checked as a protocol on the CPU from the kernels' sources."""
 import os
 import re
 
@@ -68,3 +68,27 @@ def test_what_peers_sent_is_waited_for_at_cluster_scope():
     assert {bar for how, bar in waits} >= barriers | {"full", "done"}
     assert all((how == "wait_peer") == (bar in barriers) for how, bar in waits), waits
     assert "mbarrier.arrive.relaxed" not in text
+
+
+@pytest.mark.parametrize("name", ["lr_relay_kernel.cu", "lr_chain_kernel.cu", "mlp_mma_kernel.cu", "mlp_wide_kernel.cu", "cnn_mma_kernel.cu"])
+def test_who_has_given_up_arms_and_sends_nothing(name):
+    # A barrier that counts bytes must not be armed again while it is short of some, nor be sent bytes without end that nobody
+    # armed it for: inside a round's loops both happen only while no wait of the thread has given up.
+    lines = source(name).split("\n")
+    start = next(i for i, l in enumerate(lines) if "bool ok = true;" in l)
+    first = {"lr_relay_kernel.cu": 2, "lr_chain_kernel.cu": 2}.get(name, 0)    # (armed for the first time, before the loop)
+    guard = re.compile(r"if \(!?ok\b|&& ok\b")
+    seen = []
+    for i in range(start + 1, len(lines)):
+        if not re.search(r"\b(mbar_expect_tx|send1|send_peer|send_pair|send_quad)\(", lines[i]):
+            continue
+        depth, at, held = len(lines[i]) - len(lines[i].lstrip()), i, bool(guard.search(lines[i]))
+        while not held and depth > 4 and at > start:     # the lines that enclose it, innermost first, and a skip beside it
+            at -= 1
+            here = len(lines[at]) - len(lines[at].lstrip())
+            if lines[at].strip() and not lines[at].startswith("#") and here <= depth:
+                held = bool(guard.search(lines[at])) and (here < depth or "continue" in lines[at])
+                depth = here
+        seen.append((i + 1, held))
+    assert len(seen) >= 4
+    assert [held for _, held in seen].count(False) <= first, seen
