@@ -1025,8 +1025,8 @@ aet_status aet_debug_lost_copies(aet_handle* h, uint32_t client, uint32_t round,
                                  float* U_out, float* w_out, void* cuda_stream) {
   if (!h) return AET_ERR_ARG;
   if (!h->lr_fast || h->cfg.split_mode || round < h->cfg.round_base) return fail(h, AET_ERR_CONFIG, "lost copies can be played for the regression's rounds only");
-  uint32_t at_once[9] = {};
-  for (uint32_t cl = 1; cl <= 8; ++cl) AET_CUDA(h, clusters_at_once(cl, &at_once[cl]));
+  uint32_t at_once[9];
+  AET_CUDA(h, clusters_at_once(at_once));
   const LrChoice c = choose_lr_kernel(h->cfg.n_clients, sample_size(h->cfg, round), false, at_once);
   if (c.kernel != LrKernel::kRelay) return fail(h, AET_ERR_CONFIG, "lost copies can be played for few clients only");
   if (cta >= c.cluster || max_polls == 0 || max_polls > (1u << 16)) return fail(h, AET_ERR_ARG, "cta must be below the cluster's width, max_polls in [1, 2^16]");

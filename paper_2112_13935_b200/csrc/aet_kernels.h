@@ -56,6 +56,7 @@ struct RoundLaunch {
 
 // How many clusters of 1 to 8 CTAs with an SM each the current device runs at once, 0 where it runs none (see device_info.cu).
 cudaError_t clusters_at_once(uint32_t cluster, uint32_t* out);
+cudaError_t clusters_at_once(uint32_t (&out)[9]);   // all of them, [CTAs], with one question to the runtime
 
 // One CTA waits (at most max_polls polls) on a barrier nobody signals, then sets bit 0 of *status.
 cudaError_t launch_wait_probe(uint32_t* status, uint32_t max_polls, cudaStream_t s);

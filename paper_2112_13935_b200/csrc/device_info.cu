@@ -20,17 +20,12 @@ __global__ void __launch_bounds__(kThreads, 1) whole_sm_kernel(float* p) {   // 
 // [device][CTAs], one more than the answer; 0: not asked yet.  Two host threads may ask at once and store the same value.
 std::atomic<uint32_t> g_fit[kMaxDevices][9] = {};
 
-}  // namespace
-
-cudaError_t clusters_at_once(uint32_t cluster, uint32_t* out) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (cluster < 1 || cluster > 8) return cudaErrorInvalidValue;
+cudaError_t at_once_on(int dev, uint32_t cluster, uint32_t* out) {
   std::atomic<uint32_t>* known = dev >= 0 && dev < kMaxDevices ? &g_fit[dev][cluster] : nullptr;
   uint32_t n = known ? known->load(std::memory_order_relaxed) : 0;
   if (!n) {
     int v = 0;
+    cudaError_t e;
     if (cluster == 1) {
       e = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
     } else {
@@ -52,6 +47,24 @@ cudaError_t clusters_at_once(uint32_t cluster, uint32_t* out) {
     if (known) known->store(n, std::memory_order_relaxed);
   }
   *out = n - 1;
+  return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t clusters_at_once(uint32_t cluster, uint32_t* out) {
+  int dev = 0;
+  if (cluster < 1 || cluster > 8) return cudaErrorInvalidValue;
+  if (const cudaError_t e = cudaGetDevice(&dev)) return e;
+  return at_once_on(dev, cluster, out);
+}
+
+cudaError_t clusters_at_once(uint32_t (&out)[9]) {
+  int dev = 0;
+  if (const cudaError_t e = cudaGetDevice(&dev)) return e;
+  out[0] = 0;
+  for (uint32_t cl = 1; cl <= 8; ++cl)
+    if (const cudaError_t e = at_once_on(dev, cl, &out[cl])) return e;
   return cudaSuccess;
 }
 

@@ -48,9 +48,8 @@ LrChoice choose_lr_kernel(uint32_t n_tasks, uint32_t longest, bool by_value, con
 
 cudaError_t launch_lr_rounds(const RoundLaunch& p, cudaStream_t s) {
   if (p.n_tasks == 0) return cudaSuccess;
-  uint32_t at_once[9] = {};
-  for (uint32_t cl : {1u, 2u, 4u, 6u, 8u})
-    if (const cudaError_t e = clusters_at_once(cl, &at_once[cl])) return e;
+  uint32_t at_once[9];
+  if (const cudaError_t e = clusters_at_once(at_once)) return e;
   const LrChoice c = choose_lr_kernel(p.wave_tasks ? p.wave_tasks : p.n_tasks, p.longest, p.by_value != 0, at_once);
   if (c.kernel == LrKernel::kRelay) return launch_lr_relay_rounds(p, c.cluster, s);
   if (c.kernel == LrKernel::kChain) return launch_lr_chain_rounds(p, c.cluster, s);
