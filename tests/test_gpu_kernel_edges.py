@@ -35,15 +35,17 @@ def check(cfg, w_tol=2e-5, bf16=False):
 
 
 @pytest.mark.parametrize("l2", [0.0, 1e-3])
-@pytest.mark.parametrize("n_clients", [3, 33, 74, 100, 200])    # clusters of four, of two (the most of each); one CTA; two CTAs per SM
+@pytest.mark.parametrize("n_clients", [3, 33, 74, 100, 200])    # clusters of eight, four, two (the most of the last two); one CTA; two CTAs per SM
 @pytest.mark.parametrize("first", [1, 7, 15, 31])           # rounds of first, first + 1, first + 2 samples: around blocks of 8 and 16
 def test_regression_rounds_around_whole_blocks(n_clients, first, l2):
     check(workloads.get_config("cfg5", n_clients=n_clients, n_rounds=3, sched_a=1, sched_b=first, l2=l2, lr=0.002 if n_clients < 10 else 1e-4,
                                data=dict(per_client=40)))
 
 
-# Clusters of eight (up to 15 round-tasks on this part) and of six (up to 22); blocks of sixteen, rings of three and four blocks.
-@pytest.mark.parametrize("n_clients,first,l2", [(1, 16, 0.0), (15, 33, 1e-3), (16, 1, 1e-3), (16, 48, 0.0), (22, 17, 1e-3), (22, 79, 0.0)])
+# Clusters of eight (up to 15 round-tasks on this part), of six (up to 22, rounds above 64 samples) and of four (shorter ones); blocks of
+# sixteen, rings of three and four blocks.
+@pytest.mark.parametrize("n_clients,first,l2", [(1, 16, 0.0), (15, 33, 1e-3), (16, 1, 1e-3), (16, 48, 0.0), (22, 17, 1e-3), (22, 79, 0.0),
+                                                (16, 65, 1e-3), (16, 80, 0.0), (22, 81, 1e-3), (19, 128, 1e-3)])
 def test_regression_rounds_of_few_clients(n_clients, first, l2):
     check(workloads.get_config("cfg5", n_clients=n_clients, n_rounds=3, sched_a=15, sched_b=first, l2=l2, lr=0.03 / n_clients, data=dict(per_client=40)))
 
@@ -51,9 +53,10 @@ def test_regression_rounds_of_few_clients(n_clients, first, l2):
 # A step moves a sample's own logits by eta (|x|^2 + 1), 16 eta and more here: 33 samples carry corrections far beyond the exponential's
 # range, which the walk has to shift out.  The bar: one fp32 rounding (2^-24) per step, each amplified by no more than the softmax's
 # 1/2 x 16 eta per later step that shares its class.
-@pytest.mark.parametrize("n_clients,lr", [(3, 0.2), (3, 2.0), (18, 2.0)])   # (from 20 on the checker's own loss overflows)
-def test_regression_rounds_with_steps_that_swing(n_clients, lr):
-    check(workloads.get_config("cfg5", n_clients=n_clients, n_rounds=1, sched_a=1, sched_b=33, lr=lr, data=dict(per_client=40)))
+@pytest.mark.parametrize("n_clients,lr,samples", [(3, 0.2, 33), (3, 2.0, 33), (18, 2.0, 33),    # (from 20 on the checker's own loss overflows)
+                                                  (18, 0.2, 66)])                                # clusters of six
+def test_regression_rounds_with_steps_that_swing(n_clients, lr, samples):
+    check(workloads.get_config("cfg5", n_clients=n_clients, n_rounds=1, sched_a=1, sched_b=samples, lr=lr, data=dict(per_client=40)))
 
 
 def round_rms(cfg, w0, clients):
@@ -75,7 +78,8 @@ def round_rms(cfg, w0, clients):
 # 22 bits instead of 24 would show at 50 (1.5e-7).  Crowded launches (200 clients): the kernels before left 1.5e-7 at 12 samples, 1.25e-7
 # with l2; cut operands 1.6e-7 and 1.5e-7.
 @pytest.mark.parametrize("n_clients,samples,l2,bar", [
-    *[(n, s, 0.0, bar) for n in (3, 50, 100) for s, bar in ((5, 0.46e-7), (50, 0.9e-7), (600, 2.2e-7))],   # clusters of four, of two; one CTA
+    # clusters of eight, four (of six from 65 samples on), four, two; one CTA
+    *[(n, s, 0.0, bar) for n in (3, 20, 33, 50, 100) for s, bar in ((5, 0.46e-7), (50, 0.9e-7), (600, 2.2e-7))],
     (200, 12, 0.0, 1.1e-7), (200, 12, 1e-4, 1.0e-7), (200, 50, 0.0, 1.1e-7),
 ])
 def test_regression_rounds_are_as_good_as_fp32_sums(n_clients, samples, l2, bar):
