@@ -511,6 +511,7 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
     const uint32_t grank = rank - MC;
     launch_next();
     Split pv[KG][4];   // the rows of the block before, split
+    int slot = 0;      // kb mod kGramParts
     for (uint32_t kb = 0; kb < nblk; ++kb) {
       wait(&sm.full[kb % NS], (kb / NS) & 1);
       const float* xr = rows + ((kb % NS) * kB + g) * PG + 8 * warp + 2 * tt;
@@ -538,7 +539,8 @@ __global__ void __launch_bounds__(kThreads, 1) lr_relay_kernel(RoundLaunch p) {
       }
       __syncwarp();
       if (ok && lane == 0) mbar_arrive(&sm.freed[kb % NS]);
-      float* const block = gpart + (int)(kb % kGramParts) * NG * kCoup;
+      float* const block = gpart + slot * NG * kCoup;
+      slot = slot + 1 < kGramParts ? slot + 1 : 0;
       float* part = block + warp * kCoup;
 #pragma unroll
       for (int m = 0; m < 2; ++m)
