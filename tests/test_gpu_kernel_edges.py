@@ -50,6 +50,23 @@ def test_regression_rounds_of_few_clients(n_clients, first, l2):
     check(workloads.get_config("cfg5", n_clients=n_clients, n_rounds=3, sched_a=15, sched_b=first, l2=l2, lr=0.03 / n_clients, data=dict(per_client=40)))
 
 
+# Hand-overs inside the kernels on clusters: a race between the warps that add up couplings gave a few of such runs other bits.
+@pytest.mark.parametrize("over", [
+    dict(n_clients=95, n_rounds=22, sched_a=6, sched_b=28, l2=0.0), dict(n_clients=41, n_rounds=10, sched_a=7, sched_b=9, l2=1e-4),
+    dict(n_clients=44, n_rounds=51, sched_a=5, sched_b=11, l2=0.0, topology=1), dict(n_clients=16, n_rounds=32, sched_a=4, sched_b=9, l2=1e-4, topology=1),
+])
+def test_regression_runs_repeat_bit_for_bit(over):
+    cfg = workloads.get_config("cfg5", lr=0.02 / over["n_clients"], data=dict(per_client=100), **over)
+    data, w0 = make(cfg)
+    with api.Session(cfg, to_device(data), torch.from_numpy(w0).cuda()) as s:
+        seen = set()
+        for _ in range(40):
+            s.reset()
+            s.run()
+            seen.add(b"".join(api.aet_get_node_model(s.h, c).tobytes() for c in range(cfg["n_clients"])) if cfg.get("topology") else s.model().tobytes())
+    assert len(seen) == 1, len(seen)
+
+
 # A step moves a sample's own logits by eta (|x|^2 + 1), 16 eta and more here: 33 samples carry corrections far beyond the exponential's
 # range, which the walk has to shift out.  The bar: one fp32 rounding (2^-24) per step, each amplified by no more than the softmax's
 # 1/2 x 16 eta per later step that shares its class.
