@@ -25,12 +25,13 @@
 // lr_chain_kernel.cu, where the fragments are the same).  With lambda the kernel carries D = sum_s q^(n-1-s) delta_s x_s;
 // U = D + W_start (1 - q^n) / eta.
 //
-// What bounds it: R, 1,970 of 2,340 cycles a block of sixteen in rounds of hundreds of samples; in short rounds the way from one wave to the
+// What bounds it: in rounds of hundreds of samples the way from a block's deltas to the logits of the block after next (update, product, sums,
+// two hand-overs), 2,340 cycles a block of sixteen, of which R walks 1,970 and waits 370; in short rounds the way from one wave to the
 // next (from R's last step to the next wave's first 9 us: end of the round 2, server's kernel 5, start model and first logits 2).  The
 // next kernel may come up four blocks before a round's end, so that its rows and Gram matrices are ready when the model is (from then to
 // the first step 3.0 -> 1.5 us; 16 clients 1.28 -> 1.20 ms, ring 6.22 -> 6.12).
-// Measured against four CTAs that did everything alike: 5 clients for 110 rounds on the ring 8.27 -> 6.12 ms, 16 skewed clients
-// 1.39 -> 1.20 ms, 4 clients with l2 92 -> 82 us, one round of 50 samples 13.1 -> 10.9 us.
+// Measured against four CTAs that did everything alike: 5 clients for 110 rounds on the ring 8.27 -> 6.17 ms, 16 skewed clients
+// 1.39 -> 1.22 ms, 4 clients with l2 92 -> 83 us, one round of 50 samples 13.4 -> 11.3 us.
 #include <cuda_runtime.h>
 
 #include <atomic>
